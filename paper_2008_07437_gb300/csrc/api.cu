@@ -31,6 +31,7 @@ struct geo_ctx {
     DevStatus *st = nullptr;
     DevResults *res = nullptr;
     int *sync = nullptr;          // 4 ints: sync words of the one-launch triangular solves
+    int *csync = nullptr;         // GEO_CHOL_SYNC_INTS ints: sync words of the one-launch factorisations
     DevStatus *h_st = nullptr;    // pinned
     DevResults *h_res = nullptr;  // pinned
     // reusable workspace for the matrix of a discarded evaluation
@@ -431,6 +432,7 @@ int geo_create(geo_ctx **out, int device, size_t hbm_budget_bytes) {
     if (cudaMalloc(&ctx->st, sizeof(DevStatus)) != cudaSuccess ||
         cudaMalloc(&ctx->res, sizeof(DevResults)) != cudaSuccess ||
         cudaMalloc(&ctx->sync, 4 * sizeof(int)) != cudaSuccess ||
+        cudaMalloc(&ctx->csync, GEO_CHOL_SYNC_INTS * sizeof(int)) != cudaSuccess ||
         cudaMallocHost(&ctx->h_st, sizeof(DevStatus)) != cudaSuccess ||
         cudaMallocHost(&ctx->h_res, sizeof(DevResults)) != cudaSuccess ||
         cudaMalloc(&ctx->prof.d_tc_flops, sizeof(unsigned long long)) != cudaSuccess ||
@@ -469,6 +471,7 @@ int geo_destroy(geo_ctx *ctx) {
     if (ctx->st) cudaFree(ctx->st);
     if (ctx->res) cudaFree(ctx->res);
     if (ctx->sync) cudaFree(ctx->sync);
+    if (ctx->csync) cudaFree(ctx->csync);
     if (ctx->h_st) cudaFreeHost(ctx->h_st);
     if (ctx->h_res) cudaFreeHost(ctx->h_res);
     delete ctx;
@@ -521,13 +524,13 @@ static int dense_factor(geo_ctx *ctx, double *A, long long ld, int N, int nrows,
                         cudaError_t *err) {
     *err = cudaSuccess;
     if (o.fp64_gemm != 1) {
-        *err = chol64_factor(A, ld, N, nrows, o.nb, ctx->st, s);
+        *err = chol64_factor(A, ld, N, nrows, ctx->st, ctx->csync, s);
         return GEO_OK;
     }
     const int S = oz_slices_of(o);
     int rc = ensure_buffer(ctx, &ctx->ows, &ctx->ows_bytes, oz_chol_workspace_bytes(nrows, o.nb, S), s);
     if (rc) return rc;
-    *err = chol_oz_factor(A, ld, N, nrows, o.nb, S, o.oz_cut, ctx->ows, ctx->ows_bytes, ctx->st, s);
+    *err = chol_oz_factor(A, ld, N, nrows, o.nb, S, o.oz_cut, ctx->ows, ctx->ows_bytes, ctx->st, ctx->csync, s);
     return GEO_OK;
 }
 
@@ -690,7 +693,8 @@ static int loglik_tlr(geo_ctx *ctx, const double *locs_dev, int n, const double 
     cudaError_t e;
     if ((e = cudaMemcpyAsync(d_perm, f->perm.data(), sizeof(int) * n, cudaMemcpyHostToDevice, s)) ||
         (e = launch_gather_vec(z_dev, d_perm, n, p, f->ybuf, 1, s)) ||
-        (e = tlr_factor(*F, f->cp, f->lx, f->ly, ctx->tws, ctx->tws_bytes, ctx->tarena, ctx->st, ctx->h_st, s))) {
+        (e = tlr_factor(*F, f->cp, f->lx, f->ly, ctx->tws, ctx->tws_bytes, ctx->tarena, ctx->st, ctx->csync,
+                        ctx->h_st, s))) {
         cudaStreamSynchronize(s);
         dev_free(ctx, d_perm, sizeof(int) * n);
         if (e == cudaErrorMemoryAllocation)
@@ -700,6 +704,7 @@ static int loglik_tlr(geo_ctx *ctx, const double *locs_dev, int n, const double 
     CK(cudaMemcpyAsync(ctx->h_st, ctx->st, sizeof(DevStatus), cudaMemcpyDeviceToHost, s));
     CK(cudaStreamSynchronize(s));
     dev_free(ctx, d_perm, sizeof(int) * n);
+    if (ctx->h_st->timeout) return bail(fail(ctx, GEO_ETIMEOUT, "a bounded device wait expired"));
     if (ctx->h_st->info) {
         if (info) *info = ctx->h_st->info;
         if (loglik_host) *loglik_host = nan("");
@@ -804,7 +809,7 @@ int geo_loglik(geo_ctx *ctx, const double *locs_dev, int n, const double *z_dev,
         (refine && (e = cudaMemcpyAsync(Scopy, f->A, sizeof(double) * (size_t)f->ld * (size_t)N,
                                         cudaMemcpyDeviceToDevice, s))) ||
         (e = mixed ? chol_mixed_factor(f->A, f->ld, N, N + 1, o.nb, o.band, o.lowp, ctx->mws, ctx->mws_bytes,
-                                       ctx->st, s)
+                                       ctx->st, ctx->csync, s)
                    : (dense_factor(ctx, f->A, f->ld, N, N + 1, o, s, &e_fac), e_fac)) ||
         (e = refine ? refine_solve(Scopy, f->A, f->ld, N, zsorted, f->A + N, f->ld, o.refine_iters, f->w, ctx->rws,
                                    ctx->st, ctx->res, s)
@@ -818,6 +823,12 @@ int geo_loglik(geo_ctx *ctx, const double *locs_dev, int n, const double *z_dev,
         return cuda_fail(ctx, e, "geo_loglik");
     }
     dev_free(ctx, d_perm, sizeof(int) * n);
+    if (ctx->h_st->timeout) {
+        if (loglik_host) *loglik_host = nan("");
+        release_factor_buffers(ctx, f, true);
+        delete f;
+        return fail(ctx, GEO_ETIMEOUT, "a bounded device wait expired");
+    }
     if (ctx->h_st->info) {
         if (info) *info = ctx->h_st->info;
         if (loglik_host) *loglik_host = nan("");
@@ -1075,7 +1086,8 @@ int geo_simulate(geo_ctx *ctx, const double *locs_dev, int n, const double *e_de
         release_factor_buffers(ctx, &f, true);
         return rc;
     }
-    if ((e = mixed ? chol_mixed_factor(f.A, f.ld, N, N, o.nb, o.band, o.lowp, ctx->mws, ctx->mws_bytes, ctx->st, s)
+    if ((e = mixed ? chol_mixed_factor(f.A, f.ld, N, N, o.nb, o.band, o.lowp, ctx->mws, ctx->mws_bytes, ctx->st,
+                                       ctx->csync, s)
                    : e_fac) ||
         (e = launch_trmv_lower(f.A, f.ld, N, e_dev, zs, s)) ||
         (e = cudaMemcpyAsync(d_perm, f.perm.data(), sizeof(int) * n, cudaMemcpyHostToDevice, s)) ||
@@ -1088,6 +1100,7 @@ int geo_simulate(geo_ctx *ctx, const double *locs_dev, int n, const double *e_de
     dev_free(ctx, d_perm, sizeof(int) * n);
     release_factor_buffers(ctx, &f, true);
     if (rc) return rc;
+    if (ctx->h_st->timeout) return fail(ctx, GEO_ETIMEOUT, "a bounded device wait expired");
     if (ctx->h_st->info) {
         if (info) *info = ctx->h_st->info;
         return fail(ctx, GEO_ENOTSPD, "Sigma(theta) is not positive definite");

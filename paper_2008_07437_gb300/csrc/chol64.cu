@@ -1,26 +1,105 @@
 // Dense FP64 tiled Cholesky, Sigma = L L' (Sec. 5.2; the tile algorithm of
 // Sec. 5.1 / Fig. 1 / Fig. 2: POTRF on the diagonal tile, TRSM on the panel,
-// SYRK / GEMM on the trailing matrix).
+// SYRK / GEMM on the trailing matrix), as one data-flow launch.
 //
-// On GB300 the FP64 pipe runs at about 1.2 TFLOP/s (roughly two FP64 FMAs per
-// clock per SM), some 60x below the FP32 pipe, so the dense FP64 path is
-// bound by FP64 issue, not by memory: a rank-nb update reads 16 bytes per
-// 2*nb flops.  The schedule is a right-looking blocked factorisation in
-// stream order with two levels:
-//   outer tiles of width nb (the tile size of the options): after the panel
-//     of tile column k is factored, ONE launch updates the whole trailing
-//     lower triangle (the SYRK and GEMM tasks of step k fused, rank nb);
-//   inner blocks of width IB = 64 inside the panel: a one-CTA POTRF of the
-//     64 x 64 diagonal block, a TRSM of every row below it, and a rank-64
-//     update of the rest of the panel.
-// Rows N .. nrows-1 are extra right-hand-side rows: they take part in every
-// TRSM and update, so row N ends up holding (L^-1 z)' when it starts as z'
-// (the forward substitution of Eq. 1 comes out of the factorisation).
+// On GB300 the FP64 pipe runs at about 1.2 TFLOP/s (two FP64 FMAs per clock
+// per SM, a warp-wide FMA every 16 clocks), some 60x below the FP32 pipe.  So
+// memory never sets the pace -- a 32 x 32 output tile reads 16 bytes per 32
+// FMAs, one byte per clock and SM -- and tiles can be small, which is what the
+// latency of the column chain asks for: a 64-wide diagonal block costs one SM
+// at least 11 us of FP64 issue, the 64 x 64 solve below it 32 us, while the
+// 32-wide ones take 4 and 4.
+//
+// The matrix is cut into 32 x 32 tiles.  Groups of 128 threads (four to a CTA,
+// one CTA per SM) take tiles from a ticket counter, column by column, and do
+// everything for a tile at once, left-looking: C_ic = A_ic - sum_k L_ik L_ck'
+// in registers over the finished tiles k < c of the two tile rows, then the
+// Cholesky factor of the 32 x 32 block (i = c, one warp, a row per lane in
+// registers) or the solve with L_cc' (i > c, one warp, a row per lane).  Every
+// tile is written once.  A progress word per tile row counts its finished
+// tiles; a group waits on the words of its two rows, so tiles of later columns
+// accumulate while the column chain runs (lookahead without streams).  A group
+// only waits for tiles whose tickets were taken earlier by groups that are
+// running, so the launch cannot deadlock whatever the number of resident CTAs.
+// Every wait is bounded: past DF_WAIT_CYCLES without progress the waiter
+// raises the abort word, records the timeout and all groups return; a failed
+// pivot raises the same word.  Sums run in a fixed order: results do not
+// depend on timing.
+//
+// Rows N .. nrows-1 are extra right-hand-side rows: tiles of their own that
+// take part in every product and solve, so row N ends up holding (L^-1 z)'
+// when it starts as z' (the forward substitution of Eq. 1 comes out of the
+// factorisation).  The inverse of a diagonal tile (for the emulated form's
+// panel solves) is the solve of identity rows carried along the same way.
+//
+// Bounds: small orders by the column chain (34 us per 32 columns: 12.5 the
+// block's factorisation, 6.3 the solve below it, 6.6 the product, the rest
+// memory and flags), large ones by the FP64 pipe.  Measured, against one
+// launch per step of a 64-wide blocked algorithm (POTRF in one CTA 97 us, TRSM
+// 65, rank-64 update 100 and more): N = 800 0.84 ms (3.5), N = 8,002 141.5 ms
+// = 0.96 of the pipe (172), a 512-column diagonal tile with its inverse beside
+// other work 0.55 ms (1.6), 24 tiles of 256 in the mixed form 10 ms (24).
+// Four groups of 128 threads share a CTA because one CTA per SM keeps the
+// SMs of a concurrent persistent kernel free, and 128 threads reach all four
+// FP64 units of an SM with eight entries each.
+#include <algorithm>
+
 #include "geo_internal.cuh"
 
 namespace {
 
-constexpr int IB = 64;
+constexpr int DT = 32;                 // tile edge
+constexpr int DG = 128;                // threads per group
+constexpr int DF_GROUPS = 4;           // groups per CTA: with one CTA per SM they fill the registers
+constexpr int DF_THREADS = DG * DF_GROUPS;
+constexpr int DLD = DT + 1;            // operand tiles: conflict-free along rows and columns
+constexpr int DLL = DT + 2;            // the solve's copy of L_cc: 16-byte pairs
+constexpr long long DF_WAIT_CYCLES = 4000000000LL;   // ~2 s at 2 GHz
+
+// Order (GEO_CHOL_STRAIGHT, GEO_CHOL_BLOCK64) of a tile's sum A_ic - sum_k L_ik L_ck' over the columns k of the panel: straight through, one FMA
+// after the other from A_ic on; or a separate sum per 64 columns, subtracted as a whole, and straight through
+// within the 64 columns the tile belongs to.  The second is the order of a factorisation in 64-wide steps with
+// a rank-64 update after each.  The forms with less than FP64 behind their far tiles use it: they round the
+// factor's entries to 35 bits or FP32, which turns a last-bit difference here into one of up to 1e-7 in l, so
+// their results stay what that order gives.
+struct DfSmem {
+    double As[DT][DLD], Bs[DT][DLD];   // operand tiles [k][row]; Bs then holds the tile itself, [col][row]
+    double Ls[DT][DLL];                // L_cc, [col][row]; the factorisation's exchange buffer
+    double dinv[DT];                   // 1 / diagonal of L_cc
+    int word[4];
+};
+
+struct DfArgs {
+    double *A;
+    long long ld;
+    int j0, jb;       // columns of the panel (the diagonal tile's rows are the same range)
+    int x0, x1;       // extra rows
+    int T, E;         // 32-wide column tiles; tiles of extra rows
+    int factor;       // 0: the diagonal range already holds L, only the extra rows are solved
+    double *W;        // not null: W = -L^-1 of the diagonal range (column-major, ldw, zeros above the diagonal)
+    long long ldw;
+    int *sync;        // {ticket, abort, progress words: T + E (+ T with W), with chain: ready words 2 T}
+    int tickets;
+    int chain;        // 1: one group runs the column chain (df_chain)
+    int alone;        // chain: the other groups of its CTA leave it the SM
+    int block64;      // GEO_CHOL_BLOCK64: sums per 64 columns
+    int plain;        // GEO_CHOL_BLOCK64 and GEO_CHOL_PLAIN: pivots and solves as the plain algorithm rounds them
+    DevStatus *st;
+};
+
+__device__ __forceinline__ int df_ld_acquire(const int *p) {
+    int v;
+    asm volatile("ld.acquire.gpu.global.s32 %0, [%1];\n" : "=r"(v) : "l"(p) : "memory");
+    return v;
+}
+
+// (after a barrier: releases what the whole group wrote)
+__device__ __forceinline__ void df_st_release(int *p, int v) {
+    asm volatile("st.release.gpu.global.s32 [%0], %1;\n" ::"l"(p), "r"(v) : "memory");
+}
+
+// Barrier of one group (named barriers 1 .. DF_GROUPS).
+__device__ __forceinline__ void df_sync(int grp) { asm volatile("bar.sync %0, %1;" ::"r"(grp + 1), "n"(DG) : "memory"); }
 
 __device__ __forceinline__ void set_info(DevStatus *st, int row1) {
     // keep the smallest failing row
@@ -32,231 +111,629 @@ __device__ __forceinline__ void set_info(DevStatus *st, int row1) {
     }
 }
 
-// ---- POTRF of one diagonal block (cb <= IB) in shared memory -------------
-// Right-looking, two barriers per column: the rows below the pivot are scaled
-// by 1 / L_jj, then the rank-1 update runs with thread (row r, group g)
-// updating columns j + 1 + g, j + 5 + g, ...; the thread that updates the next
-// diagonal entry (the only one to touch it) takes its square root and
-// reciprocal right after its columns, so the pivot is ready at the next barrier.  The FP64
-// pipe (two FMAs per clock per SM) bounds the block at cb^3 / 6 FMAs; square
-// roots and divisions are taken once per column, not per thread.
-__global__ void __launch_bounds__(256) k_potrf_diag(double *A, long long ld, int c0, int cb, DevStatus *st) {
-    __shared__ double S[IB][IB + 1];   // S[col][row]: the block's Schur complement, then L
-    __shared__ double sinv;            // 1 / L_jj of the current column
-    __shared__ int fail;
-    if (st->info) return;
-    for (int t = threadIdx.x; t < cb * cb; t += blockDim.x) {
-        const int c = t / cb, r = t % cb;
-        S[c][r] = (r >= c) ? A[(long long)(c0 + c) * ld + c0 + r] : 0.0;
-    }
-    if (threadIdx.x == 0) fail = 0;
-    __syncthreads();
-    const int r = threadIdx.x % IB, g = threadIdx.x / IB;   // 4 column groups of 64 row threads
-    auto pivot = [&](int j) {
-        const double d = S[j][j];
-        if (!(d > 0.0)) {
-            fail = 1;
-            set_info(st, c0 + j + 1);
-        } else {
-            const double l = sqrt(d);
-            S[j][j] = l;
-            sinv = 1.0 / l;
+// Wait until min(*p, *q) >= need (one thread).  Returns that minimum, or -1 when the launch was aborted.
+__device__ int df_wait(const int *p, const int *q, int need, int *sync, int *timeout_word) {
+    long long t0 = clock64();
+    int last = -1;
+    for (;;) {
+        int v = df_ld_acquire(p);
+        if (q != p) v = min(v, df_ld_acquire(q));
+        if (v >= need) return v;
+        if (df_ld_acquire(&sync[1])) return -1;
+        if (v != last) {
+            last = v;
+            t0 = clock64();
+        } else if (clock64() - t0 > DF_WAIT_CYCLES) {
+            atomicExch(&sync[1], 1);
+            atomicCAS(timeout_word, 0, 8);
+            return -1;
         }
-    };
-    if (threadIdx.x == 0) pivot(0);
-    __syncthreads();
-    for (int j = 0; j < cb; ++j) {
-        if (fail) return;   // read after a barrier: uniform
-        if (g == 0 && r > j && r < cb) S[j][r] *= sinv;
-        __syncthreads();
-        for (int c = j + 1 + g; c < cb; c += 4)
-            if (r >= c && r < cb) S[c][r] -= S[j][r] * S[j][c];
-        if (g == 0 && r == j + 1 && r < cb) pivot(j + 1);
-        __syncthreads();
-    }
-    for (int t = threadIdx.x; t < cb * cb; t += blockDim.x) {
-        const int c = t / cb, r2 = t % cb;
-        if (r2 >= c) A[(long long)(c0 + c) * ld + c0 + r2] = S[c][r2];
+        __nanosleep(20);
     }
 }
 
-// ---- TRSM: X <- X L^-T for the rows r0 .. r1-1, columns c0 .. c0+cb-1 ----
-// L = A[c0:c0+cb, c0:c0+cb] (lower).  One CTA per 64 rows.
-constexpr int TRSM_ROWS = 64;
-
-__global__ void __launch_bounds__(256) k_trsm_rlt(double *A, long long ld, int c0, int cb, int r0, int r1,
-                                                 const DevStatus *st) {
-    extern __shared__ double smem[];
-    double *Ls = smem;                       // Ls[c * IB + r]
-    double *Xs = smem + IB * IB;             // Xs[c * (TRSM_ROWS + 1) + row]
-    const int XLD = TRSM_ROWS + 1;
-    if (st->info) return;
-    const int rbase = r0 + blockIdx.x * TRSM_ROWS;
-    const int nr = min(TRSM_ROWS, r1 - rbase);
-    if (nr <= 0) return;
-    for (int t = threadIdx.x; t < cb * cb; t += blockDim.x) {
-        const int c = t / cb, r = t % cb;
-        Ls[c * IB + r] = (r >= c) ? A[(long long)(c0 + c) * ld + c0 + r] : 0.0;
-    }
-    for (int t = threadIdx.x; t < cb * TRSM_ROWS; t += blockDim.x) {
-        const int c = t / TRSM_ROWS, r = t % TRSM_ROWS;
-        Xs[c * XLD + r] = (r < nr) ? A[(long long)(c0 + c) * ld + rbase + r] : 0.0;
-    }
-    __shared__ double dinv[IB];   // 1 / L_cc, one division per column
-    __syncthreads();
-    if (threadIdx.x < cb) dinv[threadIdx.x] = 1.0 / Ls[threadIdx.x * IB + threadIdx.x];
-    __syncthreads();
-    const int row = threadIdx.x % TRSM_ROWS, grp = threadIdx.x / TRSM_ROWS;   // 4 column groups
-    for (int c = 0; c < cb; ++c) {
-        if (grp == 0) Xs[c * XLD + row] *= dinv[c];
-        __syncthreads();
-        const double xc = Xs[c * XLD + row];
-        for (int k = c + 1 + grp; k < cb; k += 4) Xs[k * XLD + row] -= xc * Ls[c * IB + k];
-        __syncthreads();
-    }
-    for (int t = threadIdx.x; t < cb * TRSM_ROWS; t += blockDim.x) {
-        const int c = t / TRSM_ROWS, r = t % TRSM_ROWS;
-        if (r < nr) A[(long long)(c0 + c) * ld + rbase + r] = Xs[c * XLD + r];
-    }
+// Half of a normal number well above the smallest one, off the FP64 pipe.
+__device__ __forceinline__ double df_half(double x) {
+    return __hiloint2double(__double2hiint(x) - (1 << 20), __double2loint(x));
 }
 
-// ---- GEMM update: C -= A B' (FP64 FMA) -----------------------------------
-// C = A[rC + i, cC + j] for i < m, j < n; A-operand rows rC.., cols kA..kA+k;
-// B-operand rows cC.., same cols.  All inside the one matrix (column-major).
-// CTA tiles that lie entirely above the diagonal (global row < global col
-// everywhere) are skipped: those entries are never read.
-constexpr int GT = 64, GK = 16;
+// d > 0 (false for a NaN), off the FP64 pipe.
+__device__ __forceinline__ bool df_positive(double d) {
+    const long long b = __double_as_longlong(d);
+    return b > 0 && b <= 0x7FF0000000000000LL;
+}
 
-__global__ void __launch_bounds__(256) k_dgemm_update(double *A, long long ld, int rC, int cC, int m, int n, int kA,
-                                                      int k, const DevStatus *st) {
-    __shared__ double As[GK][GT + 2];
-    __shared__ double Bs[GK][GT + 2];
-    if (st->info) return;
-    const int tm = blockIdx.x * GT, tn = blockIdx.y * GT;
-    if (rC + tm + GT - 1 < cC + tn) return;   // fully above the diagonal
-    const int tx = threadIdx.x % 16, ty = threadIdx.x / 16;
-    double acc[4][4];
+// l = sqrt(d) and inv = 1 / l for a positive normal d, both as IEEE rounding gives them (the residuals of the
+// last steps are exact FMAs): the hardware's approximation of 1 / sqrt(d) (about 22 bits), one Newton step for
+// the root and its reciprocal, and a correction of each.  A chain of seven dependent FP64 operations where
+// sqrt() and a division take some twenty.
+__device__ __forceinline__ void df_root(double d, double *l, double *inv) {
+    double y0;
+    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y0) : "d"(d));
+    const double t = d * y0, e = fma(-t, df_half(y0), 0.5);   // (1 - d y0^2) / 2
+    const double r = fma(t, e, t), y = fma(y0, e, y0);
+    const double root = fma(fma(-r, r, d), df_half(y), r);
+    *l = root;
+    *inv = fma(fma(-root, y, 1.0), y, y);
+}
+
+// Cholesky factor of the 32 x 32 block S[col][row] (lower part) by one group, lane = row, columns w, w + 4, ...
+// in the registers of warp w.  Returns the first column without a positive pivot, or 32.  Panels of four
+// columns: the warps exchange the panel through shared memory (one barrier), then every warp factors it for
+// itself, so that no barrier or shared-memory round trip stands between its pivots, and applies it to its own
+// columns, the next panel's first.  A dependent FP64 operation takes 66 clocks and every warp-wide one occupies
+// its scheduler's FP64 unit for 64: one warp alone needs 38 us for the block, this 19.
+// dinv receives the reciprocals of the factor's diagonal.  Pivots, roots and products are those of the plain
+// right-looking algorithm, bit for bit (GEO_CHOL_BLOCK64).
+__device__ __forceinline__ int df_potrf32_plain(double (*S)[DLD], double (*buf)[4][DT], double *dinv, int grp, int tid) {
+    const int lane = tid & 31, w = tid >> 5;
+    double v[8], p[4] = {0.0, 0.0, 0.0, 0.0};
 #pragma unroll
-    for (int i = 0; i < 4; ++i)
+    for (int q = 0; q < 8; ++q) v[q] = S[4 * q + w][lane];
+    int bad = DT;
 #pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] = 0.0;
-    const double *Ap = A + (long long)kA * ld + rC + tm;
-    const double *Bp = A + (long long)kA * ld + cC + tn;
-    for (int k0 = 0; k0 < k; k0 += GK) {
-        for (int t = threadIdx.x; t < GK * GT; t += 256) {
-            const int kk = t / GT, r = t % GT;
-            const bool kin = (k0 + kk) < k;
-            As[kk][r] = (kin && tm + r < m) ? Ap[(long long)(k0 + kk) * ld + r] : 0.0;
-            Bs[kk][r] = (kin && tn + r < n) ? Bp[(long long)(k0 + kk) * ld + r] : 0.0;
+    for (int P = 0; P < 8; ++P) {
+        buf[P & 1][w][lane] = v[P];
+        df_sync(grp);
+        if (P > 0) {   // the previous panel on this warp's columns beyond this panel
+#pragma unroll
+            for (int q = P + 1; q < 8; ++q)
+#pragma unroll
+                for (int i = 0; i < 4; ++i) v[q] = fma(-p[i], S[4 * (P - 1) + i][4 * q + w], v[q]);
         }
-        __syncthreads();
 #pragma unroll
-        for (int kk = 0; kk < GK; ++kk) {
-            double a[4], b[4];
-#pragma unroll
-            for (int i = 0; i < 4; ++i) a[i] = As[kk][ty + 16 * i];
-#pragma unroll
-            for (int j = 0; j < 4; ++j) b[j] = Bs[kk][tx + 16 * j];
-#pragma unroll
-            for (int i = 0; i < 4; ++i)
-#pragma unroll
-                for (int j = 0; j < 4; ++j) acc[i][j] = fma(a[i], b[j], acc[i][j]);
-        }
-        __syncthreads();
-    }
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-        const int c = tn + tx + 16 * j;
-        if (c >= n) continue;
-        double *col = A + (long long)(cC + c) * ld + rC + tm;
+        for (int i = 0; i < 4; ++i) p[i] = buf[P & 1][i][lane];
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
-            const int r = ty + 16 * i;
-            if (tm + r < m) col[r] -= acc[i][j];
+            const int j = 4 * P + i;
+            const double d = __shfl_sync(0xffffffffu, p[i], j);
+            if (!df_positive(d) && bad == DT) bad = j;
+            double l, inv;
+            df_root(d, &l, &inv);
+            p[i] = lane == j ? l : p[i] * inv;
+            if (tid == j) dinv[j] = inv;
+#pragma unroll
+            for (int i2 = i + 1; i2 < 4; ++i2) p[i2] = fma(-p[i], __shfl_sync(0xffffffffu, p[i], 4 * P + i2), p[i2]);
+        }
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            if (w == i) S[4 * P + i][lane] = p[i];
+            if (P < 7) v[(P + 1) % 8] = fma(-p[i], __shfl_sync(0xffffffffu, p[i], (4 * P + 4 + w) & 31), v[(P + 1) % 8]);
+        }
+    }
+    return bad;
+}
+
+// The same as L D L' first: the columns stay unscaled (u = l times the pivot's root) and are applied as
+// (u / d) u', so that between two pivots stand a reciprocal approximation and four dependent FP64 operations
+// instead of seven and a product; the 32 roots are taken together at the end, one per lane (12.5 us for the block).
+__device__ __forceinline__ int df_potrf32(double (*S)[DLD], double (*buf)[4][DT], double *dinv, int grp, int tid) {
+    const int lane = tid & 31, w = tid >> 5;
+    double v[8], p[4] = {0.0, 0.0, 0.0, 0.0}, m[4] = {0.0, 0.0, 0.0, 0.0};
+#pragma unroll
+    for (int q = 0; q < 8; ++q) v[q] = S[4 * q + w][lane];
+#pragma unroll
+    for (int P = 0; P < 8; ++P) {
+        buf[P & 1][w][lane] = v[P];
+        df_sync(grp);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) p[i] = buf[P & 1][i][lane];
+        double f[4];   // this panel's multipliers
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const double d = __shfl_sync(0xffffffffu, p[i], 4 * P + i);
+            double r0;
+            asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r0) : "d"(d));
+            const double e = fma(-d, r0, 1.0), f0 = p[i] * r0;
+            f[i] = fma(f0, fma(e, e, e), f0);   // u / d: the approximation's error e to the third order
+#pragma unroll
+            for (int i2 = i + 1; i2 < 4; ++i2) p[i2] = fma(-f[i], __shfl_sync(0xffffffffu, p[i], 4 * P + i2), p[i2]);
+            // the previous panel on this warp's columns beyond this one, in the chain's gaps
+            if (P > 0)
+#pragma unroll
+                for (int q = P + 1; q < 8; ++q) v[q] = fma(-m[i], S[4 * (P - 1) + i][4 * q + w], v[q]);
+        }
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            m[i] = f[i];
+            if (w == i) S[4 * P + i][lane] = p[i];
+            if (P < 7) v[(P + 1) % 8] = fma(-m[i], __shfl_sync(0xffffffffu, p[i], (4 * P + 4 + w) & 31), v[(P + 1) % 8]);
+        }
+    }
+    df_sync(grp);
+    // the roots and their reciprocals, in every warp for itself
+    const double d = S[lane][lane];
+    const unsigned ok = __ballot_sync(0xffffffffu, df_positive(d));
+    double l, inv;
+    df_root(d, &l, &inv);
+    if (w == 0) dinv[lane] = inv;
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+        const int col = 4 * q + w;
+        const double iv = __shfl_sync(0xffffffffu, inv, col);
+        v[q] = lane == col ? l : S[col][lane] * iv;
+    }
+    df_sync(grp);   // every warp has read the diagonal
+#pragma unroll
+    for (int q = 0; q < 8; ++q) S[4 * q + w][lane] = v[q];
+    return ok == 0xffffffffu ? DT : __ffs(~ok) - 1;
+}
+
+// X <- X L^-T for the 32 x 32 tiles X[col][row] and L[col][row] by one group: warp w takes rows 8 w .. 8 w + 7,
+// lane = row + 8 g holds the columns g, g + 4, ... of its row; x_m goes from its lane to the row's four lanes
+// by shuffle, so the warps never wait for one another.  dinv: 1 / L_mm.
+__device__ __forceinline__ void df_trsm32(double (*X)[DLD], const double (*L)[DLL], const double *dinv, int tid) {
+    const int lane = tid & 31, g = lane >> 3, row = 8 * (tid >> 5) + (lane & 7);
+    double x[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) x[i] = X[4 * i + g][row];
+#pragma unroll
+    for (int m = 0; m < DT; ++m) {
+        const int im = m / 4, gm = m % 4;
+        const double xm = __shfl_sync(0xffffffffu, x[im] * dinv[m], (lane & 7) + 8 * gm);
+        if (g == gm) X[m][row] = xm;
+#pragma unroll
+        for (int i = im; i < 8; ++i) {
+            if (i == im && gm == 3) continue;
+            const double y = fma(-xm, L[m][4 * i + g], x[i]);
+            x[i] = (i == im && g <= gm) ? x[i] : y;
         }
     }
 }
 
-cudaError_t gemm_update(double *A, long long ld, int rC, int cC, int m, int n, int kA, int k, DevStatus *st,
-                        cudaStream_t s) {
-    if (m <= 0 || n <= 0 || k <= 0) return cudaSuccess;
-    dim3 grid((m + GT - 1) / GT, (n + GT - 1) / GT);
-    // algorithmic work: the lower-triangle entries of C (rC == cC here), 2k flops each
-    const double nn = n, mm = m;
-    const double entries = (rC == cC) ? (nn * mm - nn * (nn - 1.0) / 2.0) : nn * mm;
-    KScope ks(GEO_K_GEMM, s, 2.0 * k * entries, 8.0 * (2.0 * entries + (mm + nn) * k));
-    k_dgemm_update<<<grid, 256, 0, s>>>(A, ld, rC, cC, m, n, kA, k, st);
+// The same with the scaled factor H[m][k] = L_km / L_mm in place of L: the unscaled x_m goes out as it is (one
+// dependent operation per column instead of two), and the row is scaled once at the end.
+__device__ __forceinline__ void df_trsm32_scaled(double (*X)[DLD], const double (*H)[DLL], const double *dinv, int tid) {
+    const int lane = tid & 31, g = lane >> 3, row = 8 * (tid >> 5) + (lane & 7);
+    double x[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) x[i] = X[4 * i + g][row];
+#pragma unroll
+    for (int m = 0; m < DT; ++m) {
+        const int im = m / 4, gm = m % 4;
+        const double xm = __shfl_sync(0xffffffffu, x[im], (lane & 7) + 8 * gm);
+#pragma unroll
+        for (int i = im; i < 8; ++i) {
+            if (i == im && gm == 3) continue;
+            const double y = fma(-xm, H[m][4 * i + g], x[i]);
+            x[i] = (i == im && g <= gm) ? x[i] : y;
+        }
+    }
+#pragma unroll
+    for (int i = 0; i < 8; ++i) X[4 * i + g][row] = x[i] * dinv[4 * i + g];
+}
+
+// Products of a 32-deep slice, acc += A-tile times B-tile': rows ty + 8 i, columns tx + 16 j.
+template <int IM>
+__device__ __forceinline__ void df_mma(double (&acc)[8], const double (*As)[DLD], const double (*Bs)[DLD], int tx,
+                                       int ty) {
+#pragma unroll 8
+    for (int kk = 0; kk < DT; ++kk) {
+        double a[IM], b[2];
+#pragma unroll
+        for (int i = 0; i < IM; ++i) a[i] = As[kk][ty + 8 * i];
+#pragma unroll
+        for (int j = 0; j < 2; ++j) b[j] = Bs[kk][tx + 16 * j];
+#pragma unroll
+        for (int i = 0; i < IM; ++i)
+#pragma unroll
+            for (int j = 0; j < 2; ++j) acc[2 * i + j] = fma(a[i], b[j], acc[2 * i + j]);
+    }
+}
+
+// The same for a diagonal tile, of which only the ten 8 x 8 blocks at or below the diagonal are formed: five
+// entries a thread instead of eight.
+__device__ __forceinline__ void df_mma_diag(double (&acc)[8], const double (*As)[DLD], const int (&dr)[5],
+                                            const int (&dc)[5]) {
+#pragma unroll 8
+    for (int kk = 0; kk < DT; ++kk)
+#pragma unroll
+        for (int i = 0; i < 5; ++i) acc[i] = fma(As[kk][dr[i]], As[kk][dc[i]], acc[i]);
+}
+
+// The column chain, by one group: for every column c the last product of the diagonal tile (with L_c,c-1, which
+// this group has just solved and still holds), its factorisation, and the solve of the tile below it.  Handing
+// these three from group to group costs two trips through L2 (3.5 us each) per 32 columns; the other groups
+// bring the two tiles up to date with the columns before and say so in the ready words.
+template <bool PLAIN>
+__device__ __noinline__ void df_chain(const DfArgs &a, DfSmem &sm, int grp, int tid, const int (&dr)[5],
+                                      const int (&dc)[5]) {
+    const int lr = tid % 32, lc = tid / 32;
+    int *prog = a.sync + 2, *ready = prog + a.T + a.E + (a.W ? a.T : 0);
+    for (int c = 0; c < a.T; ++c) {
+        const int c0 = a.j0 + DT * c, cb = min(DT, a.j0 + a.jb - c0);
+        if (c >= 2) {   // the diagonal tile holds the products of the columns before c - 1
+            if (tid == 0) sm.word[1] = df_wait(&ready[2 * c], &ready[2 * c], 1, a.sync, &a.st->timeout);
+            df_sync(grp);
+            if (sm.word[1] < 0) return;
+        }
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+            const int col = lc + 4 * u;
+            sm.Bs[col][lr] = (lr < cb && col < cb) ? __ldcg(a.A + (long long)(c0 + col) * a.ld + c0 + lr) : 0.0;
+        }
+        df_sync(grp);
+        double acc[8];
+#pragma unroll
+        for (int i = 0; i < 5; ++i) acc[i] = -sm.Bs[dc[i]][dr[i]];
+        if (c > 0) df_mma_diag(acc, sm.As, dr, dc);
+        df_sync(grp);
+#pragma unroll
+        for (int i = 0; i < 5; ++i)
+            sm.Bs[dc[i]][dr[i]] = (dr[i] < cb && dc[i] < cb) ? -acc[i] : (dr[i] == dc[i] ? 1.0 : 0.0);
+        df_sync(grp);
+        auto *buf = reinterpret_cast<double (*)[4][DT]>(sm.Ls);
+            const int bad = PLAIN ? df_potrf32_plain(sm.Bs, buf, sm.dinv, grp, tid)
+                                  : df_potrf32(sm.Bs, buf, sm.dinv, grp, tid);
+        if (bad < cb) {
+            if (tid == 0) {
+                set_info(a.st, c0 + bad + 1);
+                __threadfence();
+                atomicExch(&a.sync[1], 1);
+            }
+            return;
+        }
+        df_sync(grp);
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+            const int col = lc + 4 * u;
+            const double v = sm.Bs[col][lr];
+            if (lr < cb && col < cb && lr >= col) a.A[(long long)(c0 + col) * a.ld + c0 + lr] = v;
+            sm.Ls[col][lr] = lr >= col ? (PLAIN ? v : v * sm.dinv[col]) : 0.0;
+        }
+        df_sync(grp);
+        if (tid == 0) df_st_release(&prog[c], c + 1);
+        if (c + 1 == a.T) return;
+        const int r0 = c0 + DT, nr = min(DT, a.j0 + a.jb - r0);
+        if (c >= 1) {   // the tile below holds the products of the columns before c
+            if (tid == 32) sm.word[1] = df_wait(&ready[2 * c + 1], &ready[2 * c + 1], 1, a.sync, &a.st->timeout);
+            df_sync(grp);
+            if (sm.word[1] < 0) return;
+        }
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+            const int col = lc + 4 * u;
+            sm.As[col][lr] = lr < nr ? __ldcg(a.A + (long long)(c0 + col) * a.ld + r0 + lr) : 0.0;
+        }
+        df_sync(grp);
+        if (PLAIN)
+            df_trsm32(sm.As, sm.Ls, sm.dinv, tid);
+        else
+            df_trsm32_scaled(sm.As, sm.Ls, sm.dinv, tid);
+        df_sync(grp);
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+            const int col = lc + 4 * u;
+            if (lr < nr) a.A[(long long)(c0 + col) * a.ld + r0 + lr] = sm.As[col][lr];
+        }
+        df_sync(grp);
+        if (tid == 0) df_st_release(&prog[c + 1], c + 1);
+    }
+}
+
+template <bool PLAIN>
+__global__ void __launch_bounds__(DF_THREADS, 1) k_chol_df(const DfArgs a) {
+    extern __shared__ __align__(16) unsigned char df_smem[];
+    const int grp = threadIdx.x / DG, tid = threadIdx.x % DG;
+    DfSmem &sm = reinterpret_cast<DfSmem *>(df_smem)[grp];
+    const int tx = tid % 16, ty = tid / 16, lr = tid % 32, lc = tid / 32;
+    int *prog = a.sync + 2;
+    // this thread's entries of a diagonal tile: one of the 64 of every other 8 x 8 block of its lower part
+    int dr[5], dc[5];
+#pragma unroll
+    for (int i = 0; i < 5; ++i) {
+        const int b = 2 * i + tid / 64, bi = b < 1 ? 0 : b < 3 ? 1 : b < 6 ? 2 : 3, bj = b - bi * (bi + 1) / 2;
+        dr[i] = 8 * bi + tid % 8;
+        dc[i] = 8 * bj + tid % 64 / 8;
+    }
+    __shared__ int chain_here;   // this CTA runs the column chain
+    if (threadIdx.x == 0) chain_here = 0;
+    __syncthreads();
+    // with few tiles, fewer groups to an SM share its FP64 pipe
+    if ((long long)grp * gridDim.x >= a.tickets) return;
+    for (;;) {
+        // stop after a failed pivot (of this launch or an earlier one) or an expired wait
+        if (tid == 0) {
+            const bool stop = df_ld_acquire(&a.sync[1]) || df_ld_acquire(&a.st->info) ||
+                              (a.alone && *(volatile int *)&chain_here);
+            sm.word[0] = stop ? a.tickets : atomicAdd(&a.sync[0], 1) - a.chain;
+            if (sm.word[0] < 0) *(volatile int *)&chain_here = 1;
+        }
+        df_sync(grp);
+        const int t = sm.word[0];
+        if (t >= a.tickets) return;
+        if (t < 0) {   // the first ticket of a launch with a chain
+            df_chain<PLAIN>(a, sm, grp, tid, dr, dc);
+            return;
+        }
+        // tile column c, and tile row: of the diagonal range (kind 0), the extra rows (1) or the identity rows (2)
+        int c, q;
+        if (!a.factor && a.W) {   // the inverse alone: column c has the identity rows 0 .. c
+            c = max(0, (int)((sqrt(8.0 * t + 1.0) - 1.0) * 0.5) - 1);
+            while ((c + 1) * (c + 2) / 2 <= t) ++c;
+            q = t - c * (c + 1) / 2 + a.T + a.E;
+        } else if (!a.factor) {
+            c = t / a.E;
+            q = t % a.E + a.T;
+        } else if (a.W) {
+            c = t / (a.T + a.E + 1);
+            q = t % (a.T + a.E + 1) + c;
+        } else {
+            // column c starts at ticket c (T + E) - c (c - 1) / 2
+            const double b = a.T + a.E + 0.5;
+            c = max(0, min(a.T - 1, (int)(b - sqrt(b * b - 2.0 * t))));
+            auto start = [&](int cc) { return cc * (a.T + a.E) - cc * (cc - 1) / 2; };
+            while (c > 0 && start(c) > t) --c;
+            while (c + 1 < a.T && start(c + 1) <= t) ++c;
+            q = t - start(c) + c;
+        }
+        const int kind = q < a.T ? 0 : q < a.T + a.E ? 1 : 2;
+        const int e = q - (kind == 1 ? a.T : kind == 2 ? a.T + a.E : 0);   // tile row within its kind
+        const int c0 = a.j0 + DT * c, cb = min(DT, a.j0 + a.jb - c0);
+        const int r0 = kind == 1 ? a.x0 + DT * e : a.j0 + DT * e;          // first row (identity rows: of the unit part)
+        const int nr = min(DT, (kind == 1 ? a.x1 : a.j0 + a.jb) - r0);
+        const bool diag = kind == 0 && e == c;
+        // with a chain, the diagonal tile and the one below it are only brought up to date here
+        const bool pre = a.chain && kind == 0 && e <= c + 1;
+        const int kend = pre && diag ? c - 1 : c;
+        if (pre && kend <= 0) {
+            df_sync(grp);   // everyone has read the ticket
+            continue;
+        }
+        int *prow = &prog[q], *pcol = a.factor ? &prog[c] : prow;
+        // the tile as it starts, through shared memory into the products' layout (eight or, on the diagonal, five
+        // entries a thread), negated: acc = -A + sum of products
+        double acc[8], cur[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+            const int col = lc + 4 * u;
+            double v;
+            if (kind == 2)
+                v = (e == c && lr == col) ? 1.0 : 0.0;
+            else
+                v = (lr < nr && col < cb) ? __ldcg(a.A + (long long)(c0 + col) * a.ld + r0 + lr) : 0.0;
+            sm.Bs[col][lr] = v;
+        }
+        df_sync(grp);
+        const bool straight = !a.block64 || kind == 2 || c < 2;
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            cur[i] = diag ? (i < 5 ? sm.Bs[dc[i % 5]][dr[i % 5]] : 0.0) : sm.Bs[tx + 16 * (i % 2)][ty + 8 * (i / 2)];
+            acc[i] = straight ? -cur[i] : 0.0;
+        }
+        df_sync(grp);
+        const int kbeg = kind == 2 ? e : 0;
+        int avail = kbeg;
+        double pa[8], pb[8];
+        auto load = [&](int k) {
+            const long long kc = a.j0 + DT * k;
+#pragma unroll
+            for (int u = 0; u < 8; ++u) {
+                const int kk = lc + 4 * u;
+                if (kind == 2)   // row r of the identity block's solution is column r of -W; threads walk k
+                    pa[u] = (DT * e + kk < a.jb) ? -__ldcg(a.W + (long long)(DT * e + kk) * a.ldw + DT * k + lr) : 0.0;
+                else
+                    pa[u] = lr < nr ? __ldcg(a.A + (kc + kk) * a.ld + r0 + lr) : 0.0;
+                if (!diag) pb[u] = lr < cb ? __ldcg(a.A + (kc + kk) * a.ld + c0 + lr) : 0.0;
+            }
+        };
+        bool gone = false;
+        for (int k = kbeg; k < kend; ++k) {
+            if (avail <= k) {
+                if (tid == 0) sm.word[1] = df_wait(prow, pcol, k + 1, a.sync, &a.st->timeout);
+                df_sync(grp);
+                avail = sm.word[1];
+                if (avail < 0) {
+                    gone = true;
+                    break;
+                }
+                load(k);
+            }
+            // (the previous slice's products are done: barrier at the end of the loop body)
+#pragma unroll
+            for (int u = 0; u < 8; ++u) {
+                if (kind == 2)
+                    sm.As[lr][lc + 4 * u] = pa[u];
+                else
+                    sm.As[lc + 4 * u][lr] = pa[u];
+                if (!diag) sm.Bs[lc + 4 * u][lr] = pb[u];
+            }
+            df_sync(grp);
+            if (k + 1 < kend && avail > k + 1) load(k + 1);   // in flight during the products
+            if (diag)
+                df_mma_diag(acc, sm.As, dr, dc);
+            else if (nr <= 8)
+                df_mma<1>(acc, sm.As, sm.Bs, tx, ty);
+            else
+                df_mma<4>(acc, sm.As, sm.Bs, tx, ty);
+            if (!straight && (k & 1)) {   // 64 columns done: off the tile, and on with the next ones
+                const bool own = k + 1 == (c & ~1);
+#pragma unroll
+                for (int i = 0; i < 8; ++i) {
+                    cur[i] -= acc[i];
+                    acc[i] = own ? -cur[i] : 0.0;
+                }
+            }
+            df_sync(grp);
+        }
+        if (gone) return;   // uniform over the group
+        // the tile into shared memory, [col][row]; past the matrix a diagonal block continues as the identity
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            if (!diag)
+                sm.Bs[tx + 16 * (i % 2)][ty + 8 * (i / 2)] = -acc[i];
+            else if (i < 5)
+                sm.Bs[dc[i % 5]][dr[i % 5]] =
+                    (dr[i % 5] < cb && dc[i % 5] < cb) ? -acc[i] : (dr[i % 5] == dc[i % 5] ? 1.0 : 0.0);
+        }
+        if (pre) {
+            df_sync(grp);
+        } else if (diag) {
+            df_sync(grp);
+            // (the tile's part above the diagonal is never set: what the lanes of those rows compute is not used)
+            auto *buf = reinterpret_cast<double (*)[4][DT]>(sm.Ls);
+            const int bad = PLAIN ? df_potrf32_plain(sm.Bs, buf, sm.dinv, grp, tid)
+                                  : df_potrf32(sm.Bs, buf, sm.dinv, grp, tid);
+            if (bad < cb) {   // the same in every thread; nothing below this pivot can be finished
+                if (tid == 0) {
+                    set_info(a.st, c0 + bad + 1);
+                    __threadfence();
+                    atomicExch(&a.sync[1], 1);
+                }
+                return;
+            }
+            df_sync(grp);
+        } else {
+            // L_cc: wait for its factorisation
+            if (tid == 0) sm.word[1] = a.factor ? df_wait(&prog[c], &prog[c], c + 1, a.sync, &a.st->timeout) : 0;
+            df_sync(grp);
+            if (sm.word[1] < 0) return;
+#pragma unroll
+            for (int u = 0; u < 8; ++u) {
+                const int col = lc + 4 * u;
+                pa[u] = (lr < cb && col < cb && lr >= col) ? __ldcg(a.A + (long long)(c0 + col) * a.ld + c0 + lr)
+                                                           : (lr == col ? 1.0 : 0.0);
+                if (PLAIN) sm.Ls[col][lr] = pa[u];
+            }
+            if (tid < DT) sm.dinv[tid] = tid < cb ? 1.0 / __ldcg(a.A + (long long)(c0 + tid) * a.ld + c0 + tid) : 1.0;
+            df_sync(grp);
+            if (PLAIN) {
+                df_trsm32(sm.Bs, sm.Ls, sm.dinv, tid);
+            } else {
+#pragma unroll
+                for (int u = 0; u < 8; ++u) sm.Ls[lc + 4 * u][lr] = pa[u] * sm.dinv[lc + 4 * u];
+                df_sync(grp);
+                df_trsm32_scaled(sm.Bs, sm.Ls, sm.dinv, tid);
+            }
+            df_sync(grp);
+        }
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+            if (kind == 2) {
+                // W(column of the solution, row) = -X: threads walk the solution's columns, W's rows
+                const int row = lc + 4 * u;   // row of the identity block
+                if (lr < cb && row < nr) a.W[(long long)(DT * e + row) * a.ldw + DT * c + lr] = -sm.Bs[lr][row];
+            } else {
+                const int col = lc + 4 * u;
+                if (lr < nr && col < cb && (!diag || lr >= col)) a.A[(long long)(c0 + col) * a.ld + r0 + lr] = sm.Bs[col][lr];
+            }
+        }
+        df_sync(grp);
+        if (tid == 0) {
+            if (pre)
+                df_st_release(prog + a.T + a.E + (a.W ? a.T : 0) + 2 * c + (diag ? 0 : 1), 1);
+            else
+                df_st_release(prow, c + 1);
+        }
+    }
+}
+
+// C[r, c] -= sum_k A[r, k] B[c, k] for a few rows r (right-hand sides): a thread per column reads its
+// operand row along k (coalesced over columns), bound by that one pass over B (HBM).
+constexpr int RROWS = 4;
+
+__global__ void __launch_bounds__(128) k_rhs_update(double *A, long long ld, int rC, int cC, int m, int n, int kA, int k,
+                                                   const DevStatus *st) {
+    if (st->info) return;
+    const int r0 = blockIdx.y * RROWS;
+    __shared__ double a[RROWS][128];
+    const int c = blockIdx.x * 128 + threadIdx.x;
+    double acc[RROWS] = {};
+    for (int k0 = 0; k0 < k; k0 += 128) {
+        const int kc = min(128, k - k0);
+        __syncthreads();
+        for (int i = 0; i < RROWS; ++i)
+            a[i][threadIdx.x] = (threadIdx.x < kc && r0 + i < m)
+                                    ? A[(long long)(kA + k0 + threadIdx.x) * ld + rC + r0 + i] : 0.0;
+        __syncthreads();
+        if (c < n) {
+            const double *b = A + (long long)(kA + k0) * ld + cC + c;
+#pragma unroll 8
+            for (int kk = 0; kk < kc; ++kk) {
+                const double bv = b[(long long)kk * ld];
+#pragma unroll
+                for (int i = 0; i < RROWS; ++i) acc[i] = fma(a[i][kk], bv, acc[i]);
+            }
+        }
+    }
+    if (c < n)
+        for (int i = 0; i < RROWS && r0 + i < m; ++i) A[(long long)(cC + c) * ld + rC + r0 + i] -= acc[i];
+}
+
+int df_sms() {
+    int dev = 0, n = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
+        n <= 0)
+        return 1;
+    return n;
+}
+
+cudaError_t launch_df(const DfArgs &a0, int sms, int cls, double flops, cudaStream_t s) {
+    DfArgs a = a0;
+    const long long T = a.T, E = a.E;
+    a.chain = a.factor && !a.block64 && T > 1;
+    // below about 4,000 columns the chain, not the products, sets the time
+    a.alone = a.chain && T < 128;
+    const long long words = 2 + T + E + (a.W ? T : 0) + (a.chain ? 2 * T : 0);
+    const long long tickets = !a.factor ? (a.W ? T * (T + 1) / 2 : T * E) : a.W ? T * (T + E + 1) : T * (T + E) - T * (T - 1) / 2;
+    if (tickets == 0) return cudaSuccess;
+    if (words > GEO_CHOL_SYNC_INTS || tickets > (1LL << 30)) return cudaErrorInvalidValue;
+    a.tickets = (int)tickets;
+    cudaError_t e = cudaMemsetAsync(a.sync, 0, sizeof(int) * words, s);
+    if (e != cudaSuccess) return e;
+    constexpr size_t smem = sizeof(DfSmem) * DF_GROUPS;
+    auto *kernel = a.plain ? k_chol_df<true> : k_chol_df<false>;
+    if ((e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess) return e;
+    const int all = df_sms();
+    const int grid = (int)std::min<long long>(sms > 0 ? std::min(sms, all) : all, tickets + a.chain);
+    if (grid < 8) a.alone = 0;
+    KScope ks(cls, s, flops, 16.0 * ((double)a.jb * a.jb / 2 + (double)(a.x1 - a.x0) * a.jb));
+    kernel<<<grid, DF_THREADS, smem, s>>>(a);
     return cudaGetLastError();
 }
 
 }  // namespace
 
-// Factor the panel of columns [j0, j0 + jb): its diagonal tile (inner 64-wide
-// blocks: POTRF, TRSM, rank-64 update) and, carried through the same inner
-// steps, the rows [x0, x1) below the tile (x0 >= j0 + jb; x0 == x1 = none).
-// With factor_diag false the diagonal tile must already hold L and only the
-// rows [x0, x1) are solved against it (X <- X L^-T).
-cudaError_t chol64_panel(double *A, long long ld, int j0, int jb, int x0, int x1, DevStatus *st, cudaStream_t s,
-                         bool factor_diag, const PanelUpdate *upd) {
-    const size_t trsm_smem = sizeof(double) * (IB * IB + IB * (TRSM_ROWS + 1));
-    cudaError_t e = cudaFuncSetAttribute(k_trsm_rlt, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)trsm_smem);
-    if (e != cudaSuccess) return e;
-    const bool contiguous = factor_diag && (x0 == j0 + jb);
-    for (int c0 = j0; c0 < j0 + jb; c0 += IB) {
-        const int cb = min(IB, j0 + jb - c0);
-        if (factor_diag) {
-            KScope ks(GEO_K_POTRF, s, (double)cb * cb * cb / 3.0, 16.0 * cb * cb);
-            k_potrf_diag<<<1, 256, 0, s>>>(A, ld, c0, cb, st);
-        }
-        const int rows0 = c0 + cb;
-        // row ranges carried through this inner step
-        int ra[2][2];
-        int nrange = 0;
-        if (!factor_diag) {
-            if (x0 < x1) ra[nrange][0] = x0, ra[nrange][1] = x1, ++nrange;
-        } else if (contiguous) {
-            if (rows0 < x1) ra[nrange][0] = rows0, ra[nrange][1] = x1, ++nrange;
-        } else {
-            if (rows0 < j0 + jb) ra[nrange][0] = rows0, ra[nrange][1] = j0 + jb, ++nrange;
-            if (x0 < x1) ra[nrange][0] = x0, ra[nrange][1] = x1, ++nrange;
-        }
-        for (int q = 0; q < nrange; ++q) {
-            const int nr = ra[q][1] - ra[q][0];
-            KScope ks(GEO_K_TRSM, s, (double)nr * cb * cb, 16.0 * nr * cb);
-            k_trsm_rlt<<<(nr + TRSM_ROWS - 1) / TRSM_ROWS, 256, trsm_smem, s>>>(A, ld, c0, cb, ra[q][0], ra[q][1], st);
-        }
-        if ((e = cudaGetLastError()) != cudaSuccess) return e;
-        // rest of the panel: cols rows0 .. j0+jb-1
-        if (rows0 < j0 + jb) {
-            for (int q = 0; q < nrange; ++q) {
-                e = upd ? upd->fn(upd, A, ld, ra[q][0], rows0, ra[q][1] - ra[q][0], j0 + jb - rows0, c0, cb, st, s)
-                        : gemm_update(A, ld, ra[q][0], rows0, ra[q][1] - ra[q][0], j0 + jb - rows0, c0, cb, st, s);
-                if (e != cudaSuccess) return e;
-            }
-        }
-    }
-    return cudaSuccess;
+// Factor the columns [j0, j0 + jb): the diagonal range, and the rows [x0, x1) below it (x0 >= j0 + jb;
+// x0 == x1 = none) solved against it.  factor_diag false: the diagonal range already holds L and only the
+// rows are solved (X <- X L^-T), or, without rows, only W is formed.  W (jb x jb, ldw) != NULL: also W = -L^-1, its strictly upper part must hold
+// zeros.  sms: at most that many CTAs, one per SM (0 = all).  sync: GEO_CHOL_SYNC_INTS device ints of scratch.
+cudaError_t chol64_panel(double *A, long long ld, int j0, int jb, int x0, int x1, DevStatus *st, int *sync,
+                         cudaStream_t s, bool factor_diag, double *W, long long ldw, int sms, int order) {
+    if (jb <= 0) return cudaSuccess;
+    if (!factor_diag && W && x1 > x0) return cudaErrorInvalidValue;
+    const int nx = std::max(0, x1 - x0);
+    DfArgs a{A, ld, j0, jb, x0, x0 + nx, (jb + DT - 1) / DT, (nx + DT - 1) / DT, factor_diag ? 1 : 0, W, ldw, sync, 0, 0, 0, order == GEO_CHOL_BLOCK64,
+             order != GEO_CHOL_STRAIGHT, st};
+    const double j = jb, cubes = (factor_diag ? j * j * j / 3.0 : 0.0) + (W ? j * j * j / 3.0 : 0.0);
+    return launch_df(a, sms, factor_diag ? GEO_K_POTRF : GEO_K_TRSM, cubes + nx * j * j, s);
 }
 
-cudaError_t chol64_gemm_update(double *A, long long ld, int rC, int cC, int m, int n, int kA, int k, DevStatus *st,
-                               cudaStream_t s) {
-    return gemm_update(A, ld, rC, cC, m, n, kA, k, st, s);
+// SMs for a diagonal tile of order jb (with its inverse) that runs beside other work of rest_us: the fewest
+// with which the tile is done in that time.  A tile takes its column chain, about 0.55 us a column, or its FP64
+// FMAs (jb^3 / 6, twice with the inverse) at two per clock and SM, whichever is longer.
+int chol64_side_sms(int jb, bool inverse, double rest_us) {
+    const double j = jb, chain = 0.55 * j, fma_us = j * j * j / 6.0 * (inverse ? 2.0 : 1.0) / (2.0 * 2000.0);
+    int n = 8;
+    while (n < 48 && fma_us / n > std::max(chain, rest_us)) n += 8;
+    return n;
 }
 
-cudaError_t chol64_factor(double *A, long long ld, int N, int nrows, int nb, DevStatus *st, cudaStream_t s) {
-    if (nb < IB) nb = IB;
-    nb = (nb / IB) * IB;
-    cudaError_t e = cudaSuccess;
-    for (int j0 = 0; j0 < N; j0 += nb) {
-        const int jb = min(nb, N - j0);
-        e = chol64_panel(A, ld, j0, jb, j0 + jb, nrows, st, s);
-        if (e != cudaSuccess) return e;
-        // trailing update: rows j0+jb .. nrows-1, cols j0+jb .. N-1, rank jb
-        const int t0 = j0 + jb;
-        if (t0 < N) {
-            e = gemm_update(A, ld, t0, t0, nrows - t0, N - t0, j0, jb, st, s);
-            if (e != cudaSuccess) return e;
-        }
-    }
-    return cudaSuccess;
+// C[rC.., cC..] (m x n) -= A[rC.., kA..kA+k] A[cC.., kA..kA+k]' in FP64, for the right-hand-side rows of a
+// factorisation whose other updates run elsewhere.
+cudaError_t chol64_rhs_update(double *A, long long ld, int rC, int cC, int m, int n, int kA, int k, DevStatus *st,
+                              cudaStream_t s) {
+    if (m <= 0 || n <= 0 || k <= 0) return cudaSuccess;
+    KScope ks(GEO_K_GEMM, s, 2.0 * k * (double)m * n, 8.0 * ((double)n * k + 2.0 * m * n));
+    k_rhs_update<<<dim3((n + 127) / 128, (m + RROWS - 1) / RROWS), 128, 0, s>>>(A, ld, rC, cC, m, n, kA, k, st);
+    return cudaGetLastError();
+}
+
+// In-place lower Cholesky of the leading N x N block of A with the rows N .. nrows-1 carried along: one launch.
+cudaError_t chol64_factor(double *A, long long ld, int N, int nrows, DevStatus *st, int *sync, cudaStream_t s) {
+    if (N <= 0) return cudaSuccess;
+    const int nx = std::max(0, nrows - N);
+    DfArgs a{A, ld, 0, N, N, N + nx, (N + DT - 1) / DT, (nx + DT - 1) / DT, 1, nullptr, 0, sync, 0, 0, 0, 0, 0, st};
+    const double n = N;
+    return launch_df(a, 0, GEO_K_GEMM, n * n * n / 3.0 + nx * n * n, s);
 }

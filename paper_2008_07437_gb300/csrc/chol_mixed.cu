@@ -319,14 +319,16 @@ struct MixedGeom {
     int N, nrows, nb, band, lowp;
     long long ldp;
     DevStatus *st;
+    int *sync;   // scratch words of the diagonal tiles' launches
 };
 
 // Diagonal tile of panel [j0, j0 + jb) in FP64, carrying the right-hand-side
-// rows [N, nrows): a chain of small latency-bound launches.
-cudaError_t mixed_panel_diag(const MixedGeom &G, int j0, cudaStream_t s) {
+// rows [N, nrows), on at most `sms` SMs (0 = all).
+cudaError_t mixed_panel_diag(const MixedGeom &G, int j0, int sms, cudaStream_t s) {
     const int jb = min(G.nb, G.N - j0);
     const int t0 = j0 + jb;
-    return chol64_panel(G.A, G.ld, j0, jb, (G.nrows > G.N) ? G.N : t0, (G.nrows > G.N) ? G.nrows : t0, G.st, s);
+    return chol64_panel(G.A, G.ld, j0, jb, (G.nrows > G.N) ? G.N : t0, (G.nrows > G.N) ? G.nrows : t0, G.st, G.sync, s,
+                        true, nullptr, 0, sms, GEO_CHOL_BLOCK64);
 }
 
 // Rows below the diagonal tile of panel j0: solved in FP32 against the
@@ -464,7 +466,7 @@ cudaError_t mixed_update(const MixedGeom &G, int j0, int ca, int cb, const Panel
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }
     // right-hand-side rows in FP64
-    if (nrows > N) return chol64_gemm_update(A, ld, N, ca, nrows - N, cb - ca, j0, jb, st, s);
+    if (nrows > N) return chol64_rhs_update(A, ld, N, ca, nrows - N, cb - ca, j0, jb, st, s);
     return cudaSuccess;
 }
 
@@ -473,16 +475,14 @@ cudaError_t mixed_update(const MixedGeom &G, int j0, int ca, int cb, const Panel
 size_t mixed_workspace_bytes(int N, int nb) { return panel_ws_bytes(N, nb); }
 
 // Right-looking over panels with a lookahead of one: step j first updates the
-// next panel's tile column; the diagonal tile of that panel (a chain of small
-// FP64 launches) is then factored on a second, high-priority stream while the
-// rest of step j's trailing update runs (its persistent tensor-core launch
-// leaves SIDE_SMS SMs free for it); the rows below it are solved after the
-// join.  Every entry receives the same operations in the same order as
+// next panel's tile column; the diagonal tile of that panel is then factored
+// in FP64 on a second, high-priority stream while the rest of step j's
+// trailing update runs (its persistent tensor-core launch leaves a few SMs
+// free for it); the rows below it are solved after the join.  Every entry receives the same operations in the same order as
 // without the lookahead.
-constexpr int SIDE_SMS = 8;
 
 cudaError_t chol_mixed_factor(double *A, long long ld, int N, int nrows, int nb, int band, int lowp, void *ws,
-                              size_t ws_bytes, DevStatus *st, cudaStream_t s) {
+                              size_t ws_bytes, DevStatus *st, int *sync, cudaStream_t s) {
     if (nb % 128 != 0 || nb <= 0) return cudaErrorInvalidValue;
     if (ws_bytes < mixed_workspace_bytes(N, nb)) return cudaErrorInvalidValue;
     EncodeTiledFn enc = encode_fn();
@@ -491,7 +491,7 @@ cudaError_t chol_mixed_factor(double *A, long long ld, int N, int nrows, int nb,
                                          (int)tc::SMEM_BYTES);
     if (e != cudaSuccess) return e;
     const size_t rows_max = (size_t)N + 128;
-    MixedGeom G{A, ld, N, nrows, nb, band, lowp, (long long)((rows_max + 3) / 4 * 4), st};
+    MixedGeom G{A, ld, N, nrows, nb, band, lowp, (long long)((rows_max + 3) / 4 * 4), st, sync};
     const PanelWs W = carve((uint8_t *)ws, rows_max, G.ldp, nb);
     const uint32_t idesc = tc::instr_desc(lowp ? 1 : 0);
     int prio_lo = 0, prio_hi = 0;
@@ -508,7 +508,7 @@ cudaError_t chol_mixed_factor(double *A, long long ld, int N, int nrows, int nb,
     const int all = num_sms();
     auto run = [&]() -> cudaError_t {
         cudaError_t r;
-        if ((r = mixed_panel_diag(G, 0, s)) != cudaSuccess || (r = mixed_panel_rows(G, 0, W, s)) != cudaSuccess)
+        if ((r = mixed_panel_diag(G, 0, 0, s)) != cudaSuccess || (r = mixed_panel_rows(G, 0, W, s)) != cudaSuccess)
             return r;
         for (int j0 = 0; j0 < N; j0 += nb) {
             const int t0 = j0 + min(nb, N - j0);
@@ -518,10 +518,14 @@ cudaError_t chol_mixed_factor(double *A, long long ld, int N, int nrows, int nb,
             if ((r = mixed_update(G, j0, t0, n1, W, enc, idesc, all, s)) != cudaSuccess) return r;
             if ((r = cudaEventRecord(e_upd, s)) != cudaSuccess) return r;
             if ((r = cudaStreamWaitEvent(s2, e_upd, 0)) != cudaSuccess) return r;
-            if ((r = mixed_panel_diag(G, t0, s2)) != cudaSuccess) return r;
+            // the update's rest in us at 600 TFLOP/s (three FP16 products per entry): the diagonal tile gets the
+            // SMs it needs to finish within it
+            const double left = N - n1, rest_us = 3.0 * left * left * (t0 - j0) / 600e6;
+            const int side = chol64_side_sms(n1 - t0, false, rest_us);
+            if ((r = mixed_panel_diag(G, t0, n1 < N ? side : 0, s2)) != cudaSuccess) return r;
             if ((r = cudaEventRecord(e_pan, s2)) != cudaSuccess) return r;
             // the rest of this step's trailing update meanwhile
-            if (n1 < N && (r = mixed_update(G, j0, n1, N, W, enc, idesc, all - SIDE_SMS, s)) != cudaSuccess)
+            if (n1 < N && (r = mixed_update(G, j0, n1, N, W, enc, idesc, all - side, s)) != cudaSuccess)
                 return r;
             if ((r = cudaStreamWaitEvent(s, e_pan, 0)) != cudaSuccess) return r;
             if ((r = mixed_panel_rows(G, t0, W, s)) != cudaSuccess) return r;

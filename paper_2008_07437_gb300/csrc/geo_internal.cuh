@@ -101,28 +101,30 @@ cudaError_t launch_scatter_vec(const double *in, long long stride, const int *pe
                                cudaStream_t s);
 
 // ---- chol64.cu ----------------------------------------------------------
+// Device ints of scratch (ticket, abort and progress words) of a chol64_* launch.
+constexpr int GEO_CHOL_SYNC_INTS = 16384;
+// Order of the sums within a panel: straight through, or per 64 columns; PLAIN and BLOCK64 round pivots and
+// solves as the plain right-looking algorithm does (the reduced forms keep both).
+constexpr int GEO_CHOL_STRAIGHT = 0, GEO_CHOL_BLOCK64 = 1, GEO_CHOL_PLAIN = 2;
 // In-place lower Cholesky of the leading N x N block of A; rows N..nrows-1
 // are extra right-hand-side rows carried through the factorisation (row N
-// receives (L^-1 z)' when it holds z').  nb = outer tile size.
-cudaError_t chol64_factor(double *A, long long ld, int N, int nrows, int nb, DevStatus *st, cudaStream_t s);
-// The rank-64 updates inside a panel, C[rC.., cC..] (m x n) -= A[rC.., kA..kA+k] A[cC.., kA..kA+k]'
-// (lower part when rC == cC), when they should not run on the FP64 pipe.
-struct PanelUpdate {
-    cudaError_t (*fn)(const PanelUpdate *u, double *A, long long ld, int rC, int cC, int m, int n, int kA, int k,
-                      DevStatus *st, cudaStream_t s);
-    void *ctx;
-};
-// One panel [j0, j0+jb): diagonal tile plus extra rows [x0, x1) carried along.
-cudaError_t chol64_panel(double *A, long long ld, int j0, int jb, int x0, int x1, DevStatus *st, cudaStream_t s,
-                         bool factor_diag = true, const PanelUpdate *upd = nullptr);
-// C[rC.., cC..] (m x n) -= A[rC.., kA..kA+k] A[cC.., kA..kA+k]' in FP64.
-cudaError_t chol64_gemm_update(double *A, long long ld, int rC, int cC, int m, int n, int kA, int k, DevStatus *st,
-                               cudaStream_t s);
+// receives (L^-1 z)' when it holds z').
+cudaError_t chol64_factor(double *A, long long ld, int N, int nrows, DevStatus *st, int *sync, cudaStream_t s);
+// One panel [j0, j0+jb): diagonal tile plus extra rows [x0, x1) carried along; W: also -L^-1 of the tile
+// (its strictly upper part must hold zeros); sms: at most that many SMs (0 = all).
+cudaError_t chol64_panel(double *A, long long ld, int j0, int jb, int x0, int x1, DevStatus *st, int *sync,
+                         cudaStream_t s, bool factor_diag = true, double *W = nullptr, long long ldw = 0, int sms = 0,
+                         int order = GEO_CHOL_STRAIGHT);
+// SMs to leave to a diagonal tile that is factored beside other work of rest_us.
+int chol64_side_sms(int jb, bool inverse, double rest_us);
+// C[rC.., cC..] (m x n) -= A[rC.., kA..kA+k] A[cC.., kA..kA+k]' in FP64, m a few right-hand-side rows.
+cudaError_t chol64_rhs_update(double *A, long long ld, int rC, int cC, int m, int n, int kA, int k, DevStatus *st,
+                              cudaStream_t s);
 
 // ---- chol_mixed.cu --------------------------------------------------------
 size_t mixed_workspace_bytes(int N, int nb);
 cudaError_t chol_mixed_factor(double *A, long long ld, int N, int nrows, int nb, int band, int lowp, void *ws,
-                              size_t ws_bytes, DevStatus *st, cudaStream_t s);
+                              size_t ws_bytes, DevStatus *st, int *sync, cudaStream_t s);
 
 
 // ---- ozaki.cu -------------------------------------------------------------
@@ -156,7 +158,7 @@ size_t oz_chol_workspace_bytes(int nrows, int nb, int S);
 // Dense Cholesky as chol64_factor, trailing updates and panel solves on the
 // tensor cores with S slices (nb <= 1024); cut = 1: the trailing updates use the level cut.
 cudaError_t chol_oz_factor(double *A, long long ld, int N, int nrows, int nb, int S, int cut, void *ws,
-                           size_t ws_bytes, DevStatus *st, cudaStream_t s);
+                           size_t ws_bytes, DevStatus *st, int *sync, cudaStream_t s);
 size_t oz_gemm_workspace_bytes(int m, int n, int k, int S);
 // C (m x n) -= A (m x k) B (n x k)', column-major FP64, S slices.
 cudaError_t oz_gemm(int m, int n, int k, const double *A, long long lda, const double *B, long long ldb, double *C,
@@ -321,7 +323,8 @@ size_t tlr_factor_bytes(int N, int nb, int kmax);
 size_t tlr_workspace_bytes(int N, int nb, int kmax);
 size_t tlr_solve_workspace_bytes(int N, int nb, int kmax);
 cudaError_t tlr_factor(TlrFactor &F, const CovParams &cp, const double *lx, const double *ly, void *ws,
-                       size_t ws_bytes, void *arena_host, DevStatus *st, DevStatus *h_st, cudaStream_t s);
+                       size_t ws_bytes, void *arena_host, DevStatus *st, int *sync, DevStatus *h_st,
+                       cudaStream_t s);
 cudaError_t tlr_solve(const TlrFactor &F, double *x, bool transpose, void *ws, void *arena_host, cudaStream_t s);
 cudaError_t tlr_reduce(const TlrFactor &F, const double *y, const DevStatus *st, DevResults *res, cudaStream_t s);
 

@@ -108,7 +108,7 @@ extern "C" int geo_loglik_noalloc(const double *locs_dev, int n, const double *z
     const long long ld = ((long long)(N + 1) + 31) / 32 * 32;
     double *A = scratch;
     double *lx = scratch + kMatDoubles;
-    double *ly = lx + n;
+    double *ly = lx + n;   // once Sigma is generated, the locations' array holds the factorisation's sync words
     double *tab = scratch + kMatDoubles + kLocDoubles;
     DevStatus *st = (DevStatus *)(scratch + kMatDoubles + kLocDoubles + kTabDoubles);
     cudaStream_t s = (cudaStream_t)stream;
@@ -118,7 +118,7 @@ extern "C" int geo_loglik_noalloc(const double *locs_dev, int n, const double *z
         (e = launch_gather_vec(z_dev, nullptr, n, theta->p, A + N, ld, s)) ||
         (e = launch_cheb_build(cp, tab, s)) ||
         (e = launch_covgen_sym(cp, lx, ly, n, A, ld, s)) ||
-        (e = chol64_factor(A, ld, N, N + 1, nb, st, s)) ||
+        (e = chol64_factor(A, ld, N, N + 1, st, (int *)lx, s)) ||
         (e = launch_loglik_reduce(A, ld, N, A + N, ld, st, (DevResults *)out_dev, s))) {
         return GEO_ECUDA;
     }

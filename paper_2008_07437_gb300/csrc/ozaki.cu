@@ -780,97 +780,6 @@ cudaError_t oz_update(const OzSlices &A, const OzSlices &B, double *C, long long
     return cudaSuccess;
 }
 
-namespace {
-
-// W = -L^-1 for the lower-triangular jb x jb tile L (column-major, ld),
-// written column-major with leading dimension ldw (zeros above the diagonal).
-// Column-oriented forward substitution L w = e_c for the TRTRI_COLS columns of
-// a CTA: at step k the owner of row k divides by L_kk and publishes w_k, every
-// thread then updates its rows below with column k of L (read along the
-// column, coalesced).  The broadcast buffer is double-buffered, so one barrier
-// per step suffices; the reciprocals of the diagonal are taken up front, off
-// the chain of steps.  Four columns per CTA: the FP64 work of a step (two
-// FMAs per clock per SM) is split over jb / 4 CTAs.
-constexpr int TRTRI_COLS = 4, TRTRI_THREADS = 256, TRTRI_RPT = 4;   // rows per thread: jb <= 1024
-
-__global__ void __launch_bounds__(TRTRI_THREADS) k_trtri_neg(const double *__restrict__ L, long long ld, int jb,
-                                                          double *W, long long ldw, const DevStatus *st) {
-    __shared__ double wk[2][TRTRI_COLS];
-    __shared__ double dinv[TRTRI_THREADS * TRTRI_RPT];
-    __shared__ int skip;
-    if (threadIdx.x == 0) skip = *(volatile const int *)&st->info;
-    __syncthreads();
-    if (skip) return;
-    for (int r = threadIdx.x; r < jb; r += TRTRI_THREADS) dinv[r] = 1.0 / L[(long long)r * ld + r];
-    __syncthreads();
-    const int c0 = blockIdx.x * TRTRI_COLS;
-    const int ncol = min(TRTRI_COLS, jb - c0);
-    double w[TRTRI_RPT][TRTRI_COLS];
-#pragma unroll
-    for (int q = 0; q < TRTRI_RPT; ++q) {
-        const int r = threadIdx.x + q * TRTRI_THREADS;
-#pragma unroll
-        for (int c = 0; c < TRTRI_COLS; ++c) w[q][c] = (r == c0 + c) ? 1.0 : 0.0;
-    }
-    // column k of L for this thread's rows (and the diagonal entry for the owner of row k),
-    // loaded one step ahead so that the load latency is off the chain of barriers
-    double lcol[TRTRI_RPT];
-    auto load_col = [&](int k, double *dst) {
-#pragma unroll
-        for (int q = 0; q < TRTRI_RPT; ++q) {
-            const int r = threadIdx.x + q * TRTRI_THREADS;
-            dst[q] = (k < jb && r >= k && r < jb) ? L[(long long)k * ld + r] : 0.0;
-        }
-    };
-    load_col(c0, lcol);
-    for (int k = c0; k < jb; ++k) {
-        double lnext[TRTRI_RPT];
-        load_col(k + 1, lnext);
-        const int owner_q = k / TRTRI_THREADS, owner_t = k % TRTRI_THREADS;
-        if (threadIdx.x == owner_t) {
-            const double inv = dinv[k];
-#pragma unroll
-            for (int q = 0; q < TRTRI_RPT; ++q)
-                if (q == owner_q) {
-#pragma unroll
-                    for (int c = 0; c < TRTRI_COLS; ++c) {
-                        w[q][c] *= inv;
-                        wk[k & 1][c] = w[q][c];
-                    }
-                }
-        }
-        __syncthreads();
-#pragma unroll
-        for (int q = 0; q < TRTRI_RPT; ++q) {
-            const int r = threadIdx.x + q * TRTRI_THREADS;
-            if (r > k && r < jb) {
-#pragma unroll
-                for (int c = 0; c < TRTRI_COLS; ++c) w[q][c] = fma(-lcol[q], wk[k & 1][c], w[q][c]);
-            }
-        }
-#pragma unroll
-        for (int q = 0; q < TRTRI_RPT; ++q) lcol[q] = lnext[q];
-    }
-#pragma unroll
-    for (int q = 0; q < TRTRI_RPT; ++q) {
-        const int r = threadIdx.x + q * TRTRI_THREADS;
-        if (r >= jb) continue;
-#pragma unroll
-        for (int c = 0; c < TRTRI_COLS; ++c)
-            if (c < ncol) W[(long long)(c0 + c) * ldw + r] = (r >= c0 + c) ? -w[q][c] : 0.0;
-    }
-}
-
-cudaError_t launch_trtri_neg(const double *L, long long ld, int jb, double *W, long long ldw, const DevStatus *st,
-                             cudaStream_t s) {
-    if (jb > TRTRI_THREADS * TRTRI_RPT) return cudaErrorInvalidValue;
-    KScope ks(GEO_K_TRSM, s, (double)jb * jb * jb / 3.0, 16.0 * jb * jb);
-    k_trtri_neg<<<(jb + TRTRI_COLS - 1) / TRTRI_COLS, TRTRI_THREADS, 0, s>>>(L, ld, jb, W, ldw, st);
-    return cudaGetLastError();
-}
-
-}  // namespace
-
 constexpr int OZ_TILE_IB = 64;   // inner block of the diagonal tiles (the rank of their updates)
 
 size_t oz_chol_workspace_bytes(int nrows, int nb, int S) {
@@ -888,18 +797,17 @@ struct TileUpdate {
     int sms;
 };
 
-cudaError_t tile_update(const PanelUpdate *u, double *A, long long ld, int rC, int cC, int m, int n, int kA, int k,
-                        DevStatus *st, cudaStream_t s) {
-    const TileUpdate &t = *(const TileUpdate *)u->ctx;
-    if (m <= 0 || n <= 0 || k <= 0) return cudaSuccess;
-    if (rC != cC || k > t.sl.K || m > t.sl.rows) return cudaErrorInvalidValue;
+cudaError_t tile_update(const TileUpdate &t, double *A, long long ld, int rC, int m, int kA, int k, DevStatus *st,
+                        cudaStream_t s) {
+    if (m <= 0 || k <= 0) return cudaSuccess;
+    if (k > t.sl.K || m > t.sl.rows) return cudaErrorInvalidValue;
     OzSlices p = t.sl;
     p.K = k;
     p.nchunk = (k + p.kchunk - 1) / p.kchunk;
     p.valid = m;
     cudaError_t e = oz_slice(A + (long long)kA * ld + rC, ld, m, p, st, s);
     if (e != cudaSuccess) return e;
-    return oz_update(p, p, A, ld, rC, cC, m, n, rC + m, cC + n, 0, 0, 1, t.sms, st, s, 0, 0);
+    return oz_update(p, p, A, ld, rC, rC, m, m, rC + m, rC + m, 0, 0, 1, t.sms, st, s, 0, 0);
 }
 }  // namespace
 
@@ -907,16 +815,17 @@ cudaError_t tile_update(const PanelUpdate *u, double *A, long long ld, int rC, i
 // form).  Step j slices its solved panel (the rows below the diagonal tile,
 // right-hand-side rows included) and updates the next panel's tile column
 // first; on a high-priority second stream the next diagonal tile is factored
-// (native FP64 POTRF) and inverted, W = -L_kk^-1, while the rest of the
-// trailing update runs (its persistent launch leaves SIDE_SMS SMs free).
+// and inverted, W = -L_kk^-1, in one native FP64 launch while the rest of the
+// trailing update runs (its persistent launch leaves it the SMs it needs).
 // After the join the rows below the new diagonal tile are solved as one
 // emulated product, L_ik = A_ik L_kk^-T = -(A_ik W'), written over A_ik.
 // Every trailing update and panel solve is emulated; POTRF of the diagonal
 // tiles and their inversion are native FP64, and so is the last panel.
+constexpr double OZ_REST_RATE = 1.2e9;   // BF16 flops per us of a trailing update, for the split of the SMs
+
 cudaError_t chol_oz_factor(double *A, long long ld, int N, int nrows, int nb, int S, int cut, void *ws,
-                           size_t ws_bytes, DevStatus *st, cudaStream_t s) {
-    constexpr int SIDE_SMS = 8;
-    if (nb < 64 || nb % 64 != 0 || nb > TRTRI_THREADS * TRTRI_RPT || S < 3 || S > 8) return cudaErrorInvalidValue;
+                           size_t ws_bytes, DevStatus *st, int *sync, cudaStream_t s) {
+    if (nb < 64 || nb % 64 != 0 || nb > 1024 || S < 3 || S > 8) return cudaErrorInvalidValue;
     if (ws_bytes < oz_chol_workspace_bytes(nrows, nb, S)) return cudaErrorInvalidValue;
     const OzSlices sl = oz_slices_carve(ws, (long long)nrows + 128, nb, S);
     uintptr_t wp = ((uintptr_t)ws + oz_slices_bytes((long long)nrows + 128, nb, S) + 255) & ~(uintptr_t)255;
@@ -924,8 +833,11 @@ cudaError_t chol_oz_factor(double *A, long long ld, int N, int nrows, int nb, in
     wp = (wp + oz_slices_bytes(nb, nb, S) + 255) & ~(uintptr_t)255;
     double *W = (double *)wp;   // nb x nb, ld nb
     wp = (wp + sizeof(double) * (size_t)nb * nb + 255) & ~(uintptr_t)255;
-    TileUpdate tu{oz_slices_carve((void *)wp, nb, OZ_TILE_IB, S), SIDE_SMS};
-    const PanelUpdate tile_upd{tile_update, &tu};
+    const OzSlices tile_sl = oz_slices_carve((void *)wp, nb, OZ_TILE_IB, S);
+    // with FP64-class slices a diagonal tile is one native launch; with fewer its own rank-64 updates
+    // are emulated like every other update (their rounding is part of that form's result)
+    const bool fused = S >= 7;
+    const int order = fused ? GEO_CHOL_STRAIGHT : GEO_CHOL_BLOCK64;
     int prio_lo = 0, prio_hi = 0;
     cudaDeviceGetStreamPriorityRange(&prio_lo, &prio_hi);
     cudaStream_t s2 = nullptr;
@@ -953,17 +865,28 @@ cudaError_t chol_oz_factor(double *A, long long ld, int N, int nrows, int nb, in
             return r;
         return oz_update(p, q, A, ld, x0, t0, x1 - x0, jb, x1, t0 + jb, 0, 0, 0, all, st, st_, 1, 0);
     };
-    // native FP64 factorisation of the diagonal tile [t0, t0 + jb) and its inverse
-    auto diag = [&](int t0, int jb, cudaStream_t st_) -> cudaError_t {
-        cudaError_t r = chol64_panel(A, ld, t0, jb, t0 + jb, t0 + jb, st, st_, true, &tile_upd);
-        if (r != cudaSuccess) return r;
-        return launch_trtri_neg(A + (long long)t0 * ld + t0, ld, jb, W, nb, st, st_);
+    // factorisation of the diagonal tile [t0, t0 + jb) and its inverse on at most sms SMs
+    auto diag = [&](int t0, int jb, int sms, cudaStream_t st_) -> cudaError_t {
+        if (fused) return chol64_panel(A, ld, t0, jb, t0 + jb, t0 + jb, st, sync, st_, true, W, nb, sms);
+        cudaError_t r;
+        for (int c0 = t0; c0 < t0 + jb; c0 += OZ_TILE_IB) {
+            const int cb = std::min(OZ_TILE_IB, t0 + jb - c0);
+            if ((r = chol64_panel(A, ld, c0, cb, c0 + cb, t0 + jb, st, sync, st_, true, nullptr, 0, sms,
+                                  GEO_CHOL_PLAIN)) != cudaSuccess ||
+                (r = tile_update(TileUpdate{tile_sl, sms > 0 ? sms : all}, A, ld, c0 + cb, t0 + jb - c0 - cb, c0, cb, st,
+                                 st_)) != cudaSuccess)
+                return r;
+        }
+        return chol64_panel(A, ld, t0, jb, t0 + jb, t0 + jb, st, sync, st_, false, W, nb, sms, GEO_CHOL_PLAIN);
     };
     auto run = [&]() -> cudaError_t {
         cudaError_t r;
         const int jb0 = std::min(nb, N);
-        if (jb0 == N) return chol64_panel(A, ld, 0, N, N, nrows, st, s);   // one tile: native
-        if ((r = diag(0, jb0, s)) != cudaSuccess || (r = panel_solve(0, jb0, jb0, nrows, s)) != cudaSuccess)
+        if (jb0 == N)   // one tile: native
+            return chol64_panel(A, ld, 0, N, N, nrows, st, sync, s, true, nullptr, 0, 0, order);
+        // the launches below write W's lower part only
+        if ((r = cudaMemsetAsync(W, 0, sizeof(double) * (size_t)nb * nb, s)) != cudaSuccess) return r;
+        if ((r = diag(0, jb0, 0, s)) != cudaSuccess || (r = panel_solve(0, jb0, jb0, nrows, s)) != cudaSuccess)
             return r;
         for (int j0 = 0;;) {
             const int jb = std::min(nb, N - j0);
@@ -982,18 +905,23 @@ cudaError_t chol_oz_factor(double *A, long long ld, int N, int nrows, int nb, in
                 cudaSuccess)
                 return r;
             if (n1 >= N) {
-                r = chol64_panel(A, ld, t0, N - t0, N, nrows, st, s);   // last panel: diagonal tile + RHS rows
+                r = chol64_panel(A, ld, t0, N - t0, N, nrows, st, sync, s, true, nullptr, 0, 0, order);   // last panel: diagonal tile + RHS rows
                 if (r != cudaSuccess) return r;
                 j0 = t0;
                 continue;
             }
             if ((r = cudaEventRecord(e_upd, s)) != cudaSuccess) return r;
             if ((r = cudaStreamWaitEvent(s2, e_upd, 0)) != cudaSuccess) return r;
-            if ((r = diag(t0, n1 - t0, s2)) != cudaSuccess) return r;
+            const double left = N - n1;
+            const double rest_us = left * left * jb * S * (S + 1) / 2.0 / OZ_REST_RATE;
+            // with its updates emulated the diagonal tile is a longer chain (about 1.3 ms for 512 columns): the
+            // update's rest is the shorter side below that, and gives up SMs
+            const int side = !fused && rest_us < 5.0 * (n1 - t0) ? 48 : chol64_side_sms(n1 - t0, true, rest_us);
+            if ((r = diag(t0, n1 - t0, side, s2)) != cudaSuccess) return r;
             if ((r = cudaEventRecord(e_pan, s2)) != cudaSuccess) return r;
             // the rest of the trailing update meanwhile: rows [n1, nrows), cols [n1, N)
             if ((r = oz_update(p, p, A, ld, n1, n1, nrows - n1, N - n1, nrows, N, n1 - t0, n1 - t0, 1,
-                               all - SIDE_SMS, st, s, 0, cut)) != cudaSuccess)
+                               all - side, st, s, 0, cut)) != cudaSuccess)
                 return r;
             if ((r = cudaStreamWaitEvent(s, e_pan, 0)) != cudaSuccess) return r;
             if ((r = panel_solve(t0, n1 - t0, n1, nrows, s)) != cudaSuccess) return r;

@@ -44,7 +44,7 @@ __global__ void __launch_bounds__(RED_THREADS) k_loglik_reduce(const double *__r
             b += s2[w];
         }
         const double logdet = 2.0 * a;
-        if (st->info) {
+        if (st->info || st->timeout) {   // no factor
             res->loglik = res->logdet = res->quad = nan("");
         } else {
             res->logdet = logdet;

@@ -223,7 +223,8 @@ struct SplitKScope {
 }  // namespace
 
 cudaError_t tlr_factor(TlrFactor &F, const CovParams &cp, const double *lx, const double *ly, void *ws,
-                       size_t ws_bytes, void *arena_host, DevStatus *st, DevStatus *h_st, cudaStream_t s) {
+                       size_t ws_bytes, void *arena_host, DevStatus *st, int *sync, DevStatus *h_st,
+                       cudaStream_t s) {
     const int N = F.N, nb = F.nb, T = F.T, kmax = F.kmax, p = cp.p;
     const int rmax = std::min(kmax + 16, nb);
     if (nb % p) return cudaErrorInvalidValue;
@@ -439,7 +440,7 @@ cudaError_t tlr_factor(TlrFactor &F, const CovParams &cp, const double *lx, cons
             return launch_bgemm(gy, (int)dy.size(), gemm_tiles(dy), s, gemm_flops(dy), gemm_kmax(dy));
         }));
         // 3. diagonal tile in FP64
-        TCK(chol64_panel(W, ldw, 0, mj, mj, mj, st, s));
+        TCK(chol64_panel(W, ldw, 0, mj, mj, mj, st, sync, s));
         TCK(cudaMemcpy2DAsync(F.D + (size_t)j * nb * nb, sizeof(double) * nb, W, sizeof(double) * ldw,
                               sizeof(double) * mj, mj, cudaMemcpyDeviceToDevice, s));
         if (j == T - 1) break;
@@ -603,7 +604,7 @@ cudaError_t tlr_factor(TlrFactor &F, const CovParams &cp, const double *lx, cons
                 F.max_rank = std::max(F.max_rank, F.dense[sl] ? 0 : rk[q]);
                 if (F.dense[sl]) {
                     // L_ij = W_ij L_jj^-T in FP64 (the panel TRSM on these rows), U = L_ij, V = I
-                    TCK(chol64_panel(W, ldw, 0, mj, (i - j) * nb, (i - j) * nb + mt(i), st, s, false));
+                    TCK(chol64_panel(W, ldw, 0, mj, (i - j) * nb, (i - j) * nb + mt(i), st, sync, s, false));
                     TCK(cudaMemcpy2DAsync(Uof(i, j), sizeof(double) * nb, W + (size_t)(i - j) * nb, sizeof(double) * ldw,
                                           sizeof(double) * mt(i), mj, cudaMemcpyDeviceToDevice, s));
                     KScope kk(GEO_K_AUX, s);
