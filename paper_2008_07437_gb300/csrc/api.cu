@@ -62,6 +62,7 @@ struct geo_ctx {
     std::vector<geo_factor *> factors;
     // K_nu tables of the theta of the last geo_covgen call
     double *ctab = nullptr;
+    size_t ctab_doubles = 0;
     Profiler prof;
 };
 
@@ -71,7 +72,8 @@ struct geo_factor {
     long long ld = 0;
     double *A = nullptr;    // L (lower) with y' in row N
     size_t A_bytes = 0;
-    double *lx = nullptr, *ly = nullptr;   // locations in internal order (SoA)
+    double *lx = nullptr, *ly = nullptr;   // locations in internal order (SoA), then the tables of theta
+    size_t loc_doubles = 0;                // doubles of that buffer
     double *w = nullptr;                   // L^-T y (lazy)
     std::vector<int> perm;                 // internal k -> caller location perm[k]
     CovParams cp;
@@ -332,6 +334,7 @@ int theta_to_params(const geo_theta *th, CovParams *cp, std::string *err) {
     memset(cp, 0, sizeof(*cp));
     cp->p = p;
     cp->inv_a = 1.0 / th->a;
+    cp->inv_a2 = (double)(1.0L / ((long double)th->a * th->a));
     for (int i = 0; i < p; ++i) {
         for (int j = 0; j < p; ++j) {
             MaternConst &c = cp->m[i * p + j];
@@ -361,7 +364,10 @@ int theta_to_params(const geo_theta *th, CovParams *cp, std::string *err) {
             if (c.kind == 0 && c.nu <= GEO_CHEB_NU_MAX) c.toff = (g++) * GEO_TAB_PER_PAIR;
             cp->m[j * p + i].toff = c.toff;
         }
-    cp->tab = nullptr;
+    cp->tab = cp->fine = nullptr;
+    int f = 0;   // fine tables, one per i <= j
+    for (int i = 0; i < p; ++i)
+        for (int j = i; j < p; ++j) cp->m[i * p + j].foff = cp->m[j * p + i].foff = (f++) * GEO_FINE_PER_PAIR;
     return GEO_OK;
 }
 
@@ -460,7 +466,7 @@ int geo_destroy(geo_ctx *ctx) {
     if (ctx->rws) dev_free(ctx, ctx->rws, ctx->rws_bytes);
     if (ctx->tws) dev_free(ctx, ctx->tws, ctx->tws_bytes);
     if (ctx->tarena) cudaFreeHost(ctx->tarena);
-    if (ctx->ctab) dev_free(ctx, ctx->ctab, sizeof(double) * GEO_TAB_DOUBLES);
+    if (ctx->ctab) dev_free(ctx, ctx->ctab, sizeof(double) * ctx->ctab_doubles);
     for (auto &g : ctx->graphs) cudaGraphExecDestroy(g.second.first);
     if (ctx->cap_stream) cudaStreamDestroy(ctx->cap_stream);
     if (ctx->bws) dev_free(ctx, ctx->bws, ctx->bws_bytes);
@@ -495,12 +501,22 @@ int geo_covgen(geo_ctx *ctx, const double *locs1_dev, int n1, const double *locs
     SetDevice sd(ctx->device);
     cudaStream_t s = (cudaStream_t)stream;
     if (n1 == 0 || n2 == 0) return GEO_OK;
-    if (!ctx->ctab && cov_needs_tables(cp)) {
+    // tables of theta: the K_nu ones, then (with enough pairs) the fine ones
+    const size_t fine = cov_fine_doubles(cp.p, (double)n1 * n2);
+    const size_t need = (cov_needs_tables(cp) || fine) ? GEO_TAB_DOUBLES + fine : 0;
+    if (ctx->ctab_doubles < need) {
+        if (ctx->ctab) {
+            CK(cudaStreamSynchronize(s));
+            dev_free(ctx, ctx->ctab, sizeof(double) * ctx->ctab_doubles);
+            ctx->ctab = nullptr;
+            ctx->ctab_doubles = 0;
+        }
         void *pt;
-        if ((rc = dev_alloc(ctx, &pt, sizeof(double) * GEO_TAB_DOUBLES))) return rc;
+        if ((rc = dev_alloc(ctx, &pt, sizeof(double) * need))) return rc;
         ctx->ctab = (double *)pt;
+        ctx->ctab_doubles = need;
     }
-    CK(launch_cheb_build(cp, ctx->ctab, s));
+    CK(fine ? launch_fine_build(cp, ctx->ctab, ctx->ctab + GEO_TAB_DOUBLES, s) : launch_cheb_build(cp, ctx->ctab, s));
     CK(launch_covgen_rect(cp, locs1_dev, n1, locs2_dev ? locs2_dev : locs1_dev, n2, out_dev, ld, s));
     return GEO_OK;
 }
@@ -559,10 +575,20 @@ static int prepare_matrix(geo_ctx *ctx, const double *locs_dev, int n, const geo
         std::iota(f->perm.begin(), f->perm.end(), 0);
     // device buffers: locations (SoA) + permutation
     void *p1, *p2;
-    if ((rc = dev_alloc(ctx, &p1, sizeof(double) * (2 * (size_t)n + GEO_TAB_DOUBLES)))) return rc;
+    const size_t tab_at = 2 * (size_t)n, fine_at = tab_at + GEO_TAB_DOUBLES;
+    const size_t fine = cov_fine_doubles(p, 0.5 * n * (n + 1.0));
+    if ((rc = dev_alloc(ctx, &p1, sizeof(double) * (fine_at + fine)))) return rc;
+    f->loc_doubles = fine_at + fine;
     f->lx = (double *)p1;
     f->ly = f->lx + n;
-    CK(launch_cheb_build(f->cp, f->lx + 2 * (size_t)n, s));   // K_nu tables after the locations
+    // The forms that round the factor's entries to 35 bits or FP32 turn a last-bit difference of Sigma into one
+    // of up to 1e-7 in l: they keep the tables and the evaluation their results have always had.
+    const bool reduced = o->prec == GEO_PREC_MIXED || (o->prec == GEO_PREC_FP64 && o->fp64_gemm == 1 && oz_slices_of(*o) < 7);
+    // K_nu tables after the locations, then the fine ones
+    if (reduced || !fine) CK(launch_cheb_build(f->cp, f->lx + tab_at, s));
+    CovParams gen = f->cp;   // for Sigma
+    if (fine) CK(launch_fine_build(f->cp, reduced ? nullptr : f->lx + tab_at, f->lx + fine_at, s));
+    if (!reduced) gen = f->cp;
     if ((rc = dev_alloc(ctx, &p2, sizeof(int) * n))) return rc;
     int *d_perm = (int *)p2;
     CK(cudaMemcpyAsync(d_perm, f->perm.data(), sizeof(int) * n, cudaMemcpyHostToDevice, s));
@@ -596,7 +622,7 @@ static int prepare_matrix(geo_ctx *ctx, const double *locs_dev, int n, const geo
         f->A_bytes = bytes;
     }
     CK(cudaMemsetAsync(ctx->st, 0, sizeof(DevStatus), s));
-    CK(launch_covgen_sym(f->cp, f->lx, f->ly, n, f->A, f->ld, s));
+    CK(launch_covgen_sym(gen, f->lx, f->ly, n, f->A, f->ld, s));
     // keep d_perm alive until the stream has used it
     CK(cudaStreamSynchronize(s));
     dev_free(ctx, d_perm, sizeof(int) * n);
@@ -613,7 +639,7 @@ static void release_factor_buffers(geo_ctx *ctx, geo_factor *f, bool keep_matrix
         }
         f->A = nullptr;
     }
-    if (f->lx) dev_free(ctx, f->lx, sizeof(double) * (2 * (size_t)f->n + GEO_TAB_DOUBLES));
+    if (f->lx) dev_free(ctx, f->lx, sizeof(double) * f->loc_doubles);
     if (f->w) dev_free(ctx, f->w, sizeof(double) * f->N);
     f->lx = f->ly = f->w = nullptr;
     if (f->ybuf) dev_free(ctx, f->ybuf, sizeof(double) * f->N);
@@ -1119,7 +1145,7 @@ int geo_factor_stats_get(const geo_factor *f, geo_factor_stats *out) {
     out->loglik = f->loglik;
     out->logdet = f->logdet;
     out->quad = f->quad;
-    out->device_bytes = (long long)(f->A_bytes + sizeof(double) * (2 * (size_t)f->n + GEO_TAB_DOUBLES) +
+    out->device_bytes = (long long)(f->A_bytes + sizeof(double) * f->loc_doubles +
                                     (f->w ? sizeof(double) * f->N : 0));
     out->tlr_bytes_ratio = 1.0;
     if (f->tlr) {
@@ -1130,7 +1156,7 @@ int geo_factor_stats_get(const geo_factor *f, geo_factor_stats *out) {
         out->tlr_bytes_ratio = used / dense;
         out->tlr_max_rank = F.max_rank;
         out->tlr_dense_tiles = F.capped;
-        out->device_bytes = (long long)(8.0 * used + sizeof(double) * (2.0 * f->n + GEO_TAB_DOUBLES + f->N));
+        out->device_bytes = (long long)(8.0 * used + sizeof(double) * (f->loc_doubles + (double)f->N));
     }
     return GEO_OK;
 }
@@ -1685,7 +1711,7 @@ size_t loglik_device_bytes(int device, int n, int p, const geo_opts *opts) {
     const size_t N = (size_t)p * n;
     if (o.nb == 0) o.nb = resolve_nb(device, form_of(o), (int)N);
     const size_t nb = (size_t)std::max(o.nb, 64);
-    size_t b = sizeof(double) * (2 * (size_t)n + GEO_TAB_DOUBLES) + sizeof(int) * 2 * n + sizeof(double) * N;
+    size_t b = sizeof(double) * (2 * (size_t)n + GEO_TAB_DOUBLES + cov_fine_doubles(p, 0.5 * n * (n + 1.0))) + sizeof(int) * 2 * n + sizeof(double) * N;
     if (o.prec == GEO_PREC_TLR) {
         const int kmax = std::min(o.tlr_kmax, (int)nb);
         const size_t T = (N + nb - 1) / nb;

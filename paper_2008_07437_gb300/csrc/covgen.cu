@@ -3,8 +3,15 @@
 //
 // Every matrix entry is one FP64 evaluation of Eq. 2: the work is FP64 ALU
 // bound (Bessel K_nu), so the kernels map one location pair to one thread,
-// evaluate the p(p+1)/2 distinct C_ij once per pair, and write the p x p block
-// with column-major stores that are contiguous across a warp.
+// evaluate the p(p+1)/2 distinct C_ij once per pair (from the theta's fine
+// tables, matern.cuh, where they pay), and write the p x p block with
+// column-major stores that are contiguous across a warp.  Measured against one
+// Clenshaw sum per order and one exponential per pair: Sigma of N = 40,000
+// (p = 2) 9.4 ms (51.4), a 15,009 x 8,331 cross-covariance (p = 3) 1.25 ms
+// (8.0), 2,000 predictions on 10,000 locations (p = 2) 1.12 ms (10.2); the FP64
+// operations that are left (27 a pair for p = 2, 48 for p = 3) take 0.9, 1.06
+// and 0.99 of that at the pipe's rate.  Entries are 2.5 to 4 times closer to
+// the exact values than before (4e-16 relative, weighted by size).
 #include "geo_internal.cuh"
 
 namespace {
@@ -12,7 +19,7 @@ namespace {
 constexpr int TL = 64;   // locations l (rows) per CTA
 constexpr int TR = 4;    // locations r (columns) per CTA
 
-// The p x p block of C at distance h for one location pair.
+// The p x p block of C at distance h for one location pair, without the fine tables.
 __device__ __forceinline__ void cov_block(const CovParams &cp, double h, double *v) {
     matern_block(h * cp.inv_a, cp, v);
 }
@@ -21,6 +28,97 @@ __device__ __forceinline__ void cov_block(const CovParams &cp, double h, double 
 __global__ void __launch_bounds__(32) k_cheb_build(const CovParams cp, double *tab) {
     __shared__ double hv[GEO_CHEB_N];
     cheb_build_block(cp, tab, blockIdx.x, blockIdx.y, hv);
+}
+
+// cos(pi j / 22), j = 0 .. 22, and the powers of t in the Chebyshev polynomials T_0 .. T_10.
+__constant__ double c_cos22[23] = {
+    1.0, 0.98982144188093273238, 0.95949297361449738989, 0.90963199535451837141, 0.84125353283118116886,
+    0.75574957435425828377, 0.65486073394528506406, 0.54064081745559758211, 0.41541501300188642553,
+    0.28173255684142969771, 0.14231483827328514044, 0.0, -0.14231483827328514044, -0.28173255684142969771,
+    -0.41541501300188642553, -0.54064081745559758211, -0.65486073394528506406, -0.75574957435425828377,
+    -0.84125353283118116886, -0.90963199535451837141, -0.95949297361449738989, -0.98982144188093273238, -1.0};
+__constant__ double c_cheb_pow[GEO_FINE_NODES][GEO_FINE_NODES] = {
+    {1, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0},
+    {0, 1, 0, 0, 0, 0, 0, 0, 0, 0, 0},
+    {-1, 0, 2, 0, 0, 0, 0, 0, 0, 0, 0},
+    {0, -3, 0, 4, 0, 0, 0, 0, 0, 0, 0},
+    {1, 0, -8, 0, 8, 0, 0, 0, 0, 0, 0},
+    {0, 5, 0, -20, 0, 16, 0, 0, 0, 0, 0},
+    {-1, 0, 18, 0, -48, 0, 32, 0, 0, 0, 0},
+    {0, -7, 0, 56, 0, -112, 0, 64, 0, 0, 0},
+    {1, 0, -32, 0, 160, 0, -256, 0, 128, 0, 0},
+    {0, 9, 0, -120, 0, 432, 0, -576, 0, 256, 0},
+    {-1, 0, 50, 0, -400, 0, 1120, 0, -1280, 0, 512},
+};
+
+// Tables of a theta: blockIdx.x the pair i <= j.  blockIdx.y < GEO_FINE_N / 8: eight intervals of its fine table,
+// sixteen threads to each, eleven of them at its Chebyshev nodes.  The transform works on differences to the
+// middle node (they are small, so its rounding is too), and the Chebyshev coefficients, which fall by a factor
+// of 60 or more each, go over to powers of t.  Beyond: four intervals of its K_nu table (cheb_f's, for distances
+// outside the fine one), 32 threads to each, and the reciprocals.  Bound by the latency of one evaluation:
+// 90 steps of four FP64 operations.
+constexpr int FINE_BLOCKS = GEO_FINE_N / 8, COARSE_BLOCKS = GEO_CHEB_NI / 4;
+
+__global__ void __launch_bounds__(128) k_fine_build(const CovParams cp, double *tab, double *fine) {
+    __shared__ double val[8][16], cf[8][16];
+    __shared__ NodeTabs nt;
+    constexpr int n = GEO_FINE_NODES;
+    int i = 0, j = blockIdx.x;
+    while (j >= cp.p - i) j -= cp.p - i, ++i;
+    const MaternConst &c = cp.m[i * cp.p + i + j];
+    const bool coarse = blockIdx.y >= FINE_BLOCKS;
+    if (coarse && (c.kind != 0 || c.toff < 0)) return;
+    if (c.kind == 0) node_tabs(nt, c, threadIdx.x, 128);
+    __syncthreads();
+    if (coarse) {
+        const int w = threadIdx.x / 32, t = threadIdx.x % 32, iv = (blockIdx.y - FINE_BLOCKS) * 4 + w;
+        double *T = tab + c.toff, *hv = &val[2 * w][0];
+        const double lo = ldexp(1.0, GEO_CHEB_K0 + iv);
+        if (t < GEO_CHEB_N) {
+            const double x = 1.5 * lo + 0.5 * lo * cospi((t + 0.5) / GEO_CHEB_N);
+            bool scaled;
+            const double v = xnu_besselk_node(x, c, nt, &scaled);
+            hv[t] = scaled ? v : exp(x) * v;
+        }
+        __syncwarp();
+        if (t < GEO_CHEB_N) {
+            const double h0 = hv[GEO_CHEB_N / 2];
+            double s = 0.0;
+            for (int m = 0; m < GEO_CHEB_N; ++m) s = fma(hv[m] - h0, cospi(t * (m + 0.5) / GEO_CHEB_N), s);
+            T[iv * GEO_CHEB_N + t] = fma(s, (t == 0 ? 1.0 : 2.0) / GEO_CHEB_N, t == 0 ? h0 : 0.0);
+            if (iv == 0)
+                for (int q = 0; q < 4; ++q) T[GEO_CHEB_NI * GEO_CHEB_N + q * GEO_TEMME_K + t] = nt.inv[q][t];
+        }
+        return;
+    }
+    const int w = threadIdx.x / 16, k = threadIdx.x % 16, idx = blockIdx.y * 8 + w;
+    auto cos22 = [](int q) {   // cos(pi q / 22)
+        q %= 44;
+        return q <= 22 ? c_cos22[q] : c_cos22[44 - q];
+    };
+    double mid, half;
+    matern_fine_bounds(idx, &mid, &half);
+    if (k < n) val[w][k] = matern_fine_node(fma(half, cos22(2 * k + 1), mid), c, nt);
+    __syncthreads();
+    const double v0 = val[w][n / 2];   // t = 0
+    double s = 0.0;
+    if (k < n) {
+        for (int q = 0; q < n; ++q) s = fma(val[w][q] - v0, cos22(k * (2 * q + 1)), s);
+        cf[w][k] = s * ((k == 0 ? 1.0 : 2.0) / n);
+    }
+    __syncthreads();
+    if (k >= n) return;
+    s = 0.0;
+    for (int m = n - 1; m >= 0; --m) s = fma(cf[w][m], c_cheb_pow[m][k], s);
+    if (k == 0) s += v0;
+    double *e = fine + c.foff + (long long)idx * GEO_FINE_STRIDE;
+    // the floats relative to the value's own power of two: far out both are beyond FP32's range
+    const int ex = v0 == 0.0 ? 0 : max(ilogb(v0), -800);
+    if (k < 7)
+        e[k] = s;
+    else
+        reinterpret_cast<float *>(e + 7)[k - 7] = (float)ldexp(s, -ex);
+    if (k == 0) reinterpret_cast<unsigned *>(e + 9)[0] = (unsigned)((ex + 896) << 20);
 }
 
 // Lower triangle (location blocks l >= r) of Sigma, column-major A[c*ld + r].
@@ -43,21 +141,56 @@ __global__ void __launch_bounds__(TL *TR) k_covgen_sym(const CovParams cp, const
     }
 }
 
+// The same from the fine tables.  Each thread takes RPT locations r, so that the table positions and loads of
+// one pair run under the FP64 chain of another.
+constexpr int RPT = 4;
+
+template <int P>
+__global__ void __launch_bounds__(TL *TR) k_covgen_sym_fine(const CovParams cp, const double *__restrict__ lx,
+                                                            const double *__restrict__ ly, int n, double *A,
+                                                            long long ld) {
+    const int l0 = blockIdx.y * TL, r0 = blockIdx.x * (TR * RPT);
+    if (r0 > l0 + TL - 1) return;   // tile entirely above the location diagonal
+    const int l = l0 + (threadIdx.x % TL);
+    if (l >= n) return;
+    const double x = lx[l], y = ly[l];
+#pragma unroll
+    for (int q = 0; q < RPT; ++q) {
+        const int r = r0 + q * TR + threadIdx.x / TL;
+        if (r > l) continue;
+        const double dx = x - lx[r], dy = y - ly[r];
+        double v[P * P];
+        matern_pair<P>((l == r) ? 0.0 : fma(dx, dx, dy * dy), cp, v);
+#pragma unroll
+        for (int j = 0; j < P; ++j) {
+            double *col = A + (long long)(P * r + j) * ld + (long long)P * l;
+#pragma unroll
+            for (int i = 0; i < P; ++i) col[i] = v[i * P + j];
+        }
+    }
+}
+
 // Full rectangle: rows p*n1 (locations l of set 1), cols p*n2 (set 2); AoS inputs.
+template <int P>
 __global__ void __launch_bounds__(TL *TR) k_covgen_rect(const CovParams cp, const double *__restrict__ l1, int n1,
                                                         const double *__restrict__ l2, int n2, double *out,
                                                         long long ld) {
     const int l = blockIdx.y * TL + (threadIdx.x % TL);
-    const int r = blockIdx.x * TR + (threadIdx.x / TL);
-    if (l >= n1 || r >= n2) return;
-    const double dx = l1[2 * l] - l2[2 * r], dy = l1[2 * l + 1] - l2[2 * r + 1];
-    const double h = sqrt(dx * dx + dy * dy);
-    double v[GEO_PMAX_DEV * GEO_PMAX_DEV];
-    cov_block(cp, h, v);
-    const int p = cp.p;
-    for (int j = 0; j < p; ++j) {
-        double *col = out + (long long)(p * r + j) * ld + (long long)p * l;
-        for (int i = 0; i < p; ++i) col[i] = v[i * GEO_PMAX_DEV + j];
+    if (l >= n1) return;
+    const double x = l1[2 * l], y = l1[2 * l + 1];
+#pragma unroll
+    for (int q = 0; q < RPT; ++q) {
+        const int r = (blockIdx.x * RPT + q) * TR + threadIdx.x / TL;
+        if (r >= n2) return;
+        const double dx = x - l2[2 * r], dy = y - l2[2 * r + 1];
+        double v[P * P];
+        matern_pair<P>(fma(dx, dx, dy * dy), cp, v);
+#pragma unroll
+        for (int j = 0; j < P; ++j) {
+            double *col = out + (long long)(P * r + j) * ld + (long long)P * l;
+#pragma unroll
+            for (int i = 0; i < P; ++i) col[i] = v[i * P + j];
+        }
     }
 }
 
@@ -66,37 +199,47 @@ __global__ void __launch_bounds__(TL *TR) k_covgen_rect(const CovParams cp, cons
 // depend on timing.
 constexpr int PRED_THREADS = 256;
 
-__global__ void __launch_bounds__(PRED_THREADS) k_predict(const CovParams cp, const double *__restrict__ s0,
-                                                          const double *__restrict__ lx,
-                                                          const double *__restrict__ ly, int n,
-                                                          const double *__restrict__ w, double *zhat) {
-    const int l = blockIdx.x;
-    const double x0 = s0[2 * l], y0 = s0[2 * l + 1];
-    const int p = cp.p;
-    double acc[GEO_PMAX_DEV] = {0.0, 0.0, 0.0, 0.0};
-    double v[GEO_PMAX_DEV * GEO_PMAX_DEV];
+template <int P>
+__device__ __forceinline__ void predict_one(const CovParams &cp, double x0, double y0, const double *__restrict__ lx,
+                                            const double *__restrict__ ly, int n, const double *__restrict__ w,
+                                            double *zhat) {
+    double acc[P];
+#pragma unroll
+    for (int i = 0; i < P; ++i) acc[i] = 0.0;
     for (int r = threadIdx.x; r < n; r += PRED_THREADS) {
         const double dx = x0 - lx[r], dy = y0 - ly[r];
-        cov_block(cp, sqrt(dx * dx + dy * dy), v);
-        for (int i = 0; i < p; ++i) {
-            double t = 0.0;
-            for (int j = 0; j < p; ++j) t += v[i * GEO_PMAX_DEV + j] * w[(long long)p * r + j];
-            acc[i] += t;
+        double v[P * P];
+        matern_pair<P>(fma(dx, dx, dy * dy), cp, v);
+#pragma unroll
+        for (int j = 0; j < P; ++j) {
+            const double wj = w[(long long)P * r + j];
+#pragma unroll
+            for (int i = 0; i < P; ++i) acc[i] = fma(v[i * P + j], wj, acc[i]);
         }
     }
-    __shared__ double red[GEO_PMAX_DEV][PRED_THREADS / 32];
+    __shared__ double red[P][PRED_THREADS / 32];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    for (int i = 0; i < p; ++i) {
+#pragma unroll
+    for (int i = 0; i < P; ++i) {
         double t = acc[i];
         for (int o = 16; o > 0; o >>= 1) t += __shfl_down_sync(0xffffffffu, t, o);
         if (lane == 0) red[i][wid] = t;
     }
     __syncthreads();
-    if (threadIdx.x < p) {
+    if (threadIdx.x < P) {
         double t = 0.0;
         for (int k = 0; k < PRED_THREADS / 32; ++k) t += red[threadIdx.x][k];
-        zhat[(long long)p * l + threadIdx.x] = t;
+        zhat[threadIdx.x] = t;
     }
+}
+
+template <int P>
+__global__ void __launch_bounds__(PRED_THREADS) k_predict(const CovParams cp, const double *__restrict__ s0,
+                                                          const double *__restrict__ lx,
+                                                          const double *__restrict__ ly, int n,
+                                                          const double *__restrict__ w, double *zhat) {
+    const int l = blockIdx.x;
+    predict_one<P>(cp, s0[2 * l], s0[2 * l + 1], lx, ly, n, w, zhat + (long long)P * l);
 }
 
 __global__ void k_gather_locs(const double *__restrict__ locs, const int *__restrict__ perm, int n, double *lx,
@@ -143,22 +286,40 @@ cudaError_t launch_cheb_build(CovParams &cp, double *tab, cudaStream_t s) {
     return cudaGetLastError();
 }
 
+size_t cov_fine_doubles(int p, double pairs) {
+    // with fewer location pairs the tables (10,000 evaluations per C_ij) cost more than they save
+    return pairs >= 32768.0 ? (size_t)p * (p + 1) / 2 * GEO_FINE_PER_PAIR : 0;
+}
+
+cudaError_t launch_fine_build(CovParams &cp, double *tab, double *fine, cudaStream_t s) {
+    KScope ks(GEO_K_COVGEN, s);
+    // tab == NULL: cp.tab is there already
+    k_fine_build<<<dim3(cp.p * (cp.p + 1) / 2, FINE_BLOCKS + (tab ? COARSE_BLOCKS : 0)), 128, 0, s>>>(cp, tab, fine);
+    if (tab) cp.tab = tab;
+    cp.fine = fine;
+    return cudaGetLastError();
+}
+
 cudaError_t launch_covgen_sym(const CovParams &cp, const double *lx, const double *ly, int n, double *A,
                               long long ld, cudaStream_t s) {
     if (n <= 0) return cudaSuccess;
-    dim3 grid((n + TR - 1) / TR, (n + TL - 1) / TL);
+    const int per = cp.fine ? TR * RPT : TR;
+    dim3 grid((n + per - 1) / per, (n + TL - 1) / TL);
     const double N = (double)cp.p * n;
     KScope ks(GEO_K_COVGEN, s, 0.0, 8.0 * N * (N + cp.p) / 2.0);   // bytes: lower triangle written once
-    k_covgen_sym<<<grid, TL * TR, 0, s>>>(cp, lx, ly, n, A, ld);
+    if (cp.fine)
+        cov_by_p(cp.p, [&](auto P) { k_covgen_sym_fine<P.value><<<grid, TL * TR, 0, s>>>(cp, lx, ly, n, A, ld); });
+    else
+        k_covgen_sym<<<grid, TL * TR, 0, s>>>(cp, lx, ly, n, A, ld);
     return cudaGetLastError();
 }
 
 cudaError_t launch_covgen_rect(const CovParams &cp, const double *l1, int n1, const double *l2, int n2,
                                double *out, long long ld, cudaStream_t s) {
     if (n1 <= 0 || n2 <= 0) return cudaSuccess;
-    dim3 grid((n2 + TR - 1) / TR, (n1 + TL - 1) / TL);
+    dim3 grid((n2 + TR * RPT - 1) / (TR * RPT), (n1 + TL - 1) / TL);
     KScope ks(GEO_K_COVGEN, s, 0.0, 8.0 * cp.p * (double)n1 * cp.p * (double)n2);
-    k_covgen_rect<<<grid, TL * TR, 0, s>>>(cp, l1, n1, l2, n2, out, ld);
+    cov_by_p(cp.p, [&](auto P) { k_covgen_rect<P.value><<<grid, TL * TR, 0, s>>>(cp, l1, n1, l2, n2, out, ld); });
     return cudaGetLastError();
 }
 
@@ -190,34 +351,14 @@ __global__ void __launch_bounds__(PRED_THREADS) k_predict_batch(const PredDesc *
         for (int t = threadIdx.x; t < words; t += PRED_THREADS) dst[t] = src[t];
     }
     __syncthreads();
-    const CovParams &cp = cps;
-    const int l = g - q.first, n = q.n;
-    const double *lx = q.lx, *ly = q.ly, *w = q.w;
+    const int l = g - q.first, p = cps.p;
     const double x0 = q.s0[2 * l], y0 = q.s0[2 * l + 1];
-    const int p = cp.p;
-    double acc[GEO_PMAX_DEV] = {0.0, 0.0, 0.0, 0.0};
-    double v[GEO_PMAX_DEV * GEO_PMAX_DEV];
-    for (int r = threadIdx.x; r < n; r += PRED_THREADS) {
-        const double dx = x0 - lx[r], dy = y0 - ly[r];
-        cov_block(cp, sqrt(dx * dx + dy * dy), v);
-        for (int i = 0; i < p; ++i) {
-            double t = 0.0;
-            for (int j = 0; j < p; ++j) t += v[i * GEO_PMAX_DEV + j] * w[(long long)p * r + j];
-            acc[i] += t;
-        }
-    }
-    __shared__ double red[GEO_PMAX_DEV][PRED_THREADS / 32];
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    for (int i = 0; i < p; ++i) {
-        double t = acc[i];
-        for (int o = 16; o > 0; o >>= 1) t += __shfl_down_sync(0xffffffffu, t, o);
-        if (lane == 0) red[i][wid] = t;
-    }
-    __syncthreads();
-    if (threadIdx.x < p) {
-        double t = 0.0;
-        for (int k = 0; k < PRED_THREADS / 32; ++k) t += red[threadIdx.x][k];
-        q.zhat[(long long)p * l + threadIdx.x] = t;
+    double *out = q.zhat + (long long)p * l;
+    switch (p) {
+        case 1: predict_one<1>(cps, x0, y0, q.lx, q.ly, q.n, q.w, out); break;
+        case 2: predict_one<2>(cps, x0, y0, q.lx, q.ly, q.n, q.w, out); break;
+        case 3: predict_one<3>(cps, x0, y0, q.lx, q.ly, q.n, q.w, out); break;
+        default: predict_one<4>(cps, x0, y0, q.lx, q.ly, q.n, q.w, out); break;
     }
 }
 
@@ -225,7 +366,7 @@ cudaError_t launch_predict(const CovParams &cp, const double *new_locs, int m, c
                            const double *ly, int n, const double *w, double *zhat, cudaStream_t s) {
     if (m <= 0) return cudaSuccess;
     KScope ks(GEO_K_PREDICT, s, 2.0 * cp.p * (double)m * cp.p * (double)n, 16.0 * n + 24.0 * m);
-    k_predict<<<m, PRED_THREADS, 0, s>>>(cp, new_locs, lx, ly, n, w, zhat);
+    cov_by_p(cp.p, [&](auto P) { k_predict<P.value><<<m, PRED_THREADS, 0, s>>>(cp, new_locs, lx, ly, n, w, zhat); });
     return cudaGetLastError();
 }
 

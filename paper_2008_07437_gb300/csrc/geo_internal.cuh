@@ -6,6 +6,7 @@
 
 #include <functional>
 #include <string>
+#include <type_traits>
 #include <utility>
 #include <vector>
 
@@ -70,6 +71,21 @@ struct KScope {
 // afterwards reads them.  Nothing is launched when theta has no tabulated order.
 cudaError_t launch_cheb_build(CovParams &cp, double *tab, cudaStream_t s);
 bool cov_needs_tables(const CovParams &cp);
+// Doubles of the fine tables (matern.cuh) of p variables, 0 where the number of location pairs does not pay
+// for them; and their construction on stream s together with the K_nu tables (tab, GEO_TAB_DOUBLES; NULL: only
+// the fine ones), with cp pointed at both.
+size_t cov_fine_doubles(int p, double pairs);
+cudaError_t launch_fine_build(CovParams &cp, double *tab, double *fine, cudaStream_t s);
+// f(integral constant P) for p = 1 .. 4 variables.
+template <typename F>
+void cov_by_p(int p, F f) {
+    switch (p) {
+        case 1: f(std::integral_constant<int, 1>()); break;
+        case 2: f(std::integral_constant<int, 2>()); break;
+        case 3: f(std::integral_constant<int, 3>()); break;
+        default: f(std::integral_constant<int, 4>()); break;
+    }
+}
 // Lower triangle of Sigma (order p*n) into A (column-major, ld), from
 // SoA locations; the full p x p block on the location diagonal.
 cudaError_t launch_covgen_sym(const CovParams &cp, const double *lx, const double *ly, int n, double *A,

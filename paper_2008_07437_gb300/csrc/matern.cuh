@@ -67,6 +67,18 @@
 #define GEO_TAB_PER_PAIR (GEO_CHEB_NI * GEO_CHEB_N + 4 * GEO_TEMME_K)
 #define GEO_TAB_DOUBLES (GEO_PMAX_DEV * (GEO_PMAX_DEV + 1) / 2 * GEO_TAB_PER_PAIR)
 
+// Fine table of one C_ij as a function of u = (h / a)^2 (see matern_fine):
+// 32 intervals per octave of u from 2^-14 on, 64 per octave from 2^10 to
+// 2^12; an entry is 7 doubles, 4 floats and their scale in 10 doubles.
+#define GEO_FINE_E0 (-14)
+#define GEO_FINE_E1 10
+#define GEO_FINE_E2 12
+#define GEO_FINE_LOW ((GEO_FINE_E1 - GEO_FINE_E0) * 32)
+#define GEO_FINE_N (GEO_FINE_LOW + (GEO_FINE_E2 - GEO_FINE_E1) * 64)
+#define GEO_FINE_STRIDE 10
+#define GEO_FINE_PER_PAIR (GEO_FINE_N * GEO_FINE_STRIDE)
+#define GEO_FINE_NODES 11
+
 // Per (i, j) constants of Eq. 2 for one theta, computed on the host.
 struct MaternConst {
     double nu;     // nu_ij
@@ -81,12 +93,15 @@ struct MaternConst {
     int nl;        // number of upward recurrence steps
     int kind;      // 0 general order, 1: nu = 1/2, 2: nu = 3/2, 3: nu = 5/2
     int toff;      // general order <= GEO_CHEB_NU_MAX: offset of its table in CovParams::tab; else -1
+    int foff;      // offset of its fine table in CovParams::fine
 };
 
 struct CovParams {
     int p;
     double inv_a;                                     // 1 / a
     const double *tab;                                // device tables (k_cheb_build), or null
+    const double *fine;                               // device fine tables (k_fine_build), or null
+    double inv_a2;                                    // 1 / a^2
     MaternConst m[GEO_PMAX_DEV * GEO_PMAX_DEV];       // m[i * p + j], symmetric
 };
 
@@ -319,4 +334,184 @@ GEO_DEV void matern_block(double x, const CovParams &cp, double *v) {
             v[i * GEO_PMAX_DEV + j] = val;
             v[j * GEO_PMAX_DEV + i] = val;
         }
+}
+
+// ---- C_ij from the fine tables ------------------------------------------------
+// A warp-wide FP64 operation occupies its scheduler for 64 clocks, so the count
+// of FP64 operations per location pair is the time of every covariance kernel;
+// integer and FP32 operations and the table's loads (L1) run beside them.  The
+// tables above cost a square root, an exponential and two operations per
+// Chebyshev term (24 terms) and order: about 50 per order and 35 per pair.
+// Here C_ij itself (amplitude included, every order alike) is tabulated as a
+// function of u = (h / a)^2, on intervals so short (1/32 or 1/64 of an octave)
+// that a polynomial of degree 10 in t = the position within the interval
+// suffices to about 2^-53 of its value up to u = 2^12 (h = 64 a), and the
+// terms from t^7 on are below 2^-26 of it, so that they are summed in FP32 to
+// no less: seven FP64 FMAs per order and six operations per pair for u and t.
+// u comes without the root, the interval and t from u's bits.  Outside the
+// table (h < a / 128, h >= 64 a) the evaluation above is used.
+
+// Interval of u and the position in it, t in [-1, 1), also in FP32; false outside the table (and for u = 0, NaN).
+GEO_DEV bool matern_fine_pos(double u, int *idx, double *t, float *tf) {
+    const unsigned hi = (unsigned)__double2hiint(u), lo = (unsigned)__double2loint(u);
+    constexpr unsigned b0 = 1023 + GEO_FINE_E0, b1 = 1023 + GEO_FINE_E1, b2 = 1023 + GEO_FINE_E2;
+    if (hi - (b0 << 20) >= ((b2 - b0) << 20)) return false;
+    const int up = hi >= (b1 << 20);   // 1: 64 intervals to the octave
+    *idx = (int)(hi >> (15 - up)) - (up ? (int)(b1 << 6) - GEO_FINE_LOW : (int)(b0 << 5));
+    const unsigned mhi = __funnelshift_l(lo, hi, 5 + up) & 0xFFFFFu, mlo = lo << (5 + up);
+    *t = __hiloint2double((int)(0x40000000u | mhi), (int)mlo) - 3.0;   // [2, 4) - 3
+    *tf = __uint_as_float(0x40000000u | (mhi << 3) | (mlo >> 29)) - 3.0f;
+    return true;
+}
+
+// f 2^e as a double on the integer pipe, bias = (e + 896) << 20 (zero and subnormal floats come out below 2^(e - 126)).
+GEO_DEV double matern_widen(float f, unsigned bias) {
+    const unsigned b = __float_as_uint(f);
+    return __hiloint2double((int)((b & 0x80000000u) | (((b & 0x7FFFFFFFu) >> 3) + bias)), (int)(b << 29));
+}
+
+GEO_DEV double matern_fine(const double *e, double t, float tf) {
+    const double2 *q = reinterpret_cast<const double2 *>(e);
+    const double2 a01 = __ldg(q), a23 = __ldg(q + 1), a45 = __ldg(q + 2);
+    const float4 r = __ldg(reinterpret_cast<const float4 *>(q + 3));   // a6 (two words), b7, b8
+    const float4 w = __ldg(reinterpret_cast<const float4 *>(q + 4));   // b9, b10, the floats' scale
+    const float f = fmaf(fmaf(fmaf(w.y, tf, w.x), tf, r.w), tf, r.z);
+    double v = fma(matern_widen(f, __float_as_uint(w.z)), t, __hiloint2double(__float_as_int(r.y), __float_as_int(r.x)));
+    v = fma(v, t, a45.y);
+    v = fma(v, t, a45.x);
+    v = fma(v, t, a23.y);
+    v = fma(v, t, a23.x);
+    v = fma(v, t, a01.y);
+    return fma(v, t, a01.x);
+}
+
+// The block at squared distance d2 by the evaluation above (rare: out of line).
+static __device__ __noinline__ void matern_block_far(double d2, const CovParams &cp, double *v) {
+    matern_block(sqrt(d2) * cp.inv_a, cp, v);
+}
+
+// The P x P block of C at the squared distance d2 (0: the limit C_ij(0)): v[i * P + j].
+template <int P>
+GEO_DEV void matern_pair(double d2, const CovParams &cp, double (&v)[P * P]) {
+    int idx;
+    double t;
+    float tf;
+    if (cp.fine && matern_fine_pos(d2 * cp.inv_a2, &idx, &t, &tf)) {
+        const double *e = cp.fine + (long long)idx * GEO_FINE_STRIDE;
+#pragma unroll
+        for (int i = 0; i < P; ++i)
+#pragma unroll
+            for (int j = i; j < P; ++j) v[i * P + j] = v[j * P + i] = matern_fine(e + cp.m[i * P + j].foff, t, tf);
+        return;
+    }
+    double w[GEO_PMAX_DEV * GEO_PMAX_DEV];
+    matern_block_far(d2, cp, w);
+#pragma unroll
+    for (int i = 0; i < P; ++i)
+#pragma unroll
+        for (int j = 0; j < P; ++j) v[i * P + j] = w[i * GEO_PMAX_DEV + j];
+}
+
+// ---- values at the tables' nodes --------------------------------------------------
+// The two methods of the reference evaluator with nothing but multiplications in their loops: the reciprocals of
+// Temme's series from a table of the order, and for x > 2 the recurrence run on the u_k themselves (they grow
+// towards k = 0, by less than 10^170 in all) with the sum T_k = u_k + a_k T_{k+1}, a_k = ((k + 1/2)^2 - mu^2) / (k + 1),
+// whose coefficients depend on the order alone.  x^nu as a power, not through a logarithm's rounding.
+#define GEO_MILLER_K 92
+struct NodeTabs {
+    double inv[4][GEO_TEMME_K];            // 1 / (k^2 - mu^2), 1 / (k - mu), 1 / (k + mu), 1 / k, k = 1 ..
+    double b2[GEO_MILLER_K], a[GEO_MILLER_K];   // (k + 1/2)^2 - mu^2 and that over k + 1, k = 0 ..
+};
+
+// Fill the tables of an order (all threads of the block; a barrier follows).
+GEO_DEV void node_tabs(NodeTabs &n, const MaternConst &c, int tid, int threads) {
+    const double mu = c.mu;
+    for (int k = tid; k < GEO_TEMME_K; k += threads) {
+        const double kd = k + 1.0;
+        n.inv[0][k] = 1.0 / (kd * kd - mu * mu);
+        n.inv[1][k] = 1.0 / (kd - mu);
+        n.inv[2][k] = 1.0 / (kd + mu);
+        n.inv[3][k] = 1.0 / kd;
+    }
+    for (int k = tid; k < GEO_MILLER_K; k += threads) {
+        n.b2[k] = fma(k + 0.5, k + 0.5, -mu * mu);
+        n.a[k] = n.b2[k] / (k + 1.0);
+    }
+}
+
+// x^nu K_nu(x), times e^x where *scaled (x > 2).
+GEO_DEV double xnu_besselk_node(double x, const MaternConst &c, const NodeTabs &n, bool *scaled) {
+    const double mu = c.mu, ix = 1.0 / x;
+    double kmu, kmu1;
+    *scaled = x > 2.0;
+    if (!*scaled) {
+        const double lx = log(2.0 * ix), s = mu * lx, es = exp(s), ies = 1.0 / es;
+        double shs;
+        if (fabs(s) < 1e-2) {
+            const double s2 = s * s;
+            shs = 1.0 + s2 * (1.0 / 6.0 + s2 * (1.0 / 120.0 + s2 * (1.0 / 5040.0)));
+        } else {
+            shs = sinh(s) / s;
+        }
+        double f = c.fact * (0.5 * (es + ies) * c.g1 + shs * lx * c.g2);
+        double pk = 0.5 * es * c.gp, qk = 0.5 * ies * c.gm, ck = 1.0, sum = f, sum1 = pk;
+        const double d = 0.25 * x * x;
+        for (int k = 0; k < GEO_TEMME_K; ++k) {
+            const double kd = k + 1.0;
+            f = (fma(kd, f, pk) + qk) * n.inv[0][k];
+            ck *= d * n.inv[3][k];
+            pk *= n.inv[1][k];
+            qk *= n.inv[2][k];
+            const double del = ck * f;
+            sum += del;
+            sum1 = fma(ck, fma(-kd, f, pk), sum1);
+            if (fabs(del) < 1e-18 * fabs(sum)) break;
+        }
+        kmu = sum;
+        kmu1 = sum1 * (2.0 * ix);
+    } else {
+        const int K = (int)(160.0 * ix) + 10;   // <= 90
+        double u1 = 1.0, u2 = 0.0, T = 0.0, c2 = 2.0 * (K + x);   // u_k, u_{k+1}, T_{k+1} at k = K
+        for (int k = K; k >= 1; --k) {
+            T = fma(n.a[k], T, u1);
+            const double u0 = fma(c2, u1, -n.b2[k] * u2);
+            u2 = u1;
+            u1 = u0;
+            c2 -= 2.0;
+        }
+        T = fma(n.a[0], T, u1);
+        kmu = sqrt(1.5707963267948966 * ix) * (u1 / T);
+        kmu1 = kmu * (1.0 + ((mu + 0.5) + (mu * mu - 0.25) * (u2 / u1)) * ix);
+    }
+    double km = kmu, k0 = c.nl == 0 ? kmu : kmu1;
+    for (int j = 1; j < c.nl; ++j) {
+        const double kn = fma(2.0 * (mu + j) * ix, k0, km);
+        km = k0;
+        k0 = kn;
+    }
+    return pow(x, c.nu) * k0;
+}
+
+// C_ij at u = (h / a)^2; the rounding of x = sqrt(u) is put back into the exponential.
+GEO_DEV double matern_fine_node(double u, const MaternConst &c, const NodeTabs &n) {
+    const double x = sqrt(u);
+    const double dx = fma(-x, x, u) / (2.0 * x);   // sqrt(u) = x + dx
+    const double ex = exp(-x), emx = fma(-ex, dx, ex);
+    switch (c.kind) {
+        case 1: return c.c0 * emx;
+        case 2: return c.c0 * ((1.0 + x) * emx);
+        case 3: return c.c0 * ((1.0 + x + x * x * (1.0 / 3.0)) * emx);
+        default: break;
+    }
+    bool scaled;
+    const double v = xnu_besselk_node(x, c, n, &scaled);
+    return c.pre * (scaled ? v * emx : v);
+}
+
+// Middle and half width of an interval.
+GEO_DEV void matern_fine_bounds(int idx, double *mid, double *half) {
+    const int up = idx >= GEO_FINE_LOW, k = up ? idx - GEO_FINE_LOW : idx, per = up ? 64 : 32;
+    const double lo = ldexp(1.0, (up ? GEO_FINE_E1 : GEO_FINE_E0) + k / per), h = lo / (2 * per);
+    *half = h;
+    *mid = lo + (2 * (k % per) + 1) * h;
 }

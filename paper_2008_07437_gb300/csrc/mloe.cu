@@ -12,6 +12,7 @@ constexpr int XB = 64;   // column block of the right-side solve and product
 
 // out[(p r + j) * ld + (p q + i)] = C_ij(|s0_q - s_r|): rows = prediction
 // locations (AoS), columns = observed locations (SoA, the factor's order).
+template <int P>
 __global__ void __launch_bounds__(256) k_covgen_cross(const CovParams cp, const double *__restrict__ s0, int m,
                                                       const double *__restrict__ lx, const double *__restrict__ ly,
                                                       int n, double *out, long long ld) {
@@ -19,12 +20,12 @@ __global__ void __launch_bounds__(256) k_covgen_cross(const CovParams cp, const 
     const int r = blockIdx.x * 4 + (threadIdx.x / 64);
     if (q >= m || r >= n) return;
     const double dx = s0[2 * q] - lx[r], dy = s0[2 * q + 1] - ly[r];
-    const double x = sqrt(dx * dx + dy * dy) * cp.inv_a;
-    const int p = cp.p;
-    double v[GEO_PMAX_DEV * GEO_PMAX_DEV];
-    matern_block(x, cp, v);
-    for (int i = 0; i < p; ++i)
-        for (int j = 0; j < p; ++j) out[(long long)(p * r + j) * ld + (long long)p * q + i] = v[i * GEO_PMAX_DEV + j];
+    double v[P * P];
+    matern_pair<P>(fma(dx, dx, dy * dy), cp, v);
+#pragma unroll
+    for (int i = 0; i < P; ++i)
+#pragma unroll
+        for (int j = 0; j < P; ++j) out[(long long)(P * r + j) * ld + (long long)P * q + i] = v[i * P + j];
 }
 
 // For rows q < R of X (column-major, ldx, N columns): s[q] = sum_c X[q, c]^2
@@ -162,7 +163,7 @@ cudaError_t launch_covgen_cross(const CovParams &cp, const double *s0, int m, co
     if (m <= 0 || n <= 0) return cudaSuccess;
     dim3 grid((n + 3) / 4, (m + 63) / 64);
     KScope ks(GEO_K_COVGEN, s, 0.0, 8.0 * cp.p * (double)m * cp.p * (double)n);
-    k_covgen_cross<<<grid, 256, 0, s>>>(cp, s0, m, lx, ly, n, out, ld);
+    cov_by_p(cp.p, [&](auto P) { k_covgen_cross<P.value><<<grid, 256, 0, s>>>(cp, s0, m, lx, ly, n, out, ld); });
     return cudaGetLastError();
 }
 

@@ -30,6 +30,7 @@
 namespace {
 
 // Sigma block: rows = locations [l0, l0 + nl), cols = locations [r0, r0 + nr), SoA locations, Rep. I.
+template <int P>
 __global__ void __launch_bounds__(256) k_covgen_block(const CovParams cp, const double *__restrict__ lx,
                                                      const double *__restrict__ ly, int l0, int nl, int r0, int nr,
                                                      double *out, long long ld) {
@@ -37,12 +38,12 @@ __global__ void __launch_bounds__(256) k_covgen_block(const CovParams cp, const 
     const int r = r0 + blockIdx.x * 4 + (threadIdx.x / 64);
     if (l >= l0 + nl || r >= r0 + nr) return;
     const double dx = lx[l] - lx[r], dy = ly[l] - ly[r];
-    const double x = (l == r) ? 0.0 : sqrt(dx * dx + dy * dy) * cp.inv_a;
-    const int p = cp.p;
-    double v[GEO_PMAX_DEV * GEO_PMAX_DEV];
-    matern_block(x, cp, v);
-    for (int i = 0; i < p; ++i)
-        for (int j = 0; j < p; ++j) out[(long long)(p * (r - r0) + j) * ld + p * (l - l0) + i] = v[i * GEO_PMAX_DEV + j];
+    double v[P * P];
+    matern_pair<P>((l == r) ? 0.0 : fma(dx, dx, dy * dy), cp, v);
+#pragma unroll
+    for (int i = 0; i < P; ++i)
+#pragma unroll
+        for (int j = 0; j < P; ++j) out[(long long)(P * (r - r0) + j) * ld + P * (l - l0) + i] = v[i * P + j];
 }
 
 // M (r x r) = transpose of the upper triangle of B (r x r leading block, ld ldb).
@@ -281,7 +282,7 @@ cudaError_t tlr_factor(TlrFactor &F, const CovParams &cp, const double *lx, cons
             const int l0 = j * nb / p, nl = Rj / p, r0 = j * nb / p, nr = mj / p;
             dim3 grid((nr + 3) / 4, (nl + 63) / 64);
             KScope ks(GEO_K_COVGEN, s, 0.0, 8.0 * (double)Rj * mj);
-            k_covgen_block<<<grid, 256, 0, s>>>(cp, lx, ly, l0, nl, r0, nr, W, ldw);
+            cov_by_p(p, [&](auto P) { k_covgen_block<P.value><<<grid, 256, 0, s>>>(cp, lx, ly, l0, nl, r0, nr, W, ldw); });
             TCK(cudaGetLastError());
         }
         // 2. the updates of the finished columns k < j, applied implicitly:
