@@ -1349,28 +1349,29 @@ int geo_predict_var(geo_ctx *ctx, const geo_factor *factor, const double *new_lo
     const geo_factor *f = factor;
     const int p = f->p, N = f->N, pm = p * m;
     const long long ldx = round_up(pm, 32);
-    const size_t xbytes = sizeof(double) * (size_t)ldx * N, sbytes = sizeof(double) * pm,
-                 dbytes = sizeof(GemmDesc) * 64;
-    void *px = nullptr, *ps = nullptr, *pd = nullptr;
+    const size_t xbytes = sizeof(double) * (size_t)ldx * N, sbytes = sizeof(double) * pm;
+    void *px = nullptr, *ps = nullptr;
     auto done = [&](int code) {
         cudaStreamSynchronize(s);
         if (px) dev_free(ctx, px, xbytes);
         if (ps) dev_free(ctx, ps, sbytes);
-        if (pd) dev_free(ctx, pd, dbytes);
         return code;
     };
     int rc;
-    if ((rc = dev_alloc(ctx, &px, xbytes)) || (rc = dev_alloc(ctx, &ps, sbytes)) || (rc = dev_alloc(ctx, &pd, dbytes)))
-        return done(rc);
+    if ((rc = dev_alloc(ctx, &px, xbytes)) || (rc = dev_alloc(ctx, &ps, sbytes))) return done(rc);
     double c0d[GEO_PMAX];
     for (int i = 0; i < p; ++i) c0d[i] = f->cp.m[i * p + i].c0;
     cudaError_t e;
     // X = c0' (p m x N, the factor's location order), X <- X L^-T = (L^-1 c0)', var = C_ii(0) - |row|^2
-    if ((e = launch_covgen_cross(f->cp, new_locs_dev, m, f->lx, f->ly, f->n, (double *)px, ldx, s)) ||
-        (e = trsm_right_upper_t((double *)px, ldx, pm, f->A, f->ld, N, pd, s)) ||
+    if ((e = cudaMemsetAsync(ctx->st, 0, sizeof(DevStatus), s)) ||
+        (e = launch_covgen_cross(f->cp, new_locs_dev, m, f->lx, f->ly, f->n, (double *)px, ldx, s)) ||
+        (e = chol64_solve_rows((double *)px, ldx, pm, f->A, f->ld, N, ctx->st, ctx->csync, s)) ||
         (e = launch_row_sums((double *)px, ldx, nullptr, 0, pm, N, (double *)ps, nullptr, s)) ||
-        (e = launch_var_finish((const double *)ps, pm, p, c0d, var_dev, s)))
+        (e = launch_var_finish((const double *)ps, pm, p, c0d, var_dev, s)) ||
+        (e = cudaMemcpyAsync(ctx->h_st, ctx->st, sizeof(DevStatus), cudaMemcpyDeviceToHost, s)) ||
+        (e = cudaStreamSynchronize(s)))
         return done(cuda_fail(ctx, e, "geo_predict_var"));
+    if (ctx->h_st->timeout) return done(fail(ctx, GEO_ETIMEOUT, "a bounded device wait expired"));
     return done(GEO_OK);
 }
 

@@ -73,7 +73,9 @@ struct DfArgs {
     double *A;
     long long ld;
     int j0, jb;       // columns of the panel (the diagonal tile's rows are the same range)
-    int x0, x1;       // extra rows
+    double *X;        // extra rows x = 0 .. nx - 1: column j of the matrix at X[j * ldx + x]
+    long long ldx;
+    int nx;
     int T, E;         // 32-wide column tiles; tiles of extra rows
     int factor;       // 0: the diagonal range already holds L, only the extra rows are solved
     double *W;        // not null: W = -L^-1 of the diagonal range (column-major, ldw, zeros above the diagonal)
@@ -470,8 +472,10 @@ __global__ void __launch_bounds__(DF_THREADS, 1) k_chol_df(const DfArgs a) {
         const int kind = q < a.T ? 0 : q < a.T + a.E ? 1 : 2;
         const int e = q - (kind == 1 ? a.T : kind == 2 ? a.T + a.E : 0);   // tile row within its kind
         const int c0 = a.j0 + DT * c, cb = min(DT, a.j0 + a.jb - c0);
-        const int r0 = kind == 1 ? a.x0 + DT * e : a.j0 + DT * e;          // first row (identity rows: of the unit part)
-        const int nr = min(DT, (kind == 1 ? a.x1 : a.j0 + a.jb) - r0);
+        const int r0 = kind == 1 ? DT * e : a.j0 + DT * e;   // first row (of X, the matrix, the unit part)
+        const int nr = min(DT, (kind == 1 ? a.nx : a.j0 + a.jb) - r0);
+        double *R = kind == 1 ? a.X : a.A;
+        const long long rld = kind == 1 ? a.ldx : a.ld;
         const bool diag = kind == 0 && e == c;
         // with a chain, the diagonal tile and the one below it are only brought up to date here
         const bool pre = a.chain && kind == 0 && e <= c + 1;
@@ -491,7 +495,7 @@ __global__ void __launch_bounds__(DF_THREADS, 1) k_chol_df(const DfArgs a) {
             if (kind == 2)
                 v = (e == c && lr == col) ? 1.0 : 0.0;
             else
-                v = (lr < nr && col < cb) ? __ldcg(a.A + (long long)(c0 + col) * a.ld + r0 + lr) : 0.0;
+                v = (lr < nr && col < cb) ? __ldcg(R + (long long)(c0 + col) * rld + r0 + lr) : 0.0;
             sm.Bs[col][lr] = v;
         }
         df_sync(grp);
@@ -513,7 +517,7 @@ __global__ void __launch_bounds__(DF_THREADS, 1) k_chol_df(const DfArgs a) {
                 if (kind == 2)   // row r of the identity block's solution is column r of -W; threads walk k
                     pa[u] = (DT * e + kk < a.jb) ? -__ldcg(a.W + (long long)(DT * e + kk) * a.ldw + DT * k + lr) : 0.0;
                 else
-                    pa[u] = lr < nr ? __ldcg(a.A + (kc + kk) * a.ld + r0 + lr) : 0.0;
+                    pa[u] = lr < nr ? __ldcg(R + (kc + kk) * rld + r0 + lr) : 0.0;
                 if (!diag) pb[u] = lr < cb ? __ldcg(a.A + (kc + kk) * a.ld + c0 + lr) : 0.0;
             }
         };
@@ -615,7 +619,7 @@ __global__ void __launch_bounds__(DF_THREADS, 1) k_chol_df(const DfArgs a) {
                 if (lr < cb && row < nr) a.W[(long long)(DT * e + row) * a.ldw + DT * c + lr] = -sm.Bs[lr][row];
             } else {
                 const int col = lc + 4 * u;
-                if (lr < nr && col < cb && (!diag || lr >= col)) a.A[(long long)(c0 + col) * a.ld + r0 + lr] = sm.Bs[col][lr];
+                if (lr < nr && col < cb && (!diag || lr >= col)) R[(long long)(c0 + col) * rld + r0 + lr] = sm.Bs[col][lr];
             }
         }
         df_sync(grp);
@@ -687,7 +691,7 @@ cudaError_t launch_df(const DfArgs &a0, int sms, int cls, double flops, cudaStre
     const int all = df_sms();
     const int grid = (int)std::min<long long>(sms > 0 ? std::min(sms, all) : all, tickets + a.chain);
     if (grid < 8) a.alone = 0;
-    KScope ks(cls, s, flops, 16.0 * ((double)a.jb * a.jb / 2 + (double)(a.x1 - a.x0) * a.jb));
+    KScope ks(cls, s, flops, 16.0 * ((double)a.jb * a.jb / 2 + (double)a.nx * a.jb));
     kernel<<<grid, DF_THREADS, smem, s>>>(a);
     return cudaGetLastError();
 }
@@ -703,7 +707,7 @@ cudaError_t chol64_panel(double *A, long long ld, int j0, int jb, int x0, int x1
     if (jb <= 0) return cudaSuccess;
     if (!factor_diag && W && x1 > x0) return cudaErrorInvalidValue;
     const int nx = std::max(0, x1 - x0);
-    DfArgs a{A, ld, j0, jb, x0, x0 + nx, (jb + DT - 1) / DT, (nx + DT - 1) / DT, factor_diag ? 1 : 0, W, ldw, sync, 0, 0, 0, order == GEO_CHOL_BLOCK64,
+    DfArgs a{A, ld, j0, jb, A + x0, ld, nx, (jb + DT - 1) / DT, (nx + DT - 1) / DT, factor_diag ? 1 : 0, W, ldw, sync, 0, 0, 0, order == GEO_CHOL_BLOCK64,
              order != GEO_CHOL_STRAIGHT, st};
     const double j = jb, cubes = (factor_diag ? j * j * j / 3.0 : 0.0) + (W ? j * j * j / 3.0 : 0.0);
     return launch_df(a, sms, factor_diag ? GEO_K_POTRF : GEO_K_TRSM, cubes + nx * j * j, s);
@@ -733,7 +737,15 @@ cudaError_t chol64_rhs_update(double *A, long long ld, int rC, int cC, int m, in
 cudaError_t chol64_factor(double *A, long long ld, int N, int nrows, DevStatus *st, int *sync, cudaStream_t s) {
     if (N <= 0) return cudaSuccess;
     const int nx = std::max(0, nrows - N);
-    DfArgs a{A, ld, 0, N, N, N + nx, (N + DT - 1) / DT, (nx + DT - 1) / DT, 1, nullptr, 0, sync, 0, 0, 0, 0, 0, st};
+    DfArgs a{A, ld, 0, N, A + N, ld, nx, (N + DT - 1) / DT, (nx + DT - 1) / DT, 1, nullptr, 0, sync, 0, 0, 0, 0, 0, st};
     const double n = N;
     return launch_df(a, 0, GEO_K_GEMM, n * n * n / 3.0 + nx * n * n, s);
+}
+
+// X <- X L^-T for the rows of X (R x N, column-major, ldx), L the lower N x N factor: one launch.
+cudaError_t chol64_solve_rows(double *X, long long ldx, int R, double *L, long long ldl, int N, DevStatus *st, int *sync,
+                              cudaStream_t s) {
+    if (R <= 0 || N <= 0) return cudaSuccess;
+    DfArgs a{L, ldl, 0, N, X, ldx, R, (N + DT - 1) / DT, (R + DT - 1) / DT, 0, nullptr, 0, sync, 0, 0, 0, 0, 0, st};
+    return launch_df(a, 0, GEO_K_SOLVE, (double)R * N * N, s);
 }

@@ -131,6 +131,9 @@ cudaError_t chol64_factor(double *A, long long ld, int N, int nrows, DevStatus *
 cudaError_t chol64_panel(double *A, long long ld, int j0, int jb, int x0, int x1, DevStatus *st, int *sync,
                          cudaStream_t s, bool factor_diag = true, double *W = nullptr, long long ldw = 0, int sms = 0,
                          int order = GEO_CHOL_STRAIGHT);
+// X <- X L^-T (X: R x N column-major, ldx; L lower).
+cudaError_t chol64_solve_rows(double *X, long long ldx, int R, double *L, long long ldl, int N, DevStatus *st, int *sync,
+                              cudaStream_t s);
 // SMs to leave to a diagonal tile that is factored beside other work of rest_us.
 int chol64_side_sms(int jb, bool inverse, double rest_us);
 // C[rC.., cC..] (m x n) -= A[rC.., kA..kA+k] A[cC.., kA..kA+k]' in FP64, m a few right-hand-side rows.
@@ -191,9 +194,6 @@ cudaError_t launch_row_sums(const double *X, long long ldx, const double *Y, lon
 // X <- X L^-1 (X: R x N, L lower); arena_dev: 64 GemmDesc of device scratch.
 cudaError_t trsm_right_lower(double *X, long long ldx, int R, const double *L, long long ldl, int N, void *arena_dev,
                              cudaStream_t s);
-// X <- X L^-T (X: R x N, L lower); arena_dev: 64 GemmDesc of device scratch.
-cudaError_t trsm_right_upper_t(double *X, long long ldx, int R, const double *L, long long ldl, int N,
-                               void *arena_dev, cudaStream_t s);
 // Y = X' (X: R x C column-major, ldx; Y: C x R column-major, ldy).
 cudaError_t launch_transpose(const double *X, long long ldx, int R, int C, double *Y, long long ldy, cudaStream_t s);
 // sums[q] = sum_{c < N} Y[q * ldy + c]^2, q < R (columns of a column-major Y).
