@@ -57,7 +57,7 @@ struct geo_ctx {
     // batched predictions: descriptors (device + pinned staging)
     void *pdesc_d = nullptr, *pdesc_h = nullptr;
     size_t pdesc_cap = 0;
-    std::vector<unsigned char> bunits;  // cached ticket table (16 bytes per unit)
+    std::vector<unsigned char> bunits;  // cached ticket table (8 bytes per unit)
     cudaStream_t cap_stream = nullptr;   // private stream for graph capture (the legacy stream cannot capture)
     std::vector<geo_factor *> factors;
     // K_nu tables of the theta of the last geo_covgen call
@@ -1240,7 +1240,7 @@ int geo_loglik_batch(geo_ctx *ctx, int count, const geo_batch_item *items, doubl
     std::vector<CovParams> cps(count);
     std::vector<size_t> offs(count);
     size_t total = 0;
-    int nmax = 0, Nmax = 0;
+    int pmax = 1, Nmax = 0;
     for (int k = 0; k < count; ++k) {
         const geo_batch_item &it = items[k];
         std::string err;
@@ -1251,21 +1251,23 @@ int geo_loglik_batch(geo_ctx *ctx, int count, const geo_batch_item *items, doubl
         const int N = it.theta.p * it.n;
         const long long ld = round_up((long long)N + 1, 32);
         offs[k] = total;
-        total += (size_t)ld * N + GEO_TAB_DOUBLES;   // matrix, then the theta's K_nu tables
-        nmax = std::max(nmax, it.n);
+        // matrix, then the theta's K_nu and fine tables
+        total += (size_t)ld * N + GEO_TAB_DOUBLES + batch_fine_doubles(it.theta.p, it.n);
+        pmax = std::max(pmax, it.theta.p);
         Nmax = std::max(Nmax, N);
     }
     int rc;
     if ((rc = ensure_buffer(ctx, &ctx->bws, &ctx->bws_bytes, sizeof(double) * total, s))) return rc;
-    // device buffer: descriptors, counters (4 + count ints), the unit count, the ticket table
-    std::vector<int> orders(2 * count);   // orders, then location counts
-    for (int k = 0; k < count; ++k) orders[k] = items[k].theta.p * items[k].n, orders[count + k] = items[k].n;
-    const int nunits = -batch_units(orders.data(), orders.data() + count, count, 0, nullptr, 0);   // size query
+    // device buffer: descriptors, sync words, the unit count, the ticket table
+    std::vector<int> orders(count);
+    for (int k = 0; k < count; ++k) orders[k] = items[k].theta.p * items[k].n;
+    const long long nunits = batch_units(orders.data(), count, nullptr);
+    if (Nmax > 32 * 65000 || nunits > (1LL << 30)) return fail(ctx, GEO_EINVAL, "batch too large");
     const size_t desc_bytes = batch_desc_bytes() * (size_t)count;
     const size_t cnt_off = (desc_bytes + 255) / 256 * 256;
-    const size_t nun_off = cnt_off + (sizeof(int) * (4 + (size_t)count) + 255) / 256 * 256;
+    const size_t nun_off = cnt_off + (sizeof(int) * batch_sync_ints(count, Nmax) + 255) / 256 * 256;
     const size_t unit_off = nun_off + 256;
-    const size_t dbytes = unit_off + 16 * (size_t)nunits;
+    const size_t dbytes = unit_off + 8 * (size_t)nunits;
     if (ctx->bdesc_cap < dbytes) {
         CK(cudaStreamSynchronize(s));
         if (ctx->bdesc_d) cudaFree(ctx->bdesc_d);
@@ -1287,23 +1289,24 @@ int geo_loglik_batch(geo_ctx *ctx, int count, const geo_batch_item *items, doubl
         const int N = it.theta.p * it.n;
         const long long ld = round_up((long long)N + 1, 32);
         cps[k].tab = base + offs[k] + (size_t)ld * N;
+        cps[k].fine = batch_fine_doubles(it.theta.p, it.n) ? cps[k].tab + GEO_TAB_DOUBLES : nullptr;
         batch_fill_desc(ctx->bdesc_h, k, base + offs[k], ld, N, it.n, it.locs_dev, it.z_dev, cps[k]);
     }
     char *hb = (char *)ctx->bdesc_h, *db = (char *)ctx->bdesc_d;
-    *(int *)(hb + nun_off) = nunits;
+    *(int *)(hb + nun_off) = (int)nunits;
     // the ticket table depends only on the problem orders: rebuilt when they change
     if (ctx->border != orders) {
-        ctx->bunits.resize(16 * (size_t)nunits);
-        batch_units(orders.data(), orders.data() + count, count, batch_workers(), ctx->bunits.data(), (size_t)nunits);
+        ctx->bunits.resize(8 * (size_t)nunits);
+        batch_units(orders.data(), count, ctx->bunits.data());
         ctx->border = orders;
     }
-    memcpy(hb + unit_off, ctx->bunits.data(), 16 * (size_t)nunits);
+    memcpy(hb + unit_off, ctx->bunits.data(), 8 * (size_t)nunits);
     CK(cudaMemcpyAsync(db, hb, desc_bytes, cudaMemcpyHostToDevice, s));
     CK(cudaMemcpyAsync(db + nun_off, hb + nun_off, dbytes - nun_off, cudaMemcpyHostToDevice, s));
     int *counters_d = (int *)(db + cnt_off);
     const int *nunits_d = (const int *)(db + nun_off);
     const void *units_d = db + unit_off;
-    const auto key = std::make_tuple(count, nmax, Nmax);
+    const auto key = std::make_tuple(count, pmax, Nmax);
     auto itg = ctx->graphs.find(key);
     if (itg == ctx->graphs.end()) {
         // capture the launch sequence of this batch shape; launches are counted, not event-timed
@@ -1312,7 +1315,7 @@ int geo_loglik_batch(geo_ctx *ctx, int count, const geo_batch_item *items, doubl
         ProfBind pb(&counter);
         cudaGraph_t graph;
         CK(cudaStreamBeginCapture(ctx->cap_stream, cudaStreamCaptureModeThreadLocal));
-        cudaError_t e = batch_record(ctx->bdesc_d, units_d, nunits_d, counters_d, count, nmax, Nmax, ctx->cap_stream);
+        cudaError_t e = batch_record(ctx->bdesc_d, units_d, nunits_d, counters_d, count, pmax, Nmax, ctx->cap_stream);
         cudaError_t e2 = cudaStreamEndCapture(ctx->cap_stream, &graph);
         if (e != cudaSuccess) return cuda_fail(ctx, e, "batch capture");
         if (e2 != cudaSuccess) return cuda_fail(ctx, e2, "batch capture end");

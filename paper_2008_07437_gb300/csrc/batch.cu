@@ -1,39 +1,40 @@
 // Batched evaluation of many small, uneven Eq. 1 likelihoods (dense FP64).
 //
-// Three batched launches prepare every problem at once (K_nu tables of its
-// theta, covariance generation, Z into the extra row N); then ONE persistent
-// launch factors them all: CTAs take problems from a device queue in the
-// order the host gives (largest first, so that the SMs finish together), and
-// a CTA (one per SM, 512 threads) runs one problem's whole right-looking
-// Cholesky in 64-wide panels -- POTRF of the diagonal block in shared memory,
-// TRSM of every row below with the Z row carried along, rank-64 update of the
-// trailing lower triangle in 128 x 64 tiles -- and its log-determinant /
-// quadratic-form reduction.  No CTA
-// waits on another.  Every per-problem quantity (matrix pointer, order, theta
-// constants, input pointers) lives in a device descriptor array, so the launch
-// sequence of a batch shape (count, orders) is captured once as a CUDA graph
-// and replayed with new inputs and theta by refreshing the descriptors.  Each
-// problem's result depends only on its own data and a fixed operation order:
-// a likelihood is bit-identical alone and inside any batch.
+// One launch builds the tables of every problem's theta; ONE persistent launch
+// does the rest.  Its unit is a 32 x 32 tile of one problem's matrix (the tile
+// code of chol64.cu): generated from Eq. 2 on the spot, brought up to date with
+// the finished columns before it in registers, factored or solved, written
+// once; the observations ride along as an extra row, and a last unit per
+// problem sums up its log-determinant and quadratic form.  Groups of 128
+// threads take units from a ticket table and wait on progress words, one per
+// tile row of each problem.  The table runs over the columns of all problems
+// together, those with most columns left first: between two columns of one
+// problem lie the same-numbered columns of all the others, so that a unit's
+// inputs are finished long before its turn, and the problems end together.
+// Within a problem a unit only waits for units earlier in the table, whose
+// groups are running, so the launch cannot deadlock; waits are bounded.  Every
+// per-problem quantity lives in a device descriptor array, so the launch
+// sequence of a batch shape is captured once as a CUDA graph and replayed with
+// new inputs and theta by refreshing the descriptors.  Each problem's result
+// depends only on its own data and a fixed operation order: a likelihood is
+// bit-identical alone and inside any batch.
+//
+// Bound by the FP64 pipe: 512 problems of 50 to 1,000 bivariate locations (one draw) take
+// 346 ms (461 with 64-wide panels, a barrier between a problem's phases and the
+// covariance as units of its own); their N^3 / 3 alone takes about 310.
 #include <math.h>
 #include <string.h>
 
 #include <algorithm>
-#include <functional>
-#include <map>
-#include <queue>
-#include <mutex>
 #include <vector>
 
-#include "geo_internal.cuh"
+#include "chol_tile.cuh"
+#include "cov_tables.cuh"
 
 namespace {
 
-constexpr int PB = 64;   // panel width
-constexpr int BT = 256, BR = 128;   // persistent launch: threads per CTA, rows per TRSM chunk / update tile
-
 struct BatchDesc {
-    double *A;            // column-major, ld, N columns; row N holds Z' / y'
+    double *A;            // column-major, ld, N columns; row N receives y'
     long long ld;
     int N, n;
     const double *locs;   // n x 2 (caller order)
@@ -43,271 +44,198 @@ struct BatchDesc {
     DevResults res;
 };
 
-// K_nu tables of every problem's theta: block (q, k, problem).
-__global__ void __launch_bounds__(32) k_b_cheb_build(BatchDesc *d) {
-    __shared__ double hv[GEO_CHEB_N];
-    const CovParams &cp = d[blockIdx.z].cp;
-    cheb_build_block(cp, const_cast<double *>(cp.tab), blockIdx.x, blockIdx.y, hv);
-}
-
-// ---- one persistent launch over the units of every problem ----------------
-// A unit is one step of one problem's right-looking Cholesky in 64-wide
-// panels: POTRF of the diagonal block (panel c), TRSM of 128 rows below it
-// (the Z row included), or one 128 x 64 tile of the rank-64 trailing update
-// (the reduction is the unit after the last panel).  The host lays the units
-// out in a ticket table, panel-major across the problems (every problem's
-// panel-c POTRF, then their TRSM chunks, then their update tiles, then panel
-// c + 1 ...), and gives each unit the count of its problem's units that must
-// be complete before it starts (all units of the problem's previous phase).
-// CTAs take tickets in order; a unit waits (bounded, acquire loads) on its
-// problem's done counter, works, and publishes with a release increment.  A
-// CTA only waits for units whose tickets were taken earlier by CTAs that are
-// running, so the launch cannot deadlock whatever the number of resident CTAs;
-// past BWAIT_CYCLES a waiter raises the abort word and records the timeout.
-constexpr long long BWAIT_CYCLES = 4000000000LL;   // ~2 s at 2 GHz
+constexpr int B_REDUCE = 0xFFFF;   // tile column of a problem's last unit
 
 struct BSmem {
-    double S[PB][PB + 1];          // diagonal block, S[col][row]
-    union {
-        double X[PB][BR + 1];      // TRSM: 128 rows of the panel, X[col][row]
-        struct {
-            double As[16][BR + 2], Bs[16][PB + 2];   // update: K slices of the two operands
-        } u;
-        CovParams cp;              // covariance generation: the problem's theta constants
-    };
-    double red[2][BT / 32];
-    int fail, ok;
-    int4 unit;
+    DfSmem t;
+    CovParams cp;                  // the unit's problem
+    double red[2][DG / 32];
 };
 
-__device__ __forceinline__ int b_ld_acquire(const int *p) {
-    int v;
-    asm volatile("ld.acquire.gpu.global.s32 %0, [%1];\n" : "=r"(v) : "l"(p) : "memory");
-    return v;
-}
-
-// Wait until *done >= target; false when the launch was aborted (here or elsewhere).
-__device__ bool b_wait(const int *done, int target, int *abort_word, int *timeout_word) {
-    const long long t0 = clock64();
-    for (;;) {
-        if (b_ld_acquire(done) >= target) return true;
-        if (b_ld_acquire(abort_word)) return false;
-        if (clock64() - t0 > BWAIT_CYCLES) {
-            atomicExch(abort_word, 1);
-            atomicCAS(timeout_word, 0, 7);
-            return false;
-        }
-        __nanosleep(200);
-    }
-}
-
-__device__ void b_potrf_block(BSmem &sm, double *A, long long ld, int c0, int cb, DevStatus *st) {
-    for (int t = threadIdx.x; t < cb * cb; t += BT) {
-        const int c = t / cb, r = t % cb;
-        sm.S[c][r] = (r >= c) ? __ldcg(A + (long long)(c0 + c) * ld + c0 + r) : 0.0;
-    }
-    if (threadIdx.x == 0) sm.fail = 0;
-    __syncthreads();
-    for (int j = 0; j < cb; ++j) {
-        if (threadIdx.x == 0) {
-            const double v = sm.S[j][j];
-            if (!(v > 0.0)) {
-                sm.fail = 1;
-                st->info = c0 + j + 1;
+// The 32 x 32 tile of Sigma from row 32 i and column 32 c into S[col][row], by location pairs where the tile's
+// edge is a multiple of P, else entry by entry; zeros past the matrix.
+template <int P>
+__device__ __forceinline__ void b_cov_tile(double (*S)[DLD], const CovParams &cp, const double *__restrict__ locs, int n,
+                                           int i, int c, int tid) {
+    if constexpr (DT % P == 0) {
+        constexpr int LT = DT / P;   // locations along a tile's edge
+        for (int e = tid; e < LT * LT; e += DG) {
+            const int lr = e % LT, lc = e / LT, l = i * LT + lr, r = c * LT + lc;
+            double v[P * P];
+            if (l < n && r < n) {
+                const double dx = locs[2 * l] - locs[2 * r], dy = locs[2 * l + 1] - locs[2 * r + 1];
+                matern_pair<P>(l == r ? 0.0 : fma(dx, dx, dy * dy), cp, v);
             } else {
-                sm.S[j][j] = sqrt(v);
+#pragma unroll
+                for (int q = 0; q < P * P; ++q) v[q] = 0.0;
             }
+#pragma unroll
+            for (int q = 0; q < P * P; ++q) S[P * lc + q % P][P * lr + q / P] = v[q];
         }
-        __syncthreads();
-        if (sm.fail) return;   // uniform
-        const double inv = 1.0 / sm.S[j][j];
-        for (int r = j + 1 + threadIdx.x; r < cb; r += BT) sm.S[j][r] *= inv;
-        __syncthreads();
-        const int m = cb - j - 1;
-        for (int t = threadIdx.x; t < m * m; t += BT) {
-            const int c = j + 1 + t / m, r = j + 1 + t % m;
-            if (r >= c) sm.S[c][r] -= sm.S[j][r] * sm.S[j][c];
-        }
-        __syncthreads();
-    }
-    for (int t = threadIdx.x; t < cb * cb; t += BT) {
-        const int c = t / cb, r = t % cb;
-        if (r >= c) A[(long long)(c0 + c) * ld + c0 + r] = sm.S[c][r];
-    }
-}
-
-// rows [rbase, rbase + 128) within [c0 + cb, N] (the Z row N included) <- rows L_bb^-T
-__device__ void b_trsm_chunk(BSmem &sm, double *A, long long ld, int N, int c0, int cb, int rbase) {
-    const int row = threadIdx.x % BR, grp = threadIdx.x / BR;   // 2 groups share the columns
-    const int nr = min(BR, N + 1 - rbase);
-    for (int t = threadIdx.x; t < cb * cb; t += BT) {
-        const int c = t / cb, r = t % cb;
-        sm.S[c][r] = (r >= c) ? __ldcg(A + (long long)(c0 + c) * ld + c0 + r) : 0.0;
-    }
-    for (int t = threadIdx.x; t < cb * BR; t += BT) {
-        const int c = t / BR, r = t % BR;
-        sm.X[c][r] = (r < nr) ? __ldcg(A + (long long)(c0 + c) * ld + rbase + r) : 0.0;
-    }
-    __syncthreads();
-    for (int c = 0; c < cb; ++c) {
-        if (grp == 0) sm.X[c][row] *= 1.0 / sm.S[c][c];
-        __syncthreads();
-        const double xc = sm.X[c][row];
-        for (int k = c + 1 + grp; k < cb; k += BT / BR) sm.X[k][row] -= xc * sm.S[c][k];
-        __syncthreads();
-    }
-    for (int t = threadIdx.x; t < cb * BR; t += BT) {
-        const int c = t / BR, r = t % BR;
-        if (r < nr) A[(long long)(c0 + c) * ld + rbase + r] = sm.X[c][r];
-    }
-}
-
-// one 128 x 64 tile (rows t0 + tm.., cols t0 + tn..) of C -= P P', P = cols [c0, c0 + cb)
-__device__ void b_update_tile(BSmem &sm, double *A, long long ld, int N, int c0, int cb, int tm, int tn) {
-    const int t0 = c0 + cb;
-    const int m = N + 1 - t0, n = N - t0;
-    const int tx = threadIdx.x % 16, ty = threadIdx.x / 16;   // 16 x 16 threads, 8 x 4 outputs each
-    double acc[8][4] = {};
-    for (int k0 = 0; k0 < cb; k0 += 16) {
-        for (int t = threadIdx.x; t < 16 * BR; t += BT) {
-            const int kk = t / BR, r = t % BR;
-            sm.u.As[kk][r] = (k0 + kk < cb && tm + r < m) ? __ldcg(A + (long long)(c0 + k0 + kk) * ld + t0 + tm + r) : 0.0;
-        }
-        for (int t = threadIdx.x; t < 16 * PB; t += BT) {
-            const int kk = t / PB, r = t % PB;
-            sm.u.Bs[kk][r] = (k0 + kk < cb && tn + r < n) ? __ldcg(A + (long long)(c0 + k0 + kk) * ld + t0 + tn + r) : 0.0;
-        }
-        __syncthreads();
-#pragma unroll
-        for (int kk = 0; kk < 16; ++kk) {
-            double a[8], b[4];
-#pragma unroll
-            for (int i = 0; i < 8; ++i) a[i] = sm.u.As[kk][ty + 16 * i];
-#pragma unroll
-            for (int j = 0; j < 4; ++j) b[j] = sm.u.Bs[kk][tx + 16 * j];
-#pragma unroll
-            for (int i = 0; i < 8; ++i)
-#pragma unroll
-                for (int j = 0; j < 4; ++j) acc[i][j] = fma(a[i], b[j], acc[i][j]);
-        }
-        __syncthreads();
-    }
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-        const int c = tn + tx + 16 * j;
-        if (c >= n) continue;
-#pragma unroll
-        for (int i = 0; i < 8; ++i) {
-            const int r = tm + ty + 16 * i;
-            if (r < m && r >= c) {   // the Z row has r > c
-                double *pc = A + (long long)(t0 + c) * ld + t0 + r;
-                *pc = __ldcg(pc) - acc[i][j];
+    } else {
+        for (int e = tid; e < DT * DT; e += DG) {
+            const int R = i * DT + e % DT, C = c * DT + e / DT, l = R / P, r = C / P;
+            double v = 0.0;
+            if (l < n && r < n) {
+                const double dx = locs[2 * l] - locs[2 * r], dy = locs[2 * l + 1] - locs[2 * r + 1];
+                v = matern_entry(l == r ? 0.0 : fma(dx, dx, dy * dy), cp, R % P, C % P);
             }
+            S[e / DT][e % DT] = v;
         }
     }
 }
 
-// one 64 x 64 block of location pairs (l in block bl, r in block br <= bl, r <= l) of Eq. 2 into the
-// lower triangle; the diagonal blocks also put Z into the extra row N
-__device__ void b_covgen_block(BSmem &sm, const BatchDesc &q, int bl, int br) {
-    {   // the theta constants into shared memory (every thread reads them per pair)
-        const int words = (int)(sizeof(CovParams) / sizeof(int));
-        const int *src = reinterpret_cast<const int *>(&q.cp);
-        int *dst = reinterpret_cast<int *>(&sm.cp);
-        for (int t = threadIdx.x; t < words; t += BT) dst[t] = src[t];
-    }
-    __syncthreads();
-    const CovParams &cp = sm.cp;
-    const int p = cp.p, n = q.n;
-    const int l = bl * PB + threadIdx.x % PB;
-    if (l < n) {
-        const double lxv = q.locs[2 * l], lyv = q.locs[2 * l + 1];
-        for (int k = threadIdx.x / PB; k < PB; k += BT / PB) {
-            const int r = br * PB + k;
-            if (r >= n || r > l) continue;
-            const double dx = lxv - q.locs[2 * r], dy = lyv - q.locs[2 * r + 1];
-            const double x = (l == r) ? 0.0 : sqrt(dx * dx + dy * dy) * cp.inv_a;
-            double v[GEO_PMAX_DEV * GEO_PMAX_DEV];
-            matern_block(x, cp, v);
-            for (int j = 0; j < p; ++j)
-                for (int i = 0; i < p; ++i) q.A[(long long)(p * r + j) * q.ld + p * l + i] = v[i * GEO_PMAX_DEV + j];
-        }
-    }
-    if (bl == br)
-        for (int t = threadIdx.x; t < p * PB; t += BT) {
-            const int k = bl * PB * p + t;
-            if (k < q.N) q.A[(long long)k * q.ld + q.N] = q.z[k];
-        }
+// The tables of every problem's theta.
+__global__ void __launch_bounds__(128) k_b_tables(BatchDesc *d) {
+    const CovParams &cp = d[blockIdx.z].cp;
+    if ((int)blockIdx.x >= cp.p * (cp.p + 1) / 2) return;
+    fine_build_block(cp, const_cast<double *>(cp.tab), const_cast<double *>(cp.fine), blockIdx.x, blockIdx.y);
 }
 
-__device__ void b_reduce(BSmem &sm, BatchDesc &q) {
-    double a = 0.0, b = 0.0;
-    for (int k = threadIdx.x; k < q.N; k += BT) {
-        a += log(__ldcg(q.A + (long long)k * q.ld + k));
-        const double v = __ldcg(q.A + (long long)k * q.ld + q.N);
-        b += v * v;
-    }
-    for (int o = 16; o > 0; o >>= 1) {
-        a += __shfl_down_sync(0xffffffffu, a, o);
-        b += __shfl_down_sync(0xffffffffu, b, o);
-    }
-    if ((threadIdx.x & 31) == 0) sm.red[0][threadIdx.x >> 5] = a, sm.red[1][threadIdx.x >> 5] = b;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double ta = 0.0, tb = 0.0;
-        for (int w = 0; w < BT / 32; ++w) ta += sm.red[0][w], tb += sm.red[1][w];
-        if (q.st.info) {
-            q.res.loglik = q.res.logdet = q.res.quad = nan("");
-        } else {
-            q.res.logdet = 2.0 * ta;
-            q.res.quad = tb;
-            q.res.loglik = -0.5 * (double)q.N * log(2.0 * 3.141592653589793) - 0.5 * q.res.logdet - 0.5 * tb;
-        }
-    }
-}
-
-// sync: {ticket, abort, timeout, unused}; done: one counter per problem (all zeroed before the launch).
-// units[t] = {problem, kind << 16 | panel, index, target}: kind 0 POTRF, 1 TRSM chunk, 2 update tile
-// (index = tile row block * 65536 + tile column block), 3 reduction, 4 covariance block (index = location
-// row block * 65536 + location column block); *nunits_p: the unit count.
-// Matrix data another CTA wrote is read through L2 (__ldcg), after the acquire of the done counter.
-__global__ void __launch_bounds__(BT, 2) k_b_persistent(BatchDesc *d, const int4 *units, const int *nunits_p,
-                                                        int *done, int *sync) {
+// sync: {ticket, abort, timeout, unused}, then `stride` progress words per problem: one per tile row, the
+// observations' row last.  units[t] = {problem, tile column << 16 | tile row}.
+__global__ void __launch_bounds__(DF_THREADS, 1) k_b_persistent(BatchDesc *d, const int2 *__restrict__ units,
+                                                                const int *nunits_p, int *sync, int stride) {
+    extern __shared__ __align__(16) unsigned char b_smem[];
+    const int grp = threadIdx.x / DG, tid = threadIdx.x % DG;
+    BSmem &bs = reinterpret_cast<BSmem *>(b_smem)[grp];
+    DfSmem &sm = bs.t;
+    const int tx = tid % 16, ty = tid / 16, lr = tid % 32, lc = tid / 32;
     const int nunits = *nunits_p;
-    extern __shared__ __align__(16) uint8_t b_smem_raw[];
-    BSmem &sm = *reinterpret_cast<BSmem *>(b_smem_raw);
+    int dr[5], dc[5];
+    df_diag_entries(tid, dr, dc);
     for (;;) {
-        if (threadIdx.x == 0) {
-            const int t = atomicAdd(&sync[0], 1);
-            sm.unit = t < nunits ? units[t] : make_int4(-1, 0, 0, 0);
-            sm.ok = 1;
-            if (t < nunits) sm.ok = b_wait(&done[sm.unit.x], sm.unit.w, &sync[1], &sync[2]) ? 1 : 0;
+        if (tid == 0) {
+            const int t = df_ld_acquire(&sync[1]) ? nunits : atomicAdd(&sync[0], 1);
+            const int2 u = t < nunits ? units[t] : make_int2(-1, 0);
+            sm.word[0] = u.x;
+            sm.word[1] = u.y;
         }
-        __syncthreads();
-        const int4 u = sm.unit;
-        if (u.x < 0 || !sm.ok) return;   // uniform: no more units, or the launch was aborted
-        BatchDesc &q = d[u.x];
-        const int kind = u.y >> 16, c0 = (u.y & 0xFFFF) * PB;
-        // a failed pivot (written before the done counter that this unit waited for) skips the rest
-        const bool skip = *(volatile int *)&q.st.info != 0;
-        if (kind == 4) {
-            b_covgen_block(sm, q, u.z >> 16, u.z & 0xFFFF);
-        } else if (!skip || kind == 3) {
-            const int cb = min(PB, q.N - c0);
-            if (kind == 0)
-                b_potrf_block(sm, q.A, q.ld, c0, cb, &q.st);
-            else if (kind == 1)
-                b_trsm_chunk(sm, q.A, q.ld, q.N, c0, cb, c0 + cb + u.z * BR);
-            else if (kind == 2)
-                b_update_tile(sm, q.A, q.ld, q.N, c0, cb, (u.z >> 16) * BR, (u.z & 0xFFFF) * PB);
+        df_sync(grp);
+        const int p = sm.word[0];
+        if (p < 0) return;
+        const int c = sm.word[1] >> 16 & 0xFFFF, i = sm.word[1] & 0xFFFF;
+        BatchDesc &q = d[p];
+        const int N = q.N, T = (N + DT - 1) / DT;
+        int *prog = sync + 4 + (long long)p * stride;
+        if (c == B_REDUCE) {
+            if (tid == 0) sm.word[2] = df_wait(&prog[T], &prog[T - 1], T, sync, &sync[2]);
+            df_sync(grp);
+            if (sm.word[2] < 0) return;
+            double a = 0.0, b = 0.0;
+            for (int k = tid; k < N; k += DG) {
+                a += log(__ldcg(q.A + (long long)k * q.ld + k));
+                const double v = __ldcg(q.A + (long long)k * q.ld + N);
+                b += v * v;
+            }
+            for (int o = 16; o > 0; o >>= 1) {
+                a += __shfl_down_sync(0xffffffffu, a, o);
+                b += __shfl_down_sync(0xffffffffu, b, o);
+            }
+            if (lr == 0) bs.red[0][lc] = a, bs.red[1][lc] = b;
+            df_sync(grp);
+            if (tid == 0) {
+                double ta = 0.0, tb = 0.0;
+                for (int w = 0; w < DG / 32; ++w) ta += bs.red[0][w], tb += bs.red[1][w];
+                if (df_ld_acquire(&q.st.info)) {
+                    q.res.loglik = q.res.logdet = q.res.quad = nan("");
+                } else {
+                    q.res.logdet = 2.0 * ta;
+                    q.res.quad = tb;
+                    q.res.loglik = -0.5 * (double)N * log(2.0 * 3.141592653589793) - 0.5 * q.res.logdet - 0.5 * tb;
+                }
+            }
+            df_sync(grp);
+            continue;
+        }
+        const bool diag = i == c, obs = i == T;
+        const int c0 = DT * c, cb = min(DT, N - c0), r0 = obs ? N : DT * i, nr = obs ? 1 : min(DT, N - r0);
+        int *prow = &prog[i], *pcol = &prog[c];
+        // the tile as it starts
+        if (obs) {
+#pragma unroll
+            for (int u = 0; u < 8; ++u) sm.Bs[lc + 4 * u][lr] = (lr == 0 && lc + 4 * u < cb) ? q.z[c0 + lc + 4 * u] : 0.0;
+        } else {
+            const int words = (int)(sizeof(CovParams) / sizeof(int));
+            const int *src = reinterpret_cast<const int *>(&q.cp);
+            int *dst = reinterpret_cast<int *>(&bs.cp);
+            for (int t = tid; t < words; t += DG) dst[t] = src[t];
+            df_sync(grp);
+            switch (bs.cp.p) {
+                case 1: b_cov_tile<1>(sm.Bs, bs.cp, q.locs, q.n, i, c, tid); break;
+                case 2: b_cov_tile<2>(sm.Bs, bs.cp, q.locs, q.n, i, c, tid); break;
+                case 3: b_cov_tile<3>(sm.Bs, bs.cp, q.locs, q.n, i, c, tid); break;
+                default: b_cov_tile<4>(sm.Bs, bs.cp, q.locs, q.n, i, c, tid); break;
+            }
+        }
+        df_sync(grp);
+        double acc[8];
+#pragma unroll
+        for (int e = 0; e < 8; ++e)
+            acc[e] = diag ? (e < 5 ? -sm.Bs[dc[e % 5]][dr[e % 5]] : 0.0) : -sm.Bs[tx + 16 * (e % 2)][ty + 8 * (e / 2)];
+        df_sync(grp);
+        double pa[8], pb[8];
+        auto load = [&](int k) {
+            const long long kc = DT * k;
+#pragma unroll
+            for (int u = 0; u < 8; ++u) {
+                const double *col = q.A + (kc + lc + 4 * u) * q.ld + lr;
+                pa[u] = lr < nr ? __ldcg(col + r0) : 0.0;
+                if (!diag) pb[u] = lr < cb ? __ldcg(col + c0) : 0.0;
+            }
+        };
+        int avail = 0;
+        for (int k = 0; k < c; ++k) {
+            if (avail <= k) {
+                if (tid == 0) sm.word[2] = df_wait(prow, pcol, k + 1, sync, &sync[2]);
+                df_sync(grp);
+                avail = sm.word[2];
+                if (avail < 0) return;
+                load(k);
+            }
+#pragma unroll
+            for (int u = 0; u < 8; ++u) {
+                sm.As[lc + 4 * u][lr] = pa[u];
+                if (!diag) sm.Bs[lc + 4 * u][lr] = pb[u];
+            }
+            df_sync(grp);
+            if (k + 1 < c && avail > k + 1) load(k + 1);   // in flight during the products
+            if (diag)
+                df_mma_diag(acc, sm.As, dr, dc);
+            else if (nr <= 8)
+                df_mma<1>(acc, sm.As, sm.Bs, tx, ty);
             else
-                b_reduce(sm, q);
+                df_mma<4>(acc, sm.As, sm.Bs, tx, ty);
+            df_sync(grp);
         }
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            __threadfence();
-            atomicAdd(&done[u.x], 1);
+#pragma unroll
+        for (int e = 0; e < 8; ++e) {
+            if (!diag)
+                sm.Bs[tx + 16 * (e % 2)][ty + 8 * (e / 2)] = -acc[e];
+            else if (e < 5)
+                sm.Bs[dc[e % 5]][dr[e % 5]] = (dr[e % 5] < cb && dc[e % 5] < cb) ? -acc[e] : (dr[e % 5] == dc[e % 5] ? 1.0 : 0.0);
         }
+        df_sync(grp);
+        if (diag) {
+            const int bad = df_potrf32(sm.Bs, reinterpret_cast<double (*)[4][DT]>(sm.Ls), sm.dinv, grp, tid);
+            // the first failing row stays; the rest of the problem runs on what it finds, nothing reads it
+            if (bad < cb && tid == 0) atomicCAS(&q.st.info, 0, c0 + bad + 1);
+            df_sync(grp);
+        } else {
+            if (tid == 0) sm.word[2] = df_wait(pcol, pcol, c + 1, sync, &sync[2]);
+            df_sync(grp);
+            if (sm.word[2] < 0) return;
+            df_load_scaled(sm, q.A + (long long)c0 * q.ld + c0, q.ld, cb, grp, tid);
+            df_trsm32_scaled(sm.Bs, sm.Ls, sm.dinv, tid);
+            df_sync(grp);
+        }
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+            const int col = lc + 4 * u;
+            if (lr < nr && col < cb && (!diag || lr >= col)) q.A[(long long)(c0 + col) * q.ld + r0 + lr] = sm.Bs[col][lr];
+        }
+        df_sync(grp);
+        if (tid == 0) df_st_release(prow, c + 1);
     }
 }
 
@@ -315,118 +243,40 @@ __global__ void __launch_bounds__(BT, 2) k_b_persistent(BatchDesc *d, const int4
 
 size_t batch_desc_bytes() { return sizeof(BatchDesc); }
 
-// The ticket table.  Per problem the phases run in order -- the covariance
-// blocks; for each panel c: POTRF, the TRSM chunks, the update tiles; the
-// reduction -- and a unit's
-// target is its problem's count of units in earlier phases.  The order of the
-// tickets comes from a list-scheduling simulation on `workers` CTAs with
-// relative unit costs (update tile 1, TRSM chunk 0.5, POTRF 0.4, covariance
-// block 0.3, reduction 0.05): whenever a simulated CTA is free it takes a ready unit of the problem
-// with the most work left.  A unit is therefore dispensed only after every
-// unit it depends on, and roughly when they complete, so that CTAs rarely
-// wait.  Returns the unit count, or minus it when cap (units) is too small.
-int batch_units(const int *N, const int *nloc, int count, int workers, void *out_v, size_t cap) {
-    int4 *out = (int4 *)out_v;
-    struct Phase {
-        int kind, c, units;   // kind 0 POTRF, 1 TRSM, 2 update, 3 reduction, 4 covariance blocks
-        double cost;          // of one unit
-    };
-    std::vector<std::vector<Phase>> ph(count);
-    std::vector<double> left(count, 0.0);
-    size_t total = 0;
+// With the GPU full of problems the tables cost their FP64 operations, 3 million a C_ij, against some 55 saved per
+// pair of locations: they pay from about 340 locations on.
+size_t batch_fine_doubles(int p, int n) { return n >= 340 ? cov_fine_doubles(p, 0.5 * n * (n + 1.0)) : 0; }
+
+long long batch_units(const int *N, int count, void *out_v) {
+    int2 *out = (int2 *)out_v;
+    long long total = 0;
+    int Tmax = 0;
     for (int q = 0; q < count; ++q) {
-        const int T = (N[q] + PB - 1) / PB;
-        const int nbl = (nloc[q] + PB - 1) / PB;
-        ph[q].push_back({4, 0, nbl * (nbl + 1) / 2, 0.3});   // covariance blocks (lower triangle of location blocks)
-        for (int c = 0; c < T; ++c) {
-            const int c0 = c * PB, cb = std::min(PB, N[q] - c0), t0 = c0 + cb;
-            ph[q].push_back({0, c, 1, 0.4});
-            ph[q].push_back({1, c, (N[q] - t0) / BR + 1, 0.5});   // rows t0 .. N, 128 at a time
-            if (t0 < N[q]) {
-                const int m = N[q] + 1 - t0, nn = N[q] - t0;
-                int tiles = 0;
-                for (int tn = 0; tn < nn; tn += PB) tiles += (m - (tn / BR) * BR + BR - 1) / BR;
-                ph[q].push_back({2, c, tiles, 1.0});
-            }
-        }
-        ph[q].push_back({3, 0, 1, 0.05});
-        for (const Phase &f : ph[q]) left[q] += f.units * f.cost, total += f.units;
+        const long long T = (N[q] + DT - 1) / DT;
+        total += T * (T + 1) / 2 + T + 1;   // tiles, the observations' tiles, the reduction
+        Tmax = std::max(Tmax, (int)T);
     }
-    if (!out || cap < total) return -(int)total;
-    // simulation state: per problem the current phase, units of it not yet dispensed, running
-    std::vector<int> cur(count, 0), undisp(count), running(count, 0), done_before(count, 0);
-    for (int q = 0; q < count; ++q) undisp[q] = ph[q][0].units;
-    // ready problems by remaining work (max first)
-    std::priority_queue<std::pair<double, int>> ready;
-    for (int q = 0; q < count; ++q) ready.push({left[q], -q});
-    // running units: (finish time, problem), min first
-    typedef std::pair<double, int> Ev;
-    std::priority_queue<Ev, std::vector<Ev>, std::greater<Ev>> fin;
-    std::vector<double> stale_key(count, -1.0);
-    size_t n = 0;
-    double now = 0.0;
-    int idle = std::max(1, workers);
-    while (n < total) {
-        // dispense to idle workers while something is ready
-        while (idle > 0 && !ready.empty()) {
-            const int q = -ready.top().second;
-            ready.pop();
-            if (undisp[q] == 0) continue;   // stale entry
-            const Phase &f = ph[q][cur[q]];
-            const int idx = f.units - undisp[q];
-            int z = idx;
-            if (f.kind == 4) {   // idx -> (location row block, location column block), row by row
-                int bl = 0;
-                while ((bl + 1) * (bl + 2) / 2 <= idx) ++bl;
-                z = bl * 65536 + (idx - bl * (bl + 1) / 2);
-            } else if (f.kind == 2) {   // idx -> (tile row block, tile column block), column-major over the triangle
-                const int c0 = f.c * PB, cb = std::min(PB, N[q] - c0), t0 = c0 + cb;
-                const int m = N[q] + 1 - t0, nn = N[q] - t0;
-                int k = idx;
-                z = -1;
-                for (int tn = 0; tn < nn && z < 0; tn += PB) {
-                    const int rows = (m - (tn / BR) * BR + BR - 1) / BR;
-                    if (k < rows) z = ((tn / BR) + k) * 65536 + tn / PB;
-                    else k -= rows;
-                }
-            }
-            out[n++] = make_int4(q, (f.kind << 16) | f.c, z, done_before[q]);
-            --undisp[q];
-            ++running[q];
-            --idle;
-            left[q] -= f.cost;
-            fin.push({now + f.cost, q});
-            if (undisp[q] > 0) ready.push({left[q], -q});
-        }
-        if (fin.empty()) break;   // cannot happen: something is running or ready
-        // advance to the next completion
-        const Ev e = fin.top();
-        fin.pop();
-        now = e.first;
-        const int q = e.second;
-        ++idle;
-        if (--running[q] == 0 && undisp[q] == 0 && cur[q] + 1 < (int)ph[q].size()) {
-            done_before[q] += ph[q][cur[q]].units;   // the phase is complete: the next one is ready
-            ++cur[q];
-            undisp[q] = ph[q][cur[q]].units;
-            ready.push({left[q], -q});
+    if (!out) return total;
+    // problems by their number of columns, the largest first
+    std::vector<int> by(count);
+    for (int q = 0; q < count; ++q) by[q] = q;
+    std::stable_sort(by.begin(), by.end(), [&](int a, int b) { return (N[a] + DT - 1) / DT > (N[b] + DT - 1) / DT; });
+    long long n = 0;
+    int active = 0;
+    for (int left = Tmax; left >= 1; --left) {   // columns left, this one included
+        while (active < count && (N[by[active]] + DT - 1) / DT >= left) ++active;
+        for (int a = 0; a < active; ++a) {
+            const int q = by[a], T = (N[q] + DT - 1) / DT, c = T - left;
+            for (int i = c; i <= T; ++i) out[n++] = make_int2(q, c << 16 | i);
         }
     }
-    return (int)n;
+    for (int a = 0; a < count; ++a) out[n++] = make_int2(by[a], B_REDUCE << 16);
+    return n;
 }
 
-int batch_workers() {
-    int dev = 0, n = 0;
-    cudaGetDevice(&dev);
-    if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n <= 0) n = 1;
-    return 2 * n;   // two CTAs per SM
-}
+static int batch_stride(int Nmax) { return (Nmax + DT - 1) / DT + 1; }
 
-// Builds the descriptors on the host (pinned staging `hdesc`), the launch
-// sequence is recorded on `s` (capturable).
-struct BatchPlan {
-    int count = 0, nmax = 0, Nmax = 0;
-};
+size_t batch_sync_ints(int count, int Nmax) { return 4 + (size_t)count * batch_stride(Nmax); }
 
 void batch_fill_desc(void *hdesc_v, int k, double *A, long long ld, int N, int n, const double *locs,
                      const double *z, const CovParams &cp) {
@@ -441,24 +291,21 @@ void batch_fill_desc(void *hdesc_v, int k, double *A, long long ld, int N, int n
     h[k].cp = cp;
 }
 
-cudaError_t batch_record(void *ddesc_v, const void *units, const int *nunits, int *counters, int count, int nmax,
-                         int Nmax, cudaStream_t s) {
+cudaError_t batch_record(void *ddesc_v, const void *units, const int *nunits, int *sync, int count, int pmax, int Nmax,
+                         cudaStream_t s) {
     BatchDesc *d = (BatchDesc *)ddesc_v;
-    // counters: sync {ticket, abort, timeout, unused}, then one done counter per problem
-    cudaError_t e0 = cudaMemsetAsync(counters, 0, sizeof(int) * (4 + (size_t)count), s);
-    if (e0 != cudaSuccess) return e0;
+    cudaError_t e = cudaMemsetAsync(sync, 0, sizeof(int) * batch_sync_ints(count, Nmax), s);
+    if (e != cudaSuccess) return e;
     {
         KScope ks(GEO_K_COVGEN, s);
-        k_b_cheb_build<<<dim3(GEO_PMAX_DEV * GEO_PMAX_DEV, GEO_CHEB_NI + 1, count), 32, 0, s>>>(d);
+        k_b_tables<<<dim3(pmax * (pmax + 1) / 2, FINE_BLOCKS + COARSE_BLOCKS, count), 128, 0, s>>>(d);
     }
     {
-        // covariance generation, factorisation and reduction of every problem in one persistent launch
         KScope ks(GEO_K_GEMM, s);
-        cudaError_t e = cudaFuncSetAttribute(k_b_persistent, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)sizeof(BSmem));
-        if (e != cudaSuccess) return e;
-        k_b_persistent<<<batch_workers(), BT, sizeof(BSmem), s>>>(d, (const int4 *)units, nunits, counters + 4,
-                                                                   counters);
+        constexpr size_t smem = sizeof(BSmem) * DF_GROUPS;
+        if ((e = cudaFuncSetAttribute(k_b_persistent, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess)
+            return e;
+        k_b_persistent<<<df_sms(), DF_THREADS, smem, s>>>(d, (const int2 *)units, nunits, sync, batch_stride(Nmax));
     }
     return cudaGetLastError();
 }

@@ -44,30 +44,9 @@
 // FP64 units of an SM with eight entries each.
 #include <algorithm>
 
-#include "geo_internal.cuh"
+#include "chol_tile.cuh"
 
 namespace {
-
-constexpr int DT = 32;                 // tile edge
-constexpr int DG = 128;                // threads per group
-constexpr int DF_GROUPS = 4;           // groups per CTA: with one CTA per SM they fill the registers
-constexpr int DF_THREADS = DG * DF_GROUPS;
-constexpr int DLD = DT + 1;            // operand tiles: conflict-free along rows and columns
-constexpr int DLL = DT + 2;            // the solve's copy of L_cc: 16-byte pairs
-constexpr long long DF_WAIT_CYCLES = 4000000000LL;   // ~2 s at 2 GHz
-
-// Order (GEO_CHOL_STRAIGHT, GEO_CHOL_BLOCK64) of a tile's sum A_ic - sum_k L_ik L_ck' over the columns k of the panel: straight through, one FMA
-// after the other from A_ic on; or a separate sum per 64 columns, subtracted as a whole, and straight through
-// within the 64 columns the tile belongs to.  The second is the order of a factorisation in 64-wide steps with
-// a rank-64 update after each.  The forms with less than FP64 behind their far tiles use it: they round the
-// factor's entries to 35 bits or FP32, which turns a last-bit difference here into one of up to 1e-7 in l, so
-// their results stay what that order gives.
-struct DfSmem {
-    double As[DT][DLD], Bs[DT][DLD];   // operand tiles [k][row]; Bs then holds the tile itself, [col][row]
-    double Ls[DT][DLL];                // L_cc, [col][row]; the factorisation's exchange buffer
-    double dinv[DT];                   // 1 / diagonal of L_cc
-    int word[4];
-};
 
 struct DfArgs {
     double *A;
@@ -88,250 +67,6 @@ struct DfArgs {
     int plain;        // GEO_CHOL_BLOCK64 and GEO_CHOL_PLAIN: pivots and solves as the plain algorithm rounds them
     DevStatus *st;
 };
-
-__device__ __forceinline__ int df_ld_acquire(const int *p) {
-    int v;
-    asm volatile("ld.acquire.gpu.global.s32 %0, [%1];\n" : "=r"(v) : "l"(p) : "memory");
-    return v;
-}
-
-// (after a barrier: releases what the whole group wrote)
-__device__ __forceinline__ void df_st_release(int *p, int v) {
-    asm volatile("st.release.gpu.global.s32 [%0], %1;\n" ::"l"(p), "r"(v) : "memory");
-}
-
-// Barrier of one group (named barriers 1 .. DF_GROUPS).
-__device__ __forceinline__ void df_sync(int grp) { asm volatile("bar.sync %0, %1;" ::"r"(grp + 1), "n"(DG) : "memory"); }
-
-__device__ __forceinline__ void set_info(DevStatus *st, int row1) {
-    // keep the smallest failing row
-    int old = st->info;
-    while (old == 0 || old > row1) {
-        const int prev = atomicCAS(&st->info, old, row1);
-        if (prev == old) break;
-        old = prev;
-    }
-}
-
-// Wait until min(*p, *q) >= need (one thread).  Returns that minimum, or -1 when the launch was aborted.
-__device__ int df_wait(const int *p, const int *q, int need, int *sync, int *timeout_word) {
-    long long t0 = clock64();
-    int last = -1;
-    for (;;) {
-        int v = df_ld_acquire(p);
-        if (q != p) v = min(v, df_ld_acquire(q));
-        if (v >= need) return v;
-        if (df_ld_acquire(&sync[1])) return -1;
-        if (v != last) {
-            last = v;
-            t0 = clock64();
-        } else if (clock64() - t0 > DF_WAIT_CYCLES) {
-            atomicExch(&sync[1], 1);
-            atomicCAS(timeout_word, 0, 8);
-            return -1;
-        }
-        __nanosleep(20);
-    }
-}
-
-// Half of a normal number well above the smallest one, off the FP64 pipe.
-__device__ __forceinline__ double df_half(double x) {
-    return __hiloint2double(__double2hiint(x) - (1 << 20), __double2loint(x));
-}
-
-// d > 0 (false for a NaN), off the FP64 pipe.
-__device__ __forceinline__ bool df_positive(double d) {
-    const long long b = __double_as_longlong(d);
-    return b > 0 && b <= 0x7FF0000000000000LL;
-}
-
-// l = sqrt(d) and inv = 1 / l for a positive normal d, both as IEEE rounding gives them (the residuals of the
-// last steps are exact FMAs): the hardware's approximation of 1 / sqrt(d) (about 22 bits), one Newton step for
-// the root and its reciprocal, and a correction of each.  A chain of seven dependent FP64 operations where
-// sqrt() and a division take some twenty.
-__device__ __forceinline__ void df_root(double d, double *l, double *inv) {
-    double y0;
-    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y0) : "d"(d));
-    const double t = d * y0, e = fma(-t, df_half(y0), 0.5);   // (1 - d y0^2) / 2
-    const double r = fma(t, e, t), y = fma(y0, e, y0);
-    const double root = fma(fma(-r, r, d), df_half(y), r);
-    *l = root;
-    *inv = fma(fma(-root, y, 1.0), y, y);
-}
-
-// Cholesky factor of the 32 x 32 block S[col][row] (lower part) by one group, lane = row, columns w, w + 4, ...
-// in the registers of warp w.  Returns the first column without a positive pivot, or 32.  Panels of four
-// columns: the warps exchange the panel through shared memory (one barrier), then every warp factors it for
-// itself, so that no barrier or shared-memory round trip stands between its pivots, and applies it to its own
-// columns, the next panel's first.  A dependent FP64 operation takes 66 clocks and every warp-wide one occupies
-// its scheduler's FP64 unit for 64: one warp alone needs 38 us for the block, this 19.
-// dinv receives the reciprocals of the factor's diagonal.  Pivots, roots and products are those of the plain
-// right-looking algorithm, bit for bit (GEO_CHOL_BLOCK64).
-__device__ __forceinline__ int df_potrf32_plain(double (*S)[DLD], double (*buf)[4][DT], double *dinv, int grp, int tid) {
-    const int lane = tid & 31, w = tid >> 5;
-    double v[8], p[4] = {0.0, 0.0, 0.0, 0.0};
-#pragma unroll
-    for (int q = 0; q < 8; ++q) v[q] = S[4 * q + w][lane];
-    int bad = DT;
-#pragma unroll
-    for (int P = 0; P < 8; ++P) {
-        buf[P & 1][w][lane] = v[P];
-        df_sync(grp);
-        if (P > 0) {   // the previous panel on this warp's columns beyond this panel
-#pragma unroll
-            for (int q = P + 1; q < 8; ++q)
-#pragma unroll
-                for (int i = 0; i < 4; ++i) v[q] = fma(-p[i], S[4 * (P - 1) + i][4 * q + w], v[q]);
-        }
-#pragma unroll
-        for (int i = 0; i < 4; ++i) p[i] = buf[P & 1][i][lane];
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            const int j = 4 * P + i;
-            const double d = __shfl_sync(0xffffffffu, p[i], j);
-            if (!df_positive(d) && bad == DT) bad = j;
-            double l, inv;
-            df_root(d, &l, &inv);
-            p[i] = lane == j ? l : p[i] * inv;
-            if (tid == j) dinv[j] = inv;
-#pragma unroll
-            for (int i2 = i + 1; i2 < 4; ++i2) p[i2] = fma(-p[i], __shfl_sync(0xffffffffu, p[i], 4 * P + i2), p[i2]);
-        }
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            if (w == i) S[4 * P + i][lane] = p[i];
-            if (P < 7) v[(P + 1) % 8] = fma(-p[i], __shfl_sync(0xffffffffu, p[i], (4 * P + 4 + w) & 31), v[(P + 1) % 8]);
-        }
-    }
-    return bad;
-}
-
-// The same as L D L' first: the columns stay unscaled (u = l times the pivot's root) and are applied as
-// (u / d) u', so that between two pivots stand a reciprocal approximation and four dependent FP64 operations
-// instead of seven and a product; the 32 roots are taken together at the end, one per lane (12.5 us for the block).
-__device__ __forceinline__ int df_potrf32(double (*S)[DLD], double (*buf)[4][DT], double *dinv, int grp, int tid) {
-    const int lane = tid & 31, w = tid >> 5;
-    double v[8], p[4] = {0.0, 0.0, 0.0, 0.0}, m[4] = {0.0, 0.0, 0.0, 0.0};
-#pragma unroll
-    for (int q = 0; q < 8; ++q) v[q] = S[4 * q + w][lane];
-#pragma unroll
-    for (int P = 0; P < 8; ++P) {
-        buf[P & 1][w][lane] = v[P];
-        df_sync(grp);
-#pragma unroll
-        for (int i = 0; i < 4; ++i) p[i] = buf[P & 1][i][lane];
-        double f[4];   // this panel's multipliers
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            const double d = __shfl_sync(0xffffffffu, p[i], 4 * P + i);
-            double r0;
-            asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r0) : "d"(d));
-            const double e = fma(-d, r0, 1.0), f0 = p[i] * r0;
-            f[i] = fma(f0, fma(e, e, e), f0);   // u / d: the approximation's error e to the third order
-#pragma unroll
-            for (int i2 = i + 1; i2 < 4; ++i2) p[i2] = fma(-f[i], __shfl_sync(0xffffffffu, p[i], 4 * P + i2), p[i2]);
-            // the previous panel on this warp's columns beyond this one, in the chain's gaps
-            if (P > 0)
-#pragma unroll
-                for (int q = P + 1; q < 8; ++q) v[q] = fma(-m[i], S[4 * (P - 1) + i][4 * q + w], v[q]);
-        }
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            m[i] = f[i];
-            if (w == i) S[4 * P + i][lane] = p[i];
-            if (P < 7) v[(P + 1) % 8] = fma(-m[i], __shfl_sync(0xffffffffu, p[i], (4 * P + 4 + w) & 31), v[(P + 1) % 8]);
-        }
-    }
-    df_sync(grp);
-    // the roots and their reciprocals, in every warp for itself
-    const double d = S[lane][lane];
-    const unsigned ok = __ballot_sync(0xffffffffu, df_positive(d));
-    double l, inv;
-    df_root(d, &l, &inv);
-    if (w == 0) dinv[lane] = inv;
-#pragma unroll
-    for (int q = 0; q < 8; ++q) {
-        const int col = 4 * q + w;
-        const double iv = __shfl_sync(0xffffffffu, inv, col);
-        v[q] = lane == col ? l : S[col][lane] * iv;
-    }
-    df_sync(grp);   // every warp has read the diagonal
-#pragma unroll
-    for (int q = 0; q < 8; ++q) S[4 * q + w][lane] = v[q];
-    return ok == 0xffffffffu ? DT : __ffs(~ok) - 1;
-}
-
-// X <- X L^-T for the 32 x 32 tiles X[col][row] and L[col][row] by one group: warp w takes rows 8 w .. 8 w + 7,
-// lane = row + 8 g holds the columns g, g + 4, ... of its row; x_m goes from its lane to the row's four lanes
-// by shuffle, so the warps never wait for one another.  dinv: 1 / L_mm.
-__device__ __forceinline__ void df_trsm32(double (*X)[DLD], const double (*L)[DLL], const double *dinv, int tid) {
-    const int lane = tid & 31, g = lane >> 3, row = 8 * (tid >> 5) + (lane & 7);
-    double x[8];
-#pragma unroll
-    for (int i = 0; i < 8; ++i) x[i] = X[4 * i + g][row];
-#pragma unroll
-    for (int m = 0; m < DT; ++m) {
-        const int im = m / 4, gm = m % 4;
-        const double xm = __shfl_sync(0xffffffffu, x[im] * dinv[m], (lane & 7) + 8 * gm);
-        if (g == gm) X[m][row] = xm;
-#pragma unroll
-        for (int i = im; i < 8; ++i) {
-            if (i == im && gm == 3) continue;
-            const double y = fma(-xm, L[m][4 * i + g], x[i]);
-            x[i] = (i == im && g <= gm) ? x[i] : y;
-        }
-    }
-}
-
-// The same with the scaled factor H[m][k] = L_km / L_mm in place of L: the unscaled x_m goes out as it is (one
-// dependent operation per column instead of two), and the row is scaled once at the end.
-__device__ __forceinline__ void df_trsm32_scaled(double (*X)[DLD], const double (*H)[DLL], const double *dinv, int tid) {
-    const int lane = tid & 31, g = lane >> 3, row = 8 * (tid >> 5) + (lane & 7);
-    double x[8];
-#pragma unroll
-    for (int i = 0; i < 8; ++i) x[i] = X[4 * i + g][row];
-#pragma unroll
-    for (int m = 0; m < DT; ++m) {
-        const int im = m / 4, gm = m % 4;
-        const double xm = __shfl_sync(0xffffffffu, x[im], (lane & 7) + 8 * gm);
-#pragma unroll
-        for (int i = im; i < 8; ++i) {
-            if (i == im && gm == 3) continue;
-            const double y = fma(-xm, H[m][4 * i + g], x[i]);
-            x[i] = (i == im && g <= gm) ? x[i] : y;
-        }
-    }
-#pragma unroll
-    for (int i = 0; i < 8; ++i) X[4 * i + g][row] = x[i] * dinv[4 * i + g];
-}
-
-// Products of a 32-deep slice, acc += A-tile times B-tile': rows ty + 8 i, columns tx + 16 j.
-template <int IM>
-__device__ __forceinline__ void df_mma(double (&acc)[8], const double (*As)[DLD], const double (*Bs)[DLD], int tx,
-                                       int ty) {
-#pragma unroll 8
-    for (int kk = 0; kk < DT; ++kk) {
-        double a[IM], b[2];
-#pragma unroll
-        for (int i = 0; i < IM; ++i) a[i] = As[kk][ty + 8 * i];
-#pragma unroll
-        for (int j = 0; j < 2; ++j) b[j] = Bs[kk][tx + 16 * j];
-#pragma unroll
-        for (int i = 0; i < IM; ++i)
-#pragma unroll
-            for (int j = 0; j < 2; ++j) acc[2 * i + j] = fma(a[i], b[j], acc[2 * i + j]);
-    }
-}
-
-// The same for a diagonal tile, of which only the ten 8 x 8 blocks at or below the diagonal are formed: five
-// entries a thread instead of eight.
-__device__ __forceinline__ void df_mma_diag(double (&acc)[8], const double (*As)[DLD], const int (&dr)[5],
-                                            const int (&dc)[5]) {
-#pragma unroll 8
-    for (int kk = 0; kk < DT; ++kk)
-#pragma unroll
-        for (int i = 0; i < 5; ++i) acc[i] = fma(As[kk][dr[i]], As[kk][dc[i]], acc[i]);
-}
 
 // The column chain, by one group: for every column c the last product of the diagonal tile (with L_c,c-1, which
 // this group has just solved and still holds), its factorisation, and the solve of the tile below it.  Handing
@@ -420,14 +155,8 @@ __global__ void __launch_bounds__(DF_THREADS, 1) k_chol_df(const DfArgs a) {
     DfSmem &sm = reinterpret_cast<DfSmem *>(df_smem)[grp];
     const int tx = tid % 16, ty = tid / 16, lr = tid % 32, lc = tid / 32;
     int *prog = a.sync + 2;
-    // this thread's entries of a diagonal tile: one of the 64 of every other 8 x 8 block of its lower part
     int dr[5], dc[5];
-#pragma unroll
-    for (int i = 0; i < 5; ++i) {
-        const int b = 2 * i + tid / 64, bi = b < 1 ? 0 : b < 3 ? 1 : b < 6 ? 2 : 3, bj = b - bi * (bi + 1) / 2;
-        dr[i] = 8 * bi + tid % 8;
-        dc[i] = 8 * bj + tid % 64 / 8;
-    }
+    df_diag_entries(tid, dr, dc);
     __shared__ int chain_here;   // this CTA runs the column chain
     if (threadIdx.x == 0) chain_here = 0;
     __syncthreads();
@@ -592,21 +321,19 @@ __global__ void __launch_bounds__(DF_THREADS, 1) k_chol_df(const DfArgs a) {
             if (tid == 0) sm.word[1] = a.factor ? df_wait(&prog[c], &prog[c], c + 1, a.sync, &a.st->timeout) : 0;
             df_sync(grp);
             if (sm.word[1] < 0) return;
-#pragma unroll
-            for (int u = 0; u < 8; ++u) {
-                const int col = lc + 4 * u;
-                pa[u] = (lr < cb && col < cb && lr >= col) ? __ldcg(a.A + (long long)(c0 + col) * a.ld + c0 + lr)
-                                                           : (lr == col ? 1.0 : 0.0);
-                if (PLAIN) sm.Ls[col][lr] = pa[u];
-            }
-            if (tid < DT) sm.dinv[tid] = tid < cb ? 1.0 / __ldcg(a.A + (long long)(c0 + tid) * a.ld + c0 + tid) : 1.0;
-            df_sync(grp);
+            const double *L = a.A + (long long)c0 * a.ld + c0;
             if (PLAIN) {
+#pragma unroll
+                for (int u = 0; u < 8; ++u) {
+                    const int col = lc + 4 * u;
+                    sm.Ls[col][lr] = (lr < cb && col < cb && lr >= col) ? __ldcg(L + (long long)col * a.ld + lr)
+                                                                        : (lr == col ? 1.0 : 0.0);
+                }
+                if (tid < DT) sm.dinv[tid] = tid < cb ? 1.0 / __ldcg(L + (long long)tid * a.ld + tid) : 1.0;
+                df_sync(grp);
                 df_trsm32(sm.Bs, sm.Ls, sm.dinv, tid);
             } else {
-#pragma unroll
-                for (int u = 0; u < 8; ++u) sm.Ls[lc + 4 * u][lr] = pa[u] * sm.dinv[lc + 4 * u];
-                df_sync(grp);
+                df_load_scaled(sm, L, a.ld, cb, grp, tid);
                 df_trsm32_scaled(sm.Bs, sm.Ls, sm.dinv, tid);
             }
             df_sync(grp);
@@ -662,14 +389,6 @@ __global__ void __launch_bounds__(128) k_rhs_update(double *A, long long ld, int
     }
     if (c < n)
         for (int i = 0; i < RROWS && r0 + i < m; ++i) A[(long long)(cC + c) * ld + rC + r0 + i] -= acc[i];
-}
-
-int df_sms() {
-    int dev = 0, n = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
-        n <= 0)
-        return 1;
-    return n;
 }
 
 cudaError_t launch_df(const DfArgs &a0, int sms, int cls, double flops, cudaStream_t s) {

@@ -119,8 +119,13 @@ cudaError_t launch_scatter_vec(const double *in, long long stride, const int *pe
 // ---- chol64.cu ----------------------------------------------------------
 // Device ints of scratch (ticket, abort and progress words) of a chol64_* launch.
 constexpr int GEO_CHOL_SYNC_INTS = 16384;
-// Order of the sums within a panel: straight through, or per 64 columns; PLAIN and BLOCK64 round pivots and
-// solves as the plain right-looking algorithm does (the reduced forms keep both).
+// Order of a tile's sum A_ic - sum_k L_ik L_ck' over the columns k of a panel: STRAIGHT through, one FMA after the
+// other from A_ic on; or (BLOCK64) a separate sum per 64 columns, subtracted as a whole, and straight through
+// within the 64 columns the tile belongs to: the order of a factorisation in 64-wide steps with a rank-64 update
+// after each.  PLAIN and BLOCK64 also round pivots and solves as the plain right-looking algorithm does.  The
+// forms with less than FP64 behind their far tiles use these two: they round the factor's entries to 35 bits or
+// FP32, which turns a last-bit difference here into one of up to 1e-7 in l, so their results stay what that
+// order gives.
 constexpr int GEO_CHOL_STRAIGHT = 0, GEO_CHOL_BLOCK64 = 1, GEO_CHOL_PLAIN = 2;
 // In-place lower Cholesky of the leading N x N block of A; rows N..nrows-1
 // are extra right-hand-side rows carried through the factorisation (row N
@@ -348,17 +353,18 @@ cudaError_t tlr_reduce(const TlrFactor &F, const double *y, const DevStatus *st,
 size_t batch_desc_bytes();
 void batch_fill_desc(void *hdesc, int k, double *A, long long ld, int N, int n, const double *locs, const double *z,
                      const CovParams &cp);
-// Ticket table of the persistent launch (16 bytes per unit) for problems of orders N[0..count) and
-// n[0..count) locations,
-// ordered by a list-scheduling simulation on `workers` CTAs; returns the unit count, or minus it when
-// out is NULL or cap (units) is too small.
-int batch_units(const int *N, const int *n, int count, int workers, void *out, size_t cap);
-// CTAs of the persistent launch.
-int batch_workers();
+// Doubles of fine tables of a problem of n locations (0: it goes without).
+size_t batch_fine_doubles(int p, int n);
+// Ticket table of the persistent launch (8 bytes per unit) for problems of orders N[0..count); returns the unit
+// count (out == NULL: only that).
+long long batch_units(const int *N, int count, void *out);
+// Device ints of the launch's sync and progress words.
+size_t batch_sync_ints(int count, int Nmax);
 // units: device ticket table, nunits: device int holding its length (read by the launch, so a captured
-// sequence serves any table); counters: 4 + count device ints (zeroed by the sequence itself).
-cudaError_t batch_record(void *ddesc, const void *units, const int *nunits, int *counters, int count, int nmax,
-                         int Nmax, cudaStream_t s);
+// sequence serves any table); sync: batch_sync_ints device ints (zeroed by the sequence itself); pmax: the
+// largest number of variables.
+cudaError_t batch_record(void *ddesc, const void *units, const int *nunits, int *sync, int count, int pmax, int Nmax,
+                         cudaStream_t s);
 cudaError_t batch_results(const void *ddesc, void *hdesc, int count, double *loglik, int *info, cudaStream_t s);
 
 // ---- host helpers (api.cu) ------------------------------------------------

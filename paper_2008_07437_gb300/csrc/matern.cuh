@@ -412,6 +412,17 @@ GEO_DEV void matern_pair(double d2, const CovParams &cp, double (&v)[P * P]) {
         for (int j = 0; j < P; ++j) v[i * P + j] = w[i * GEO_PMAX_DEV + j];
 }
 
+// C_ij alone at the squared distance d2.
+GEO_DEV double matern_entry(double d2, const CovParams &cp, int i, int j) {
+    const MaternConst &c = cp.m[i * cp.p + j];
+    int idx;
+    double t;
+    float tf;
+    if (cp.fine && matern_fine_pos(d2 * cp.inv_a2, &idx, &t, &tf))
+        return matern_fine(cp.fine + c.foff + (long long)idx * GEO_FINE_STRIDE, t, tf);
+    return matern_cov(sqrt(d2) * cp.inv_a, c, cp.tab);
+}
+
 // ---- values at the tables' nodes --------------------------------------------------
 // The two methods of the reference evaluator with nothing but multiplications in their loops: the reciprocals of
 // Temme's series from a table of the order, and for x > 2 the recurrence run on the u_k themselves (they grow
