@@ -172,6 +172,11 @@ def load_library(path: str = LIB_PATH) -> ctypes.CDLL:
 # argument marshalling
 # ----------------------------------------------------------------------------
 
+def _doubles(values):
+    values = [float(v) for v in values]
+    return (ctypes.c_double * max(1, len(values)))(*values)
+
+
 @dataclass
 class Theta:
     """theta = (sigma^2_1..p, a, nu_1..p, beta) of Eq. 2 (Sec. 4.2)."""
@@ -199,12 +204,10 @@ class Theta:
         return b
 
     def to_c(self):
+        # ctypes arrays, not numpy ones: a batch converts hundreds of these per call
         p = len(self.sigma2)
-        keep = (np.ascontiguousarray(self.sigma2, dtype=np.float64),
-                np.ascontiguousarray(self.nu, dtype=np.float64),
-                np.ascontiguousarray(self.beta_matrix(), dtype=np.float64).reshape(-1))
-        th = geo_theta(p, keep[0].ctypes.data_as(_c_double_p), keep[1].ctypes.data_as(_c_double_p),
-                       keep[2].ctypes.data_as(_c_double_p), float(self.a))
+        keep = (_doubles(self.sigma2), _doubles(self.nu), _doubles(self.beta_matrix().reshape(-1).tolist()))
+        th = geo_theta(p, keep[0], keep[1], keep[2], float(self.a))
         return th, keep
 
     @staticmethod

@@ -247,24 +247,23 @@ int ensure_buffer(geo_ctx *ctx, void **buf, size_t *have, size_t need, cudaStrea
     return GEO_OK;
 }
 
-// G1(mu) = (1/Gamma(1-mu) - 1/Gamma(1+mu)) / (2 mu), G2(mu) = (1/Gamma(1-mu) + 1/Gamma(1+mu)) / 2.
+// G1(mu) = (1/Gamma(1-mu) - 1/Gamma(1+mu)) / (2 mu), G2(mu) = (1/Gamma(1-mu) + 1/Gamma(1+mu)) / 2, from
+// rp = 1/Gamma(1+mu) and fact = mu pi / sin(mu pi) = Gamma(1+mu) Gamma(1-mu).
 // Near mu = 0 the difference cancels: G1 is even in mu and equals
 // -(a2 + a4 mu^2 + a6 mu^4 + ...), a_k the Taylor coefficients of 1/Gamma(z).
-void temme_gammas(double mu, double *g1, double *g2, double *gp, double *gm, double *fact) {
-    const long double m = mu;
-    const long double rp = 1.0L / tgammal(1.0L + m), rm = 1.0L / tgammal(1.0L - m);
-    *gp = (double)tgammal(1.0L + m);
-    *gm = (double)tgammal(1.0L - m);
-    *g2 = (double)(0.5L * (rm + rp));
+void temme_gammas(double mu, long double gp, long double fact, MaternConst *c) {
+    const long double m = mu, rp = 1.0L / gp, rm = gp / fact;
+    c->gp = (double)gp;
+    c->gm = (double)(fact / gp);
+    c->g2 = (double)(0.5L * (rm + rp));
     if (fabsl(m) < 1e-3L) {
         const double u = mu * mu;
         // a2 = Euler's constant; a4, a6 of the series of 1/Gamma(z)
-        *g1 = -(0.5772156649015328606 + u * (-0.042002635034095235529 + u * (-0.04219773455554433675)));
+        c->g1 = -(0.5772156649015328606 + u * (-0.042002635034095235529 + u * (-0.04219773455554433675)));
     } else {
-        *g1 = (double)((rm - rp) / (2.0L * m));
+        c->g1 = (double)((rm - rp) / (2.0L * m));
     }
-    const long double pi = 3.141592653589793238462643383279502884L;
-    *fact = (mu == 0.0) ? 1.0 : (double)(m * pi / sinl(m * pi));
+    c->fact = (double)fact;
 }
 
 }  // namespace
@@ -335,25 +334,31 @@ int theta_to_params(const geo_theta *th, CovParams *cp, std::string *err) {
     cp->p = p;
     cp->inv_a = 1.0 / th->a;
     cp->inv_a2 = (double)(1.0L / ((long double)th->a * th->a));
+    // Gamma(nu + 1) / Gamma(nu) = nu, and one Gamma(1 + mu) per order gives the others by recurrence and
+    // reflection: long double functions are software on this host (about 1.5 us a call), and a batch has hundreds
+    // of thetas (44 calls a bivariate theta before, 70 us; now three)
     for (int i = 0; i < p; ++i) {
-        for (int j = 0; j < p; ++j) {
+        for (int j = i; j < p; ++j) {
             MaternConst &c = cp->m[i * p + j];
             const double nui = th->nu[i], nuj = th->nu[j];
             const double nij = 0.5 * (nui + nuj);
-            const long double ri = tgammal((long double)nui + 1.0L) / tgammal((long double)nui);
-            const long double rj = tgammal((long double)nuj + 1.0L) / tgammal((long double)nuj);
-            const long double rho = (long double)B[i][j] * sqrtl(ri) * sqrtl(rj) * tgammal((long double)nij) /
-                                    tgammal((long double)nij + 1.0L);
+            const long double rho = (long double)B[i][j] * sqrtl((long double)nui) * sqrtl((long double)nuj) / (long double)nij;
             const long double c0 = rho * sqrtl((long double)th->sigma2[i]) * sqrtl((long double)th->sigma2[j]);
             c.nu = nij;
             c.c0 = (double)c0;
-            c.pre = (double)(c0 / (powl(2.0L, (long double)nij - 1.0L) * tgammal((long double)nij)));
             const int nl = (int)floor(nij + 0.5);
             c.nl = nl;
             c.mu = nij - nl;
-            temme_gammas(c.mu, &c.g1, &c.g2, &c.gp, &c.gm, &c.fact);
             c.kind = (nij == 0.5) ? 1 : (nij == 1.5) ? 2 : (nij == 2.5) ? 3 : 0;
             c.toff = -1;
+            const long double pi = 3.141592653589793238462643383279502884L, m = c.mu;
+            const long double gp = tgammal(1.0L + m), fact = (c.mu == 0.0) ? 1.0L : m * pi / sinl(m * pi);
+            long double g = gp;   // Gamma(nu) = Gamma(mu + nl)
+            for (int k = 1; k < nl; ++k) g *= m + k;
+            if (nl == 0) g /= m;
+            c.pre = (double)(c0 / (exp2l((long double)nij - 1.0L) * g));
+            temme_gammas(c.mu, gp, fact, &c);
+            cp->m[j * p + i] = c;
         }
     }
     // K_nu tables for the general orders nu_ij <= GEO_CHEB_NU_MAX, one per i <= j
