@@ -155,12 +155,12 @@ cudaError_t chol_mixed_factor(double *A, long long ld, int N, int nrows, int nb,
 // FP64-accurate products on the BF16 tensor cores: the rows of an operand
 // as S BF16 digit slices with a power-of-two exponent per row and K chunk.
 struct OzSlices {
-    void *d;                  // S slices of rows x Kp BF16 digits (row-major, K contiguous)
+    void *d;                  // BF16 digits, row-major: per row and 16 columns the 16 digits of every slice in turn
     int *e;                   // row exponents, nchunk x rows
     int S, K, Kp, kchunk, nchunk;
+    int Sg;                   // slices with their padding (a multiple of 4)
     long long rows;           // capacity: row stride of the exponent array
     long long valid;          // rows holding data (extent of the tensor maps)
-    long long slice_stride;   // elements between slices
     int *be;                  // per 32-row block exponent maxima: 2 nchunk x bstride (all rows, reference rows)
     long long bstride;
     long long ref_rows;       // rows that set the level cut's reference scale (-1: every sliced row)

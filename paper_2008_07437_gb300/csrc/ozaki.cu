@@ -43,25 +43,41 @@
 //               against the largest (far from the diagonal in a spatially
 //               ordered covariance) skip levels or vanish entirely.
 //
-// The kernel is persistent (one CTA per SM) over 128 x BN output tiles, the
-// K range in chunks of BK.  TMEM (512 columns) holds 512 / BN level
-// accumulators of 128 x BN FP32: with BN = 64 all eight levels of 8 slices
-// fit and a tile is one pass over K; with BN = 128 (used from 6 slices on,
-// where the 128-row A operand read per 128 x 64 MMA otherwise keeps the MMA
-// issue path twice as busy as the math) the level groups run as passes over
-// K, each loading only the slices its levels use and writing its part of C.
-//   warp 0, one lane: TMA producer, ring of K chunks (32 or 64-byte rows,
-//     swizzled to match), each chunk holding the digit slices of the A rows
-//     (128 x BK BF16 each) and of the B rows (BN x BK each);
+// The digits lie interleaved: per operand row and 16 columns (the K of one MMA)
+// the 16 digits of four slices fill one 128-byte line.  A TMA box of 128 such
+// lines brings four slices at once, and a slice is a 32-byte step of the
+// operand descriptor within the 128-byte swizzle, the step that usually
+// advances K.  With the slices apart a chunk of 8 slices took 24 boxes of
+// 32-byte lines a tile, with almost no MMAs 0.73 ms for the product below; now
+// 6 boxes, 0.61 ms.
+//
+// The kernel is persistent (one CTA per SM) over 128 x 128 output tiles, the
+// K range in chunks of 16.  TMEM (512 columns) holds four level accumulators
+// of 128 x 128 FP32, so the levels run as passes of four over K, each loading
+// only the slices its levels use and writing its part of C.  (64-column tiles
+// would hold eight levels, but the 128-row A operand read per MMA then keeps
+// shared memory twice as busy as the math: 4 slices 0.56 ms against 0.34 for
+// C 8192 x 4096, K = 512, 5 slices 0.76 against 0.57.)
+//   warp 0, one lane: TMA producer, ring of slots, each with four digit slices
+//     of a K chunk of the A rows (128 lines of 128 bytes) and of the B rows
+//     (128 lines); a pass that reads at most four takes one slot per chunk;
 //   warp 1: allocates the 512 TMEM columns; one lane issues tcgen05.mma
-//     kind::f16 (M 128, N BN, K 16) level by level from precomputed shared
+//     kind::f16 (M 128, N 128, K 16) level by level from precomputed shared
 //     memory descriptors and commits chunks back to the producer;
 //   warps 2-9: epilogue; tcgen05.ld of each level, releasing that
 //     accumulator slot as soon as it is read (the MMAs of the next pass or
 //     tile may start into it while the epilogue folds the values in
-//     registers), then the FP64 read-modify-write of C (with the level cut,
-//     C comes through shared memory by cp.async, four columns at a time,
-//     double-buffered, so that no register waits on a load of C).
+//     registers), then the FP64 read-modify-write of C, which comes through
+//     shared memory by cp.async twelve columns ahead, the first of them
+//     before the tile's MMAs are done.
+// What bounds it: without the cut the MMAs (77 of 64 ideal cycles each: two
+// 4 KB operands per MMA take all of shared memory's bandwidth), 8 slices 67 us
+// a tile of K = 512; with few levels left the epilogue's FP64 work and loads of
+// C, 7 us a pass (28 before the loads ran ahead).  The single-thread roles count
+// along where they stand in the ring: a 64-bit division per chunk there took as
+// long as ten MMAs.  C 8192 x 4096, K = 512: 8 slices 1.02 -> 0.93 ms, 6 slices
+// 0.91 -> 0.64, 4 slices 0.56 -> 0.34; the updates of N = 40,000 with the level cut
+// 343 -> 305 ms.
 // With the level cut each CTA first computes the cut of all its tiles into a
 // shared-memory table, and the MMA thread counts the products it issues
 // (the device-side tensor work of the profile).
@@ -80,42 +96,32 @@ namespace {
 using namespace tc;
 
 constexpr int OZ_BM = 128;        // output rows per tile (MMA M, TMEM lanes)
+constexpr int OZ_BN = 128;        // output columns per tile (MMA N)
 constexpr int OZ_KALIGN = 32;     // slice arrays: K padded to a multiple of 32 (64-byte rows)
 constexpr int OZ_EPI_WARPS = 8;
 constexpr int OZ_THREADS = 64 + 32 * OZ_EPI_WARPS;
 constexpr int OZ_TMEM_COLS = 512;
-constexpr int OZ_SMEM_CAP = 200 * 1024;   // the ring of K chunks; the rest: level-cut table, C staging
+constexpr int OZ_A_BYTES = OZ_BM * 128, OZ_SLOT_BYTES = (OZ_BM + OZ_BN) * 128;   // one group of one K chunk
+constexpr int OZ_SLOTS = 6;               // ring of K chunks
+constexpr int OZ_CPT = OZ_BN / 2;         // columns per epilogue thread
+constexpr int OZ_CD = 12, OZ_CQ = 4;      // C columns in flight per epilogue thread, columns per copy group
+constexpr size_t OZ_SMEM = (size_t)OZ_SLOTS * OZ_SLOT_BYTES + sizeof(double) * OZ_EPI_WARPS * OZ_CD * 32 + 1024;
 constexpr int OZ_LC_CAP = 8192;           // tiles per CTA whose level cut is computed up front
 constexpr int OZ_GROUP = 8;       // row blocks swept together (operand reuse in L2)
 constexpr int OZ_LPW = 4;         // levels folded into one 64-bit word
 constexpr int OZ_E_NONE = -4096;  // block exponent of rows that are all zero (or absent)
 
-// Tile width BN (MMA N), K chunk BK (16: 32-byte rows, 32-byte swizzle; 32:
-// 64-byte rows, 64-byte swizzle).  TMEM holds 512 / BN level accumulators, so
-// the S levels are processed in passes of WPP words over the whole K range;
-// each pass loads only the slices its levels use.
-template <int S, int BN, int BK>
+// TMEM holds 512 / OZ_BN = 4 level accumulators, one word of levels, so the S levels are processed in passes of a
+// word over the whole K range; each pass loads only the groups of four slices its levels use.
+template <int S>
 struct OzCfg {
-    static constexpr int NWT = (S + OZ_LPW - 1) / OZ_LPW;            // words of <= 4 levels (levels 2 .. S+1)
-    static constexpr int WPP = OZ_TMEM_COLS / (BN * OZ_LPW);          // words per pass
-    static constexpr int PASSES = (NWT + WPP - 1) / WPP;
-    static constexpr int WREG = WPP < NWT ? WPP : NWT;                // words an epilogue thread holds
-    static constexpr int A_BYTES = OZ_BM * BK * 2;
-    static constexpr int B_BYTES = BN * BK * 2;
-    static constexpr int STAGE_BYTES = S * (A_BYTES + B_BYTES);      // the widest pass uses every slice
-    static constexpr int STAGES = (OZ_SMEM_CAP / STAGE_BYTES) < 6 ? (OZ_SMEM_CAP / STAGE_BYTES) : 6;
-    static constexpr size_t SMEM = (size_t)STAGES * STAGE_BYTES + 1024;
-    static constexpr int CPT = BN / 2;                                // columns per epilogue thread
+    static constexpr int PASSES = (S + OZ_LPW - 1) / OZ_LPW;   // words of <= 4 levels (levels 2 .. S+1)
+    static constexpr int NG = (S + 3) / 4;                     // groups of four slices
     // levels of pass g: [lev_lo, lev_hi]; slices it reads: 1 .. tmax
-    __host__ __device__ static constexpr int lev_lo(int g) { return 2 + OZ_LPW * WPP * g; }
-    __host__ __device__ static constexpr int lev_hi(int g) {
-        return (1 + OZ_LPW * WPP * (g + 1)) < (S + 1) ? (1 + OZ_LPW * WPP * (g + 1)) : (S + 1);
-    }
-    __host__ __device__ static constexpr int tmax(int g) { return (lev_hi(g) - 1) < S ? (lev_hi(g) - 1) : S; }
-    // last level of word w (its unit is 2^(2 - 7 hi))
-    __host__ __device__ static constexpr int word_hi(int w) {
-        return (5 + OZ_LPW * w) < (S + 1) ? (5 + OZ_LPW * w) : (S + 1);
-    }
+    __host__ __device__ static constexpr int lev_lo(int g) { return 2 + OZ_LPW * g; }
+    // (also the word's unit, 2^(2 - 7 lev_hi))
+    __host__ __device__ static constexpr int lev_hi(int g) { return (5 + OZ_LPW * g) < (S + 1) ? (5 + OZ_LPW * g) : (S + 1); }
+    __host__ __device__ static constexpr int tmax(int g) { return lev_hi(g) - 1; }
 };
 
 struct OzArgs {
@@ -123,11 +129,11 @@ struct OzArgs {
     long long ldc;
     int r0, c0;          // global row / col of the region's first output
     int m_end, n_end;    // outputs with global row >= m_end or col >= n_end are not written
-    int mt, nt;          // 128-row x BN-col tiles of the region
+    int mt, nt;          // 128 x 128 tiles of the region
     int tri;             // write only global row >= global col; skip tiles entirely above the diagonal
     int overwrite;       // 1: C = -A B' (C is not read)
     int a_off, b_off;    // slice row of the region's first row (A) / first column (B)
-    int nk;              // K chunks of BK
+    int nk;              // K chunks of 16
     const int *ea, *eb;  // per-row exponents of the A / B slices
     // level cut: per 32-row block maxima of the row exponents over every row (ba, bb) and over the
     // reference rows (ra, rb) of the A / B slices, nba / nbb blocks; cut = 0 keeps every level
@@ -137,7 +143,7 @@ struct OzArgs {
     DevStatus *st;
 };
 
-__device__ __forceinline__ long long ntiles_all(const OzArgs &a) { return (long long)a.mt * a.nt; }
+__device__ __forceinline__ int ntiles_all(const OzArgs &a) { return a.mt * a.nt; }
 
 __device__ __forceinline__ void cp_async8(double *dst, const double *src) {
     asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(smem_u32(dst)), "l"(src) : "memory");
@@ -149,29 +155,28 @@ __device__ __forceinline__ void cp_async_wait() {
 }
 
 // Highest level an output tile keeps (< 2: the tile is skipped); eref = E_A + E_B.
-template <int S, int BN>
+template <int S>
 __device__ __forceinline__ int oz_lcut(const OzArgs &a, int ar, int br, int eref) {
     if (!a.cut) return S + 1;
     int ei = OZ_E_NONE, ej = OZ_E_NONE;
-    const int a1 = min((ar + OZ_BM - 1) >> 5, a.nba - 1), b1 = min((br + BN - 1) >> 5, a.nbb - 1);
+    const int a1 = min((ar + OZ_BM - 1) >> 5, a.nba - 1), b1 = min((br + OZ_BN - 1) >> 5, a.nbb - 1);
     for (int b = ar >> 5; b <= a1; ++b) ei = max(ei, a.ba[b]);
     for (int b = br >> 5; b <= b1; ++b) ej = max(ej, a.bb[b]);
     if (ei == OZ_E_NONE || ej == OZ_E_NONE) return 1;   // every row of one side is zero: nothing to add
     return S + 1 - max(0, eref - ei - ej) / 7;
 }
 
-template <int BN>
-__device__ __forceinline__ bool oz_tile(const OzArgs &a, long long L, int *gr, int *gc, int *ar, int *br) {
-    const long long per_band = (long long)OZ_GROUP * a.nt;
-    const long long band = L / per_band;
+__device__ __forceinline__ bool oz_tile(const OzArgs &a, int L, int *gr, int *gc, int *ar, int *br) {
+    const unsigned per_band = (unsigned)OZ_GROUP * a.nt;
+    const unsigned band = (unsigned)L / per_band;
     const int i0 = (int)band * OZ_GROUP;
-    const int gm = min(OZ_GROUP, a.mt - i0);
-    const long long w = L - band * per_band;
+    const unsigned gm = min(OZ_GROUP, a.mt - i0);
+    const unsigned w = (unsigned)L - band * per_band;
     const int j = (int)(w / gm), i = i0 + (int)(w % gm);
     *gr = a.r0 + i * OZ_BM;
-    *gc = a.c0 + j * BN;
+    *gc = a.c0 + j * OZ_BN;
     *ar = a.a_off + i * OZ_BM;
-    *br = a.b_off + j * BN;
+    *br = a.b_off + j * OZ_BN;
     return !(a.tri && *gr + OZ_BM - 1 < *gc);
 }
 
@@ -183,32 +188,15 @@ __device__ __forceinline__ double pow2i(int e) {
     return __longlong_as_double((long long)(e + 1023) << 52);
 }
 
-template <int BK>
-__device__ __forceinline__ uint64_t oz_desc(uint32_t saddr) {
-    if constexpr (BK == 16) {
-        uint64_t d = 0;   // SWIZZLE_32B: 8 rows x 32 bytes = 256-byte groups
-        d |= (uint64_t)((saddr >> 4) & 0x3FFF);
-        d |= (uint64_t)1 << 16;
-        d |= (uint64_t)(256 >> 4) << 32;
-        d |= (uint64_t)1 << 46;
-        d |= (uint64_t)6 << 61;
-        return d;
-    } else {
-        return smem_desc_sw64(saddr);
-    }
-}
-
-template <int S, int BN, int BK>
+// LOW_FIRST: the passes from the last levels up instead of down to them (without the level cut).
+template <int S, bool LOW_FIRST>
 __global__ void __launch_bounds__(OZ_THREADS, 1)
     k_oz_update(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapB,
                 const OzArgs args) {
-    using Cfg = OzCfg<S, BN, BK>;
-    constexpr int ST = Cfg::STAGES;
-    constexpr int STAGE_BYTES = Cfg::STAGE_BYTES;
-    constexpr int A_BYTES = Cfg::A_BYTES, B_BYTES = Cfg::B_BYTES;
-    constexpr int PASSES = Cfg::PASSES, CPT = Cfg::CPT, WREG = Cfg::WREG;
+    using Cfg = OzCfg<S>;
+    constexpr int ST = OZ_SLOTS, NG = Cfg::NG, PASSES = Cfg::PASSES, CPT = OZ_CPT;
     extern __shared__ uint8_t smem_raw[];
-    constexpr int NSLOT = OZ_TMEM_COLS / BN;   // accumulator slots of BN columns
+    constexpr int NSLOT = OZ_TMEM_COLS / OZ_BN;   // accumulator slots
     __shared__ uint64_t full_bar[ST], empty_bar[ST], acc_full, slot_empty[NSLOT], drain_bar;
     __shared__ uint32_t tmem_slot;
     __shared__ int skip, emax_a, emax_b;
@@ -239,23 +227,23 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
     // the level cut of this CTA's tiles (the i-th tile it visits is L = blockIdx.x + i gridDim.x),
     // computed once here so that no role waits on the exponent loads inside its tile loop
     __shared__ uint8_t lc_tab[OZ_LC_CAP];
-    __shared__ __align__(16) double c_stage[OZ_EPI_WARPS * 2 * 4 * 32];   // epilogue: C columns in flight
     if (args.cut) {
-        const long long mine = (ntiles_all(args) - blockIdx.x + gridDim.x - 1) / gridDim.x;
+        const int mine = (int)((ntiles_all(args) - blockIdx.x + gridDim.x - 1) / gridDim.x);
         for (int i = threadIdx.x; i < OZ_LC_CAP && i < mine; i += OZ_THREADS) {
             int gr, gc, ar, br;
-            const long long L = blockIdx.x + (long long)i * gridDim.x;
-            lc_tab[i] = oz_tile<BN>(args, L, &gr, &gc, &ar, &br) ? (uint8_t)max(0, oz_lcut<S, BN>(args, ar, br, eref))
+            const int L = (int)(blockIdx.x + (unsigned)i * gridDim.x);
+            lc_tab[i] = oz_tile(args, L, &gr, &gc, &ar, &br) ? (uint8_t)max(0, oz_lcut<S>(args, ar, br, eref))
                                                                  : (uint8_t)0;
         }
         __syncthreads();
     }
-    auto tile_lc = [&](long long i, int ar, int br) -> int {
+    double *c_stage = reinterpret_cast<double *>((((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023) + ST * OZ_SLOT_BYTES);
+    auto tile_lc = [&](int i, int ar, int br) -> int {
         if (!args.cut) return S + 1;
-        return i < OZ_LC_CAP ? (int)lc_tab[i] : oz_lcut<S, BN>(args, ar, br, eref);
+        return i < OZ_LC_CAP ? (int)lc_tab[i] : oz_lcut<S>(args, ar, br, eref);
     };
     uint8_t *smem = (uint8_t *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
-    const long long ntiles = (long long)args.mt * args.nt;
+    const int ntiles = ntiles_all(args);
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < ST; ++s) {
@@ -282,106 +270,122 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
 
     if (warp == 0) {
         if (lane == 0) {
-            long long g = 0;   // chunks issued
+            // the ring's position and phase are counted along: a division per chunk in this one thread costs more
+            // than the chunk's MMAs
+            int s = 0, filled = 0;
+            uint32_t ph = 0;
             bool ok = true;
-            for (long long L = blockIdx.x, it = 0; L < ntiles && ok; L += gridDim.x, ++it) {
+            for (int L = blockIdx.x, it = 0; L < ntiles && ok; L += gridDim.x, ++it) {
                 int gr, gc, ar, br;
-                if (!oz_tile<BN>(args, L, &gr, &gc, &ar, &br)) continue;
+                if (!oz_tile(args, L, &gr, &gc, &ar, &br)) continue;
                 const int lc = tile_lc(it, ar, br);
 #pragma unroll
-                for (int ps = 0; ps < PASSES; ++ps) {
+                for (int pi = 0; pi < PASSES; ++pi) {
+                    const int ps = LOW_FIRST ? PASSES - 1 - pi : pi;
                     if (Cfg::lev_lo(ps) > lc) break;   // every level of this pass (and later ones) is cut
-                    const int tm = min(Cfg::tmax(ps), lc - 1);
-                    for (int kb = 0; kb < args.nk && ok; ++kb, ++g) {
-                        const int s = (int)(g % ST);
-                        if (g >= ST && !mbar_wait(&empty_bar[s], (uint32_t)(((g / ST) & 1) ^ 1), tword, 21)) {
-                            ok = false;
-                            break;
+                    const int ng = (min(Cfg::tmax(ps), lc - 1) + 3) / 4;   // groups of slices the pass reads
+                    for (int kb = 0; kb < args.nk && ok; ++kb)
+                        for (int gi = 0; gi < ng; ++gi) {
+                            // (a fresh barrier counts as past its odd phase: the first round does not wait)
+                            if (!mbar_wait(&empty_bar[s], ph ^ 1, tword, 21)) {
+                                ok = false;
+                                break;
+                            }
+                            uint8_t *base = smem + (size_t)s * OZ_SLOT_BYTES;
+                            mbar_arrive_expect_tx(&full_bar[s], (uint32_t)OZ_SLOT_BYTES);
+                            tma_load_2d(&mapA, &full_bar[s], base, (kb * NG + gi) * 64, ar);
+                            tma_load_2d(&mapB, &full_bar[s], base + OZ_A_BYTES, (kb * NG + gi) * 64, br);
+                            if (filled < ST) ++filled;
+                            if (++s == ST) s = 0, ph ^= 1;
                         }
-                        uint8_t *base = smem + (size_t)s * STAGE_BYTES;
-                        mbar_arrive_expect_tx(&full_bar[s], (uint32_t)(tm * (A_BYTES + B_BYTES)));
-                        for (int t = 0; t < tm; ++t) {
-                            tma_load_3d(&mapA, &full_bar[s], base + t * A_BYTES, kb * BK, ar, t);
-                            tma_load_3d(&mapB, &full_bar[s], base + S * A_BYTES + t * B_BYTES, kb * BK, br, t);
-                        }
-                    }
                 }
             }
-            if (!ok) {
-                for (long long q = (g > ST ? g - ST : 0); q < g; ++q)
-                    mbar_wait(&full_bar[q % ST], (uint32_t)((q / ST) & 1), tword, 22);
-            }
+            if (!ok)   // the copies in flight, newest first
+                for (int q = 0; q < filled; ++q) {
+                    if (s == 0) s = ST, ph ^= 1;
+                    --s;
+                    mbar_wait(&full_bar[s], ph, tword, 22);
+                }
         }
     } else if (warp == 1) {
         if (lane == 0) {
-            const uint32_t idesc = instr_desc_f16(1, OZ_BM, BN);
-            long long g = 0;
-            int use[NSLOT];   // jobs that have used each accumulator slot so far
-#pragma unroll
-            for (int j = 0; j < NSLOT; ++j) use[j] = 0;
+            const uint32_t idesc = instr_desc_f16(1, OZ_BM, OZ_BN);
+            int s = 0;
+            uint32_t ph = 0;
+            uint32_t used = 0, uph = 0;   // per accumulator slot: used before; parity of its last release
             unsigned long long nmma = 0;
             bool ok = true;
-            for (long long L = blockIdx.x, it = 0; L < ntiles && ok; L += gridDim.x, ++it) {
+            for (int L = blockIdx.x, it = 0; L < ntiles && ok; L += gridDim.x, ++it) {
                 int gr, gc, ar, br;
-                if (!oz_tile<BN>(args, L, &gr, &gc, &ar, &br)) continue;
+                if (!oz_tile(args, L, &gr, &gc, &ar, &br)) continue;
                 const int lc = tile_lc(it, ar, br);
 #pragma unroll
-                for (int ps = 0; ps < PASSES; ++ps) {
+                for (int pi = 0; pi < PASSES; ++pi) {
+                    const int ps = LOW_FIRST ? PASSES - 1 - pi : pi;
                     if (!ok || Cfg::lev_lo(ps) > lc) break;
                     // every slot of the pass takes part in the release protocol; only levels <= lc get MMAs
                     const int llo = Cfg::lev_lo(ps), lhi = Cfg::lev_hi(ps);
-                    for (int kb = 0; kb < args.nk; ++kb, ++g) {
-                        const int s = (int)(g % ST);
-                        if (!mbar_wait(&full_bar[s], (uint32_t)((g / ST) & 1), tword, 23)) {
-                            ok = false;
-                            break;
+                    const int ng = (min(Cfg::tmax(ps), lc - 1) + 3) / 4;
+                    for (int kb = 0; kb < args.nk; ++kb) {
+                        uint64_t da[NG], db[NG];
+                        uint64_t *done[NG];
+#pragma unroll
+                        for (int gi = 0; gi < NG; ++gi) {
+                            if (gi >= ng) continue;
+                            if (!mbar_wait(&full_bar[s], ph, tword, 23)) {
+                                ok = false;
+                                break;
+                            }
+                            const uint32_t a0 = smem_u32(smem + (size_t)s * OZ_SLOT_BYTES);
+                            da[gi] = smem_desc_sw128(a0);
+                            db[gi] = smem_desc_sw128(a0 + OZ_A_BYTES);
+                            done[gi] = &empty_bar[s];
+                            if (++s == ST) s = 0, ph ^= 1;
                         }
+                        if (!ok) break;
                         fence_after_sync();
-                        const uint32_t a0 = smem_u32(smem + (size_t)s * STAGE_BYTES);
-                        const uint64_t da0 = oz_desc<BK>(a0), db0 = oz_desc<BK>(a0 + S * A_BYTES);
 #pragma unroll
-                        for (int kk = 0; kk < BK / 16; ++kk) {
-#pragma unroll
-                            for (int l = 2; l <= S + 1; ++l) {
-                                if (l < llo || l > lhi) continue;
-                                const int tlo = (l - S > 1) ? l - S : 1, thi = (l - 1 < S) ? l - 1 : S;
-                                const int slot = l - llo;
-                                if (kb == 0 && kk == 0 && use[slot] >= 1) {
+                        for (int l = 2; l <= S + 1; ++l) {
+                            if (l < llo || l > lhi) continue;
+                            const int tlo = (l - S > 1) ? l - S : 1, thi = (l - 1 < S) ? l - 1 : S;
+                            const int slot = l - llo;
+                            if (kb == 0) {
+                                if (used >> slot & 1) {
                                     // the epilogue has read this slot's previous contents (per-slot release)
-                                    if (!mbar_wait(&slot_empty[slot], (uint32_t)((use[slot] - 1) & 1), tword, 25)) {
+                                    if (!mbar_wait(&slot_empty[slot], uph >> slot & 1, tword, 25)) {
                                         ok = false;
                                         break;
                                     }
                                     fence_after_sync();
+                                    uph ^= 1u << slot;
                                 }
-                                if (l > lc) continue;
-                                nmma += (unsigned long long)(thi - tlo + 1);
-#pragma unroll
-                                for (int t = tlo; t <= thi; ++t) {
-                                    const int u = l - t;
-                                    const uint32_t acc = tmem + (uint32_t)((l - llo) * BN);
-                                    // start-address field += offset / 16 (no carry: smem addresses < 2^18)
-                                    mma_f16(acc, da0 + (uint64_t)(((t - 1) * A_BYTES + kk * 32) >> 4),
-                                            db0 + (uint64_t)(((u - 1) * B_BYTES + kk * 32) >> 4), idesc,
-                                            (kb != 0 || kk != 0 || t != tlo) ? 1u : 0u);
-                                }
+                                used |= 1u << slot;
                             }
-                            if (!ok) break;
+                            if (l > lc) continue;
+                            nmma += (unsigned long long)(thi - tlo + 1);
+#pragma unroll
+                            for (int t = tlo; t <= thi; ++t) {
+                                const int u = l - t;
+                                // slice t: group (t - 1) / 4, 32-byte step (t - 1) % 4 (the start-address field
+                                // counts 16 bytes; no carry: smem addresses < 2^18)
+                                mma_f16(tmem + (uint32_t)(slot * OZ_BN), da[(t - 1) / 4] + (uint64_t)(((t - 1) % 4) * 2),
+                                        db[(u - 1) / 4] + (uint64_t)(((u - 1) % 4) * 2), idesc,
+                                        (kb != 0 || t != tlo) ? 1u : 0u);
+                            }
                         }
                         if (!ok) break;
-                        mma_commit(&empty_bar[s]);
+#pragma unroll
+                        for (int gi = 0; gi < NG; ++gi)
+                            if (gi < ng) mma_commit(done[gi]);
                     }
                     if (!ok) break;
                     mma_commit(&acc_full);
-#pragma unroll
-                    for (int l = 2; l <= S + 1; ++l)
-                        if (l >= llo && l <= lhi) ++use[l - llo];
                 }
             }
             // every MMA issued so far has completed before TMEM can be freed
             mma_commit(&drain_bar);
             mbar_wait(&drain_bar, 0, tword, 26);
-            if (args.tc_flops) atomicAdd(args.tc_flops, nmma * (unsigned long long)(2 * OZ_BM * BN * 16));
+            if (args.tc_flops) atomicAdd(args.tc_flops, nmma * (unsigned long long)(2 * OZ_BM * OZ_BN * 16));
         }
         __syncwarp();
     } else {
@@ -390,37 +394,53 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
         const int row = q * 32 + lane;
         int job = 0;
         bool ok = true;
-        // C entries of this thread's row, CQ columns at a time, double-buffered through shared
-        // memory by cp.async: the copies for the next columns are in flight while the current
-        // ones are updated, and no register waits on a load of C
-        constexpr int CQ = 4;
-        double *cbuf = &c_stage[(warp - 2) * 2 * CQ * 32];
-        for (long long L = blockIdx.x, it = 0; L < ntiles && ok; L += gridDim.x, ++it) {
+        // C entries of this thread's row come through shared memory by cp.async, OZ_CD columns ahead, the first of
+        // them while the tile's MMAs still run: a load of C takes about a microsecond, and with four columns in
+        // flight these waits were 28 us a pass
+        double *cbuf = c_stage + (warp - 2) * OZ_CD * 32 + lane;
+        for (int L = blockIdx.x, it = 0; L < ntiles && ok; L += gridDim.x, ++it) {
             int gr, gc, ar, br;
-            if (!oz_tile<BN>(args, L, &gr, &gc, &ar, &br)) continue;
+            if (!oz_tile(args, L, &gr, &gc, &ar, &br)) continue;
             const int lc = tile_lc(it, ar, br);
             const int grow = gr + row;
             const int er = (grow < args.m_end) ? args.ea[ar + row] : 0;
+            double *cp = args.C + (long long)(gc + h * CPT) * args.ldc + grow;
+            const int *eb = args.eb + br + h * CPT;
+            const int c_all = min(CPT, args.n_end - (gc + h * CPT));
+            const int eb0 = lane < c_all ? eb[lane] : 0, eb1 = 32 + lane < c_all ? eb[32 + lane] : 0;
+            int c_end = c_all;   // this thread's columns, in a triangle up to its row
+            if (args.tri) c_end = min(c_end, grow - (gc + h * CPT) + 1);
+            if (grow >= args.m_end) c_end = 0;
 #pragma unroll
-            for (int ps = 0; ps < PASSES; ++ps) {
+            for (int pi = 0; pi < PASSES; ++pi) {
+                const int ps = LOW_FIRST ? PASSES - 1 - pi : pi;
                 if (Cfg::lev_lo(ps) > lc) break;
+                const bool over = args.overwrite && pi == 0;
+                const int c_load = over ? 0 : c_end;
+                const double *cs = cp;   // the next column to stage
+                auto stage = [&](int j0) {
+#pragma unroll
+                    for (int jj = 0; jj < OZ_CQ; ++jj, cs += args.ldc)
+                        if (j0 + jj < c_load) cp_async8(&cbuf[(j0 + jj) % OZ_CD * 32], cs);
+                    cp_async_commit();
+                };
+#pragma unroll
+                for (int j0 = 0; j0 < OZ_CD; j0 += OZ_CQ) stage(j0);
                 ok = mbar_wait(&acc_full, (uint32_t)(job & 1), tword, 24);
                 ok = __all_sync(0xffffffffu, ok);   // every lane takes part in tcgen05.ld
                 if (!ok) break;
                 fence_after_sync();
                 const int llo = Cfg::lev_lo(ps), lhi = Cfg::lev_hi(ps);
-                const int w0 = ps * Cfg::WPP;
-                long long acc[WREG][CPT];
+                long long acc[CPT];
 #pragma unroll
                 for (int l = 2; l <= S + 1; ++l) {
                     if (l < llo || l > lhi) continue;
-                    const int wi = (l - 2) / OZ_LPW - w0;   // word of this level within the pass
                     const bool first = ((l - 2) % OZ_LPW) == 0;
                     const bool live = l <= lc;   // a cut level's slot holds stale values: taken as 0
 #pragma unroll
                     for (int c32 = 0; c32 < CPT / 32; ++c32) {
                         float v[32];
-                        tmem_ld32(tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)((l - llo) * BN + h * CPT + c32 * 32),
+                        tmem_ld32(tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)((l - llo) * OZ_BN + h * CPT + c32 * 32),
                                   v);
                         if (c32 == CPT / 32 - 1) {
                             // this warp has read the slot: the MMAs of the next job may overwrite it
@@ -431,69 +451,32 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
 #pragma unroll
                         for (int j = 0; j < 32; ++j) {
                             const long long d = live ? (long long)__float2int_rn(v[j]) : 0;   // exact, below 2^24
-                            acc[wi][c32 * 32 + j] = first ? d : acc[wi][c32 * 32 + j] * 128 + d;
+                            acc[c32 * 32 + j] = first ? d : acc[c32 * 32 + j] * 128 + d;
                         }
                     }
                 }
                 ++job;
-                if (grow < args.m_end) {
-                    const bool over = args.overwrite && ps == 0;
-                    auto live_col = [&](int j) {
-                        const int gcol = gc + h * CPT + j;
-                        return gcol < args.n_end && !(args.tri && grow < gcol);
-                    };
-                    auto stage = [&](int j0, int b) {
+                double *cw = cp;
 #pragma unroll
-                        for (int jj = 0; jj < CQ; ++jj)
-                            if (live_col(j0 + jj))
-                                cp_async8(&cbuf[(b * CQ + jj) * 32 + lane],
-                                          args.C + (long long)(gc + h * CPT + j0 + jj) * args.ldc + grow);
-                        cp_async_commit();
-                    };
-                    if (!args.cut || over) {
-                        // every level kept: the MMAs, not these loads, set the pace
+                for (int j0 = 0; j0 < CPT; j0 += OZ_CQ) {
+                    cp_async_wait<OZ_CD / OZ_CQ - 1>();
 #pragma unroll
-                        for (int j = 0; j < CPT; ++j) {
-                            if (!live_col(j)) continue;
-                            const int e = er + args.eb[br + h * CPT + j];
-                            double *pc = args.C + (long long)(gc + h * CPT + j) * args.ldc + grow;
-                            double c = over ? 0.0 : *pc;
-#pragma unroll
-                            for (int wi = WREG - 1; wi >= 0; --wi) {
-                                if (w0 + wi >= Cfg::NWT || 2 + OZ_LPW * (w0 + wi) > lc) continue;
-                                c = fma(-(double)acc[wi][j], pow2i(e + 2 - 7 * Cfg::word_hi(w0 + wi)), c);
-                            }
-                            *pc = c;
-                        }
-                        continue;
+                    for (int jj = 0; jj < OZ_CQ; ++jj, cw += args.ldc) {
+                        const int j = j0 + jj;
+                        // the columns' exponents sit in the warp's lanes
+                        const int e = er + __shfl_sync(0xffffffffu, j < 32 ? eb0 : eb1, j % 32);
+                        double c = over ? 0.0 : cbuf[j % OZ_CD * 32];
+                        c = fma(-(double)acc[j], pow2i(e + 2 - 7 * lhi), c);
+                        if (j < c_end) *cw = c;
                     }
-                    stage(0, 0);
-#pragma unroll
-                    for (int j0 = 0; j0 < CPT; j0 += CQ) {
-                        const int b = (j0 / CQ) & 1;
-                        if (j0 + CQ < CPT) {
-                            stage(j0 + CQ, b ^ 1);
-                            cp_async_wait<1>();
-                        } else {
-                            cp_async_wait<0>();
-                        }
-#pragma unroll
-                        for (int jj = 0; jj < CQ; ++jj) {
-                            const int j = j0 + jj;
-                            if (!live_col(j)) continue;
-                            const int e = er + args.eb[br + h * CPT + j];
-                            double c = cbuf[(b * CQ + jj) * 32 + lane];
-#pragma unroll
-                            for (int wi = WREG - 1; wi >= 0; --wi) {
-                                if (w0 + wi >= Cfg::NWT || 2 + OZ_LPW * (w0 + wi) > lc) continue;
-                                c = fma(-(double)acc[wi][j], pow2i(e + 2 - 7 * Cfg::word_hi(w0 + wi)), c);
-                            }
-                            args.C[(long long)(gc + h * CPT + j) * args.ldc + grow] = c;
-                        }
-                    }
+                    if (j0 + OZ_CD < CPT)
+                        stage(j0 + OZ_CD);
+                    else
+                        cp_async_commit();   // an empty group keeps the count
                 }
             }
         }
+        cp_async_wait<0>();
     }
     fence_before_sync();
     __syncthreads();
@@ -506,8 +489,8 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
 
 // Digit slices of rows [0, R) of the column-major FP64 panel P (ld), columns
 // [k0, k0 + kc) for the K chunk blockIdx.y (kc = kchunk, the last one
-// shorter): slice t of row r at out[t * slice_stride + r * Kp + k] (BF16,
-// zero for k beyond the panel), the row exponent at exps[chunk * exp_stride + r].
+// shorter): digit t (from 0) of row r, column k at out[(r Kp + k / 16 * 16) Sg + 16 t + k % 16]
+// (BF16, zero for k beyond the panel), the row exponent at exps[chunk * exp_stride + r].
 // Per 32-row block b the largest exponent of its non-zero rows goes to
 // bexps[2 chunk bstride + b], and that of its non-zero rows below ref_rows to
 // bexps[(2 chunk + 1) bstride + b] (OZ_E_NONE where there is none).
@@ -546,7 +529,7 @@ __device__ __forceinline__ unsigned int oz_bf16_bits(int d) {
 }
 
 __global__ void __launch_bounds__(256) k_oz_slice(const double *P, long long ld, int R, int K, int kchunk, int S,
-                                                  __nv_bfloat16 *out, long long slice_stride, int Kp, int *exps,
+                                                  __nv_bfloat16 *out, int Sg, int Kp, int *exps,
                                                   long long exp_stride, int *bexps, long long bstride, int ref_rows,
                                                   const DevStatus *st) {
     __shared__ unsigned long long tile[32][33];
@@ -600,7 +583,7 @@ __global__ void __launch_bounds__(256) k_oz_slice(const double *P, long long ld,
             long long X[4];
 #pragma unroll
             for (int i = 0; i < 4; ++i) X[i] = oz_scaled_int(tile[cq + i][r], kshift);
-            unsigned int *o = reinterpret_cast<unsigned int *>(out + (long long)(r0 + r) * Kp + c0 + cq);
+            unsigned int *o = reinterpret_cast<unsigned int *>(out + ((long long)(r0 + r) * Kp + (c0 + cq) / 16 * 16) * Sg + cq % 16);
             for (int sl = S - 1; sl >= 1; --sl) {
                 int d[4];
 #pragma unroll
@@ -611,7 +594,7 @@ __global__ void __launch_bounds__(256) k_oz_slice(const double *P, long long ld,
                 uint2 v;
                 v.x = oz_bf16_bits(d[0]) | (oz_bf16_bits(d[1]) << 16);
                 v.y = oz_bf16_bits(d[2]) | (oz_bf16_bits(d[3]) << 16);
-                *reinterpret_cast<uint2 *>(o + (long long)sl * slice_stride / 2) = v;
+                *reinterpret_cast<uint2 *>(o + sl * 8) = v;
             }
             uint2 v;   // leading digits, |X| <= 64
             v.x = oz_bf16_bits((int)X[0]) | (oz_bf16_bits((int)X[1]) << 16);
@@ -622,60 +605,29 @@ __global__ void __launch_bounds__(256) k_oz_slice(const double *P, long long ld,
     }
 }
 
-template <int S, int BN, int BK>
+template <int S, bool LOW_FIRST = false>
 cudaError_t launch_oz_kernel(const CUtensorMap &ma, const CUtensorMap &mb, const OzArgs &a, int grid,
                              cudaStream_t s) {
-    using Cfg = OzCfg<S, BN, BK>;
-    static_assert(Cfg::STAGES >= 2, "shared memory holds fewer than two chunks");
-    cudaError_t e = cudaFuncSetAttribute(k_oz_update<S, BN, BK>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)Cfg::SMEM);
+    static_assert(OZ_SLOTS >= 2 * OzCfg<S>::NG, "shared memory holds fewer than two chunks");
+    cudaError_t e = cudaFuncSetAttribute(k_oz_update<S, LOW_FIRST>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)OZ_SMEM);
     if (e != cudaSuccess) return e;
-    k_oz_update<S, BN, BK><<<grid, OZ_THREADS, Cfg::SMEM, s>>>(ma, mb, a);
+    k_oz_update<S, LOW_FIRST><<<grid, OZ_THREADS, OZ_SMEM, s>>>(ma, mb, a);
     return cudaGetLastError();
 }
 
-// Kernel shape per slice count (measured on GB300 with C 8192 x 8192, K = 512):
-// with 6 or more slices the 128-column tile in passes of four levels keeps the
-// tensor pipe busiest (8 slices: 1,290 against 1,063 TFLOP/s of BF16 work for
-// the single-pass 64-column tile); with fewer the passes get short and the
-// 64-column single pass wins (5 slices: 902 against 655).  With the level cut
-// at 5 slices the 128-column tile wins again: the second pass (the last
-// level) is cut on most tiles, so the epilogue, which sets the pace of cut
-// tiles, works on half as many C entries per MMA (N = 100,000: 4.3 against
-// 5.8 s per factorisation).
-struct OzShape {
-    int bn, bk;
-};
-
-OzShape oz_shape(int S, int cut) { return (S >= 6 || (S == 5 && cut)) ? OzShape{128, 16} : OzShape{64, 32}; }
-
-template <int S>
-cudaError_t launch_oz_shape(OzShape sh, const CUtensorMap &ma, const CUtensorMap &mb, const OzArgs &a, int grid,
-                            cudaStream_t s) {
-    if constexpr (S >= 6) {
-        return launch_oz_kernel<S, 128, 16>(ma, mb, a, grid, s);
-    } else if constexpr (S == 5) {
-        if (sh.bn == 128) return launch_oz_kernel<S, 128, 16>(ma, mb, a, grid, s);
-        return launch_oz_kernel<S, 64, 32>(ma, mb, a, grid, s);
-    } else {
-        return launch_oz_kernel<S, 64, 32>(ma, mb, a, grid, s);
-    }
-}
-
-// 3-D tensor map over the slices: (k, row, slice), box bk x rows_box x 1,
-// swizzle = the K chunk's row width (32 or 64 bytes).
-cudaError_t slice_map(CUtensorMap *map, const OzSlices &sl, int chunk, int rows_box, int bk) {
+// 2-D tensor map over the digits of a K chunk: (interleaved columns, row), box 64 (four slices of 16 columns:
+// one 128-byte line) x rows_box, swizzled by lines.
+cudaError_t slice_map(CUtensorMap *map, const OzSlices &sl, int chunk, int rows_box) {
     tc::EncodeTiledFn enc = tc::encode_fn();
     if (!enc) return cudaErrorNotSupported;
-    void *base = (__nv_bfloat16 *)sl.d + (size_t)chunk * sl.kchunk;   // 64-byte aligned: kchunk is a multiple of 32
-    cuuint64_t dims[3] = {(cuuint64_t)std::min(sl.kchunk, sl.Kp - chunk * sl.kchunk), (cuuint64_t)sl.valid,
-                          (cuuint64_t)sl.S};
-    cuuint64_t strides[2] = {(cuuint64_t)sl.Kp * 2, (cuuint64_t)sl.slice_stride * 2};
-    cuuint32_t box[3] = {(cuuint32_t)bk, (cuuint32_t)rows_box, 1};
-    cuuint32_t es[3] = {1, 1, 1};
-    CUresult cr = enc(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, base, dims, strides, box, es,
-                      CU_TENSOR_MAP_INTERLEAVE_NONE, bk == 16 ? CU_TENSOR_MAP_SWIZZLE_32B : CU_TENSOR_MAP_SWIZZLE_64B,
-                      CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    void *base = (__nv_bfloat16 *)sl.d + (size_t)chunk * sl.kchunk * sl.Sg;   // kchunk is a multiple of 32
+    cuuint64_t dims[2] = {(cuuint64_t)std::min(sl.kchunk, sl.Kp - chunk * sl.kchunk) * sl.Sg, (cuuint64_t)sl.valid};
+    cuuint64_t strides[1] = {(cuuint64_t)sl.Kp * sl.Sg * 2};
+    cuuint32_t box[2] = {64, (cuuint32_t)rows_box};
+    cuuint32_t es[2] = {1, 1};
+    CUresult cr = enc(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, base, dims, strides, box, es,
+                      CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                      CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     return cr == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
 }
 
@@ -686,7 +638,7 @@ int oz_kmax(int S) { return (4096 / S) / OZ_KALIGN * OZ_KALIGN; }
 size_t oz_slices_bytes(long long rows, int K, int S) {
     const long long Kp = (K + OZ_KALIGN - 1) / OZ_KALIGN * OZ_KALIGN;
     const int nchunk = (K + oz_kmax(S) - 1) / oz_kmax(S);
-    return (size_t)S * (size_t)rows * (size_t)Kp * 2 + sizeof(int) * (size_t)rows * nchunk +
+    return (size_t)((S + 3) / 4 * 4) * (size_t)rows * (size_t)Kp * 2 + sizeof(int) * (size_t)rows * nchunk +
            sizeof(int) * 2 * (size_t)((rows + 31) / 32) * nchunk + 768;
 }
 
@@ -699,9 +651,9 @@ OzSlices oz_slices_carve(void *ws, long long rows, int K, int S) {
     o.Kp = (K + OZ_KALIGN - 1) / OZ_KALIGN * OZ_KALIGN;
     o.nchunk = (K + o.kchunk - 1) / o.kchunk;
     o.valid = rows;
-    o.slice_stride = (long long)rows * o.Kp;
+    o.Sg = (S + 3) / 4 * 4;
     o.d = ws;
-    uintptr_t e = (uintptr_t)ws + (size_t)S * o.slice_stride * 2;
+    uintptr_t e = (uintptr_t)ws + (size_t)o.Sg * rows * o.Kp * 2;
     o.e = (int *)((e + 255) & ~(uintptr_t)255);
     o.bstride = (rows + 31) / 32;
     o.be = (int *)(((uintptr_t)(o.e + rows * o.nchunk) + 255) & ~(uintptr_t)255);
@@ -714,7 +666,7 @@ cudaError_t oz_slice(const double *P, long long ld, int R, const OzSlices &o, co
     if (R > o.rows || R > o.valid) return cudaErrorInvalidValue;
     dim3 grid((R + 31) / 32, o.nchunk);
     KScope ks(GEO_K_AUX, s, 0.0, (double)R * o.K * (16.0 + 2.0 * o.S));
-    k_oz_slice<<<grid, 256, 0, s>>>(P, ld, R, o.K, o.kchunk, o.S, (__nv_bfloat16 *)o.d, o.slice_stride, o.Kp, o.e,
+    k_oz_slice<<<grid, 256, 0, s>>>(P, ld, R, o.K, o.kchunk, o.S, (__nv_bfloat16 *)o.d, o.Sg, o.Kp, o.e,
                                     o.rows, o.be, o.bstride, o.ref_rows < 0 ? R : (int)std::min<long long>(o.ref_rows, R),
                                     st);
     return cudaGetLastError();
@@ -734,9 +686,8 @@ cudaError_t oz_update(const OzSlices &A, const OzSlices &B, double *C, long long
     a.c0 = c0;
     a.m_end = m_end;
     a.n_end = n_end;
-    const OzShape sh = oz_shape(S, cut);
     a.mt = (rows + OZ_BM - 1) / OZ_BM;
-    a.nt = (cols + sh.bn - 1) / sh.bn;
+    a.nt = (cols + OZ_BN - 1) / OZ_BN;
     a.tri = tri;
     a.a_off = a_off;
     a.overwrite = 0;
@@ -747,13 +698,14 @@ cudaError_t oz_update(const OzSlices &A, const OzSlices &B, double *C, long long
     a.nbb = (int)((B.valid + 31) / 32);
     a.tc_flops = t_prof ? t_prof->d_tc_flops : nullptr;
     const long long ntiles = (long long)a.mt * a.nt;
+    if (ntiles > (1LL << 30)) return cudaErrorInvalidValue;   // the kernel counts tiles in 32 bits
     const int grid = (int)std::min<long long>(ntiles, std::max(1, std::min(grid_cap, tc::num_sms())));
     // algorithmic work: 2 K flops per output written (lower triangle when tri)
     const double rr = rows, cc = cols;
     const double outs = tri ? std::max(0.0, rr * cc - cc * (cc - 1.0) / 2.0) : rr * cc;
     for (int ch = 0; ch < A.nchunk; ++ch) {
         const int kc = std::min(A.kchunk, A.K - ch * A.kchunk);
-        a.nk = (kc + sh.bk - 1) / sh.bk;
+        a.nk = (kc + 15) / 16;
         a.ea = A.e + (long long)ch * A.rows;
         a.eb = B.e + (long long)ch * B.rows;
         a.ba = A.be + 2LL * ch * A.bstride;
@@ -762,18 +714,19 @@ cudaError_t oz_update(const OzSlices &A, const OzSlices &B, double *C, long long
         a.rb = a.bb + B.bstride;
         CUtensorMap ma, mb;
         cudaError_t e;
-        if ((e = slice_map(&ma, A, ch, OZ_BM, sh.bk)) != cudaSuccess ||
-            (e = slice_map(&mb, B, ch, sh.bn, sh.bk)) != cudaSuccess)
+        if ((e = slice_map(&ma, A, ch, OZ_BM)) != cudaSuccess ||
+            (e = slice_map(&mb, B, ch, OZ_BN)) != cudaSuccess)
             return e;
         a.overwrite = (overwrite && ch == 0) ? 1 : 0;   // later K chunks accumulate onto the first
         KScope ks(GEO_K_TCGEMM, s, 2.0 * kc * outs, 16.0 * outs + 2.0 * S * kc * (rr + cc));
         switch (S) {
-            case 3: e = launch_oz_shape<3>(sh, ma, mb, a, grid, s); break;
-            case 4: e = launch_oz_shape<4>(sh, ma, mb, a, grid, s); break;
-            case 5: e = launch_oz_shape<5>(sh, ma, mb, a, grid, s); break;
-            case 6: e = launch_oz_shape<6>(sh, ma, mb, a, grid, s); break;
-            case 7: e = launch_oz_shape<7>(sh, ma, mb, a, grid, s); break;
-            default: e = launch_oz_shape<8>(sh, ma, mb, a, grid, s); break;
+            case 3: e = launch_oz_kernel<3>(ma, mb, a, grid, s); break;
+            case 4: e = launch_oz_kernel<4>(ma, mb, a, grid, s); break;
+            // five slices without the cut add their last level first (the sums' rounding is part of the form's result)
+            case 5: e = cut ? launch_oz_kernel<5>(ma, mb, a, grid, s) : launch_oz_kernel<5, true>(ma, mb, a, grid, s); break;
+            case 6: e = launch_oz_kernel<6>(ma, mb, a, grid, s); break;
+            case 7: e = launch_oz_kernel<7>(ma, mb, a, grid, s); break;
+            default: e = launch_oz_kernel<8>(ma, mb, a, grid, s); break;
         }
         if (e != cudaSuccess) return e;
     }
