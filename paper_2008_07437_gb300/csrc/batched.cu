@@ -261,6 +261,7 @@ __global__ void __launch_bounds__(LA_THREADS) k_house_qr(const QrDesc *__restric
     // thin Q: start from [I; 0] and apply H_c for c = r-1 .. 0
     double *Q = q.Q;
     const long long ldq = q.ldq;
+    if (!Q) return;   // only R was wanted
     for (int j = warp; j < r; j += LA_WARPS)
         for (int i = lane; i < m; i += 32) Q[(long long)j * ldq + i] = (i == j) ? 1.0 : 0.0;
     __syncthreads();
@@ -391,6 +392,10 @@ __global__ void __launch_bounds__(QT, 1) k_house_qr_cl(const QrDesc *__restrict_
     // thin Q: [I; 0] on this CTA's rows, then H_c for c = r-1 .. 0
     double *Q = q.Q;
     const long long ldq = q.ldq;
+    if (!Q) {   // only R was wanted
+        cluster.sync();
+        return;
+    }
     for (int j = warp; j < r; j += nw)
         for (int i = row0 + lane; i < row1; i += 32) Q[(long long)j * ldq + i] = (i == j) ? 1.0 : 0.0;
     __syncthreads();
@@ -432,23 +437,203 @@ __global__ void __launch_bounds__(QT, 1) k_house_qr_cl(const QrDesc *__restrict_
     cluster.sync();   // no CTA leaves while another still reads its shared memory
 }
 
+// ---- the same with the whole block in the shared memory of a cluster ---------
+// Columns are dealt out to the CTAs in turn (column j to CTA j % QC), all rows
+// of each in shared memory: a reflector needs no exchange of partial dots, only
+// the reflector itself, which its column's CTA stores into the others' shared
+// memory before the step's one cluster barrier.  A warp takes a column, or two
+// at once so that their sums share the shuffles; the norm of the next column
+// comes out of its update.  The reflectors also go to global memory (in place),
+// from where the thin Q, which takes the block's place in shared memory, is
+// accumulated without any exchange.  With Rt only R is formed: R' goes to Rt
+// and the block is left as it is.  Bound by the FP64 units of eight SMs:
+// m = 900, r = 216 3.6 ms, R alone 2.2 (16.5 with the rows split over the CTAs
+// and two exchanges a column).
+constexpr int QCT = 512, QCW = QCT / 32;
+
+size_t house_qr_col_smem(int m, int r) {
+    return sizeof(double) * ((size_t)((r + QC - 1) / QC) * m + 2 * (size_t)(m + 2) + QR_MAX + 4);
+}
+
+// 1 / sqrt(d) and 1 / d of a positive normal d: the hardware's approximations (20 bits and more) and one step of
+// Halley's iteration.
+__device__ __forceinline__ double fast_rsqrt(double d) {
+    double y;
+    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(d));
+    const double e = fma(-(d * y), y, 1.0);
+    return fma(y * e, fma(0.375, e, 0.5), y);
+}
+__device__ __forceinline__ double fast_rcp(double d) {
+    double y;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(d));
+    const double e = fma(-d, y, 1.0);
+    return fma(y, fma(e, e, e), y);
+}
+
+// y_j -= tau (v'y_j) v for two columns (b2: the second one exists), rows [c, m); v in shared memory, row i at
+// v[i].  nrm: receives |y[c1..]|^2 of the first column over the rows from c1 on (NULL: not wanted).
+__device__ __forceinline__ void qr_apply(const double *v, double tau, double *y1, double *y2, bool b2, int c, int m, int c1,
+                                         double *nrm, int lane) {
+    double d1 = 0.0, d2 = 0.0;
+    const double *z2 = b2 ? y2 : y1;
+    for (int i = c + lane; i < m; i += 32) {
+        const double vi = v[i];
+        d1 = fma(vi, y1[i], d1);
+        d2 = fma(vi, z2[i], d2);
+    }
+    // lanes 0-15 sum the first column, 16-31 the second
+    double a = (lane < 16 ? d1 : d2) + __shfl_xor_sync(0xffffffffu, lane < 16 ? d2 : d1, 16);
+    for (int o = 8; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
+    a *= -tau;
+    d1 = __shfl_sync(0xffffffffu, a, 0);
+    d2 = __shfl_sync(0xffffffffu, a, 16);
+    double s = 0.0;
+    for (int i = c + lane; i < m; i += 32) {
+        const double vi = v[i], n1 = fma(d1, vi, y1[i]);
+        y1[i] = n1;
+        if (b2) y2[i] = fma(d2, vi, y2[i]);
+        if (nrm && i >= c1) s = fma(n1, n1, s);
+    }
+    if (nrm) {
+        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+        if (lane == 0) *nrm = s;
+    }
+}
+
+__global__ void __launch_bounds__(QCT, 1) k_house_qr_col(const QrDesc *__restrict__ d, int count) {
+    cg::cluster_group cluster = cg::this_cluster();
+    const int tile = blockIdx.x / QC;
+    if (tile >= count) return;   // uniform over the cluster
+    const int rank = (int)cluster.block_rank();
+    const QrDesc q = d[tile];
+    const int m = q.m, r = q.r, nloc = (r + QC - 1) / QC;
+    extern __shared__ double csm[];
+    double *Ys = csm;                          // [nloc][m]
+    double *vb = Ys + (size_t)nloc * m;        // [2][m + 2]: reflector (row i at i), then tau at m
+    double *taus = vb + 2 * (m + 2);           // [QR_MAX]
+    double *sc = taus + QR_MAX;                // norm of the next column; alpha, v0, tau of the current one
+    const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
+    for (int lj = warp; lj < nloc; lj += QCW) {
+        const int j = lj * QC + rank;
+        if (j < r)
+            for (int i = lane; i < m; i += 32) Ys[(size_t)lj * m + i] = q.Y[(long long)j * q.ldy + i];
+    }
+    __syncthreads();
+    if (rank == 0 && warp == 0) {
+        double s = 0.0;
+        for (int i = lane; i < m; i += 32) s = fma(Ys[i], Ys[i], s);
+        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+        if (lane == 0) sc[0] = s;
+    }
+    cluster.sync();   // every CTA runs (its shared memory may be written); the first norm
+    for (int c = 0; c < r; ++c) {
+        double *v = vb + (c & 1) * (m + 2);
+        if (rank == c % QC) {
+            double *x = Ys + (size_t)(c / QC) * m;
+            if (warp == 0 && lane == 0) {
+                const double nrm2 = sc[0], x0 = x[c];
+                double alpha = 0.0, v0 = 1.0, tau = 0.0;
+                if (nrm2 > 0.0) {
+                    const double nrm = sqrt(nrm2);
+                    alpha = (x0 >= 0.0) ? -nrm : nrm;
+                    v0 = x0 - alpha;
+                    // v'v = v0^2 + (nrm2 - x0^2) = 2 nrm (nrm + |x0|)
+                    tau = 1.0 / (nrm * (nrm + fabs(x0)));
+                }
+                sc[1] = alpha;
+                sc[2] = v0;
+                sc[3] = tau;
+            }
+            __syncthreads();
+            const double alpha = sc[1], v0 = sc[2], tau = sc[3];
+            for (int i = c + threadIdx.x; i < m; i += QCT) {
+                const double vi = i == c ? v0 : x[i];
+                for (int k = 0; k < QC; ++k) cluster.map_shared_rank(v, k)[i] = vi;
+                if (q.Q) q.Y[(long long)c * q.ldy + i] = vi;
+            }
+            if (threadIdx.x < QC) cluster.map_shared_rank(v, threadIdx.x)[m] = tau;
+            __syncthreads();
+            if (threadIdx.x == 0) x[c] = alpha;   // R's diagonal
+        }
+        cluster.sync();
+        const double tau = v[m];
+        if (threadIdx.x == 0) taus[c] = tau;
+        // the columns after c on this CTA; the next column (if it is here) first, alone
+        const int l0 = (c + QC - rank) / QC;   // first local column with j > c
+        const bool own = rank == (c + 1) % QC && c + 1 < r;
+        if (own && warp == 0) qr_apply(v, tau, Ys + (size_t)l0 * m, nullptr, false, c, m, c + 1, sc, lane);
+        const int lf = l0 + (own ? 1 : 0), nl = (r - rank + QC - 1) / QC - lf;   // the others
+        // one column a warp while there are warps enough, else two
+        const int w = own ? warp - 1 : warp, nw = own ? QCW - 1 : QCW;
+        if (w >= 0) {
+            if (nl <= nw) {
+                if (w < nl) qr_apply(v, tau, Ys + (size_t)(lf + w) * m, nullptr, false, c, m, 0, nullptr, lane);
+            } else {
+                for (int p = w; 2 * p < nl; p += nw)
+                    qr_apply(v, tau, Ys + (size_t)(lf + 2 * p) * m, Ys + (size_t)(lf + 2 * p + 1) * m, 2 * p + 1 < nl, c, m, 0,
+                             nullptr, lane);
+            }
+        }
+        __syncthreads();
+    }
+    if (q.Rt) {   // column j of R is row j of the lower triangular R'
+        for (int lj = warp; lj < nloc; lj += QCW) {
+            const int j = lj * QC + rank;
+            if (j < r)
+                for (int c = lane; c < r; c += 32) q.Rt[(long long)c * q.ldr + j] = c <= j ? Ys[(size_t)lj * m + c] : 0.0;
+        }
+    }
+    if (!q.Q) {
+        cluster.sync();   // no CTA leaves while another may still write its shared memory
+        return;
+    }
+    __threadfence();
+    cluster.sync();       // the reflectors in global memory
+    for (int lj = warp; lj < nloc; lj += QCW) {
+        const int j = lj * QC + rank;
+        for (int i = lane; i < m; i += 32) Ys[(size_t)lj * m + i] = (i == j) ? 1.0 : 0.0;
+    }
+    auto fetch = [&](int c) {
+        for (int i = c + threadIdx.x; i < m; i += QCT) vb[(c & 1) * (m + 2) + i] = __ldcg(q.Y + (long long)c * q.ldy + i);
+    };
+    fetch(r - 1);
+    __syncthreads();
+    for (int c = r - 1; c >= 0; --c) {
+        if (c > 0) fetch(c - 1);
+        const double *v = vb + (c & 1) * (m + 2);
+        const double tau = taus[c];
+        const int lf = (c + QC - 1 - rank) / QC, nl = (r - rank + QC - 1) / QC - lf;   // local columns with j >= c
+        if (nl <= QCW) {
+            if (warp < nl) qr_apply(v, tau, Ys + (size_t)(lf + warp) * m, nullptr, false, c, m, 0, nullptr, lane);
+        } else {
+            for (int p = warp; 2 * p < nl; p += QCW)
+                qr_apply(v, tau, Ys + (size_t)(lf + 2 * p) * m, Ys + (size_t)(lf + 2 * p + 1) * m, 2 * p + 1 < nl, c, m, 0,
+                         nullptr, lane);
+        }
+        __syncthreads();
+    }
+    for (int lj = warp; lj < nloc; lj += QCW) {
+        const int j = lj * QC + rank;
+        if (j < r)
+            for (int i = lane; i < m; i += 32) q.Q[(long long)j * q.ldq + i] = Ys[(size_t)lj * m + i];
+    }
+}
+
 // ---- one-sided Jacobi SVD of an r x r block M (Hestenes) --------------------
-// Rotates column pairs of M (and accumulates V) until every pair is
-// orthogonal to relative 1e-13 or the sweep budget is spent (pairs whose
-// columns both have norms below `skip` are not rotated); on exit the
-// column norms of M are the singular values (unsorted), M = U S V' with
-// U = M_col / norm.  Pairs are processed in round-robin order, r/2 disjoint
-// pairs per round, one warp per pair.
+// Rotates column pairs of M until every pair is orthogonal to relative 1e-13 or
+// the sweep budget is spent (pairs whose columns both have norms below `skip`
+// are not rotated); on exit the column norms of M are the singular values
+// (unsorted) and the columns over their norms the left singular vectors.
+// Pairs are processed in round-robin order, r/2 disjoint pairs per round, one
+// warp per pair.
 __global__ void __launch_bounds__(LA_THREADS) k_jacobi_svd(const SvdDesc *__restrict__ d, int count, int max_sweeps) {
     const int pi = blockIdx.x;
     if (pi >= count) return;
     const SvdDesc s = d[pi];
     const int r = s.r;
-    double *M = s.M, *V = s.V;
+    double *M = s.M;
     const long long ld = s.ld;
     const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
-    for (int j = warp; j < r; j += LA_WARPS)
-        for (int i = lane; i < r; i += 32) V[(long long)j * ld + i] = (i == j) ? 1.0 : 0.0;
     __shared__ int rotated;
     const int rr = r + (r & 1);   // round-robin over an even count (index r = dummy)
     for (int sweep = 0; sweep < max_sweeps; ++sweep) {
@@ -488,12 +673,6 @@ __global__ void __launch_bounds__(LA_THREADS) k_jacobi_svd(const SvdDesc *__rest
                     ma[i] = cs * x - sn * y;
                     mb[i] = sn * x + cs * y;
                 }
-                double *va = V + (long long)a * ld, *vb = V + (long long)b * ld;
-                for (int i = lane; i < r; i += 32) {
-                    const double x = va[i], y = vb[i];
-                    va[i] = cs * x - sn * y;
-                    vb[i] = sn * x + cs * y;
-                }
                 if (lane == 0) rotated = 1;
             }
             __syncthreads();
@@ -510,128 +689,175 @@ __global__ void __launch_bounds__(LA_THREADS) k_jacobi_svd(const SvdDesc *__rest
     }
 }
 
-// ---- the same one-sided Jacobi SVD on a cluster of JC CTAs ------------------
-// One FP64 SM needs ~13 ms per sweep at r = 232, so the SVD of a tile is
-// spread over a thread-block cluster: CTA c holds rows [c rs, (c+1) rs) of M
-// and V in shared memory.  Each round (r/2 disjoint pairs, the same circle
-// order), two threads per pair form partial (alpha, beta, gamma) over the
-// CTA's rows, the partials are exchanged through distributed shared memory
-// (one cluster barrier, double-buffered), every CTA sums them in rank order
-// (so every CTA takes the same rotation decisions, bit for bit) and rotates
-// its own rows.  Column norms are reduced the same way at the end.  r <= 256.
-constexpr int JC = 8, JT = 256, JR_MAX = 256, JLD = JR_MAX / JC + 1;
+// ---- the same on a cluster of JC CTAs, by blocks of columns ------------------
+// The columns form 2 JC blocks of at most 16; a CTA holds two, all rows of them
+// in shared memory.  A sweep is 2 JC - 1 rounds of the circle method over the
+// blocks: in a round a CTA meets every column of its one block with every
+// column of the other (b steps of b disjoint pairs; the pairs within the two
+// blocks come first in a sweep), then the blocks move on to the neighbours'
+// other buffer through distributed shared memory: one cluster barrier a round,
+// where rows dealt out to the CTAs need one per step.  Sixteen threads take a
+// pair, its columns in registers between the dot product and the rotation; the
+// squared norms are carried along (and taken afresh every round and when one
+// shrinks much).  A warp-wide FP64 operation holds its scheduler for 64
+// clocks, so what counts is their number: five per entry of a pair, and some
+// twenty for the angle, from the hardware's approximations refined.
+// r = 216: 1.1 ms a sweep where every pair rotates (3.6).  r <= 256.
+constexpr int JC = 8, JT = 256, JR_MAX = 256, JBM = JR_MAX / (2 * JC);
 
-size_t jacobi_cl_smem(int r) {
-    return sizeof(double) * (2 * (size_t)r * JLD + 2 * 3 * (JR_MAX / 2) + JR_MAX);
-}
+size_t jacobi_cl_smem(int b, int rows) { return sizeof(double) * (2 * 2 * (size_t)b * rows + 2 * 2 * JBM); }
 
-__global__ void __launch_bounds__(JT, 1) k_jacobi_svd_cl(const SvdDesc *__restrict__ d, int count, int max_sweeps) {
+template <int NR>   // rows / 16
+__global__ void __launch_bounds__(JT, 1) k_jacobi_svd_cl(const SvdDesc *__restrict__ d, int count, int max_sweeps, int bmax) {
     cg::cluster_group cluster = cg::this_cluster();
     const int tile = blockIdx.x / JC;
     if (tile >= count) return;   // uniform over the cluster
     const int rank = (int)cluster.block_rank();
+    constexpr int ROWS = 16 * NR;
     extern __shared__ double sm[];
     const SvdDesc s = d[tile];
-    const int r = s.r;
+    const int r = s.r, b = (r + 2 * JC - 1) / (2 * JC);
     const long long ld = s.ld;
-    const int rs = (r + JC - 1) / JC;
-    const int row0 = rank * rs, nrow = max(0, min(rs, r - row0));
-    double *Ms = sm;                          // [r][JLD], rows of this CTA
-    double *Vs = Ms + (size_t)r * JLD;
-    double *P = Vs + (size_t)r * JLD;         // [2][3][JR_MAX / 2]
-    double *nrm = P + 2 * 3 * (JR_MAX / 2);   // [JR_MAX]
-    for (int e = threadIdx.x; e < r * rs; e += JT) {
-        const int c = e / rs, i = e % rs;
-        Ms[c * JLD + i] = (i < nrow) ? s.M[(long long)c * ld + row0 + i] : 0.0;
-        Vs[c * JLD + i] = (i < nrow && row0 + i == c) ? 1.0 : 0.0;
-    }
-    __syncthreads();
-    const int rr = r + (r & 1), npairs = rr / 2;
-    const int p = threadIdx.x >> 1, half = threadIdx.x & 1;
+    const size_t blk = (size_t)bmax * ROWS;           // doubles of one block buffer
+    double *norms = sm + 4 * blk;                     // [2 buffers][2 blocks][JBM]
+    __shared__ int flags[2][JC], mine;
+    auto col = [&](int buf, int w, int c) { return sm + (buf * 2 + w) * blk + (size_t)c * ROWS; };
+    auto nrm = [&](int buf, int w) { return norms + (buf * 2 + w) * JBM; };
+    const int g = threadIdx.x / 16, l = threadIdx.x % 16;   // pair slot, lane within it
     const double skip2 = s.skip * s.skip;
-    int buf = 0;
-    for (int sweep = 0; sweep < max_sweeps; ++sweep) {
-        int rotated = 0;
-        for (int round = 0; round < rr - 1; ++round) {
-            int a = -1, b = -1;
-            double al = 0.0, be = 0.0, ga = 0.0;
-            if (p < npairs) {
-                a = (p == 0) ? 0 : 1 + (p - 1 + round) % (rr - 1);
-                b = 1 + (rr - 2 - p + round) % (rr - 1);
-                if (a >= r || b >= r || a == b) {
-                    a = -1;
-                } else if (a > b) {
-                    const int t = a;
-                    a = b;
-                    b = t;
-                }
-                if (a >= 0)
-                    for (int i = half; i < nrow; i += 2) {
-                        const double x = Ms[a * JLD + i], y = Ms[b * JLD + i];
-                        al = fma(x, x, al);
-                        be = fma(y, y, be);
-                        ga = fma(x, y, ga);
-                    }
+    // blocks rank (w = 0) and JC + rank (w = 1)
+    for (int w = 0; w < 2; ++w)
+        for (int c = g; c < b; c += JT / 16) {
+            const int j = (w * JC + rank) * b + c;
+            for (int i = l; i < ROWS; i += 16) col(0, w, c)[i] = (j < r && i < r) ? s.M[(long long)j * ld + i] : 0.0;
+        }
+    cluster.sync();   // every CTA runs: its shared memory may be written
+    int buf = 0, sweep = 0, rotated = 0;
+    auto sum16 = [](double v) {
+        for (int o = 8; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+        return v;
+    };
+    // one pair per slot: columns xa (squared norm *na) and xb (*nb); act = the slot has a pair.  Every lane of the
+    // warp takes part in the shuffles.
+    auto pair = [&](double *xa, double *xb, double *na, double *nb, bool act) {
+        double al = 0.0, be = 0.0;
+        if (act) al = *na, be = *nb;
+        act = act && !(al < skip2 && be < skip2);
+        if (!__any_sync(0xffffffffu, act)) return;
+        double x[NR], y[NR], ga = 0.0;
+#pragma unroll
+        for (int i = 0; i < NR; ++i) {
+            x[i] = act ? xa[16 * i + l] : 0.0;
+            y[i] = act ? xb[16 * i + l] : 0.0;
+            ga = fma(x[i], y[i], ga);
+        }
+        ga = sum16(ga);
+        const bool rot = act && ga * ga > 1e-26 * (al * be);
+        if (!__any_sync(0xffffffffu, rot)) return;
+        // t = tan of the angle: the smaller root of t^2 + 2 zeta t - 1, zeta = (be - al) / (2 ga)
+        double cs = 1.0, sn = 0.0, t = 0.0;
+        if (rot) {
+            const double dd = be - al, h = fma(dd, dd, 4.0 * (ga * ga));
+            t = 2.0 * ga * fast_rcp(fabs(dd) + h * fast_rsqrt(h));
+            if (dd < 0.0) t = -t;
+            cs = fast_rsqrt(fma(t, t, 1.0));
+            sn = cs * t;
+        }
+#pragma unroll
+        for (int i = 0; i < NR; ++i) {
+            const double xn = fma(cs, x[i], -(sn * y[i]));
+            y[i] = fma(sn, x[i], cs * y[i]);
+            x[i] = xn;
+            if (rot) {
+                xa[16 * i + l] = x[i];
+                xb[16 * i + l] = y[i];
             }
-            al += __shfl_xor_sync(0xffffffffu, al, 1);
-            be += __shfl_xor_sync(0xffffffffu, be, 1);
-            ga += __shfl_xor_sync(0xffffffffu, ga, 1);
-            double *Pb = P + buf * 3 * (JR_MAX / 2);
-            if (half == 0 && p < npairs) {
-                Pb[p] = al;
-                Pb[JR_MAX / 2 + p] = be;
-                Pb[JR_MAX + p] = ga;
+        }
+        double an = fma(-t, ga, al), bn = fma(t, ga, be);
+        // a norm that lost most of itself is summed afresh
+        const bool fresh = rot && (an < 0.1 * al || bn < 0.1 * be);
+        if (__any_sync(0xffffffffu, fresh)) {
+            double u = 0.0, v = 0.0;
+#pragma unroll
+            for (int i = 0; i < NR; ++i) u = fma(x[i], x[i], u), v = fma(y[i], y[i], v);
+            u = sum16(u);
+            v = sum16(v);
+            if (fresh) an = u, bn = v;
+        }
+        if (rot) {
+            rotated = 1;
+            if (l == 0) *na = an, *nb = bn;
+        }
+    };
+    __syncthreads();
+    for (; sweep < max_sweeps; ++sweep) {
+        rotated = 0;
+        for (int round = 0; round < 2 * JC - 1; ++round) {
+            for (int c = g; c < 2 * JBM; c += JT / 16) {   // norms of the blocks as they are now (32 of 16 slots: two each)
+                const int w = c / JBM, cc = c % JBM;
+                double u = 0.0;
+                if (cc < b)
+                    for (int i = 0; i < NR; ++i) u = fma(col(buf, w, cc)[16 * i + l], col(buf, w, cc)[16 * i + l], u);
+                u = sum16(u);
+                if (cc < b && l == 0) nrm(buf, w)[cc] = u;
+            }
+            __syncthreads();
+            if (round == 0) {
+                // pairs within the blocks: slots 0-7 the first block, 8-15 the second
+                const int bb = b + (b & 1), w = g / 8, p = g % 8;
+                for (int st = 0; st < bb - 1; ++st) {
+                    int a = (p == 0) ? 0 : 1 + (p - 1 + st) % (bb - 1);
+                    int c = 1 + (bb - 2 - p + st) % (bb - 1);
+                    const bool act = p < bb / 2 && a < b && c < b && a != c;
+                    if (!act) a = c = 0;
+                    pair(col(buf, w, min(a, c)), col(buf, w, max(a, c)), nrm(buf, w) + min(a, c), nrm(buf, w) + max(a, c), act);
+                    __syncthreads();
+                }
+            }
+            for (int st = 0; st < b; ++st) {
+                const bool act = g < b;
+                const int a = act ? g : 0, c = act ? (g + st) % b : 0;
+                pair(col(buf, 0, a), col(buf, 1, c), nrm(buf, 0) + a, nrm(buf, 1) + c, act);
+                __syncthreads();
+            }
+            // the circle method's move: first block 0 stays, the first blocks move up, the second ones down
+            const int t0 = rank == 0 ? 0 : min(rank + 1, JC - 1), w0 = rank == JC - 1 ? 1 : 0;
+            const int t1 = rank == 0 ? 1 : rank - 1, w1 = rank == 0 ? 0 : 1;
+            double *to0 = cluster.map_shared_rank(col(buf ^ 1, w0, 0), t0), *to1 = cluster.map_shared_rank(col(buf ^ 1, w1, 0), t1);
+            for (int e = threadIdx.x; e < b * ROWS; e += JT) {
+                to0[e] = col(buf, 0, 0)[e];
+                to1[e] = col(buf, 1, 0)[e];
+            }
+            if (round == 2 * JC - 2) {   // the sweep's end: did anything rotate anywhere?
+                if (threadIdx.x == 0) mine = 0;
+                __syncthreads();
+                if (rotated) mine = 1;
+                __syncthreads();
+                if (threadIdx.x < JC) cluster.map_shared_rank(&flags[sweep & 1][0], threadIdx.x)[rank] = mine;
             }
             cluster.sync();
-            if (a >= 0) {
-                double A = 0.0, B = 0.0, G = 0.0;
-                for (int c = 0; c < JC; ++c) {
-                    const double *rp = cluster.map_shared_rank(Pb, c);
-                    A += rp[p];
-                    B += rp[JR_MAX / 2 + p];
-                    G += rp[JR_MAX + p];
+            buf ^= 1;
+        }
+        int any = 0;
+        for (int k = 0; k < JC; ++k) any |= flags[sweep & 1][k];
+        if (!any) break;   // the same decision in every CTA
+    }
+    // after whole sweeps the blocks are where they began
+    for (int w = 0; w < 2; ++w)
+        for (int c = g; c < JBM; c += JT / 16) {
+            const int j = (w * JC + rank) * b + c;
+            const bool in = c < b && j < r;
+            double u = 0.0;
+            if (in)
+                for (int i = l; i < ROWS; i += 16) {
+                    const double x = col(buf, w, c)[i];
+                    u = fma(x, x, u);
+                    if (i < r) s.M[(long long)j * ld + i] = x;
                 }
-                if (!(A < skip2 && B < skip2) && !(fabs(G) <= 1e-13 * sqrt(A * B) || G == 0.0)) {
-                    const double zeta = (B - A) / (2.0 * G);
-                    const double t = copysign(1.0, zeta) / (fabs(zeta) + sqrt(1.0 + zeta * zeta));
-                    const double cs = 1.0 / sqrt(1.0 + t * t), sn = cs * t;
-                    for (int i = half; i < nrow; i += 2) {
-                        const double x = Ms[a * JLD + i], y = Ms[b * JLD + i];
-                        Ms[a * JLD + i] = cs * x - sn * y;
-                        Ms[b * JLD + i] = sn * x + cs * y;
-                        const double u = Vs[a * JLD + i], v = Vs[b * JLD + i];
-                        Vs[a * JLD + i] = cs * u - sn * v;
-                        Vs[b * JLD + i] = sn * u + cs * v;
-                    }
-                    rotated = 1;
-                }
-            }
-            __syncthreads();   // rotated columns before the next round's partials
-            buf ^= 1;          // the other partial buffer: free since this round's barrier
+            u = sum16(u);
+            if (in && l == 0) s.sigma[j] = sqrt(u);
         }
-        if (!__syncthreads_or(rotated)) break;   // the same decision in every CTA
-    }
-    // singular values = column norms
-    for (int c = threadIdx.x; c < r; c += JT) {
-        double t = 0.0;
-        for (int i = 0; i < nrow; ++i) t = fma(Ms[c * JLD + i], Ms[c * JLD + i], t);
-        nrm[c] = t;
-    }
-    cluster.sync();
-    if (rank == 0)
-        for (int c = threadIdx.x; c < r; c += JT) {
-            double t = 0.0;
-            for (int q = 0; q < JC; ++q) t += cluster.map_shared_rank(nrm, q)[c];
-            s.sigma[c] = sqrt(t);
-        }
-    for (int e = threadIdx.x; e < r * rs; e += JT) {
-        const int c = e / rs, i = e % rs;
-        if (i < nrow) {
-            s.M[(long long)c * ld + row0 + i] = Ms[c * JLD + i];
-            s.V[(long long)c * ld + row0 + i] = Vs[c * JLD + i];
-        }
-    }
-    cluster.sync();   // no CTA leaves while another still reads its shared memory
+    cluster.sync();   // no CTA leaves while another still writes its shared memory
 }
 
 // ---- Gaussian test matrices: counter-based SplitMix64 -> Box-Muller ---------
@@ -710,29 +936,38 @@ cudaError_t launch_bgemm(const GemmDesc *d_desc, int count, int max_tiles, cudaS
     return cudaGetLastError();
 }
 
-cudaError_t launch_house_qr(const QrDesc *d_desc, int count, int mmax, int rmax, cudaStream_t s, double flops) {
-    if (count <= 0) return cudaSuccess;
-    KScope ks(GEO_K_TLR, s, flops, 0.0);
-    if (rmax > QR_MAX) {
-        k_house_qr<<<count, LA_THREADS, 0, s>>>(d_desc, count);
-        return cudaGetLastError();
-    }
-    const size_t smem = house_qr_cl_smem(mmax);
-    cudaError_t e = cudaFuncSetAttribute(k_house_qr_cl, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+template <typename K, typename... A>
+static cudaError_t launch_clusters(K kernel, int count, int ctas, int threads, size_t smem, cudaStream_t s, A... args) {
+    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)count * QC);
-    cfg.blockDim = dim3(QT);
+    cfg.gridDim = dim3((unsigned)count * ctas);
+    cfg.blockDim = dim3(threads);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = s;
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = QC;
+    at[0].val.clusterDim.x = ctas;
     at[0].val.clusterDim.y = 1;
     at[0].val.clusterDim.z = 1;
     cfg.attrs = at;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, k_house_qr_cl, d_desc, count);
+    return cudaLaunchKernelEx(&cfg, kernel, args...);
+}
+
+bool house_qr_in_smem(int mmax, int rmax) { return rmax <= QR_MAX && house_qr_col_smem(mmax, rmax) <= 226 * 1024; }
+
+cudaError_t launch_house_qr(const QrDesc *d_desc, int count, int mmax, int rmax, cudaStream_t s, double flops) {
+    if (count <= 0) return cudaSuccess;
+    KScope ks(GEO_K_TLR, s, flops, 0.0);
+    // the block in a cluster's shared memory where it fits (m = 900: r = 240); else its rows over a cluster
+    if (house_qr_in_smem(mmax, rmax))
+        return launch_clusters(k_house_qr_col, count, QC, QCT, house_qr_col_smem(mmax, rmax), s, d_desc, count);
+    if (rmax > QR_MAX) {
+        k_house_qr<<<count, LA_THREADS, 0, s>>>(d_desc, count);
+        return cudaGetLastError();
+    }
+    return launch_clusters(k_house_qr_cl, count, QC, QT, house_qr_cl_smem(mmax), s, d_desc, count);
 }
 
 cudaError_t launch_jacobi_svd(const SvdDesc *d_desc, int count, int max_sweeps, int rmax, cudaStream_t s,
@@ -743,22 +978,16 @@ cudaError_t launch_jacobi_svd(const SvdDesc *d_desc, int count, int max_sweeps, 
         k_jacobi_svd<<<count, LA_THREADS, 0, s>>>(d_desc, count, max_sweeps);
         return cudaGetLastError();
     }
-    const size_t smem = jacobi_cl_smem(rmax);
-    cudaError_t e = cudaFuncSetAttribute(k_jacobi_svd_cl, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)count * JC);
-    cfg.blockDim = dim3(JT);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = s;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = JC;
-    at[0].val.clusterDim.y = 1;
-    at[0].val.clusterDim.z = 1;
-    cfg.attrs = at;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, k_jacobi_svd_cl, d_desc, count, max_sweeps);
+    const int b = (rmax + 2 * JC - 1) / (2 * JC), nr = (rmax + 15) / 16;
+    auto go = [&](auto NR) {
+        return launch_clusters(k_jacobi_svd_cl<NR.value>, count, JC, JT, jacobi_cl_smem(b, 16 * NR.value), s, d_desc, count,
+                               max_sweeps, b);
+    };
+    if (nr <= 4) return go(std::integral_constant<int, 4>());
+    if (nr <= 8) return go(std::integral_constant<int, 8>());
+    if (nr <= 12) return go(std::integral_constant<int, 12>());
+    if (nr <= 14) return go(std::integral_constant<int, 14>());
+    return go(std::integral_constant<int, 16>());
 }
 
 cudaError_t launch_gaussian(double *O, long long n, unsigned long long seed, cudaStream_t s) {

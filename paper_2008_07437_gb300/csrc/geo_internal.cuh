@@ -260,17 +260,19 @@ struct GemmDesc {           // C = alpha op(A) op(B) + beta C, column-major
     long long ldc;
     double alpha, beta;
 };
-struct QrDesc {             // in-place Householder QR of Y (m x r), thin Q out
+struct QrDesc {             // Householder QR of Y (m x r), in place, thin Q out (Q == NULL: R only)
     int m, r;
     double *Y;
     long long ldy;
     double *Q;
     long long ldq;
     double *tau, *v0;       // r entries each
+    double *Rt;             // with house_qr_in_smem and not NULL: R' (r x r lower, ldr); with Q == NULL Y is then left as it is
+    long long ldr;
 };
-struct SvdDesc {            // one-sided Jacobi SVD of M (r x r): M <- M V, V, sigma
+struct SvdDesc {            // one-sided Jacobi SVD of M (r x r): M <- M V, sigma = its column norms
     int r;
-    double *M, *V;
+    double *M;
     long long ld;
     double *sigma;
     double skip;            // pairs of columns both below this norm are left alone (0 = none)
@@ -282,6 +284,7 @@ cudaError_t launch_bgemm(const GemmDesc *d_desc, int count, int max_tiles, cudaS
 void bgemm_splitk_scratch(double *ws, size_t bytes);
 constexpr size_t TLR_SPLITK_BYTES = 8u << 20;
 // mmax, rmax: the largest m and r of the batch (the cluster kernel serves r <= 256).
+bool house_qr_in_smem(int mmax, int rmax);   // whether the launch keeps the blocks in shared memory
 cudaError_t launch_house_qr(const QrDesc *d_desc, int count, int mmax, int rmax, cudaStream_t s, double flops);
 // rmax: the largest r of the batch (the cluster kernel serves r <= 256).
 cudaError_t launch_jacobi_svd(const SvdDesc *d_desc, int count, int max_sweeps, int rmax, cudaStream_t s,
@@ -326,12 +329,13 @@ struct TlrR2Desc {
     double *M;
     long long ldm;
 };
-struct TlrSelDesc {
+struct TlrSelDesc {         // X = the selected columns of M over their norms
     int r, k;
-    const double *M, *Vj;
-    double *Msel, *Vsel;
+    const double *M;
+    double *X;
     long long ld;
     const int *sel;
+    const double *sigma;
 };
 struct TlrTrsmDesc {
     const double *L;

@@ -11,8 +11,9 @@
 //      W_i -= P_i [U_jk]' per tile, in chunks of the stacked rank);
 //   3. factor the diagonal tile in FP64 (the dense POTRF of the tile algorithm);
 //   4. compress each W_ij, i > j, by a randomized SVD: Y = W Omega (Gaussian
-//      sketch), Q = qr(Y), B' = W' Q, Q2 R2 = qr(B'), R2' = X S Yj' (one-sided
-//      Jacobi), keep the singular values above tol: U = Q X S, V = Q2 Yj; a tile
+//      sketch), Q = qr(Y), B' = W' Q, R2 of qr(B'), R2' = X S Yj' (one-sided
+//      Jacobi, X S alone), keep the singular values above tol: U = Q X, V = B' X
+//      (= Q2 Yj S: neither Q2 nor Yj is formed); a tile
 //      whose sketch is too narrow is redone with the widest sketch;
 //   5. V_ij <- L_jj^-1 V_ij (the TRSM of the tile algorithm on the V factor only).
 // The paper's own TLR kernels (HiCMA) update in low-rank form and recompress
@@ -56,7 +57,7 @@ __global__ void k_copy_r2t(const TlrR2Desc *__restrict__ d, int count) {
     q.M[(long long)c * q.ldm + rr] = (c <= rr) ? q.B[(long long)rr * q.ldb + c] : 0.0;
 }
 
-// Gather the selected columns: Msel[:, c] = M[:, sel[c]], Vsel[:, c] = Vj[:, sel[c]].
+// The selected left singular vectors: X[:, c] = M[:, sel[c]] / sigma[sel[c]].
 __global__ void k_gather_sel(const TlrSelDesc *__restrict__ d, int count) {
     if ((int)blockIdx.y >= count) return;
     const TlrSelDesc q = d[blockIdx.y];
@@ -64,8 +65,7 @@ __global__ void k_gather_sel(const TlrSelDesc *__restrict__ d, int count) {
     if (t >= q.r * q.k) return;
     const int c = t / q.r, rr = t % q.r;
     const int src = q.sel[c];
-    q.Msel[(long long)c * q.ld + rr] = q.M[(long long)src * q.ld + rr];
-    q.Vsel[(long long)c * q.ld + rr] = q.Vj[(long long)src * q.ld + rr];
+    q.X[(long long)c * q.ld + rr] = q.M[(long long)src * q.ld + rr] / q.sigma[src];
 }
 
 // Left lower triangular solve on a 64-row block: X = L[c0:c0+cb, c0:c0+cb]^-1 X, for
@@ -203,7 +203,7 @@ size_t tlr_factor_bytes(int N, int nb, int kmax) {
 size_t tlr_workspace_bytes(int N, int nb, int kmax) {
     const size_t T = ((size_t)N + nb - 1) / nb;
     const size_t rmax = std::min((size_t)kmax + 16, (size_t)nb);
-    const size_t per_tile = (5 * (size_t)nb * rmax + 4 * rmax * rmax + 4 * rmax) * sizeof(double);
+    const size_t per_tile = (5 * (size_t)nb * rmax + 2 * rmax * rmax + 4 * rmax) * sizeof(double);
     return sizeof(double) * ((size_t)N * nb                   // column panel W
                              + (size_t)nb * rmax                // Omega
                              + (size_t)nb * TLR_KCHUNK          // stacked U_jk chunk
@@ -245,8 +245,8 @@ cudaError_t tlr_factor(TlrFactor &F, const CovParams &cp, const double *lx, cons
     double *Mb = (double *)take(sizeof(double) * (size_t)T * TLR_MAXK_PER_CHUNK * kmax * kmax);
     double *Zb = (double *)take(sizeof(double) * (size_t)TLR_KCHUNK * rmax);
     double *Tb = (double *)take(sizeof(double) * (size_t)T * TLR_KCHUNK * rmax);
-    // per tile: Y, Q, B', Q2 (nb x rmax), M, Vj, Ms, Vs (rmax^2), sigma, tau, v0, spare (rmax), saved Y (nb x rmax)
-    const size_t per_tile = 5 * (size_t)nb * rmax + 4 * (size_t)rmax * rmax + 4 * (size_t)rmax;
+    // per tile: Y, Q, B', a copy of B' (nb x rmax), M, X (rmax^2), sigma, tau, v0, spare (rmax), saved Y (nb x rmax)
+    const size_t per_tile = 5 * (size_t)nb * rmax + 2 * (size_t)rmax * rmax + 4 * (size_t)rmax;
     double *TW = (double *)take(sizeof(double) * (size_t)T * per_tile);
     SplitKScope splitk(take(TLR_SPLITK_BYTES), TLR_SPLITK_BYTES);
     Arena arena;
@@ -303,7 +303,7 @@ cudaError_t tlr_factor(TlrFactor &F, const CovParams &cp, const double *lx, cons
             // on itself and spread the dense band).
             rwant[q] = std::min(rmax, std::max(32, (hint + 16 + 31) / 32 * 32));
         }
-        auto Ysave = [&](int q) { return tb(q) + 4 * (size_t)nb * rmax + 4 * (size_t)rmax * rmax + 4 * (size_t)rmax; };
+        auto Ysave = [&](int q) { return tb(q) + 4 * (size_t)nb * rmax + 2 * (size_t)rmax * rmax + 4 * (size_t)rmax; };
         // for each chunk of row j's finished columns: Qc, and P_i for the tiles i in `rows`
         // (i - j in 0 .. nt), then apply(Kc, has) with has[i - j] = some rank of the chunk in row i
         auto chunk_loop = [&](const std::vector<int> &rows, auto &&apply) -> cudaError_t {
@@ -464,23 +464,24 @@ cudaError_t tlr_factor(TlrFactor &F, const CovParams &cp, const double *lx, cons
             std::vector<int> rows_b;
             int r = 0;
             for (int q : todo) r = std::max(r, std::min(std::min(pass == 0 ? rwant[q] : rmax, mj), mt(j + 1 + q)));
+            const bool r_direct = house_qr_in_smem(nb, r);
             for (int q : todo) {
                 const int i = j + 1 + q;
                 const int mi = mt(i);
                 const int rr = std::min(std::min(pass == 0 ? rwant[q] : rmax, mj), mi);
                 double *b = tb(q);
-                double *Y = b, *Q = b + (size_t)nb * rmax, *Bt = Q + (size_t)nb * rmax, *Q2 = Bt + (size_t)nb * rmax;
-                double *M = Q2 + (size_t)nb * rmax, *Vj = M + (size_t)rmax * rmax, *Ms = Vj + (size_t)rmax * rmax;
-                double *Vs = Ms + (size_t)rmax * rmax, *sig = Vs + (size_t)rmax * rmax, *tau = sig + rmax;
+                double *Y = b, *Q = b + (size_t)nb * rmax, *Bt = Q + (size_t)nb * rmax, *B2 = Bt + (size_t)nb * rmax;
+                double *M = B2 + (size_t)nb * rmax, *sig = M + 2 * (size_t)rmax * rmax, *tau = sig + rmax;
                 double *v0 = tau + rmax;
                 double *Wi = W + (size_t)(i - j) * nb;
                 // the first rr columns of the saved sketch (the QR works in place)
                 TCK(cudaMemcpyAsync(Y, Ysave(q), sizeof(double) * (size_t)nb * rr, cudaMemcpyDeviceToDevice, s));
-                dq1.push_back({mi, rr, Y, nb, Q, nb, tau, v0});
+                dq1.push_back({mi, rr, Y, nb, Q, nb, tau, v0, nullptr, 0});
                 db.push_back({mj, rr, mi, 1, 0, Wi, ldw, Q, nb, Bt, nb, 1.0, 0.0});
-                dq2.push_back({mj, rr, Bt, nb, Q2, nb, tau, v0});
-                dr.push_back({rr, Bt, nb, M, rmax});
-                dsv.push_back({rr, M, Vj, rmax, sig, F.tol / 16.0});
+                // R2' straight into M, or from a factored copy of B'
+                dq2.push_back({mj, rr, r_direct ? Bt : B2, nb, nullptr, 0, tau, v0, r_direct ? M : nullptr, rmax});
+                dr.push_back({rr, B2, nb, M, rmax});
+                dsv.push_back({rr, M, rmax, sig, F.tol / 16.0});
                 rused[q] = rr;
                 rows_b.push_back(i);
             }
@@ -510,23 +511,27 @@ cudaError_t tlr_factor(TlrFactor &F, const CovParams &cp, const double *lx, cons
                 if (ce) return ce;
                 return launch_bgemm(h2, (int)dt2.size(), gemm_tiles(dt2), s, gemm_flops(dt2), gemm_kmax(dt2));
             }));
+            if (!r_direct)
+                for (const QrDesc &q : dq2)
+                    TCK(cudaMemcpyAsync(q.Y, q.Y - (size_t)nb * rmax, sizeof(double) * (size_t)nb * q.r,
+                                        cudaMemcpyDeviceToDevice, s));
             QrDesc *q2 = push(arena, dq2, s, &e);
             TCK(e);
-            TCK(launch_house_qr(q2, (int)dq2.size(), nb, r, s, 4.0 * (double)dq2.size() * nb * r * r));
-            TlrR2Desc *r2 = push(arena, dr, s, &e);
-            TCK(e);
-            {
+            TCK(launch_house_qr(q2, (int)dq2.size(), nb, r, s, 2.0 * (double)dq2.size() * nb * r * r));
+            if (!r_direct) {
+                TlrR2Desc *r2 = push(arena, dr, s, &e);
+                TCK(e);
                 KScope kk(GEO_K_AUX, s);
                 k_copy_r2t<<<dim3((r * r + 255) / 256, (unsigned)dr.size()), 256, 0, s>>>(r2, (int)dr.size());
                 TCK(cudaGetLastError());
             }
             SvdDesc *sv = push(arena, dsv, s, &e);
             TCK(e);
-            TCK(launch_jacobi_svd(sv, (int)dsv.size(), 30, r, s, 3.0 * 12.0 * (double)dsv.size() * r * r * r));
+            TCK(launch_jacobi_svd(sv, (int)dsv.size(), 30, r, s, 12.0 * 5.0 * (double)dsv.size() * r * r * r));
             // singular values to the host
             for (size_t t = 0; t < todo.size(); ++t) {
                 const int q = todo[t];
-                double *sig = tb(q) + 4 * (size_t)nb * rmax + 4 * (size_t)rmax * rmax;
+                double *sig = tb(q) + 4 * (size_t)nb * rmax + 2 * (size_t)rmax * rmax;
                 TCK(cudaMemcpyAsync(h_sigma + (size_t)t * rmax, sig, sizeof(double) * rused[q], cudaMemcpyDeviceToHost,
                                     s));
             }
@@ -572,7 +577,7 @@ cudaError_t tlr_factor(TlrFactor &F, const CovParams &cp, const double *lx, cons
                     return dense_update(late, Kc, has);
                 }));
         }
-        // U = Q (M Vj)[:, sel], V = Q2 Vj[:, sel]
+        // U = Q X, V = B' X
         {
             std::vector<int> hsel;
             std::vector<size_t> selpos(nt);
@@ -617,12 +622,11 @@ cudaError_t tlr_factor(TlrFactor &F, const CovParams &cp, const double *lx, cons
                 const int i = j + 1 + q, k = rk[q];
                 if (k == 0 || F.dense[slot(i, j)]) continue;
                 double *b = tb(q);
-                double *Q = b + (size_t)nb * rmax, *Q2 = Q + 2 * (size_t)nb * rmax;
-                double *M = Q2 + (size_t)nb * rmax, *Vj = M + (size_t)rmax * rmax, *Ms = Vj + (size_t)rmax * rmax;
-                double *Vs = Ms + (size_t)rmax * rmax;
-                dg.push_back({rused[q], k, M, Vj, Ms, Vs, rmax, dsel + selpos[q]});
-                du.push_back({mt(i), k, rused[q], 0, 0, Q, nb, Ms, rmax, Uof(i, j), nb, 1.0, 0.0});
-                dv.push_back({mj, k, rused[q], 0, 0, Q2, nb, Vs, rmax, Vof(i, j), nb, 1.0, 0.0});
+                double *Q = b + (size_t)nb * rmax, *Bt = Q + (size_t)nb * rmax;
+                double *M = Bt + 2 * (size_t)nb * rmax, *X = M + (size_t)rmax * rmax, *sig = X + (size_t)rmax * rmax;
+                dg.push_back({rused[q], k, M, X, rmax, dsel + selpos[q], sig});
+                du.push_back({mt(i), k, rused[q], 0, 0, Q, nb, X, rmax, Uof(i, j), nb, 1.0, 0.0});
+                dv.push_back({mj, k, rused[q], 0, 0, Bt, nb, X, rmax, Vof(i, j), nb, 1.0, 0.0});
             }
             if (!dg.empty()) {
                 TlrSelDesc *g = push(arena, dg, s, &e);
