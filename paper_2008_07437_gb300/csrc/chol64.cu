@@ -359,36 +359,38 @@ __global__ void __launch_bounds__(DF_THREADS, 1) k_chol_df(const DfArgs a) {
     }
 }
 
-// C[r, c] -= sum_k A[r, k] B[c, k] for a few rows r (right-hand sides): a thread per column reads its
-// operand row along k (coalesced over columns), bound by that one pass over B (HBM).
-constexpr int RROWS = 4;
-
-__global__ void __launch_bounds__(128) k_rhs_update(double *A, long long ld, int rC, int cC, int m, int n, int kA, int k,
-                                                   const DevStatus *st) {
+// C[r, c] -= sum_k A[r, k] B[c, k] for RR rows r (right-hand sides): a thread per column reads its operand row
+// along k, coalesced over columns, sixteen loads in flight.  Bound by the loads' latency and the FP64 FMAs of
+// one warp, k of 64 clocks each per row; so the usual single row has its own form (k = 256 on average 31 us a
+// launch, 105 with the FMAs of four rows), whose sums are the same.
+template <int RR>
+__global__ void __launch_bounds__(64) k_rhs_update(double *A, long long ld, int rC, int cC, int m, int n, int kA, int k,
+                                                  const DevStatus *st) {
     if (st->info) return;
-    const int r0 = blockIdx.y * RROWS;
-    __shared__ double a[RROWS][128];
-    const int c = blockIdx.x * 128 + threadIdx.x;
-    double acc[RROWS] = {};
-    for (int k0 = 0; k0 < k; k0 += 128) {
-        const int kc = min(128, k - k0);
+    const int r0 = blockIdx.y * RR;
+    __shared__ double a[RR][256];
+    const int c = blockIdx.x * 64 + threadIdx.x;
+    double acc[RR] = {};
+    for (int k0 = 0; k0 < k; k0 += 256) {
+        const int kc = min(256, k - k0);
         __syncthreads();
-        for (int i = 0; i < RROWS; ++i)
-            a[i][threadIdx.x] = (threadIdx.x < kc && r0 + i < m)
-                                    ? A[(long long)(kA + k0 + threadIdx.x) * ld + rC + r0 + i] : 0.0;
+        for (int t = threadIdx.x; t < RR * kc; t += 64)
+            a[t % RR][t / RR] = (r0 + t % RR < m) ? A[(long long)(kA + k0 + t / RR) * ld + rC + r0 + t % RR] : 0.0;
         __syncthreads();
         if (c < n) {
             const double *b = A + (long long)(kA + k0) * ld + cC + c;
-#pragma unroll 8
+#pragma unroll 16
             for (int kk = 0; kk < kc; ++kk) {
                 const double bv = b[(long long)kk * ld];
 #pragma unroll
-                for (int i = 0; i < RROWS; ++i) acc[i] = fma(a[i][kk], bv, acc[i]);
+                for (int i = 0; i < RR; ++i) acc[i] = fma(a[i][kk], bv, acc[i]);
             }
         }
     }
     if (c < n)
-        for (int i = 0; i < RROWS && r0 + i < m; ++i) A[(long long)(cC + c) * ld + rC + r0 + i] -= acc[i];
+#pragma unroll
+        for (int i = 0; i < RR; ++i)
+            if (r0 + i < m) A[(long long)(cC + c) * ld + rC + r0 + i] -= acc[i];
 }
 
 cudaError_t launch_df(const DfArgs &a0, int sms, int cls, double flops, cudaStream_t s) {
@@ -448,7 +450,10 @@ cudaError_t chol64_rhs_update(double *A, long long ld, int rC, int cC, int m, in
                               cudaStream_t s) {
     if (m <= 0 || n <= 0 || k <= 0) return cudaSuccess;
     KScope ks(GEO_K_GEMM, s, 2.0 * k * (double)m * n, 8.0 * ((double)n * k + 2.0 * m * n));
-    k_rhs_update<<<dim3((n + 127) / 128, (m + RROWS - 1) / RROWS), 128, 0, s>>>(A, ld, rC, cC, m, n, kA, k, st);
+    if (m == 1)
+        k_rhs_update<1><<<(n + 63) / 64, 64, 0, s>>>(A, ld, rC, cC, m, n, kA, k, st);
+    else
+        k_rhs_update<4><<<dim3((n + 63) / 64, (m + 3) / 4), 64, 0, s>>>(A, ld, rC, cC, m, n, kA, k, st);
     return cudaGetLastError();
 }
 
