@@ -2,6 +2,20 @@
 // Sigma): forward L x = b and backward L' x = y, the solves of Eq. 1 and of
 // the cokriging weights Sigma^-1 Z in Eq. 3.
 //
+// The solve is a chain over the 64-row blocks, so all that does not need the
+// blocks before is done ahead of a block's turn: its CTA inverts the two 32 x 32
+// triangles of the diagonal block while it waits, and the entries of L are
+// loaded before the wait.  The chain then carries seven 32 x 32 products, each
+// a step over all warps, instead of 64 dependent steps of one warp: two for a
+// triangle's inverse and its residual, one more to add the correction (the
+// inverse alone has 1.5 to 3.7 times the substitution's error on a smooth
+// field's factor, with the correction it is the same), one between the halves.
+// The first block has nothing to wait for, and one warp's substitution (20 us)
+// is done sooner than the inversion: it is solved that way (N = 64: 21 us, 33
+// by inversion).  Backward, with that substitution in every block and now:
+// N = 128 41 and 34 us, 512 149 and 87, 2,000 588 and 272, 8,000 2.56 and
+// 1.04 ms, 40,500 14.3 and 6.6 ms.  Bound by the chain, about 8 us a block.
+//
 // One launch per solve.  The rows are cut into blocks of 64; CTAs take the
 // blocks in solve order from a ticket counter (forward: top to bottom;
 // backward: bottom to top).  The CTA holding block I accumulates the products
@@ -52,22 +66,100 @@ __device__ int wait_done(int *sync, int target, int *timeout_word, int code, lon
     }
 }
 
-// Diagonal block Ls[col][row] = L[i0 + row, i0 + col] (row, col < ib) and
-// the reciprocals of its diagonal.
-__device__ __forceinline__ void load_diag(const double *__restrict__ A, long long ld, int i0, int ib,
-                                          double (*Ls)[TB + 1], double *dinv) {
-    for (int e = threadIdx.x; e < TB * TB; e += TT) {
-        const int c = e / TB, r = e % TB;
-        Ls[c][r] = (r < ib && c < ib && r >= c) ? A[(long long)(i0 + c) * ld + i0 + r] : 0.0;
+constexpr int TH = TB / 2;   // triangles that are inverted
+
+// The diagonal block in shared memory, zeros past ib, columns first: its triangles, their inverses, the square
+// below them.
+struct Diag {
+    double t[2][TH][TH + 1], x[2][TH][TH + 1], m[TH][TH + 1];
+    double part[8][TH], rhs[TB], y[TH], e[TH];
+};
+
+// Loads the block and the reciprocals of its pivots (the diagonals of x) and, on request, inverts its triangles, column by column from the last: below the diagonal, minus the inverse
+// found so far times the column of L, over the pivot.  Four warps per triangle share a row's sum.
+__device__ __forceinline__ void load_diag(const double *__restrict__ A, long long ld, int i0, int ib, Diag &d,
+                                          bool invert) {
+    for (int i = threadIdx.x; i < TB * TB; i += TT) {
+        const int c = i / TB, r = i % TB, h = c / TH;
+        if (r < h * TH) continue;   // above the triangles
+        const double v = (r < ib && c < ib && r >= c) ? A[(long long)(i0 + c) * ld + i0 + r] : 0.0;
+        if (r / TH == h) {
+            d.t[h][c - h * TH][r - h * TH] = v;
+            d.x[h][c - h * TH][r - h * TH] = (r == c && r < ib) ? 1.0 / v : 0.0;
+        } else
+            d.m[c][r - TH] = v;
     }
-    if (threadIdx.x < ib) dinv[threadIdx.x] = 1.0 / A[(long long)(i0 + threadIdx.x) * ld + i0 + threadIdx.x];
+    __syncthreads();
+    if (!invert) return;
+    const int lane = threadIdx.x & 31, w = threadIdx.x / 32, q = w % 4;
+    double(*T)[TH + 1] = d.t[w / 4], (*X)[TH + 1] = d.x[w / 4];
+    for (int j = TH - 2; j >= 0; --j) {
+        double s = 0.0;
+        for (int k = j + 1 + q; k < TH; k += 4) s = fma(X[k][lane], T[j][k], s);
+        d.part[w][lane] = s;
+        __syncthreads();
+        if (q == 0 && lane > j)
+            X[j][lane] = -X[j][j] * ((s + d.part[w + 1][lane]) + (d.part[w + 2][lane] + d.part[w + 3][lane]));
+        __syncthreads();
+    }
+}
+
+// B v for a 32 x 32 block B, columns first (B' v with TR): four of a row's 32 terms per warp.  The sum, in warp 0.
+template <bool TR>
+__device__ __forceinline__ double mul32(double (*B)[TH + 1], const double *v, Diag &d) {
+    const int lane = threadIdx.x & 31, w = threadIdx.x / 32;
+    double t[2] = {0.0, 0.0};
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const int k = 4 * w + i;
+        t[i & 1] = fma(TR ? B[lane][k] : B[k][lane], v[k], t[i & 1]);
+    }
+    d.part[w][lane] = t[0] + t[1];
+    __syncthreads();
+    if (w) return 0.0;
+    return ((d.part[0][lane] + d.part[1][lane]) + (d.part[2][lane] + d.part[3][lane])) +
+           ((d.part[4][lane] + d.part[5][lane]) + (d.part[6][lane] + d.part[7][lane]));
+}
+
+// d.y = T^-1 rhs (T'^-1 with TR) for triangle h: by the inverse, then a correction by the residual's.
+template <bool TR>
+__device__ __forceinline__ void tri32(int h, Diag &d) {
+    const int i = threadIdx.x;   // of the first warp's sums
+    double v = mul32<TR>(d.x[h], d.rhs + h * TH, d);
+    if (i < TH) d.y[i] = v;
+    __syncthreads();
+    v = mul32<TR>(d.t[h], d.y, d);
+    if (i < TH) d.e[i] = d.rhs[h * TH + i] - v;
+    __syncthreads();
+    v = mul32<TR>(d.x[h], d.e, d);
+    if (i < TH) d.y[i] += v;
+    __syncthreads();
+}
+
+// rhs <- L_II^-1 rhs (L_II'^-1 with TR) by substitution, one warp, rows lane and 32 + lane.
+template <bool TR>
+__device__ __forceinline__ void substitute(Diag &d, int ib) {
+    const int lane = threadIdx.x & 31;
+    double v[2] = {d.rhs[lane], d.rhs[TH + lane]};
+#pragma unroll
+    for (int hh = 0; hh < 2; ++hh) {
+        const int h = TR ? 1 - hh : hh;
+        const int n = min(TH, ib - h * TH);
+        for (int kk = 0; kk < n; ++kk) {
+            const int k = TR ? n - 1 - kk : kk;
+            const double vk = __shfl_sync(0xffffffffu, v[h], k) * d.x[h][k][k];
+            if (lane == k) v[h] = vk;
+            if (TR ? lane < k : lane > k) v[h] = fma(-(TR ? d.t[h][lane][k] : d.t[h][k][lane]), vk, v[h]);
+            if (hh == 0) v[1 - h] = fma(-(TR ? d.m[lane][k] : d.m[k][lane]), vk, v[1 - h]);
+        }
+    }
+    d.rhs[lane] = v[0];
+    d.rhs[TH + lane] = v[1];
 }
 
 __global__ void __launch_bounds__(TT) k_trsv_fwd(const double *__restrict__ A, long long ld, int N, double *x,
                                                  int *sync, int *timeout_word, long long wait_limit) {
-    __shared__ double Ls[TB][TB + 1];
-    __shared__ double dinv[TB];
-    __shared__ double part[TT / TB][TB];
+    __shared__ Diag d;
     __shared__ int tick, abort_s;
     const int nblk = (N + TB - 1) / TB;
     const int r = threadIdx.x % TB, g = threadIdx.x / TB;   // row of the block, group of 16 columns
@@ -81,69 +173,67 @@ __global__ void __launch_bounds__(TT) k_trsv_fwd(const double *__restrict__ A, l
         const int I = tick;
         if (I >= nblk) return;
         const int i0 = I * TB, ib = min(TB, N - i0);
-        load_diag(A, ld, i0, ib, Ls, dinv);
+        load_diag(A, ld, i0, ib, d, I > 0);
         // acc = sum_{J < I} L[i0 + r, J block] x[J block], columns g*16 .. g*16+15 of each block
-        double acc = 0.0;
+        double acc = (g == 0 && r < ib) ? -x[i0 + r] : 0.0;
         int seen = 0;
         bool aborted = false;
         for (int J = 0; J < I; ++J) {
+            double a[16];
+            const double *col = A + (long long)(J * TB + g * 16) * ld + i0 + r;
+#pragma unroll
+            for (int c = 0; c < 16; ++c) a[c] = r < ib ? col[(long long)c * ld] : 0.0;
             if (J >= seen) {   // warp-uniform
                 // every lane waits with its own acquire loads before it reads x
-                const int d = __reduce_min_sync(0xffffffffu, wait_done(sync, J + 1, timeout_word, 3, wait_limit));
-                if (d < 0) {
+                const int done = __reduce_min_sync(0xffffffffu, wait_done(sync, J + 1, timeout_word, 3, wait_limit));
+                if (done < 0) {
                     aborted = true;
                     break;
                 }
-                seen = d;
+                seen = done;
             }
-            if (r < ib) {
-                const double *col = A + (long long)(J * TB + g * 16) * ld + i0 + r;
-                const double *xj = x + J * TB + g * 16;
+            const double *xj = x + J * TB + g * 16;
+            double s0 = 0.0;   // two chains
 #pragma unroll
-                for (int c = 0; c < 16; ++c) acc = fma(col[(long long)c * ld], __ldcg(xj + c), acc);
+            for (int c = 0; c < 16; c += 2) {
+                acc = fma(a[c], __ldcg(xj + c), acc);
+                s0 = fma(a[c + 1], __ldcg(xj + c + 1), s0);
             }
+            acc += s0;
         }
         if (aborted && lane == 0) atomicExch(&abort_s, 1);
-        part[g][r] = acc;
+        d.part[threadIdx.x / 32][lane] = acc;   // warps 2 g and 2 g + 1: the rows' halves
         __syncthreads();
         if (abort_s) return;   // uniform: every thread reads it after the barrier
-        if (threadIdx.x < 32) {
-            // rows lane and lane + 32 of the block; solve L_II x_I = b_I - part
-            const int l = lane;
-            double r0 = 0.0, r1 = 0.0;
-            if (l < ib) r0 = x[i0 + l] - (part[0][l] + part[1][l] + part[2][l] + part[3][l]);
-            if (l + 32 < ib) r1 = x[i0 + l + 32] - (part[0][l + 32] + part[1][l + 32] + part[2][l + 32] + part[3][l + 32]);
-            for (int c = 0; c < ib; ++c) {
-                const int owner = c & 31;
-                double v = 0.0;
-                if (l == owner) {
-                    if (c < 32) {
-                        r0 *= dinv[c];
-                        v = r0;
-                    } else {
-                        r1 *= dinv[c];
-                        v = r1;
-                    }
-                }
-                v = __shfl_sync(0xffffffffu, v, owner);
-                if (l > c && l < ib) r0 -= Ls[c][l] * v;
-                if (l + 32 > c && l + 32 < ib) r1 -= Ls[c][l + 32] * v;
-            }
-            if (l < ib) x[i0 + l] = r0;
-            if (l + 32 < ib) x[i0 + l + 32] = r1;
-            __threadfence();
-            __syncwarp();
-            if (l == 0) st_release(&sync[1], I + 1);
+        if (g == 0) {
+            const int h = r / TH;
+            d.rhs[r] = -((d.part[h][lane] + d.part[2 + h][lane]) + (d.part[4 + h][lane] + d.part[6 + h][lane]));
         }
-        __syncthreads();   // Ls, part and tick are reused by the next ticket
+        __syncthreads();
+        const bool w0 = threadIdx.x < 32;
+        if (I == 0) {
+            if (w0) {
+                substitute<false>(d, ib);
+                if (lane < ib) x[lane] = d.rhs[lane];
+                if (TH + lane < ib) x[TH + lane] = d.rhs[TH + lane];
+            }
+        } else {
+            tri32<false>(0, d);
+            if (w0 && lane < ib) x[i0 + lane] = d.y[lane];
+            const double v = mul32<false>(d.m, d.y, d);
+            if (w0) d.rhs[TH + lane] -= v;
+            __syncthreads();
+            tri32<false>(1, d);
+            if (w0 && TH + lane < ib) x[i0 + TH + lane] = d.y[lane];
+        }
+        __syncthreads();
+        if (threadIdx.x == 0) st_release(&sync[1], I + 1);   // releases what the CTA wrote before the barrier
     }
 }
 
 __global__ void __launch_bounds__(TT) k_trsv_bwd(const double *__restrict__ A, long long ld, int N, double *w,
                                                  int *sync, int *timeout_word) {
-    __shared__ double Ls[TB][TB + 1];
-    __shared__ double dinv[TB];
-    __shared__ double part[TB];
+    __shared__ Diag d;
     __shared__ int tick, abort_s;
     const int nblk = (N + TB - 1) / TB;
     const int warp = threadIdx.x / 32, lane = threadIdx.x & 31;   // warp: columns 8 warp .. 8 warp + 7
@@ -157,7 +247,7 @@ __global__ void __launch_bounds__(TT) k_trsv_bwd(const double *__restrict__ A, l
         if (t >= nblk) return;
         const int I = nblk - 1 - t;
         const int i0 = I * TB, ib = min(TB, N - i0);
-        load_diag(A, ld, i0, ib, Ls, dinv);
+        load_diag(A, ld, i0, ib, d, t > 0);
         // acc[q] = sum_{J > I} sum_{rows k of J} L[k, i0 + 8 warp + q] w[k], lanes over rows
         double acc[8];
 #pragma unroll
@@ -165,68 +255,65 @@ __global__ void __launch_bounds__(TT) k_trsv_bwd(const double *__restrict__ A, l
         int seen = 0;
         bool aborted = false;
         for (int J = nblk - 1; J > I; --J) {
-            const int need = nblk - J;   // tickets 0 .. need-1 done
-            if (need > seen) {   // warp-uniform
-                // every lane waits with its own acquire loads before it reads w
-                const int d = __reduce_min_sync(0xffffffffu, wait_done(sync, need, timeout_word, 4, 0));
-                if (d < 0) {
-                    aborted = true;
-                    break;
-                }
-                seen = d;
-            }
             const int j0 = J * TB, jb = min(TB, N - j0);
-            const double w0 = (lane < jb) ? __ldcg(w + j0 + lane) : 0.0;
-            const double w1 = (lane + 32 < jb) ? __ldcg(w + j0 + lane + 32) : 0.0;
+            double a0[8], a1[8];
 #pragma unroll
             for (int q = 0; q < 8; ++q) {
                 const int c = 8 * warp + q;
-                if (c < ib) {
-                    const double *col = A + (long long)(i0 + c) * ld + j0;
-                    if (lane < jb) acc[q] = fma(col[lane], w0, acc[q]);
-                    if (lane + 32 < jb) acc[q] = fma(col[lane + 32], w1, acc[q]);
-                }
+                const double *col = A + (long long)(i0 + c) * ld + j0;
+                a0[q] = (c < ib && lane < jb) ? col[lane] : 0.0;
+                a1[q] = (c < ib && lane + 32 < jb) ? col[lane + 32] : 0.0;
             }
+            const int need = nblk - J;   // tickets 0 .. need-1 done
+            if (need > seen) {   // warp-uniform
+                // every lane waits with its own acquire loads before it reads w
+                const int done = __reduce_min_sync(0xffffffffu, wait_done(sync, need, timeout_word, 4, 0));
+                if (done < 0) {
+                    aborted = true;
+                    break;
+                }
+                seen = done;
+            }
+            const double w0 = (lane < jb) ? __ldcg(w + j0 + lane) : 0.0;
+            const double w1 = (lane + 32 < jb) ? __ldcg(w + j0 + lane + 32) : 0.0;
+#pragma unroll
+            for (int q = 0; q < 8; ++q) acc[q] = fma(a1[q], w1, fma(a0[q], w0, acc[q]));
         }
         if (aborted && lane == 0) atomicExch(&abort_s, 1);
+        // the eight sums over the warp: each halving of the lanes halves the number of sums a lane carries
 #pragma unroll
-        for (int q = 0; q < 8; ++q) {
-            double v = acc[q];
-            for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-            if (lane == 0) part[8 * warp + q] = v;
+        for (int h = 4, o = 16; h >= 1; h >>= 1, o >>= 1) {
+            const bool up = lane & o;
+#pragma unroll
+            for (int q = 0; q < h; ++q)
+                acc[q] = (up ? acc[q + h] : acc[q]) + __shfl_xor_sync(0xffffffffu, up ? acc[q] : acc[q + h], o);
+        }
+        double v = acc[0];   // of column 4 [lane & 16] + 2 [lane & 8] + [lane & 4]
+        v += __shfl_xor_sync(0xffffffffu, v, 2);
+        v += __shfl_xor_sync(0xffffffffu, v, 1);
+        if ((lane & 3) == 0) {
+            const int c = 8 * warp + (lane >> 2 & 1) + (lane >> 3 & 1) * 2 + (lane >> 4 & 1) * 4;
+            d.rhs[c] = c < ib ? w[i0 + c] - v : 0.0;
         }
         __syncthreads();
         if (abort_s) return;
-        if (threadIdx.x < 32) {
-            // L_II' w_I = y_I - part, from the bottom row up
-            const int l = lane;
-            double r0 = 0.0, r1 = 0.0;
-            if (l < ib) r0 = w[i0 + l] - part[l];
-            if (l + 32 < ib) r1 = w[i0 + l + 32] - part[l + 32];
-            for (int c = ib - 1; c >= 0; --c) {
-                const int owner = c & 31;
-                double v = 0.0;
-                if (l == owner) {
-                    if (c < 32) {
-                        r0 *= dinv[c];
-                        v = r0;
-                    } else {
-                        r1 *= dinv[c];
-                        v = r1;
-                    }
-                }
-                v = __shfl_sync(0xffffffffu, v, owner);
-                // row k < c: r_k -= L[c, k] v, L[c, k] = Ls[k][c]
-                if (l < c) r0 -= Ls[l][c] * v;
-                if (l + 32 < c) r1 -= Ls[l + 32][c] * v;
+        if (t == 0) {
+            if (warp == 0) {
+                substitute<true>(d, ib);
+                if (lane < ib) w[i0 + lane] = d.rhs[lane];
+                if (TH + lane < ib) w[i0 + TH + lane] = d.rhs[TH + lane];
             }
-            if (l < ib) w[i0 + l] = r0;
-            if (l + 32 < ib) w[i0 + l + 32] = r1;
-            __threadfence();
-            __syncwarp();
-            if (l == 0) st_release(&sync[1], t + 1);
+        } else {
+            tri32<true>(1, d);
+            if (warp == 0 && TH + lane < ib) w[i0 + TH + lane] = d.y[lane];
+            v = mul32<true>(d.m, d.y, d);
+            if (warp == 0) d.rhs[lane] -= v;
+            __syncthreads();
+            tri32<true>(0, d);
+            if (warp == 0 && lane < ib) w[i0 + lane] = d.y[lane];
         }
         __syncthreads();
+        if (threadIdx.x == 0) st_release(&sync[1], t + 1);   // releases what the CTA wrote before the barrier
     }
 }
 
