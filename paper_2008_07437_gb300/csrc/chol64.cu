@@ -36,8 +36,8 @@
 // block's factorisation, 6.3 the solve below it, 6.6 the product, the rest
 // memory and flags), large ones by the FP64 pipe.  Measured, against one
 // launch per step of a 64-wide blocked algorithm (POTRF in one CTA 97 us, TRSM
-// 65, rank-64 update 100 and more): N = 800 0.84 ms (3.5), N = 8,002 141.5 ms
-// = 0.96 of the pipe (172), a 512-column diagonal tile with its inverse beside
+// 65, rank-64 update 100 and more): N = 800 0.84 ms (3.5), N = 8,002 142 ms
+// = 0.95 of the pipe (172), a 512-column diagonal tile with its inverse beside
 // other work 0.55 ms (1.6), 24 tiles of 256 in the mixed form 10 ms (24).
 // Four groups of 128 threads share a CTA because one CTA per SM keeps the
 // SMs of a concurrent persistent kernel free, and 128 threads reach all four
@@ -228,7 +228,12 @@ __global__ void __launch_bounds__(DF_THREADS, 1) k_chol_df(const DfArgs a) {
             sm.Bs[col][lr] = v;
         }
         df_sync(grp);
-        const bool straight = !a.block64 || kind == 2 || c < 2;
+        // Sums of blk tile columns are formed on their own and then taken off the tile: its entries are rounded
+        // once per 512 columns, not once per column (N = 40,000: l within 3.9e-14 of the 8-slice form, 4.7e-13
+        // with one sum over all columns; 0.3 % of the time)
+        const int blk = a.block64 ? 2 : 16;
+        const bool straight = kind == 2 || c < blk;
+        bool based = straight;   // acc holds the tile too, not only a sum
 #pragma unroll
         for (int i = 0; i < 8; ++i) {
             cur[i] = diag ? (i < 5 ? sm.Bs[dc[i % 5]][dr[i % 5]] : 0.0) : sm.Bs[tx + 16 * (i % 2)][ty + 8 * (i / 2)];
@@ -279,8 +284,8 @@ __global__ void __launch_bounds__(DF_THREADS, 1) k_chol_df(const DfArgs a) {
                 df_mma<1>(acc, sm.As, sm.Bs, tx, ty);
             else
                 df_mma<4>(acc, sm.As, sm.Bs, tx, ty);
-            if (!straight && (k & 1)) {   // 64 columns done: off the tile, and on with the next ones
-                const bool own = k + 1 == (c & ~1);
+            if (!straight && (k & (blk - 1)) == blk - 1) {   // a block done: off the tile, and on with the next one
+                const bool own = based = k + 1 == (c & -blk);
 #pragma unroll
                 for (int i = 0; i < 8; ++i) {
                     cur[i] -= acc[i];
@@ -290,6 +295,10 @@ __global__ void __launch_bounds__(DF_THREADS, 1) k_chol_df(const DfArgs a) {
             df_sync(grp);
         }
         if (gone) return;   // uniform over the group
+        if (!based) {
+#pragma unroll
+            for (int i = 0; i < 8; ++i) acc[i] -= cur[i];
+        }
         // the tile into shared memory, [col][row]; past the matrix a diagonal block continues as the identity
 #pragma unroll
         for (int i = 0; i < 8; ++i) {
