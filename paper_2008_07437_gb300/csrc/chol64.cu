@@ -228,11 +228,12 @@ __global__ void __launch_bounds__(DF_THREADS, 1) k_chol_df(const DfArgs a) {
             sm.Bs[col][lr] = v;
         }
         df_sync(grp);
-        // Sums of blk tile columns are formed on their own and then taken off the tile: its entries are rounded
-        // once per 512 columns, not once per column (N = 40,000: l within 3.9e-14 of the 8-slice form, 4.7e-13
-        // with one sum over all columns; 0.3 % of the time)
-        const int blk = a.block64 ? 2 : 16;
-        const bool straight = kind == 2 || c < blk;
+        // Past 8,192 columns, sums of 1,024 are formed on their own and then taken off the tile: its entries are
+        // rounded once per block, not once per column (N = 40,000: l within 6.8e-14 of the 8-slice form, 4.7e-13
+        // with one sum).  Below that one sum does: N = 8,002 2.7e-12 from 64 exact bits, 2.9e-12 in 960-wide
+        // panels, and blocks cost 0.3 % there, 1 % of the prediction variances.
+        const int blk = a.block64 ? 2 : 32;
+        const bool straight = kind == 2 || c < (a.block64 ? 2 : 256);
         bool based = straight;   // acc holds the tile too, not only a sum
 #pragma unroll
         for (int i = 0; i < 8; ++i) {
