@@ -109,14 +109,14 @@ def class_roofline(cls):
     return "alu", FP64_PEAK_TFLOPS, "derived: 152 SMs x 2 FP64 FMA/clk x 2 flop x 2.07 GHz"
 
 
-KERNEL_NAMES = {"gemm": "k_dgemm_update (FP64 FMA trailing/panel updates)",
+KERNEL_NAMES = {"gemm": "k_chol_df (native FP64 Cholesky: products, pivots and solves of its 32 x 32 tiles in one launch)",
                 "oz": "k_oz_update (tcgen05 BF16 digit products, exact FP32 accumulation: emulated FP64 "
                       "trailing updates and panel solves)",
                 "sgemm": "k_sgemm_nt (FP32 SIMT diagonal/band and panel updates)",
                 "tcgemm": "k_tc_update (tcgen05 FP16x2 updates beyond the band)",
                 "covgen": "k_covgen_sym (FP64 Matern + Bessel K_nu)"}
-TLR_KERNEL_NAMES = {"gemm": "k_bgemm + k_dgemm_update (FP64 low-rank updates of the tile column, diagonal tiles)",
-                    "tlr": "k_house_qr + k_jacobi_svd_cl (FP64 compression of the tiles)",
+TLR_KERNEL_NAMES = {"gemm": "k_bgemm (FP64 low-rank updates of the tile column, diagonal tiles)",
+                    "tlr": "k_house_qr_col + k_jacobi_svd_cl (FP64 compression of the tiles)",
                     "covgen": "k_covgen_block (FP64 Matern + Bessel K_nu)"}
 METRIC = "loglik evals/s"
 
@@ -582,8 +582,8 @@ def run_ours(args):
                       "evals_per_s": 1e3 / ms_ref, "loglik": ll_ref,
                       "rel_dl": abs(ll - ll_ref) / abs(ll_ref),
                       "speedup": ms_ref / (ms / args.steps),
-                      "k_dgemm_update_frac_of_fp64_peak": (g["flops"] / (g["ms"] * 1e-3) / 1e12 / FP64_PEAK_TFLOPS
-                                                           if g["ms"] > 0 else None)}
+                      "k_chol_df_frac_of_fp64_peak": (g["flops"] / (g["ms"] * 1e-3) / 1e12 / FP64_PEAK_TFLOPS
+                                                      if g["ms"] > 0 else None)}
     tlr_accuracy = None
     if tlr and args.tlr_ref and (rank == 0 or world == 1):
         tol = w.extra.get("tlr_tol", 1e-9)
@@ -640,16 +640,15 @@ def run_ours(args):
     other = sum(prof[k]["ms"] for k in ("covgen", "reduce", "solve", "predict")) / args.steps
     chol_ms = max(ms / args.steps - other, 1e-9)
     chol_tflops = (N ** 3 / 3.0) / (chol_ms * 1e-3) / 1e12
-    # DRAM bytes per launch: an ncu capture of a full rank-960 trailing update
-    # (N = 8,000) measured 0.822 x the algorithmic bytes; scaled to this run's
-    # average launch (FP64 update kernel only)
-    traffic = 0.822 * dk["bytes"] / max(dk["launches"], 1) if dom == "gemm" and not tlr else None
+    # DRAM bytes per launch.  The native Cholesky is one left-looking launch whose re-reads grow with N, and a
+    # capture at this size takes too many passes: null.
+    traffic = None
     if dom == "tcgemm" and emulated and w.extra.get("oz_cut") and w.extra.get("oz_slices", 8) == 8:
         # k_oz_update with the level cut: an ncu capture of every launch of one evaluation at
-        # N = 16,000 measured DRAM read + write = 0.967 x the algorithmic bytes the library counts
+        # N = 16,000 measured DRAM read + write = 1.322 x the algorithmic bytes the library counts
         # (16 B per output written, the digit slices); scaled to this run's launches (8 slices, the
         # captured kernel; other slice counts have no capture: null)
-        traffic = 0.967 * dk["bytes"] / max(dk["launches"], 1)
+        traffic = 1.322 * dk["bytes"] / max(dk["launches"], 1)
     dtype = "f64"
     if emulated:
         dtype = "f64 (emulated: bf16 digit products, exact fp32 accumulation, %d slices)" % w.extra.get("oz_slices", 8)
@@ -1221,7 +1220,7 @@ def run_mloe(args):
            "mloe": ml, "mmom": mm, "phases_ms": {"GEN": gen, "FACT": fact, "COMP": comp},
            "form": ("native FP64 FMA updates" if args.mloe_form == "native"
                     else "FP64 updates and panel solves on the tensor cores (8 digit slices, level cut)"),
-           "roofline": {"bound": bound, "kernel": ("k_dgemm_update" if cls == "gemm" else "k_oz_update") +
+           "roofline": {"bound": bound, "kernel": ("k_chol_df" if cls == "gemm" else "k_oz_update") +
                         " (both factorisations)", "achieved": ach,
                         "peak": peak, "unit": "TFLOP/s", "frac": ach / peak, "peak_source": peak_src,
                         "traffic": None},

@@ -73,7 +73,7 @@ typedef struct {
 
 /* Options of a likelihood evaluation.  geo_opts_default fills the defaults. */
 typedef struct {
-    int nb;             /* tile size of the tiled Cholesky (default 960) */
+    int nb;             /* tile size of the tiled Cholesky (default 960; native FP64 checks it and uses 32 x 32 tiles) */
     int prec;           /* GEO_PREC_* (default GEO_PREC_FP64) */
     int band;           /* MIXED: tiles with 0 < |i - j| <= band stay FP32 (default 4) */
     int lowp;           /* MIXED: 0 = FP16 operands with a per-tile power-of-two scale, 1 = BF16 */
@@ -319,13 +319,11 @@ int geo_mle_best(const geo_mle_state *state, double *sigma2, double *a, double *
  * Batched log-likelihoods of many small, uneven problems (Eq. 1 for each),
  * dense FP64, in the callers' location order.  One launch builds the K_nu
  * tables of every theta; one persistent launch does the rest for the whole
- * batch: its CTAs walk a table of units (a 64 x 64 block of location pairs of
- * Eq. 2, the POTRF of a 64-wide diagonal block, the TRSM of 128 rows below
- * it, a 128 x 64 tile of the trailing update, the reduction), each unit
- * waiting (bounded) on its problem's progress counter.  The table's order
- * comes from a list-scheduling simulation on the host (cached while the
- * problem sizes stay the same).  The launch sequence of a batch shape (count
- * and largest order) is captured once as a CUDA graph and replayed, with the
+ * batch: groups of threads walk a table of units (32 x 32 tiles of the
+ * matrices, column by column over all problems, and a reduction per problem),
+ * each unit waiting (bounded) on its problem's progress words.  The launch
+ * sequence of a batch shape (count, largest p and largest order) is captured
+ * once as a CUDA graph and replayed, with the
  * per-problem inputs, theta and units refreshed in device memory.  A
  * problem's result depends only on its own inputs: it is bit-identical alone
  * and in any batch.  GEO_ETIMEOUT if a bounded wait expired.
@@ -561,7 +559,7 @@ int geo_server_profile_read(geo_server *server, geo_kstat *out);
  *   locs_dev  n x 2 locations (device, caller-owned); used in the caller's order
  *   z_dev     N = p*n observations in Representation I (device)
  *   theta     host struct as for geo_loglik
- *   nb        tile size (>= 64)
+ *   nb        >= 64 (checked; the factorisation is one launch over 32 x 32 tiles)
  *   out_dev   3 doubles (device, caller-owned): l(theta), log|Sigma|, Z' Sigma^-1 Z;
  *             l is NaN when Sigma is not positive definite
  *   info_dev  NULL or one int (device): 0, or the 1-based failing row

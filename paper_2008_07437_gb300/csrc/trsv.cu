@@ -21,13 +21,13 @@
 // backward: bottom to top).  The CTA holding block I accumulates the products
 // with the blocks already solved, waiting on a `done` counter for the ones
 // that are not (a block completes only after its predecessor, so one counter
-// suffices), then solves its diagonal block with one warp and publishes it.
+// suffices), then solves its diagonal block and publishes it.
 // A CTA only waits on blocks whose tickets were taken earlier by CTAs that
 // are running, so the solve cannot deadlock whatever the number of resident
 // CTAs.  Every wait is bounded: past WAIT_CYCLES the CTA raises an abort word
 // that makes every other waiter give up too, records the timeout and leaves
 // the solve unfinished.  Sums run in a fixed order: the result does not
-// depend on timing.  Each pass streams the lower triangle once (HBM-bound).
+// depend on timing.  Each pass streams the lower triangle once.
 //
 // sync: 4 device ints {ticket, done, abort, unused}, zeroed before each launch.
 #include "geo_internal.cuh"
