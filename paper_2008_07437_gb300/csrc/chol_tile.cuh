@@ -71,24 +71,42 @@ __device__ __forceinline__ double df_half(double x) {
     return __hiloint2double(__double2hiint(x) - (1 << 20), __double2loint(x));
 }
 
-// d > 0 (false for a NaN), off the FP64 pipe.
+// d > 0 and finite (false for a NaN), off the FP64 pipe.
 __device__ __forceinline__ bool df_positive(double d) {
     const long long b = __double_as_longlong(d);
-    return b > 0 && b <= 0x7FF0000000000000LL;
+    return b > 0 && b < 0x7FF0000000000000LL;
 }
 
-// l = sqrt(d) and inv = 1 / l for a positive normal d, both as IEEE rounding gives them (the residuals of the
-// last steps are exact FMAs): the hardware's approximation of 1 / sqrt(d) (about 22 bits), one Newton step for
-// the root and its reciprocal, and a correction of each.  A chain of seven dependent FP64 operations where
-// sqrt() and a division take some twenty.
+// Pivots outside 2^-800 .. 2^900 would come too near the ends of the range for the approximations and residuals below
+// (variances of 1e-300, say): a tile with such a diagonal entry (ext, the same in every thread) is factored as D S D
+// with powers of two, which is exact.  The scale of a row by its diagonal entry; and one over it.
+__device__ __forceinline__ double df_row_scale(double d) {
+    const unsigned h = (unsigned)__double2hiint(d);   // (a negative d fails anyway)
+    return __hiloint2double((1023 + (h < (1023u - 800u) << 20 ? 500 : h < (1023u + 900u) << 20 ? 0 : -450)) << 20, 0);
+}
+__device__ __forceinline__ double df_inv_scale(double s) { return __hiloint2double((2046 << 20) - __double2hiint(s), 0); }
+__device__ __forceinline__ bool df_extreme(double d) {
+    return (unsigned)__double2hiint(d) - ((1023u - 800u) << 20) >= (1700u << 20);
+}
+
+// l = sqrt(d) and inv = 1 / l for a d of 2^-960 .. 2^960, both as IEEE rounding gives them, by the method of
+// P. Markstein ("Computation of elementary functions on the IBM RISC System/6000 processor", IBM J. Res. Dev. 34,
+// 1990): the hardware's approximation of 1 / sqrt(d) (about 22 bits), one Newton step for the root and its reciprocal,
+// and a correction of each by its residual, which an FMA gives exactly.  Before its last rounding each is within 2^-85
+// or so of the value, so that only one a hair's breadth from the middle of two doubles could go the other way: none of
+// 2^28 did over all those exponents.  The reciprocal's one exception is the method's: a root with a mantissa of ones,
+// of a d one or two units below an even power of two, has its reciprocal one unit above the correction's result (which
+// is a power of two), and d's bits show that before the chain begins.  A chain of seven
+// dependent FP64 operations where sqrt() and a division take some twenty.
 __device__ __forceinline__ void df_root(double d, double *l, double *inv) {
     double y0;
     asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y0) : "d"(d));
     const double t = d * y0, e = fma(-t, df_half(y0), 0.5);   // (1 - d y0^2) / 2
     const double r = fma(t, e, t), y = fma(y0, e, y0);
-    const double root = fma(fma(-r, r, d), df_half(y), r);
+    const bool below = (__double2hiint(d) & 0x1FFFFF) == 0xFFFFF && (unsigned)__double2loint(d) >= 0xFFFFFFFEu;
+    const double root = fma(fma(-r, r, d), df_half(y), r), rec = fma(fma(-root, y, 1.0), y, y);
     *l = root;
-    *inv = fma(fma(-root, y, 1.0), y, y);
+    *inv = __hiloint2double(__double2hiint(rec), below ? 1 : __double2loint(rec));
 }
 
 // Cholesky factor of the 32 x 32 block S[col][row] (lower part) by one group, lane = row, columns w, w + 4, ...
@@ -104,6 +122,15 @@ __device__ __forceinline__ int df_potrf32_plain(double (*S)[DLD], double (*buf)[
     double v[8], p[4] = {0.0, 0.0, 0.0, 0.0};
 #pragma unroll
     for (int q = 0; q < 8; ++q) v[q] = S[4 * q + w][lane];
+    // (nothing is written before the first barrier)
+    const double dg = S[lane][lane];
+    const bool ext = __any_sync(0xffffffffu, df_extreme(dg));
+    double sc = 1.0;
+    if (ext) {
+        sc = df_row_scale(dg);
+#pragma unroll
+        for (int q = 0; q < 8; ++q) v[q] *= sc * __shfl_sync(0xffffffffu, sc, 4 * q + w);
+    }
     int bad = DT;
 #pragma unroll
     for (int P = 0; P < 8; ++P) {
@@ -135,6 +162,13 @@ __device__ __forceinline__ int df_potrf32_plain(double (*S)[DLD], double (*buf)[
             if (P < 7) v[(P + 1) % 8] = fma(-p[i], __shfl_sync(0xffffffffu, p[i], (4 * P + 4 + w) & 31), v[(P + 1) % 8]);
         }
     }
+    if (ext) {
+        df_sync(grp);   // every warp has read the columns
+        const double si = df_inv_scale(sc);
+#pragma unroll
+        for (int q = 0; q < 8; ++q) S[4 * q + w][lane] *= si;
+        if (w == 0) dinv[lane] *= sc;
+    }
     return bad;
 }
 
@@ -146,6 +180,15 @@ __device__ __forceinline__ int df_potrf32(double (*S)[DLD], double (*buf)[4][DT]
     double v[8], p[4] = {0.0, 0.0, 0.0, 0.0}, m[4] = {0.0, 0.0, 0.0, 0.0};
 #pragma unroll
     for (int q = 0; q < 8; ++q) v[q] = S[4 * q + w][lane];
+    // (nothing is written before the first barrier)
+    const double dg = S[lane][lane];
+    const bool ext = __any_sync(0xffffffffu, df_extreme(dg));
+    double sc = 1.0;
+    if (ext) {
+        sc = df_row_scale(dg);
+#pragma unroll
+        for (int q = 0; q < 8; ++q) v[q] *= sc * __shfl_sync(0xffffffffu, sc, 4 * q + w);
+    }
 #pragma unroll
     for (int P = 0; P < 8; ++P) {
         buf[P & 1][w][lane] = v[P];
@@ -180,7 +223,8 @@ __device__ __forceinline__ int df_potrf32(double (*S)[DLD], double (*buf)[4][DT]
     const unsigned ok = __ballot_sync(0xffffffffu, df_positive(d));
     double l, inv;
     df_root(d, &l, &inv);
-    if (w == 0) dinv[lane] = inv;
+    if (w == 0) dinv[lane] = inv * sc;
+    const double si = df_inv_scale(sc);
 #pragma unroll
     for (int q = 0; q < 8; ++q) {
         const int col = 4 * q + w;
@@ -189,7 +233,7 @@ __device__ __forceinline__ int df_potrf32(double (*S)[DLD], double (*buf)[4][DT]
     }
     df_sync(grp);   // every warp has read the diagonal
 #pragma unroll
-    for (int q = 0; q < 8; ++q) S[4 * q + w][lane] = v[q];
+    for (int q = 0; q < 8; ++q) S[4 * q + w][lane] = ext ? v[q] * si : v[q];
     return ok == 0xffffffffu ? DT : __ffs(~ok) - 1;
 }
 
