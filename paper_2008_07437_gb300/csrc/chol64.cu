@@ -409,7 +409,21 @@ cudaError_t launch_df(const DfArgs &a0, int sms, int cls, double flops, cudaStre
     a.chain = a.factor && !a.block64 && T > 1;
     // below about 4,000 columns the chain, not the products, sets the time
     a.alone = a.chain && T < 128;
-    const long long words = 2 + T + E + (a.W ? T : 0) + (a.chain ? 2 * T : 0);
+    const long long fixed = 2 + T + (a.W ? T : 0) + (a.chain ? 2 * T : 0), room = GEO_CHOL_SYNC_INTS - fixed;
+    if (E > room) {   // rows past what the words hold, once the others are done
+        if (room <= 0) return cudaErrorInvalidValue;
+        DfArgs head = a0, rest = a0;
+        head.E = (int)room;
+        head.nx = DT * head.E;
+        rest.factor = 0;
+        rest.W = nullptr;
+        rest.X += head.nx;
+        rest.nx -= head.nx;
+        rest.E -= head.E;
+        const cudaError_t e = launch_df(head, sms, cls, flops, s);
+        return e != cudaSuccess ? e : launch_df(rest, sms, cls, 0.0, s);
+    }
+    const long long words = fixed + E;
     const long long tickets = !a.factor ? (a.W ? T * (T + 1) / 2 : T * E) : a.W ? T * (T + E + 1) : T * (T + E) - T * (T - 1) / 2;
     if (tickets == 0) return cudaSuccess;
     if (words > GEO_CHOL_SYNC_INTS || tickets > (1LL << 30)) return cudaErrorInvalidValue;
