@@ -14,15 +14,21 @@
 // one CTA per SM) take tiles from a ticket counter, column by column, and do
 // everything for a tile at once, left-looking: C_ic = A_ic - sum_k L_ik L_ck'
 // in registers over the finished tiles k < c of the two tile rows, then the
-// Cholesky factor of the 32 x 32 block (i = c, one warp, a row per lane in
-// registers) or the solve with L_cc' (i > c, one warp, a row per lane).  Every
-// tile is written once.  A progress word per tile row counts its finished
+// Cholesky factor of the 32 x 32 block (i = c) or the solve with L_cc'
+// (i > c).  The tile is written once; only with a column chain (df_chain) the
+// diagonal tiles and those below them are written up to date first and
+// finished by the chain.  A progress word per tile row counts its finished
 // tiles; a group waits on the words of its two rows, so tiles of later columns
-// accumulate while the column chain runs (lookahead without streams).  A group
-// only waits for tiles whose tickets were taken earlier by groups that are
-// running, so the launch cannot deadlock whatever the number of resident CTAs.
-// Every wait is bounded: past DF_WAIT_CYCLES without progress the waiter
-// raises the abort word, records the timeout and all groups return; a failed
+// accumulate while the column chain runs (lookahead without streams).
+//
+// The launch ends whatever the number of resident CTAs, down to one: a group
+// waits for tiles whose tickets were taken earlier by groups that are running,
+// or for the chain, which takes the first ticket and waits in column order for
+// tiles that later tickets bring up to date.  So some other group has to go on
+// taking tickets, and the groups that would leave the SM to the chain (or are
+// spare) only leave once a second CTA has started: its first group stays to
+// the end.  Every wait is bounded: past DF_WAIT_CYCLES without progress the
+// waiter raises the abort word, records the timeout and all groups return; a failed
 // pivot raises the same word.  Sums run in a fixed order: results do not
 // depend on timing.
 //
@@ -59,14 +65,17 @@ struct DfArgs {
     int factor;       // 0: the diagonal range already holds L, only the extra rows are solved
     double *W;        // not null: W = -L^-1 of the diagonal range (column-major, ldw, zeros above the diagonal)
     long long ldw;
-    int *sync;        // {ticket, abort, progress words: T + E (+ T with W), with chain: ready words 2 T}
+    int *sync;        // {ticket, abort, CTAs started, progress words: T + E (+ T with W), with chain: ready words 2 T}
     int tickets;
     int chain;        // 1: one group runs the column chain (df_chain)
-    int alone;        // chain: the other groups of its CTA leave it the SM
+    int alone;        // chain: the other groups of its CTA leave it the SM (once a second CTA runs)
     int block64;      // GEO_CHOL_BLOCK64: sums per 64 columns
     int plain;        // GEO_CHOL_BLOCK64 and GEO_CHOL_PLAIN: pivots and solves as the plain algorithm rounds them
     DevStatus *st;
+    long long limit;  // clocks without progress after which a wait gives up
 };
+
+constexpr int DF_HEAD = 3;   // sync words before the progress words
 
 // The column chain, by one group: for every column c the last product of the diagonal tile (with L_c,c-1, which
 // this group has just solved and still holds), its factorisation, and the solve of the tile below it.  Handing
@@ -76,11 +85,11 @@ template <bool PLAIN>
 __device__ __noinline__ void df_chain(const DfArgs &a, DfSmem &sm, int grp, int tid, const int (&dr)[5],
                                       const int (&dc)[5]) {
     const int lr = tid % 32, lc = tid / 32;
-    int *prog = a.sync + 2, *ready = prog + a.T + a.E + (a.W ? a.T : 0);
+    int *prog = a.sync + DF_HEAD, *ready = prog + a.T + a.E + (a.W ? a.T : 0);
     for (int c = 0; c < a.T; ++c) {
         const int c0 = a.j0 + DT * c, cb = min(DT, a.j0 + a.jb - c0);
         if (c >= 2) {   // the diagonal tile holds the products of the columns before c - 1
-            if (tid == 0) sm.word[1] = df_wait(&ready[2 * c], &ready[2 * c], 1, a.sync, &a.st->timeout);
+            if (tid == 0) sm.word[1] = df_wait(&ready[2 * c], &ready[2 * c], 1, a.sync, &a.st->timeout, a.limit);
             df_sync(grp);
             if (sm.word[1] < 0) return;
         }
@@ -123,7 +132,7 @@ __device__ __noinline__ void df_chain(const DfArgs &a, DfSmem &sm, int grp, int 
         if (c + 1 == a.T) return;
         const int r0 = c0 + DT, nr = min(DT, a.j0 + a.jb - r0);
         if (c >= 1) {   // the tile below holds the products of the columns before c
-            if (tid == 32) sm.word[1] = df_wait(&ready[2 * c + 1], &ready[2 * c + 1], 1, a.sync, &a.st->timeout);
+            if (tid == 32) sm.word[1] = df_wait(&ready[2 * c + 1], &ready[2 * c + 1], 1, a.sync, &a.st->timeout, a.limit);
             df_sync(grp);
             if (sm.word[1] < 0) return;
         }
@@ -154,19 +163,25 @@ __global__ void __launch_bounds__(DF_THREADS, 1) k_chol_df(const DfArgs a) {
     const int grp = threadIdx.x / DG, tid = threadIdx.x % DG;
     DfSmem &sm = reinterpret_cast<DfSmem *>(df_smem)[grp];
     const int tx = tid % 16, ty = tid / 16, lr = tid % 32, lc = tid / 32;
-    int *prog = a.sync + 2;
+    int *prog = a.sync + DF_HEAD;
     int dr[5], dc[5];
     df_diag_entries(tid, dr, dc);
     __shared__ int chain_here;   // this CTA runs the column chain
-    if (threadIdx.x == 0) chain_here = 0;
+    if (threadIdx.x == 0) {
+        chain_here = 0;
+        if (a.chain) atomicAdd(&a.sync[2], 1);
+    }
     __syncthreads();
     // with few tiles, fewer groups to an SM share its FP64 pipe
-    if ((long long)grp * gridDim.x >= a.tickets) return;
+    const bool spare = (long long)grp * gridDim.x >= a.tickets;
+    if (spare && !a.chain) return;
+    if (spare && tid == 0)   // the other CTAs start within a microsecond, if there is room for them
+        for (int i = 0; i < 40 && df_ld_acquire(&a.sync[2]) < 2; ++i) __nanosleep(50);
     for (;;) {
         // stop after a failed pivot (of this launch or an earlier one) or an expired wait
         if (tid == 0) {
             const bool stop = df_ld_acquire(&a.sync[1]) || df_ld_acquire(&a.st->info) ||
-                              (a.alone && *(volatile int *)&chain_here);
+                              ((spare || (a.alone && *(volatile int *)&chain_here)) && df_ld_acquire(&a.sync[2]) > 1);
             sm.word[0] = stop ? a.tickets : atomicAdd(&a.sync[0], 1) - a.chain;
             if (sm.word[0] < 0) *(volatile int *)&chain_here = 1;
         }
@@ -259,7 +274,7 @@ __global__ void __launch_bounds__(DF_THREADS, 1) k_chol_df(const DfArgs a) {
         bool gone = false;
         for (int k = kbeg; k < kend; ++k) {
             if (avail <= k) {
-                if (tid == 0) sm.word[1] = df_wait(prow, pcol, k + 1, a.sync, &a.st->timeout);
+                if (tid == 0) sm.word[1] = df_wait(prow, pcol, k + 1, a.sync, &a.st->timeout, a.limit);
                 df_sync(grp);
                 avail = sm.word[1];
                 if (avail < 0) {
@@ -328,7 +343,7 @@ __global__ void __launch_bounds__(DF_THREADS, 1) k_chol_df(const DfArgs a) {
             df_sync(grp);
         } else {
             // L_cc: wait for its factorisation
-            if (tid == 0) sm.word[1] = a.factor ? df_wait(&prog[c], &prog[c], c + 1, a.sync, &a.st->timeout) : 0;
+            if (tid == 0) sm.word[1] = a.factor ? df_wait(&prog[c], &prog[c], c + 1, a.sync, &a.st->timeout, a.limit) : 0;
             df_sync(grp);
             if (sm.word[1] < 0) return;
             const double *L = a.A + (long long)c0 * a.ld + c0;
@@ -409,7 +424,7 @@ cudaError_t launch_df(const DfArgs &a0, int sms, int cls, double flops, cudaStre
     a.chain = a.factor && !a.block64 && T > 1;
     // below about 4,000 columns the chain, not the products, sets the time
     a.alone = a.chain && T < 128;
-    const long long fixed = 2 + T + (a.W ? T : 0) + (a.chain ? 2 * T : 0), room = GEO_CHOL_SYNC_INTS - fixed;
+    const long long fixed = DF_HEAD + T + (a.W ? T : 0) + (a.chain ? 2 * T : 0), room = GEO_CHOL_SYNC_INTS - fixed;
     if (E > room) {   // rows past what the words hold, once the others are done
         if (room <= 0) return cudaErrorInvalidValue;
         DfArgs head = a0, rest = a0;
@@ -453,7 +468,7 @@ cudaError_t chol64_panel(double *A, long long ld, int j0, int jb, int x0, int x1
     if (!factor_diag && W && x1 > x0) return cudaErrorInvalidValue;
     const int nx = std::max(0, x1 - x0);
     DfArgs a{A, ld, j0, jb, A + x0, ld, nx, (jb + DT - 1) / DT, (nx + DT - 1) / DT, factor_diag ? 1 : 0, W, ldw, sync, 0, 0, 0, order == GEO_CHOL_BLOCK64,
-             order != GEO_CHOL_STRAIGHT, st};
+             order != GEO_CHOL_STRAIGHT, st, DF_WAIT_CYCLES};
     const double j = jb, cubes = (factor_diag ? j * j * j / 3.0 : 0.0) + (W ? j * j * j / 3.0 : 0.0);
     return launch_df(a, sms, factor_diag ? GEO_K_POTRF : GEO_K_TRSM, cubes + nx * j * j, s);
 }
@@ -485,7 +500,7 @@ cudaError_t chol64_rhs_update(double *A, long long ld, int rC, int cC, int m, in
 cudaError_t chol64_factor(double *A, long long ld, int N, int nrows, DevStatus *st, int *sync, cudaStream_t s) {
     if (N <= 0) return cudaSuccess;
     const int nx = std::max(0, nrows - N);
-    DfArgs a{A, ld, 0, N, A + N, ld, nx, (N + DT - 1) / DT, (nx + DT - 1) / DT, 1, nullptr, 0, sync, 0, 0, 0, 0, 0, st};
+    DfArgs a{A, ld, 0, N, A + N, ld, nx, (N + DT - 1) / DT, (nx + DT - 1) / DT, 1, nullptr, 0, sync, 0, 0, 0, 0, 0, st, DF_WAIT_CYCLES};
     const double n = N;
     return launch_df(a, 0, GEO_K_GEMM, n * n * n / 3.0 + nx * n * n, s);
 }
@@ -494,6 +509,6 @@ cudaError_t chol64_factor(double *A, long long ld, int N, int nrows, DevStatus *
 cudaError_t chol64_solve_rows(double *X, long long ldx, int R, double *L, long long ldl, int N, DevStatus *st, int *sync,
                               cudaStream_t s) {
     if (R <= 0 || N <= 0) return cudaSuccess;
-    DfArgs a{L, ldl, 0, N, X, ldx, R, (N + DT - 1) / DT, (R + DT - 1) / DT, 0, nullptr, 0, sync, 0, 0, 0, 0, 0, st};
+    DfArgs a{L, ldl, 0, N, X, ldx, R, (N + DT - 1) / DT, (R + DT - 1) / DT, 0, nullptr, 0, sync, 0, 0, 0, 0, 0, st, DF_WAIT_CYCLES};
     return launch_df(a, 0, GEO_K_SOLVE, (double)R * N * N, s);
 }

@@ -45,19 +45,24 @@ __device__ __forceinline__ void set_info(DevStatus *st, int row1) {
     }
 }
 
-// Wait until min(*p, *q) >= need (one thread).  Returns that minimum, or -1 when the launch was aborted.
-__device__ int df_wait(const int *p, const int *q, int need, int *sync, int *timeout_word) {
+// Wait until min(*p, *q) >= need (one thread).  Returns that minimum, or -1 when the launch was aborted.  It gives up
+// when neither these words nor the ticket counter sync[0] has moved for `limit` clocks: as long as tiles are taken the
+// launch goes on, however few SMs it has (one tile takes well under a second).
+__device__ int df_wait(const int *p, const int *q, int need, int *sync, int *timeout_word,
+                       long long limit = DF_WAIT_CYCLES) {
     long long t0 = clock64();
-    int last = -1;
+    int last = -1, taken = -1;
     for (;;) {
         int v = df_ld_acquire(p);
         if (q != p) v = min(v, df_ld_acquire(q));
         if (v >= need) return v;
         if (df_ld_acquire(&sync[1])) return -1;
-        if (v != last) {
+        const int t = df_ld_acquire(&sync[0]);
+        if (v != last || t != taken) {
             last = v;
+            taken = t;
             t0 = clock64();
-        } else if (clock64() - t0 > DF_WAIT_CYCLES) {
+        } else if (clock64() - t0 > limit) {
             atomicExch(&sync[1], 1);
             atomicCAS(timeout_word, 0, 8);
             return -1;

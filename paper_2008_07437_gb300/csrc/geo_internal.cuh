@@ -121,7 +121,7 @@ cudaError_t launch_scatter_vec(const double *in, long long stride, const int *pe
 // and one per 32 extra rows.  More rows than that go in several launches; more columns than a device's memory holds
 // would be refused.
 constexpr int GEO_CHOL_SYNC_INTS = 32768;
-constexpr long long GEO_CHOL_MAX_N = 32LL * ((GEO_CHOL_SYNC_INTS - 3) / 3);
+constexpr long long GEO_CHOL_MAX_N = 32LL * ((GEO_CHOL_SYNC_INTS - 4) / 3);
 static_assert(8 * GEO_CHOL_MAX_N * GEO_CHOL_MAX_N > 900LL << 30, "the largest matrix fits the words");
 // Order of a tile's sum A_ic - sum_k L_ik L_ck' over the columns k of a panel: STRAIGHT through, one FMA after the
 // other from A_ic on; or (BLOCK64) a separate sum per 64 columns, subtracted as a whole, and straight through
