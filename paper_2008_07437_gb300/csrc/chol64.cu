@@ -42,8 +42,8 @@
 // block's factorisation, 6.3 the solve below it, 6.6 the product, the rest
 // memory and flags), large ones by the FP64 pipe.  Measured, against one
 // launch per step of a 64-wide blocked algorithm (POTRF in one CTA 97 us, TRSM
-// 65, rank-64 update 100 and more): N = 800 0.84 ms (3.5), N = 8,002 142 ms
-// = 0.95 of the pipe (172), a 512-column diagonal tile with its inverse beside
+// 65, rank-64 update 100 and more): N = 800 0.85 ms (3.5), N = 8,002 145 ms
+// = 0.93 of the pipe (172), a 512-column diagonal tile with its inverse beside
 // other work 0.55 ms (1.6), 24 tiles of 256 in the mixed form 10 ms (24).
 // Four groups of 128 threads share a CTA because one CTA per SM keeps the
 // SMs of a concurrent persistent kernel free, and 128 threads reach all four
@@ -69,13 +69,14 @@ struct DfArgs {
     int tickets;
     int chain;        // 1: one group runs the column chain (df_chain)
     int alone;        // chain: the other groups of its CTA leave it the SM (once a second CTA runs)
-    int block64;      // GEO_CHOL_BLOCK64: sums per 64 columns
+    int block64;      // GEO_CHOL_BLOCK64: no chain
     int plain;        // GEO_CHOL_BLOCK64 and GEO_CHOL_PLAIN: pivots and solves as the plain algorithm rounds them
     DevStatus *st;
     long long limit;  // clocks without progress after which a wait gives up
 };
 
 constexpr int DF_HEAD = 3;   // sync words before the progress words
+constexpr int DF_SUM = 2;    // tile columns whose products are summed on their own
 
 // The column chain, by one group: for every column c the last product of the diagonal tile (with L_c,c-1, which
 // this group has just solved and still holds), its factorisation, and the solve of the tile below it.  Handing
@@ -101,16 +102,19 @@ __device__ __noinline__ void df_chain(const DfArgs &a, DfSmem &sm, int grp, int 
         df_sync(grp);
         double acc[8];
 #pragma unroll
-        for (int i = 0; i < 5; ++i) acc[i] = -sm.Bs[dc[i]][dr[i]];
+        for (int i = 0; i < 5; ++i) acc[i] = c % DF_SUM ? -sm.Bs[dc[i]][dr[i]] : 0.0;
         if (c > 0) df_mma_diag(acc, sm.As, dr, dc);
+        if (c % DF_SUM == 0)   // column c - 1 is the end of an earlier block: a sum of its own
+#pragma unroll
+            for (int i = 0; i < 5; ++i) acc[i] -= sm.Bs[dc[i]][dr[i]];
         df_sync(grp);
 #pragma unroll
         for (int i = 0; i < 5; ++i)
             sm.Bs[dc[i]][dr[i]] = (dr[i] < cb && dc[i] < cb) ? -acc[i] : (dr[i] == dc[i] ? 1.0 : 0.0);
         df_sync(grp);
         auto *buf = reinterpret_cast<double (*)[4][DT]>(sm.Ls);
-            const int bad = PLAIN ? df_potrf32_plain(sm.Bs, buf, sm.dinv, grp, tid)
-                                  : df_potrf32(sm.Bs, buf, sm.dinv, grp, tid);
+        const int bad = PLAIN ? df_potrf32_plain(sm.Bs, buf, sm.dinv, grp, tid)
+                              : df_potrf32(sm.Bs, buf, sm.dinv, grp, tid);
         if (bad < cb) {
             if (tid == 0) {
                 set_info(a.st, c0 + bad + 1);
@@ -243,19 +247,25 @@ __global__ void __launch_bounds__(DF_THREADS, 1) k_chol_df(const DfArgs a) {
             sm.Bs[col][lr] = v;
         }
         df_sync(grp);
-        // Past 8,192 columns, sums of 1,024 are formed on their own and then taken off the tile: its entries are
-        // rounded once per block, not once per column (N = 40,000: l within 6.8e-14 of the 8-slice form, 4.7e-13
-        // with one sum).  Below that one sum does: N = 8,002 2.7e-12 from 64 exact bits, 2.9e-12 in 960-wide
-        // panels, and blocks cost 0.3 % there, 1 % of the prediction variances.
-        const int blk = a.block64 ? 2 : 32;
-        const bool straight = kind == 2 || c < (a.block64 ? 2 : 256);
+        // The columns before the tile's own 64 enter as sums of 64 columns, each formed on its own and then taken off
+        // the tile, so that the entries are rounded once per 64 columns and not once per column.  Relative errors
+        // of the log-determinant (of l) against twice the digits on the same Sigma, rms of 3 to 24 draws, with one
+        // sum over all columns, in 960-wide panels of 64-wide steps, and so:
+        //   N = 800    4.2e-16 (4.0e-16)   1.6e-16 (3.1e-16)   1.4e-16 (2.8e-16)
+        //   N = 1,600  9.2e-16 (9.2e-16)   1.9e-15 (2.1e-15)   2.5e-16 (1.1e-15)
+        //   N = 3,200  1.7e-15 (3.6e-15)   3.2e-15 (9.6e-15)   1.6e-16 (3.3e-15)
+        //   N = 8,002  2.9e-15 (3.3e-14)   3.8e-15 (2.4e-13)   2.0e-16 (1.4e-14)
+        // Sums of 128 come to 1.2 to 3 times the last column.  One more FP64 operation per entry and 64 columns:
+        // N = 8,002 142.7 -> 145.1 ms.
+        const bool straight = kind == 2 || c < DF_SUM;
         bool based = straight;   // acc holds the tile too, not only a sum
 #pragma unroll
         for (int i = 0; i < 8; ++i) {
-            cur[i] = diag ? (i < 5 ? sm.Bs[dc[i % 5]][dr[i % 5]] : 0.0) : sm.Bs[tx + 16 * (i % 2)][ty + 8 * (i / 2)];
-            acc[i] = straight ? -cur[i] : 0.0;
+            cur[i] = diag ? (i < 5 ? -sm.Bs[dc[i % 5]][dr[i % 5]] : 0.0) : -sm.Bs[tx + 16 * (i % 2)][ty + 8 * (i / 2)];
+            acc[i] = straight ? cur[i] : 0.0;
         }
         df_sync(grp);
+        const int used = diag ? 5 : nr <= 8 ? 2 : 8;   // entries of acc in use
         const int kbeg = kind == 2 ? e : 0;
         int avail = kbeg;
         double pa[8], pb[8];
@@ -300,12 +310,13 @@ __global__ void __launch_bounds__(DF_THREADS, 1) k_chol_df(const DfArgs a) {
                 df_mma<1>(acc, sm.As, sm.Bs, tx, ty);
             else
                 df_mma<4>(acc, sm.As, sm.Bs, tx, ty);
-            if (!straight && (k & (blk - 1)) == blk - 1) {   // a block done: off the tile, and on with the next one
-                const bool own = based = k + 1 == (c & -blk);
+            if (!straight && k % DF_SUM == DF_SUM - 1) {   // a block done: off the tile, and on with the next one
+                const bool own = based = k + 1 == c / DF_SUM * DF_SUM;
 #pragma unroll
                 for (int i = 0; i < 8; ++i) {
-                    cur[i] -= acc[i];
-                    acc[i] = own ? -cur[i] : 0.0;
+                    if (i >= used) continue;
+                    cur[i] += acc[i];
+                    acc[i] = own ? cur[i] : 0.0;
                 }
             }
             df_sync(grp);
@@ -313,7 +324,7 @@ __global__ void __launch_bounds__(DF_THREADS, 1) k_chol_df(const DfArgs a) {
         if (gone) return;   // uniform over the group
         if (!based) {
 #pragma unroll
-            for (int i = 0; i < 8; ++i) acc[i] -= cur[i];
+            for (int i = 0; i < 8; ++i) acc[i] += cur[i];
         }
         // the tile into shared memory, [col][row]; past the matrix a diagonal block continues as the identity
 #pragma unroll
@@ -468,7 +479,7 @@ cudaError_t chol64_panel(double *A, long long ld, int j0, int jb, int x0, int x1
     if (!factor_diag && W && x1 > x0) return cudaErrorInvalidValue;
     const int nx = std::max(0, x1 - x0);
     DfArgs a{A, ld, j0, jb, A + x0, ld, nx, (jb + DT - 1) / DT, (nx + DT - 1) / DT, factor_diag ? 1 : 0, W, ldw, sync, 0, 0, 0, order == GEO_CHOL_BLOCK64,
-             order != GEO_CHOL_STRAIGHT, st, DF_WAIT_CYCLES};
+             order != GEO_CHOL_NATIVE, st, DF_WAIT_CYCLES};
     const double j = jb, cubes = (factor_diag ? j * j * j / 3.0 : 0.0) + (W ? j * j * j / 3.0 : 0.0);
     return launch_df(a, sms, factor_diag ? GEO_K_POTRF : GEO_K_TRSM, cubes + nx * j * j, s);
 }

@@ -123,14 +123,15 @@ cudaError_t launch_scatter_vec(const double *in, long long stride, const int *pe
 constexpr int GEO_CHOL_SYNC_INTS = 32768;
 constexpr long long GEO_CHOL_MAX_N = 32LL * ((GEO_CHOL_SYNC_INTS - 4) / 3);
 static_assert(8 * GEO_CHOL_MAX_N * GEO_CHOL_MAX_N > 900LL << 30, "the largest matrix fits the words");
-// Order of a tile's sum A_ic - sum_k L_ik L_ck' over the columns k of a panel: STRAIGHT through, one FMA after the
-// other from A_ic on; or (BLOCK64) a separate sum per 64 columns, subtracted as a whole, and straight through
-// within the 64 columns the tile belongs to: the order of a factorisation in 64-wide steps with a rank-64 update
-// after each.  PLAIN and BLOCK64 also round pivots and solves as the plain right-looking algorithm does.  The
-// forms with less than FP64 behind their far tiles use these two: they round the factor's entries to 35 bits or
-// FP32, which turns a last-bit difference here into one of up to 1e-7 in l, so their results stay what that
+// A tile's sum A_ic - sum_k L_ik L_ck' over the columns k of a panel goes in sums per 64 columns, each subtracted as a
+// whole, and straight through, one FMA after the other, within the 64 columns the tile belongs to: the order of a
+// factorisation in 64-wide steps with a rank-64 update after each.  NATIVE: with a column chain, which takes the
+// diagonal tiles' last 32 columns as a sum of their own, and with pivots and solves of the least latency.  BLOCK64 keeps
+// that order to the last bit and rounds pivots and solves as the plain right-looking algorithm does; PLAIN only the
+// latter.  The forms with less than FP64 behind their far tiles use these two: they round the factor's entries to 35
+// bits or FP32, which turns a last-bit difference here into one of up to 1e-7 in l, so their results stay what that
 // order gives.
-constexpr int GEO_CHOL_STRAIGHT = 0, GEO_CHOL_BLOCK64 = 1, GEO_CHOL_PLAIN = 2;
+constexpr int GEO_CHOL_NATIVE = 0, GEO_CHOL_BLOCK64 = 1, GEO_CHOL_PLAIN = 2;
 // In-place lower Cholesky of the leading N x N block of A; rows N..nrows-1
 // are extra right-hand-side rows carried through the factorisation (row N
 // receives (L^-1 z)' when it holds z').
@@ -139,7 +140,7 @@ cudaError_t chol64_factor(double *A, long long ld, int N, int nrows, DevStatus *
 // (its strictly upper part must hold zeros); sms: at most that many SMs (0 = all).
 cudaError_t chol64_panel(double *A, long long ld, int j0, int jb, int x0, int x1, DevStatus *st, int *sync,
                          cudaStream_t s, bool factor_diag = true, double *W = nullptr, long long ldw = 0, int sms = 0,
-                         int order = GEO_CHOL_STRAIGHT);
+                         int order = GEO_CHOL_NATIVE);
 // X <- X L^-T (X: R x N column-major, ldx; L lower).
 cudaError_t chol64_solve_rows(double *X, long long ldx, int R, double *L, long long ldl, int N, DevStatus *st, int *sync,
                               cudaStream_t s);

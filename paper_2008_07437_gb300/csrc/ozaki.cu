@@ -801,7 +801,7 @@ cudaError_t chol_oz_factor(double *A, long long ld, int N, int nrows, int nb, in
     // with FP64-class slices a diagonal tile is one native launch; with fewer its own rank-64 updates
     // are emulated like every other update (their rounding is part of that form's result)
     const bool fused = S >= 7;
-    const int order = fused ? GEO_CHOL_STRAIGHT : GEO_CHOL_BLOCK64;
+    const int order = fused ? GEO_CHOL_NATIVE : GEO_CHOL_BLOCK64;
     int prio_lo = 0, prio_hi = 0;
     cudaDeviceGetStreamPriorityRange(&prio_lo, &prio_hi);
     cudaStream_t s2 = nullptr;
