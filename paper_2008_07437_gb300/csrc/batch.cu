@@ -110,6 +110,7 @@ __global__ void __launch_bounds__(DF_THREADS, 1) k_b_persistent(BatchDesc *d, co
             const int2 u = t < nunits ? units[t] : make_int2(-1, 0);
             sm.word[0] = u.x;
             sm.word[1] = u.y;
+            sm.word[3] = u.x >= 0 && df_ld_acquire(&d[u.x].st.info);
         }
         df_sync(grp);
         const int p = sm.word[0];
@@ -148,9 +149,18 @@ __global__ void __launch_bounds__(DF_THREADS, 1) k_b_persistent(BatchDesc *d, co
             df_sync(grp);
             continue;
         }
+        int *prow = &prog[i], *pcol = &prog[c];
+        if (sm.word[3]) {   // a pivot of this problem has failed: its units only pass their turn on, in order
+            if (tid == 0) {
+                sm.word[2] = df_wait(prow, prow, c, sync, &sync[2]);
+                if (sm.word[2] >= 0) df_st_release(prow, c + 1);
+            }
+            df_sync(grp);
+            if (sm.word[2] < 0) return;
+            continue;
+        }
         const bool diag = i == c, obs = i == T;
         const int c0 = DT * c, cb = min(DT, N - c0), r0 = obs ? N : DT * i, nr = obs ? 1 : min(DT, N - r0);
-        int *prow = &prog[i], *pcol = &prog[c];
         // the tile as it starts
         if (obs) {
 #pragma unroll
@@ -218,7 +228,7 @@ __global__ void __launch_bounds__(DF_THREADS, 1) k_b_persistent(BatchDesc *d, co
         df_sync(grp);
         if (diag) {
             const int bad = df_potrf32(sm.Bs, reinterpret_cast<double (*)[4][DT]>(sm.Ls), sm.dinv, grp, tid);
-            // the first failing row stays; the rest of the problem runs on what it finds, nothing reads it
+            // the first failing row stays; units that are under way go on with what they find, nothing reads it
             if (bad < cb && tid == 0) atomicCAS(&q.st.info, 0, c0 + bad + 1);
             df_sync(grp);
         } else {
