@@ -447,7 +447,8 @@ int geo_server_destroy(geo_server *server);
  * candidate FP32 band, and keeps the fastest.  Each candidate gets one
  * warm-up and `samples` timed evaluations (CUDA events on `stream`; 0 = 3);
  * its time is their median.  Candidates that are not valid for the form are
- * skipped.  The choice is cached for the whole process, per device, form
+ * skipped.  Native FP64 runs the same launches whatever nb: there the first
+ * valid candidate is timed and kept.  The choice is cached for the whole process, per device, form
  * (FP64, FP64 with tensor-core updates, mixed, TLR) and order bucket (powers
  * of two of N): geo_loglik with opts->nb = 0 on any context of that device
  * takes the tuned nb and, in the mixed form, the tuned band (defaults when

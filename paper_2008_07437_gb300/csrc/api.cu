@@ -1530,7 +1530,9 @@ int geo_autotune(geo_ctx *ctx, const double *locs_dev, int n, const double *z_de
     CK(cudaEventCreate(&e1));
     int bnb = -1, bband = -1;
     double bms = 1e300;
-    for (int c = 0; c < n_nb; ++c) {
+    // native FP64 factors without tiles of nb: the first valid candidate is as good as any
+    const bool native = form_of(o) == GEO_PREC_FP64;
+    for (int c = 0; c < n_nb && !(native && bnb >= 0); ++c) {
         for (int b = 0; b < (tune_band ? n_band : 1); ++b) {
             o.nb = nb_cand[c];
             if (tune_band) o.band = band_cand[b];
