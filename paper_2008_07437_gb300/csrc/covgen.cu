@@ -83,21 +83,33 @@ __global__ void __launch_bounds__(TL *TR) k_covgen_sym_fine(const CovParams cp, 
     }
 }
 
-// Full rectangle: rows p*n1 (locations l of set 1), cols p*n2 (set 2); AoS inputs.
-template <int P>
+// Full rectangle: rows p*n1 (locations l of set 1), cols p*n2 (set 2); AoS inputs.  Without the fine tables one pair a
+// thread: an evaluation is a long chain then, and there are too few pairs to hide four after one another (order 3.5,
+// 100 x 100: 917 us so, 293 with one).
+template <int P, bool FINE>
 __global__ void __launch_bounds__(TL *TR) k_covgen_rect(const CovParams cp, const double *__restrict__ l1, int n1,
                                                         const double *__restrict__ l2, int n2, double *out,
                                                         long long ld) {
+    constexpr int RP = FINE ? RPT : 1;
     const int l = blockIdx.y * TL + (threadIdx.x % TL);
     if (l >= n1) return;
     const double x = l1[2 * l], y = l1[2 * l + 1];
 #pragma unroll
-    for (int q = 0; q < RPT; ++q) {
-        const int r = (blockIdx.x * RPT + q) * TR + threadIdx.x / TL;
+    for (int q = 0; q < RP; ++q) {
+        const int r = (blockIdx.x * RP + q) * TR + threadIdx.x / TL;
         if (r >= n2) return;
-        const double dx = x - l2[2 * r], dy = y - l2[2 * r + 1];
+        const double dx = x - l2[2 * r], dy = y - l2[2 * r + 1], d2 = fma(dx, dx, dy * dy);
         double v[P * P];
-        matern_pair<P>(fma(dx, dx, dy * dy), cp, v);
+        if constexpr (FINE) {
+            matern_pair<P>(d2, cp, v);
+        } else {
+            double w[GEO_PMAX_DEV * GEO_PMAX_DEV];
+            cov_block(cp, sqrt(d2), w);
+#pragma unroll
+            for (int i = 0; i < P; ++i)
+#pragma unroll
+                for (int j = 0; j < P; ++j) v[i * P + j] = w[i * GEO_PMAX_DEV + j];
+        }
 #pragma unroll
         for (int j = 0; j < P; ++j) {
             double *col = out + (long long)(P * r + j) * ld + (long long)P * l;
@@ -230,9 +242,15 @@ cudaError_t launch_covgen_sym(const CovParams &cp, const double *lx, const doubl
 cudaError_t launch_covgen_rect(const CovParams &cp, const double *l1, int n1, const double *l2, int n2,
                                double *out, long long ld, cudaStream_t s) {
     if (n1 <= 0 || n2 <= 0) return cudaSuccess;
-    dim3 grid((n2 + TR * RPT - 1) / (TR * RPT), (n1 + TL - 1) / TL);
+    const int per = cp.fine ? TR * RPT : TR;
+    dim3 grid((n2 + per - 1) / per, (n1 + TL - 1) / TL);
     KScope ks(GEO_K_COVGEN, s, 0.0, 8.0 * cp.p * (double)n1 * cp.p * (double)n2);
-    cov_by_p(cp.p, [&](auto P) { k_covgen_rect<P.value><<<grid, TL * TR, 0, s>>>(cp, l1, n1, l2, n2, out, ld); });
+    cov_by_p(cp.p, [&](auto P) {
+        if (cp.fine)
+            k_covgen_rect<P.value, true><<<grid, TL * TR, 0, s>>>(cp, l1, n1, l2, n2, out, ld);
+        else
+            k_covgen_rect<P.value, false><<<grid, TL * TR, 0, s>>>(cp, l1, n1, l2, n2, out, ld);
+    });
     return cudaGetLastError();
 }
 
