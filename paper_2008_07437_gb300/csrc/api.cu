@@ -370,6 +370,9 @@ int theta_to_params(const geo_theta *th, CovParams *cp, std::string *err) {
             cp->m[j * p + i].toff = c.toff;
         }
     cp->tab = cp->fine = nullptr;
+    cp->far = 1;
+    for (int q = 0; q < p * p; ++q)
+        if (cp->m[q].nu > 6.0) cp->far = 0;
     int f = 0;   // fine tables, one per i <= j
     for (int i = 0; i < p; ++i)
         for (int j = i; j < p; ++j) cp->m[i * p + j].foff = cp->m[j * p + i].foff = (f++) * GEO_FINE_PER_PAIR;

@@ -26,13 +26,13 @@ __constant__ double c_cheb_pow[GEO_FINE_NODES][GEO_FINE_NODES] = {
     {-1, 0, 50, 0, -400, 0, 1120, 0, -1280, 0, 512},
 };
 
-// Tables of a theta, one block of 128 threads of those of a pair i <= j.  by < GEO_FINE_N / 8: eight intervals of its fine table,
-// sixteen threads to each, eleven of them at its Chebyshev nodes.  The transform works on differences to the
+// Tables of a theta, one block of 128 threads of those of a pair i <= j.  by < FINE_BLOCKS: eight intervals of its fine
+// table, sixteen threads to each, eleven of them at its Chebyshev nodes.  The transform works on differences to the
 // middle node (they are small, so its rounding is too), and the Chebyshev coefficients, which fall by a factor
 // of 60 or more each, go over to powers of t.  Beyond: four intervals of its K_nu table (cheb_f's, for distances
 // outside the fine one), 32 threads to each, and the reciprocals.  Bound by the latency of one evaluation:
 // 90 steps of four FP64 operations.
-constexpr int FINE_BLOCKS = GEO_FINE_N / 8, COARSE_BLOCKS = GEO_CHEB_NI / 4;
+constexpr int FINE_BLOCKS = GEO_FINE_ALL / 8, COARSE_BLOCKS = GEO_CHEB_NI / 4;
 
 __device__ __forceinline__ void fine_build_block(const CovParams &cp, double *tab, double *fine, int pair, int by) {
     __shared__ double val[8][16], cf[8][16];
@@ -73,7 +73,10 @@ __device__ __forceinline__ void fine_build_block(const CovParams &cp, double *ta
     };
     double mid, half;
     matern_fine_bounds(idx, &mid, &half);
-    if (k < n) val[w][k] = matern_fine_node(fma(half, cos22(2 * k + 1), mid), c, nt);
+    if (k < n) {
+        const double at = fma(half, cos22(2 * k + 1), mid);
+        val[w][k] = idx >= GEO_FINE_N && idx < GEO_FINE_N + GEO_FINE_FAR ? matern_far_node(at, c, nt) : matern_fine_node(at, c, nt);
+    }
     __syncthreads();
     const double v0 = val[w][n / 2];   // t = 0
     double s = 0.0;

@@ -69,14 +69,21 @@
 
 // Fine table of one C_ij as a function of u = (h / a)^2 (see matern_fine):
 // 32 intervals per octave of u from 2^-14 on, 64 per octave from 2^10 to
-// 2^12; an entry is 7 doubles, 4 floats and their scale in 10 doubles.
+// 2^12; an entry is 7 doubles, 4 floats and their scale in 10 doubles.  Then
+// the far part, e^x C_ij as a function of x = h / a from 2^6 to 2^10, and the
+// near part, C_ij of u from 2^-30 to 2^-14, both 8 intervals per octave.
 #define GEO_FINE_E0 (-14)
 #define GEO_FINE_E1 10
 #define GEO_FINE_E2 12
 #define GEO_FINE_LOW ((GEO_FINE_E1 - GEO_FINE_E0) * 32)
 #define GEO_FINE_N (GEO_FINE_LOW + (GEO_FINE_E2 - GEO_FINE_E1) * 64)
+#define GEO_FINE_X1 10
+#define GEO_FINE_EN (-30)
+#define GEO_FINE_FAR ((GEO_FINE_X1 - GEO_FINE_E2 / 2) * 8)
+#define GEO_FINE_NEAR ((GEO_FINE_E0 - GEO_FINE_EN) * 8)
+#define GEO_FINE_ALL (GEO_FINE_N + GEO_FINE_FAR + GEO_FINE_NEAR)
 #define GEO_FINE_STRIDE 10
-#define GEO_FINE_PER_PAIR (GEO_FINE_N * GEO_FINE_STRIDE)
+#define GEO_FINE_PER_PAIR (GEO_FINE_ALL * GEO_FINE_STRIDE)
 #define GEO_FINE_NODES 11
 
 // Per (i, j) constants of Eq. 2 for one theta, computed on the host.
@@ -98,6 +105,7 @@ struct MaternConst {
 
 struct CovParams {
     int p;
+    int far;                                          // the fine tables' far part holds for these orders (all <= 6)
     double inv_a;                                     // 1 / a
     const double *tab;                                // device tables (k_cheb_build), or null
     const double *fine;                               // device fine tables (k_fine_build), or null
@@ -348,8 +356,21 @@ GEO_DEV void matern_block(double x, const CovParams &cp, double *v) {
 // suffices to about 2^-53 of its value up to u = 2^12 (h = 64 a), and the
 // terms from t^7 on are below 2^-26 of it, so that they are summed in FP32 to
 // no less: seven FP64 FMAs per order and six operations per pair for u and t.
-// u comes without the root, the interval and t from u's bits.  Outside the
-// table (h < a / 128, h >= 64 a) the evaluation above is used.
+// u comes without the root, the interval and t from u's bits.
+//
+// Further out C falls faster than its intervals could follow, but e^x C does
+// not: there (64 <= x < 1024) it is tabulated as a function of x = sqrt(u), an
+// eighth of an octave to an interval, seventeen half-widths from the
+// singularity at 0 (the terms fall like 34^-k: below 2^-53 after ten, 2^-34
+// from the seventh on), and e^-x put back; up to order 6, for x^(nu - 1/2) with
+// more has larger seventh terms than FP32 can hold.  Likewise close in (2^-30 <= u <
+// 2^-14), as C itself, where only that singularity matters.  A warp with pairs
+// on both sides of a bound pays for both, so the outer parts have to be cheap:
+// with the evaluation above in their place, domains of 100 ranges and more, or
+// of a hundredth of one, were up to 11 % slower than without any fine table
+// (9 million pairs, order 1/2, a = 0.005: 1.61 ms, 1.43 without; now 0.89, and
+// 0.31 where all pairs lie in the middle part).  Closer than 2^-15 a, and for
+// higher orders from 64 to 1,024 a, it is used still.
 
 // Interval of u and the position in it, t in [-1, 1), also in FP32; false outside the table (and for u = 0, NaN).
 GEO_DEV bool matern_fine_pos(double u, int *idx, double *t, float *tf) {
@@ -385,6 +406,32 @@ GEO_DEV double matern_fine(const double *e, double t, float tf) {
     return fma(v, t, a01.x);
 }
 
+// The same for the outer parts; *scale is what the value is to be multiplied by.
+GEO_DEV bool matern_outer_pos(double u, bool far, int *idx, double *t, float *tf, double *scale) {
+    constexpr unsigned bn = 1023 + GEO_FINE_EN, b0 = 1023 + GEO_FINE_E0;
+    constexpr double x2 = 1 << GEO_FINE_E2, x3 = 1 << 2 * GEO_FINE_X1;
+    unsigned hi = (unsigned)__double2hiint(u), lo;
+    int first;
+    *scale = 1.0;
+    if (hi - (bn << 20) < ((b0 - bn) << 20)) {
+        lo = (unsigned)__double2loint(u);
+        first = GEO_FINE_N + GEO_FINE_FAR - (int)(bn << 3);
+    } else if (u >= (far ? x2 : x3)) {
+        const double x = sqrt(fmin(u, x3));   // from 1,024 ranges on C is below 2^-1074 of C(0): the factor is 0
+        *scale = exp(-x);
+        hi = min((unsigned)__double2hiint(x), ((1023u + GEO_FINE_X1) << 20) - 1);
+        lo = (unsigned)__double2loint(x);
+        first = GEO_FINE_N - (int)((1023 + GEO_FINE_E2 / 2) << 3);
+    } else {
+        return false;
+    }
+    *idx = (int)(hi >> 17) + first;
+    const unsigned mhi = __funnelshift_l(lo, hi, 3) & 0xFFFFFu, mlo = lo << 3;
+    *t = __hiloint2double((int)(0x40000000u | mhi), (int)mlo) - 3.0;
+    *tf = __uint_as_float(0x40000000u | (mhi << 3) | (mlo >> 29)) - 3.0f;
+    return true;
+}
+
 // The block at squared distance d2 by the evaluation above (rare: out of line).
 static __device__ __noinline__ void matern_block_far(double d2, const CovParams &cp, double *v) {
     matern_block(sqrt(d2) * cp.inv_a, cp, v);
@@ -394,15 +441,27 @@ static __device__ __noinline__ void matern_block_far(double d2, const CovParams 
 template <int P>
 GEO_DEV void matern_pair(double d2, const CovParams &cp, double (&v)[P * P]) {
     int idx;
-    double t;
+    double t, scale;
     float tf;
-    if (cp.fine && matern_fine_pos(d2 * cp.inv_a2, &idx, &t, &tf)) {
-        const double *e = cp.fine + (long long)idx * GEO_FINE_STRIDE;
+    if (cp.fine) {
+        const double u = d2 * cp.inv_a2;
+        if (matern_fine_pos(u, &idx, &t, &tf)) {
+            const double *e = cp.fine + (long long)idx * GEO_FINE_STRIDE;
 #pragma unroll
-        for (int i = 0; i < P; ++i)
+            for (int i = 0; i < P; ++i)
 #pragma unroll
-            for (int j = i; j < P; ++j) v[i * P + j] = v[j * P + i] = matern_fine(e + cp.m[i * P + j].foff, t, tf);
-        return;
+                for (int j = i; j < P; ++j) v[i * P + j] = v[j * P + i] = matern_fine(e + cp.m[i * P + j].foff, t, tf);
+            return;
+        }
+        if (matern_outer_pos(u, cp.far, &idx, &t, &tf, &scale)) {
+            const double *e = cp.fine + (long long)idx * GEO_FINE_STRIDE;
+#pragma unroll
+            for (int i = 0; i < P; ++i)
+#pragma unroll
+                for (int j = i; j < P; ++j)
+                    v[i * P + j] = v[j * P + i] = scale * matern_fine(e + cp.m[i * P + j].foff, t, tf);
+            return;
+        }
     }
     double w[GEO_PMAX_DEV * GEO_PMAX_DEV];
     matern_block_far(d2, cp, w);
@@ -416,10 +475,13 @@ GEO_DEV void matern_pair(double d2, const CovParams &cp, double (&v)[P * P]) {
 GEO_DEV double matern_entry(double d2, const CovParams &cp, int i, int j) {
     const MaternConst &c = cp.m[i * cp.p + j];
     int idx;
-    double t;
+    double t, scale;
     float tf;
-    if (cp.fine && matern_fine_pos(d2 * cp.inv_a2, &idx, &t, &tf))
-        return matern_fine(cp.fine + c.foff + (long long)idx * GEO_FINE_STRIDE, t, tf);
+    if (cp.fine) {
+        const double u = d2 * cp.inv_a2, *e = cp.fine + c.foff;
+        if (matern_fine_pos(u, &idx, &t, &tf)) return matern_fine(e + (long long)idx * GEO_FINE_STRIDE, t, tf);
+        if (matern_outer_pos(u, cp.far, &idx, &t, &tf, &scale)) return scale * matern_fine(e + (long long)idx * GEO_FINE_STRIDE, t, tf);
+    }
     return matern_cov(sqrt(d2) * cp.inv_a, c, cp.tab);
 }
 
@@ -519,10 +581,28 @@ GEO_DEV double matern_fine_node(double u, const MaternConst &c, const NodeTabs &
     return c.pre * (scaled ? v * emx : v);
 }
 
-// Middle and half width of an interval.
+// e^x C_ij at x > 2, the far part.
+GEO_DEV double matern_far_node(double x, const MaternConst &c, const NodeTabs &n) {
+    switch (c.kind) {
+        case 1: return c.c0;
+        case 2: return c.c0 * (1.0 + x);
+        case 3: return c.c0 * (1.0 + x + x * x * (1.0 / 3.0));
+        default: break;
+    }
+    bool scaled;
+    return c.pre * xnu_besselk_node(x, c, n, &scaled);
+}
+
+// Middle and half width of an interval: of x in the far part, else of u.
 GEO_DEV void matern_fine_bounds(int idx, double *mid, double *half) {
-    const int up = idx >= GEO_FINE_LOW, k = up ? idx - GEO_FINE_LOW : idx, per = up ? 64 : 32;
-    const double lo = ldexp(1.0, (up ? GEO_FINE_E1 : GEO_FINE_E0) + k / per), h = lo / (2 * per);
+    int k = idx, per = 32, e = GEO_FINE_E0;
+    if (idx >= GEO_FINE_N + GEO_FINE_FAR)
+        k -= GEO_FINE_N + GEO_FINE_FAR, per = 8, e = GEO_FINE_EN;
+    else if (idx >= GEO_FINE_N)
+        k -= GEO_FINE_N, per = 8, e = GEO_FINE_E2 / 2;
+    else if (idx >= GEO_FINE_LOW)
+        k -= GEO_FINE_LOW, per = 64, e = GEO_FINE_E1;
+    const double lo = ldexp(1.0, e + k / per), h = lo / (2 * per);
     *half = h;
     *mid = lo + (2 * (k % per) + 1) * h;
 }
