@@ -23,6 +23,9 @@
 // ---------------------------------------------------------------------------
 // Context, factor
 // ---------------------------------------------------------------------------
+// Tables of any theta: made with the context, so that geo_covgen allocates nothing and can be captured in a graph.
+constexpr size_t GEO_CTAB_DOUBLES = GEO_TAB_DOUBLES + GEO_PMAX * (GEO_PMAX + 1) / 2 * (size_t)GEO_FINE_PER_PAIR;
+
 struct geo_ctx {
     int device = 0;
     size_t budget = 0;      // 0 = no cap
@@ -60,9 +63,8 @@ struct geo_ctx {
     std::vector<unsigned char> bunits;  // cached ticket table (8 bytes per unit)
     cudaStream_t cap_stream = nullptr;   // private stream for graph capture (the legacy stream cannot capture)
     std::vector<geo_factor *> factors;
-    // K_nu tables of the theta of the last geo_covgen call
+    // tables of the theta of the last geo_covgen call, K_nu and fine ones (GEO_CTAB_DOUBLES)
     double *ctab = nullptr;
-    size_t ctab_doubles = 0;
     Profiler prof;
 };
 
@@ -447,6 +449,7 @@ int geo_create(geo_ctx **out, int device, size_t hbm_budget_bytes) {
         cudaMalloc(&ctx->res, sizeof(DevResults)) != cudaSuccess ||
         cudaMalloc(&ctx->sync, 4 * sizeof(int)) != cudaSuccess ||
         cudaMalloc(&ctx->csync, GEO_CHOL_SYNC_INTS * sizeof(int)) != cudaSuccess ||
+        cudaMalloc(&ctx->ctab, GEO_CTAB_DOUBLES * sizeof(double)) != cudaSuccess ||
         cudaMallocHost(&ctx->h_st, sizeof(DevStatus)) != cudaSuccess ||
         cudaMallocHost(&ctx->h_res, sizeof(DevResults)) != cudaSuccess ||
         cudaMalloc(&ctx->prof.d_tc_flops, sizeof(unsigned long long)) != cudaSuccess ||
@@ -474,7 +477,6 @@ int geo_destroy(geo_ctx *ctx) {
     if (ctx->rws) dev_free(ctx, ctx->rws, ctx->rws_bytes);
     if (ctx->tws) dev_free(ctx, ctx->tws, ctx->tws_bytes);
     if (ctx->tarena) cudaFreeHost(ctx->tarena);
-    if (ctx->ctab) dev_free(ctx, ctx->ctab, sizeof(double) * ctx->ctab_doubles);
     for (auto &g : ctx->graphs) cudaGraphExecDestroy(g.second.first);
     if (ctx->cap_stream) cudaStreamDestroy(ctx->cap_stream);
     if (ctx->bws) dev_free(ctx, ctx->bws, ctx->bws_bytes);
@@ -486,6 +488,7 @@ int geo_destroy(geo_ctx *ctx) {
     if (ctx->res) cudaFree(ctx->res);
     if (ctx->sync) cudaFree(ctx->sync);
     if (ctx->csync) cudaFree(ctx->csync);
+    if (ctx->ctab) cudaFree(ctx->ctab);
     if (ctx->h_st) cudaFreeHost(ctx->h_st);
     if (ctx->h_res) cudaFreeHost(ctx->h_res);
     delete ctx;
@@ -514,19 +517,6 @@ int geo_covgen(geo_ctx *ctx, const double *locs1_dev, int n1, const double *locs
     bool closed = true;
     for (int q = 0; q < cp.p * cp.p; ++q) closed = closed && cp.m[q].kind != 0;
     const size_t fine = cov_fine_doubles(cp.p, (closed ? 0.2 : 1.0) * n1 * n2);
-    const size_t need = (cov_needs_tables(cp) || fine) ? GEO_TAB_DOUBLES + fine : 0;
-    if (ctx->ctab_doubles < need) {
-        if (ctx->ctab) {
-            CK(cudaStreamSynchronize(s));
-            dev_free(ctx, ctx->ctab, sizeof(double) * ctx->ctab_doubles);
-            ctx->ctab = nullptr;
-            ctx->ctab_doubles = 0;
-        }
-        void *pt;
-        if ((rc = dev_alloc(ctx, &pt, sizeof(double) * need))) return rc;
-        ctx->ctab = (double *)pt;
-        ctx->ctab_doubles = need;
-    }
     CK(fine ? launch_fine_build(cp, ctx->ctab, ctx->ctab + GEO_TAB_DOUBLES, s) : launch_cheb_build(cp, ctx->ctab, s));
     CK(launch_covgen_rect(cp, locs1_dev, n1, locs2_dev ? locs2_dev : locs1_dev, n2, out_dev, ld, s));
     return GEO_OK;
