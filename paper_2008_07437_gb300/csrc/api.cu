@@ -63,6 +63,7 @@ struct geo_ctx {
     std::vector<unsigned char> bunits;  // cached ticket table (8 bytes per unit)
     cudaStream_t cap_stream = nullptr;   // private stream for graph capture (the legacy stream cannot capture)
     std::vector<geo_factor *> factors;
+    std::vector<geo_factor *> building;  // factors of the running call that hold fine tables, not kept yet
     // tables of the theta of the last geo_covgen call, K_nu and fine ones (GEO_CTAB_DOUBLES)
     double *ctab = nullptr;
     Profiler prof;
@@ -76,6 +77,8 @@ struct geo_factor {
     size_t A_bytes = 0;
     double *lx = nullptr, *ly = nullptr;   // locations in internal order (SoA), then the tables of theta
     size_t loc_doubles = 0;                // doubles of that buffer
+    double *fine = nullptr;                // the fine ones in it (may be missing: the K_nu tables do then)
+    size_t loc_base() const { return 2 * (size_t)n + GEO_TAB_DOUBLES; }   // without them
     double *w = nullptr;                   // L^-T y (lazy)
     std::vector<int> perm;                 // internal k -> caller location perm[k]
     CovParams cp;
@@ -84,6 +87,9 @@ struct geo_factor {
     TlrFactor *tlr = nullptr;
     size_t tlr_bytes = 0;
     double *ybuf = nullptr;                // L^-1 Z (TLR form)
+    ~geo_factor() {
+        if (ctx) ctx->building.erase(std::remove(ctx->building.begin(), ctx->building.end(), this), ctx->building.end());
+    }
 };
 
 thread_local Profiler *t_prof = nullptr;
@@ -158,16 +164,25 @@ int cuda_fail(geo_ctx *ctx, cudaError_t e, const char *where) {
         if (_e != cudaSuccess) return cuda_fail(ctx, _e, #call);   \
     } while (0)
 
+void drop_fine(geo_ctx *ctx, geo_factor *f);
+
 int dev_alloc(geo_ctx *ctx, void **ptr, size_t bytes) {
     *ptr = nullptr;
     if (bytes == 0) return GEO_OK;
-    if (ctx->budget && ctx->used + bytes > ctx->budget)
-        return fail(ctx, GEO_ENOMEM, "HBM budget exceeded: need " + std::to_string(bytes) + " bytes, " +
-                                         std::to_string(ctx->budget - ctx->used) + " left");
-    cudaError_t e = cudaMalloc(ptr, bytes);
-    if (e != cudaSuccess) {
+    for (;;) {
+        cudaError_t e = cudaErrorMemoryAllocation;
+        const bool over = ctx->budget && ctx->used + bytes > ctx->budget;
+        if (!over && (e = cudaMalloc(ptr, bytes)) == cudaSuccess) break;
         cudaGetLastError();
         *ptr = nullptr;
+        // the running call's fine tables only save time: they make room first
+        if (!ctx->building.empty()) {
+            drop_fine(ctx, ctx->building.back());
+            continue;
+        }
+        if (over)
+            return fail(ctx, GEO_ENOMEM, "HBM budget exceeded: need " + std::to_string(bytes) + " bytes, " +
+                                             std::to_string(ctx->budget - ctx->used) + " left");
         return fail(ctx, GEO_ENOMEM, std::string("cudaMalloc: ") + cudaGetErrorString(e));
     }
     ctx->used += bytes;
@@ -178,6 +193,38 @@ void dev_free(geo_ctx *ctx, void *ptr, size_t bytes) {
     if (!ptr) return;
     cudaFree(ptr);
     ctx->used -= bytes;
+}
+
+// Give back the fine tables of a factor of the running call: what is before them moves to a buffer of its own, and what
+// is launched from now on uses the K_nu tables.
+void drop_fine(geo_ctx *ctx, geo_factor *f) {
+    ctx->building.erase(std::remove(ctx->building.begin(), ctx->building.end(), f), ctx->building.end());
+    const size_t bytes = sizeof(double) * f->loc_base();
+    void *p = nullptr;
+    cudaDeviceSynchronize();   // launches that read the tables
+    CovParams cp = f->cp;
+    cp.fine = nullptr;
+    double *lx = nullptr;
+    // (the K_nu tables anew: as a call without fine tables makes them, so that its results are the same)
+    if (cudaMalloc(&p, bytes) != cudaSuccess || cudaMemcpy(p, f->lx, bytes, cudaMemcpyDeviceToDevice) != cudaSuccess ||
+        launch_cheb_build(cp, (lx = (double *)p) + 2 * (size_t)f->n, 0) != cudaSuccess || cudaDeviceSynchronize() != cudaSuccess) {
+        cudaGetLastError();
+        cudaFree(p);
+        return;
+    }
+    dev_free(ctx, f->lx, sizeof(double) * f->loc_doubles);
+    ctx->used += bytes;
+    f->loc_doubles = f->loc_base();
+    f->lx = lx;
+    f->ly = lx + f->n;
+    f->fine = nullptr;
+    f->cp = cp;
+}
+
+// The call has ended well and the caller keeps f.
+void keep_factor(geo_ctx *ctx, geo_factor *f) {
+    ctx->building.erase(std::remove(ctx->building.begin(), ctx->building.end(), f), ctx->building.end());
+    ctx->factors.push_back(f);
 }
 
 struct SetDevice {
@@ -574,22 +621,29 @@ static int prepare_matrix(geo_ctx *ctx, const double *locs_dev, int n, const geo
         morton_perm_host(h_locs.data(), n, f->perm.data());
     else
         std::iota(f->perm.begin(), f->perm.end(), 0);
-    // device buffers: locations (SoA) + permutation
+    // device buffers: locations (SoA), the K_nu tables after them, and the permutation
     void *p1, *p2;
-    const size_t tab_at = 2 * (size_t)n, fine_at = tab_at + GEO_TAB_DOUBLES;
-    const size_t fine = cov_fine_doubles(p, 0.5 * n * (n + 1.0));
-    if ((rc = dev_alloc(ctx, &p1, sizeof(double) * (fine_at + fine)))) return rc;
-    f->loc_doubles = fine_at + fine;
+    size_t fine = cov_fine_doubles(p, 0.5 * n * (n + 1.0));
+    const std::string err0 = ctx->err;
+    if ((rc = dev_alloc(ctx, &p1, sizeof(double) * (f->loc_base() + fine))) == GEO_ENOMEM && fine) {
+        fine = 0;   // they only save time
+        ctx->err = err0;
+        rc = dev_alloc(ctx, &p1, sizeof(double) * f->loc_base());
+    }
+    if (rc) return rc;
+    f->loc_doubles = f->loc_base() + fine;
     f->lx = (double *)p1;
     f->ly = f->lx + n;
+    double *tab = f->lx + 2 * (size_t)n;
     // The forms that round the factor's entries to 35 bits or FP32 turn a last-bit difference of Sigma into one
     // of up to 1e-7 in l: they keep the tables and the evaluation their results have always had.
     const bool reduced = o->prec == GEO_PREC_MIXED || (o->prec == GEO_PREC_FP64 && o->fp64_gemm == 1 && oz_slices_of(*o) < 7);
-    // K_nu tables after the locations, then the fine ones
-    if (reduced || !fine) CK(launch_cheb_build(f->cp, f->lx + tab_at, s));
-    CovParams gen = f->cp;   // for Sigma
-    if (fine) CK(launch_fine_build(f->cp, reduced ? nullptr : f->lx + tab_at, f->lx + fine_at, s));
-    if (!reduced) gen = f->cp;
+    if (reduced || !fine) CK(launch_cheb_build(f->cp, tab, s));
+    if (fine) {
+        f->fine = tab + GEO_TAB_DOUBLES;
+        CK(launch_fine_build(f->cp, reduced ? nullptr : tab, f->fine, s));
+        ctx->building.push_back(f);
+    }
     if ((rc = dev_alloc(ctx, &p2, sizeof(int) * n))) return rc;
     int *d_perm = (int *)p2;
     CK(cudaMemcpyAsync(d_perm, f->perm.data(), sizeof(int) * n, cudaMemcpyHostToDevice, s));
@@ -622,6 +676,8 @@ static int prepare_matrix(geo_ctx *ctx, const double *locs_dev, int n, const geo
         f->A = (double *)pa;
         f->A_bytes = bytes;
     }
+    CovParams gen = f->cp;   // for Sigma
+    if (reduced) gen.fine = nullptr;
     CK(cudaMemsetAsync(ctx->st, 0, sizeof(DevStatus), s));
     CK(launch_covgen_sym(gen, f->lx, f->ly, n, f->A, f->ld, s));
     // keep d_perm alive until the stream has used it
@@ -640,9 +696,10 @@ static void release_factor_buffers(geo_ctx *ctx, geo_factor *f, bool keep_matrix
         }
         f->A = nullptr;
     }
+    ctx->building.erase(std::remove(ctx->building.begin(), ctx->building.end(), f), ctx->building.end());
     if (f->lx) dev_free(ctx, f->lx, sizeof(double) * f->loc_doubles);
     if (f->w) dev_free(ctx, f->w, sizeof(double) * f->N);
-    f->lx = f->ly = f->w = nullptr;
+    f->lx = f->ly = f->w = f->fine = nullptr;
     if (f->ybuf) dev_free(ctx, f->ybuf, sizeof(double) * f->N);
     f->ybuf = nullptr;
     if (f->tlr) {
@@ -717,6 +774,8 @@ static int loglik_tlr(geo_ctx *ctx, const double *locs_dev, int n, const double 
     f->ybuf = (double *)py;
     if ((rc = dev_alloc(ctx, &pp, sizeof(int) * n))) return bail(rc);
     int *d_perm = (int *)pp;
+    // the factorisation below allocates too, but holds on to f's buffer: from here on its tables stay
+    ctx->building.erase(std::remove(ctx->building.begin(), ctx->building.end(), f), ctx->building.end());
     cudaError_t e;
     if ((e = cudaMemcpyAsync(d_perm, f->perm.data(), sizeof(int) * n, cudaMemcpyHostToDevice, s)) ||
         (e = launch_gather_vec(z_dev, d_perm, n, p, f->ybuf, 1, s)) ||
@@ -747,7 +806,7 @@ static int loglik_tlr(geo_ctx *ctx, const double *locs_dev, int n, const double 
     f->quad = ctx->h_res->quad;
     if (loglik_host) *loglik_host = f->loglik;
     if (keep) {
-        ctx->factors.push_back(f);
+        keep_factor(ctx, f);
         *keep = f;
     } else {
         release_factor_buffers(ctx, f, false);
@@ -869,7 +928,7 @@ int geo_loglik(geo_ctx *ctx, const double *locs_dev, int n, const double *z_dev,
     f->quad = ctx->h_res->quad;
     if (loglik_host) *loglik_host = f->loglik;
     if (keep) {
-        ctx->factors.push_back(f);
+        keep_factor(ctx, f);
         *keep = f;
     } else {
         release_factor_buffers(ctx, f, true);
@@ -1242,6 +1301,16 @@ int geo_loglik_batch(geo_ctx *ctx, int count, const geo_batch_item *items, doubl
     std::vector<size_t> offs(count);
     size_t total = 0;
     int pmax = 1, Nmax = 0;
+    bool fine = true;   // the fine tables, if there is room for them
+    auto lay_out = [&]() {
+        total = 0;
+        for (int k = 0; k < count; ++k) {
+            const int p = items[k].theta.p, N = p * items[k].n;
+            offs[k] = total;
+            // matrix, then the theta's K_nu and fine tables
+            total += (size_t)round_up((long long)N + 1, 32) * N + GEO_TAB_DOUBLES + (fine ? batch_fine_doubles(p, items[k].n) : 0);
+        }
+    };
     for (int k = 0; k < count; ++k) {
         const geo_batch_item &it = items[k];
         std::string err;
@@ -1249,16 +1318,19 @@ int geo_loglik_batch(geo_ctx *ctx, int count, const geo_batch_item *items, doubl
             return fail(ctx, GEO_EINVAL, "batch item " + std::to_string(k) + ": bad size or pointer");
         int rc = theta_to_params(&it.theta, &cps[k], &err);
         if (rc) return fail(ctx, rc, "batch item " + std::to_string(k) + ": " + err);
-        const int N = it.theta.p * it.n;
-        const long long ld = round_up((long long)N + 1, 32);
-        offs[k] = total;
-        // matrix, then the theta's K_nu and fine tables
-        total += (size_t)ld * N + GEO_TAB_DOUBLES + batch_fine_doubles(it.theta.p, it.n);
         pmax = std::max(pmax, it.theta.p);
-        Nmax = std::max(Nmax, N);
+        Nmax = std::max(Nmax, it.theta.p * it.n);
     }
+    lay_out();
     int rc;
-    if ((rc = ensure_buffer(ctx, &ctx->bws, &ctx->bws_bytes, sizeof(double) * total, s))) return rc;
+    const std::string err0 = ctx->err;
+    if ((rc = ensure_buffer(ctx, &ctx->bws, &ctx->bws_bytes, sizeof(double) * total, s)) == GEO_ENOMEM) {
+        fine = false;
+        ctx->err = err0;
+        lay_out();
+        rc = ensure_buffer(ctx, &ctx->bws, &ctx->bws_bytes, sizeof(double) * total, s);
+    }
+    if (rc) return rc;
     // device buffer: descriptors, sync words, the unit count, the ticket table
     std::vector<int> orders(count);
     for (int k = 0; k < count; ++k) orders[k] = items[k].theta.p * items[k].n;
@@ -1290,7 +1362,7 @@ int geo_loglik_batch(geo_ctx *ctx, int count, const geo_batch_item *items, doubl
         const int N = it.theta.p * it.n;
         const long long ld = round_up((long long)N + 1, 32);
         cps[k].tab = base + offs[k] + (size_t)ld * N;
-        cps[k].fine = batch_fine_doubles(it.theta.p, it.n) ? cps[k].tab + GEO_TAB_DOUBLES : nullptr;
+        cps[k].fine = fine && batch_fine_doubles(it.theta.p, it.n) ? cps[k].tab + GEO_TAB_DOUBLES : nullptr;
         batch_fill_desc(ctx->bdesc_h, k, base + offs[k], ld, N, it.n, it.locs_dev, it.z_dev, cps[k]);
     }
     char *hb = (char *)ctx->bdesc_h, *db = (char *)ctx->bdesc_d;
