@@ -163,7 +163,6 @@ struct OzSlices {
     void *d;                  // BF16 digits, row-major: per row and 16 columns the 16 digits of every slice in turn
     int *e;                   // row exponents, nchunk x rows
     int S, K, Kp, kchunk, nchunk;
-    int Sg;                   // slices with their padding (a multiple of 4)
     long long rows;           // capacity: row stride of the exponent array
     long long valid;          // rows holding data (extent of the tensor maps)
     int *be;                  // per 32-row block exponent maxima: 2 nchunk x bstride (all rows, reference rows)

@@ -44,8 +44,10 @@
 //               ordered covariance) skip levels or vanish entirely.
 //
 // The digits lie interleaved: per operand row and 16 columns (the K of one MMA)
-// the 16 digits of four slices fill one 128-byte line.  A TMA box of 128 such
-// lines brings four slices at once, and a slice is a 32-byte step of the
+// the 16 digits of every slice in turn, 32 bytes a slice.  A TMA box of 128
+// lines of 128 bytes brings four slices at once (the last one of a chunk may
+// reach into the next chunk's, which no MMA reads, so that S need not be a
+// multiple of 4), and a slice is a 32-byte step of the
 // operand descriptor within the 128-byte swizzle, the step that usually
 // advances K.  With the slices apart a chunk of 8 slices took 24 boxes of
 // 32-byte lines a tile, with almost no MMAs 0.73 ms for the product below; now
@@ -293,8 +295,8 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
                             }
                             uint8_t *base = smem + (size_t)s * OZ_SLOT_BYTES;
                             mbar_arrive_expect_tx(&full_bar[s], (uint32_t)OZ_SLOT_BYTES);
-                            tma_load_2d(&mapA, &full_bar[s], base, (kb * NG + gi) * 64, ar);
-                            tma_load_2d(&mapB, &full_bar[s], base + OZ_A_BYTES, (kb * NG + gi) * 64, br);
+                            tma_load_2d(&mapA, &full_bar[s], base, (kb * S + 4 * gi) * 16, ar);
+                            tma_load_2d(&mapB, &full_bar[s], base + OZ_A_BYTES, (kb * S + 4 * gi) * 16, br);
                             if (filled < ST) ++filled;
                             if (++s == ST) s = 0, ph ^= 1;
                         }
@@ -489,7 +491,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
 
 // Digit slices of rows [0, R) of the column-major FP64 panel P (ld), columns
 // [k0, k0 + kc) for the K chunk blockIdx.y (kc = kchunk, the last one
-// shorter): digit t (from 0) of row r, column k at out[(r Kp + k / 16 * 16) Sg + 16 t + k % 16]
+// shorter): digit t (from 0) of row r, column k at out[(r Kp + k / 16 * 16) S + 16 t + k % 16]
 // (BF16, zero for k beyond the panel), the row exponent at exps[chunk * exp_stride + r].
 // Per 32-row block b the largest exponent of its non-zero rows goes to
 // bexps[2 chunk bstride + b], and that of its non-zero rows below ref_rows to
@@ -530,7 +532,7 @@ __device__ __forceinline__ unsigned int oz_digit_pair(unsigned int u0, unsigned 
 }
 
 __global__ void __launch_bounds__(256) k_oz_slice(const double *P, long long ld, int R, int K, int kchunk, int S,
-                                                  __nv_bfloat16 *out, int Sg, int Kp, int *exps,
+                                                  __nv_bfloat16 *out, int Kp, int *exps,
                                                   long long exp_stride, int *bexps, long long bstride, int ref_rows,
                                                   const DevStatus *st) {
     __shared__ unsigned long long tile[32][33];
@@ -600,7 +602,7 @@ __global__ void __launch_bounds__(256) k_oz_slice(const double *P, long long ld,
                 hi[i] = (unsigned int)(y >> 28);
                 lead[i] = (unsigned int)(y >> (7 * (S - 1)));
             }
-            unsigned int *o = reinterpret_cast<unsigned int *>(out + ((long long)(r0 + r) * Kp + (c0 + cq) / 16 * 16) * Sg + cq % 16);
+            unsigned int *o = reinterpret_cast<unsigned int *>(out + ((long long)(r0 + r) * Kp + (c0 + cq) / 16 * 16) * S + cq % 16);
 #pragma unroll
             for (int t = 0; t < 7; ++t)
                 if (t < S - 1) {
@@ -627,13 +629,14 @@ cudaError_t launch_oz_kernel(const CUtensorMap &ma, const CUtensorMap &mb, const
 }
 
 // 2-D tensor map over the digits of a K chunk: (interleaved columns, row), box 64 (four slices of 16 columns:
-// one 128-byte line) x rows_box, swizzled by lines.
+// one 128-byte line; past the chunk's end zeros) x rows_box, swizzled by lines.  Every box starts at a multiple of
+// 16 columns, 32 bytes.
 cudaError_t slice_map(CUtensorMap *map, const OzSlices &sl, int chunk, int rows_box) {
     tc::EncodeTiledFn enc = tc::encode_fn();
     if (!enc) return cudaErrorNotSupported;
-    void *base = (__nv_bfloat16 *)sl.d + (size_t)chunk * sl.kchunk * sl.Sg;   // kchunk is a multiple of 32
-    cuuint64_t dims[2] = {(cuuint64_t)std::min(sl.kchunk, sl.Kp - chunk * sl.kchunk) * sl.Sg, (cuuint64_t)sl.valid};
-    cuuint64_t strides[1] = {(cuuint64_t)sl.Kp * sl.Sg * 2};
+    void *base = (__nv_bfloat16 *)sl.d + (size_t)chunk * sl.kchunk * sl.S;   // kchunk is a multiple of 32
+    cuuint64_t dims[2] = {(cuuint64_t)std::min(sl.kchunk, sl.Kp - chunk * sl.kchunk) * sl.S, (cuuint64_t)sl.valid};
+    cuuint64_t strides[1] = {(cuuint64_t)sl.Kp * sl.S * 2};
     cuuint32_t box[2] = {64, (cuuint32_t)rows_box};
     cuuint32_t es[2] = {1, 1};
     CUresult cr = enc(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, base, dims, strides, box, es,
@@ -649,7 +652,7 @@ int oz_kmax(int S) { return (4096 / S) / OZ_KALIGN * OZ_KALIGN; }
 size_t oz_slices_bytes(long long rows, int K, int S) {
     const long long Kp = (K + OZ_KALIGN - 1) / OZ_KALIGN * OZ_KALIGN;
     const int nchunk = (K + oz_kmax(S) - 1) / oz_kmax(S);
-    return (size_t)((S + 3) / 4 * 4) * (size_t)rows * (size_t)Kp * 2 + sizeof(int) * (size_t)rows * nchunk +
+    return (size_t)S * (size_t)rows * (size_t)Kp * 2 + sizeof(int) * (size_t)rows * nchunk +
            sizeof(int) * 2 * (size_t)((rows + 31) / 32) * nchunk + 768;
 }
 
@@ -662,9 +665,8 @@ OzSlices oz_slices_carve(void *ws, long long rows, int K, int S) {
     o.Kp = (K + OZ_KALIGN - 1) / OZ_KALIGN * OZ_KALIGN;
     o.nchunk = (K + o.kchunk - 1) / o.kchunk;
     o.valid = rows;
-    o.Sg = (S + 3) / 4 * 4;
     o.d = ws;
-    uintptr_t e = (uintptr_t)ws + (size_t)o.Sg * rows * o.Kp * 2;
+    uintptr_t e = (uintptr_t)ws + (size_t)o.S * rows * o.Kp * 2;
     o.e = (int *)((e + 255) & ~(uintptr_t)255);
     o.bstride = (rows + 31) / 32;
     o.be = (int *)(((uintptr_t)(o.e + rows * o.nchunk) + 255) & ~(uintptr_t)255);
@@ -677,7 +679,7 @@ cudaError_t oz_slice(const double *P, long long ld, int R, const OzSlices &o, co
     if (R > o.rows || R > o.valid) return cudaErrorInvalidValue;
     dim3 grid((R + 31) / 32, o.nchunk);
     KScope ks(GEO_K_AUX, s, 0.0, (double)R * o.K * (16.0 + 2.0 * o.S));
-    k_oz_slice<<<grid, 256, 0, s>>>(P, ld, R, o.K, o.kchunk, o.S, (__nv_bfloat16 *)o.d, o.Sg, o.Kp, o.e,
+    k_oz_slice<<<grid, 256, 0, s>>>(P, ld, R, o.K, o.kchunk, o.S, (__nv_bfloat16 *)o.d, o.Kp, o.e,
                                     o.rows, o.be, o.bstride, o.ref_rows < 0 ? R : (int)std::min<long long>(o.ref_rows, R),
                                     st);
     return cudaGetLastError();
