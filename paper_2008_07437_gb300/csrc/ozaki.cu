@@ -136,6 +136,7 @@ struct OzArgs {
     int overwrite;       // 1: C = -A B' (C is not read)
     int a_off, b_off;    // slice row of the region's first row (A) / first column (B)
     int nk;              // K chunks of 16
+    int split;           // CTAs per tile, each of which forms it and updates 1 / split of its columns (1, 2 or 4)
     const int *ea, *eb;  // per-row exponents of the A / B slices
     // level cut: per 32-row block maxima of the row exponents over every row (ba, bb) and over the
     // reference rows (ra, rb) of the A / B slices, nba / nbb blocks; cut = 0 keeps every level
@@ -182,6 +183,12 @@ __device__ __forceinline__ bool oz_tile(const OzArgs &a, int L, int *gr, int *gc
     return !(a.tri && *gr + OZ_BM - 1 < *gc);
 }
 
+// A CTA's first tile and the step to its next one; SPLIT: args.split CTAs to a tile.
+template <bool SPLIT>
+__device__ __forceinline__ unsigned oz_first(const OzArgs &a) { return SPLIT ? blockIdx.x / (unsigned)a.split : blockIdx.x; }
+template <bool SPLIT>
+__device__ __forceinline__ unsigned oz_step(const OzArgs &a) { return SPLIT ? gridDim.x / (unsigned)a.split : gridDim.x; }
+
 // 2^e as a double (0 below the normal range, where the scaled terms are
 // below 2^-1000 and vanish against any entry of C that matters).
 __device__ __forceinline__ double pow2i(int e) {
@@ -190,8 +197,9 @@ __device__ __forceinline__ double pow2i(int e) {
     return __longlong_as_double((long long)(e + 1023) << 52);
 }
 
-// LOW_FIRST: the passes from the last levels up instead of down to them (without the level cut).
-template <int S, bool LOW_FIRST>
+// LOW_FIRST: the passes from the last levels up instead of down to them (without the level cut).  SPLIT: args.split
+// CTAs to a tile (a form of its own: the columns' bounds cost registers that large products need).
+template <int S, bool LOW_FIRST, bool SPLIT>
 __global__ void __launch_bounds__(OZ_THREADS, 1)
     k_oz_update(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapB,
                 const OzArgs args) {
@@ -230,10 +238,10 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
     // computed once here so that no role waits on the exponent loads inside its tile loop
     __shared__ uint8_t lc_tab[OZ_LC_CAP];
     if (args.cut) {
-        const int mine = (int)((ntiles_all(args) - blockIdx.x + gridDim.x - 1) / gridDim.x);
+        const int mine = (int)((ntiles_all(args) - oz_first<SPLIT>(args) + oz_step<SPLIT>(args) - 1) / oz_step<SPLIT>(args));
         for (int i = threadIdx.x; i < OZ_LC_CAP && i < mine; i += OZ_THREADS) {
             int gr, gc, ar, br;
-            const int L = (int)(blockIdx.x + (unsigned)i * gridDim.x);
+            const int L = (int)(oz_first<SPLIT>(args) + (unsigned)i * oz_step<SPLIT>(args));
             lc_tab[i] = oz_tile(args, L, &gr, &gc, &ar, &br) ? (uint8_t)max(0, oz_lcut<S>(args, ar, br, eref))
                                                                  : (uint8_t)0;
         }
@@ -277,7 +285,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
             int s = 0, filled = 0;
             uint32_t ph = 0;
             bool ok = true;
-            for (int L = blockIdx.x, it = 0; L < ntiles && ok; L += gridDim.x, ++it) {
+            for (int L = oz_first<SPLIT>(args), it = 0; L < ntiles && ok; L += oz_step<SPLIT>(args), ++it) {
                 int gr, gc, ar, br;
                 if (!oz_tile(args, L, &gr, &gc, &ar, &br)) continue;
                 const int lc = tile_lc(it, ar, br);
@@ -317,7 +325,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
             uint32_t used = 0, uph = 0;   // per accumulator slot: used before; parity of its last release
             unsigned long long nmma = 0;
             bool ok = true;
-            for (int L = blockIdx.x, it = 0; L < ntiles && ok; L += gridDim.x, ++it) {
+            for (int L = oz_first<SPLIT>(args), it = 0; L < ntiles && ok; L += oz_step<SPLIT>(args), ++it) {
                 int gr, gc, ar, br;
                 if (!oz_tile(args, L, &gr, &gc, &ar, &br)) continue;
                 const int lc = tile_lc(it, ar, br);
@@ -387,7 +395,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
             // every MMA issued so far has completed before TMEM can be freed
             mma_commit(&drain_bar);
             mbar_wait(&drain_bar, 0, tword, 26);
-            if (args.tc_flops) atomicAdd(args.tc_flops, nmma * (unsigned long long)(2 * OZ_BM * OZ_BN * 16));
+            if (args.tc_flops && (!SPLIT || blockIdx.x % args.split == 0)) atomicAdd(args.tc_flops, nmma * (unsigned long long)(2 * OZ_BM * OZ_BN * 16));
         }
         __syncwarp();
     } else {
@@ -400,7 +408,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
         // them while the tile's MMAs still run: a load of C takes about a microsecond, and with four columns in
         // flight these waits were 28 us a pass
         double *cbuf = c_stage + (warp - 2) * OZ_CD * 32 + lane;
-        for (int L = blockIdx.x, it = 0; L < ntiles && ok; L += gridDim.x, ++it) {
+        for (int L = oz_first<SPLIT>(args), it = 0; L < ntiles && ok; L += oz_step<SPLIT>(args), ++it) {
             int gr, gc, ar, br;
             if (!oz_tile(args, L, &gr, &gc, &ar, &br)) continue;
             const int lc = tile_lc(it, ar, br);
@@ -413,6 +421,14 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
             int c_end = c_all;   // this thread's columns, in a triangle up to its row
             if (args.tri) c_end = min(c_end, grow - (gc + h * CPT) + 1);
             if (grow >= args.m_end) c_end = 0;
+            int c_begin = 0;
+            if constexpr (SPLIT) {
+                c_begin = (int)(blockIdx.x % args.split) * (CPT / args.split);
+                c_end = min(c_end, c_begin + CPT / args.split);
+            }
+            // the warp's columns: what lies past them is not converted or stored (a product of few columns or rows
+            // would pay for a whole tile's FP64 operations, 8 us a pass)
+            const int c_warp = __reduce_max_sync(0xffffffffu, max(c_end, 0));
 #pragma unroll
             for (int pi = 0; pi < PASSES; ++pi) {
                 const int ps = LOW_FIRST ? PASSES - 1 - pi : pi;
@@ -423,7 +439,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
                 auto stage = [&](int j0) {
 #pragma unroll
                     for (int jj = 0; jj < OZ_CQ; ++jj, cs += args.ldc)
-                        if (j0 + jj < c_load) cp_async8(&cbuf[(j0 + jj) % OZ_CD * 32], cs);
+                        if ((!SPLIT || j0 + jj >= c_begin) && j0 + jj < c_load) cp_async8(&cbuf[(j0 + jj) % OZ_CD * 32], cs);
                     cp_async_commit();
                 };
 #pragma unroll
@@ -461,6 +477,12 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
                 double *cw = cp;
 #pragma unroll
                 for (int j0 = 0; j0 < CPT; j0 += OZ_CQ) {
+                    if (j0 >= c_warp) break;
+                    if (SPLIT && j0 < c_begin) {   // another CTA's
+                        cw += OZ_CQ * args.ldc;
+                        stage(j0 + OZ_CD);
+                        continue;
+                    }
                     cp_async_wait<OZ_CD / OZ_CQ - 1>();
 #pragma unroll
                     for (int jj = 0; jj < OZ_CQ; ++jj, cw += args.ldc) {
@@ -622,9 +644,10 @@ template <int S, bool LOW_FIRST = false>
 cudaError_t launch_oz_kernel(const CUtensorMap &ma, const CUtensorMap &mb, const OzArgs &a, int grid,
                              cudaStream_t s) {
     static_assert(OZ_SLOTS >= 2 * OzCfg<S>::NG, "shared memory holds fewer than two chunks");
-    cudaError_t e = cudaFuncSetAttribute(k_oz_update<S, LOW_FIRST>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)OZ_SMEM);
+    auto *kernel = a.split > 1 ? k_oz_update<S, LOW_FIRST, true> : k_oz_update<S, LOW_FIRST, false>;
+    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)OZ_SMEM);
     if (e != cudaSuccess) return e;
-    k_oz_update<S, LOW_FIRST><<<grid, OZ_THREADS, OZ_SMEM, s>>>(ma, mb, a);
+    kernel<<<grid, OZ_THREADS, OZ_SMEM, s>>>(ma, mb, a);
     return cudaGetLastError();
 }
 
@@ -712,7 +735,13 @@ cudaError_t oz_update(const OzSlices &A, const OzSlices &B, double *C, long long
     a.tc_flops = t_prof ? t_prof->d_tc_flops : nullptr;
     const long long ntiles = (long long)a.mt * a.nt;
     if (ntiles > (1LL << 30)) return cudaErrorInvalidValue;   // the kernel counts tiles in 32 bits
-    const int grid = (int)std::min<long long>(ntiles, std::max(1, std::min(grid_cap, tc::num_sms())));
+    const int ctas = std::max(1, std::min(grid_cap, tc::num_sms()));
+    // few tiles: the epilogue's FP64 operations, 8 us a pass over a tile, on two or four SMs each (the MMAs are done in
+    // every one of them; C 100 x 1000, K = 32, 5 slices 76 -> 62 us a call, 64
+    // with 64-column tiles)
+    a.split = 1;
+    while (a.split < 4 && ntiles * a.split * 2 <= ctas) a.split *= 2;
+    const int grid = (int)std::min<long long>(ntiles * a.split, ctas);
     // algorithmic work: 2 K flops per output written (lower triangle when tri)
     const double rr = rows, cc = cols;
     const double outs = tri ? std::max(0.0, rr * cc - cc * (cc - 1.0) / 2.0) : rr * cc;
