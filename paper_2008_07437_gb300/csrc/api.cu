@@ -23,7 +23,8 @@
 // ---------------------------------------------------------------------------
 // Context, factor
 // ---------------------------------------------------------------------------
-// Tables of any theta: made with the context, so that geo_covgen allocates nothing and can be captured in a graph.
+// Tables of any theta: allocated by the context's first geo_covgen that needs some and never again, so that a captured
+// one keeps its buffer.
 constexpr size_t GEO_CTAB_DOUBLES = GEO_TAB_DOUBLES + GEO_PMAX * (GEO_PMAX + 1) / 2 * (size_t)GEO_FINE_PER_PAIR;
 
 struct geo_ctx {
@@ -496,7 +497,6 @@ int geo_create(geo_ctx **out, int device, size_t hbm_budget_bytes) {
         cudaMalloc(&ctx->res, sizeof(DevResults)) != cudaSuccess ||
         cudaMalloc(&ctx->sync, 4 * sizeof(int)) != cudaSuccess ||
         cudaMalloc(&ctx->csync, GEO_CHOL_SYNC_INTS * sizeof(int)) != cudaSuccess ||
-        cudaMalloc(&ctx->ctab, GEO_CTAB_DOUBLES * sizeof(double)) != cudaSuccess ||
         cudaMallocHost(&ctx->h_st, sizeof(DevStatus)) != cudaSuccess ||
         cudaMallocHost(&ctx->h_res, sizeof(DevResults)) != cudaSuccess ||
         cudaMalloc(&ctx->prof.d_tc_flops, sizeof(unsigned long long)) != cudaSuccess ||
@@ -564,6 +564,18 @@ int geo_covgen(geo_ctx *ctx, const double *locs1_dev, int n1, const double *locs
     bool closed = true;
     for (int q = 0; q < cp.p * cp.p; ++q) closed = closed && cp.m[q].kind != 0;
     const size_t fine = cov_fine_doubles(cp.p, (closed ? 0.2 : 1.0) * n1 * n2);
+    if (!ctx->ctab && (fine || cov_needs_tables(cp))) {
+        // (in a capture too: nothing of it goes to the stream)
+        cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+        CK(cudaThreadExchangeStreamCaptureMode(&mode));
+        const cudaError_t e = cudaMalloc(&ctx->ctab, GEO_CTAB_DOUBLES * sizeof(double));
+        cudaThreadExchangeStreamCaptureMode(&mode);
+        if (e != cudaSuccess) {
+            cudaGetLastError();
+            ctx->ctab = nullptr;
+            return fail(ctx, GEO_ENOMEM, std::string("cudaMalloc: ") + cudaGetErrorString(e));
+        }
+    }
     CK(fine ? launch_fine_build(cp, ctx->ctab, ctx->ctab + GEO_TAB_DOUBLES, s) : launch_cheb_build(cp, ctx->ctab, s));
     CK(launch_covgen_rect(cp, locs1_dev, n1, locs2_dev ? locs2_dev : locs1_dev, n2, out_dev, ld, s));
     return GEO_OK;
