@@ -563,7 +563,7 @@ int geo_covgen(geo_ctx *ctx, const double *locs1_dev, int n1, const double *locs
     // it takes five times the pairs (one variable of order 1/2: 256 x 256 49 us without, 70 with, 404 x 404 66 and 71)
     bool closed = true;
     for (int q = 0; q < cp.p * cp.p; ++q) closed = closed && cp.m[q].kind != 0;
-    const size_t fine = cov_fine_doubles(cp.p, (closed ? 0.2 : 1.0) * n1 * n2);
+    const size_t fine = cov_fine_doubles(cp, (closed ? 0.2 : 1.0) * n1 * n2);
     if (!ctx->ctab && (fine || cov_needs_tables(cp))) {
         // (in a capture too: nothing of it goes to the stream)
         cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
@@ -635,7 +635,7 @@ static int prepare_matrix(geo_ctx *ctx, const double *locs_dev, int n, const geo
         std::iota(f->perm.begin(), f->perm.end(), 0);
     // device buffers: locations (SoA), the K_nu tables after them, and the permutation
     void *p1, *p2;
-    size_t fine = cov_fine_doubles(p, 0.5 * n * (n + 1.0));
+    size_t fine = cov_fine_doubles(f->cp, 0.5 * n * (n + 1.0));
     const std::string err0 = ctx->err;
     if ((rc = dev_alloc(ctx, &p1, sizeof(double) * (f->loc_base() + fine))) == GEO_ENOMEM && fine) {
         fine = 0;   // they only save time
@@ -1320,7 +1320,7 @@ int geo_loglik_batch(geo_ctx *ctx, int count, const geo_batch_item *items, doubl
             const int p = items[k].theta.p, N = p * items[k].n;
             offs[k] = total;
             // matrix, then the theta's K_nu and fine tables
-            total += (size_t)round_up((long long)N + 1, 32) * N + GEO_TAB_DOUBLES + (fine ? batch_fine_doubles(p, items[k].n) : 0);
+            total += (size_t)round_up((long long)N + 1, 32) * N + GEO_TAB_DOUBLES + (fine ? batch_fine_doubles(cps[k], items[k].n) : 0);
         }
     };
     for (int k = 0; k < count; ++k) {
@@ -1374,7 +1374,7 @@ int geo_loglik_batch(geo_ctx *ctx, int count, const geo_batch_item *items, doubl
         const int N = it.theta.p * it.n;
         const long long ld = round_up((long long)N + 1, 32);
         cps[k].tab = base + offs[k] + (size_t)ld * N;
-        cps[k].fine = fine && batch_fine_doubles(it.theta.p, it.n) ? cps[k].tab + GEO_TAB_DOUBLES : nullptr;
+        cps[k].fine = fine && batch_fine_doubles(cps[k], it.n) ? cps[k].tab + GEO_TAB_DOUBLES : nullptr;
         batch_fill_desc(ctx->bdesc_h, k, base + offs[k], ld, N, it.n, it.locs_dev, it.z_dev, cps[k]);
     }
     char *hb = (char *)ctx->bdesc_h, *db = (char *)ctx->bdesc_d;

@@ -255,7 +255,7 @@ size_t batch_desc_bytes() { return sizeof(BatchDesc); }
 
 // With the GPU full of problems the tables cost their FP64 operations, 3 million a C_ij, against some 55 saved per
 // pair of locations: they pay from about 340 locations on.
-size_t batch_fine_doubles(int p, int n) { return n >= 340 ? cov_fine_doubles(p, 0.5 * n * (n + 1.0)) : 0; }
+size_t batch_fine_doubles(const CovParams &cp, int n) { return n >= 340 ? cov_fine_doubles(cp, 0.5 * n * (n + 1.0)) : 0; }
 
 long long batch_units(const int *N, int count, void *out_v) {
     int2 *out = (int2 *)out_v;

@@ -216,6 +216,13 @@ size_t cov_fine_doubles(int p, double pairs) {
     return pairs >= 32768.0 ? (size_t)p * (p + 1) / 2 * GEO_FINE_PER_PAIR : 0;
 }
 
+size_t cov_fine_doubles(const CovParams &cp, double pairs) {
+    // the tables' floats go down to 2^-800 (64 a out, C is 2^-93 of C(0)): covariances smaller than that go without
+    for (int q = 0; q < cp.p * cp.p; ++q)
+        if (cp.m[q].c0 != 0.0 && fabs(cp.m[q].c0) < 0x1p-700) return 0;
+    return cov_fine_doubles(cp.p, pairs);
+}
+
 cudaError_t launch_fine_build(CovParams &cp, double *tab, double *fine, cudaStream_t s) {
     KScope ks(GEO_K_COVGEN, s);
     // tab == NULL: cp.tab is there already

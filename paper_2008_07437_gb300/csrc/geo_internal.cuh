@@ -74,7 +74,8 @@ bool cov_needs_tables(const CovParams &cp);
 // Doubles of the fine tables (matern.cuh) of p variables, 0 where the number of location pairs does not pay
 // for them; and their construction on stream s together with the K_nu tables (tab, GEO_TAB_DOUBLES; NULL: only
 // the fine ones), with cp pointed at both.
-size_t cov_fine_doubles(int p, double pairs);
+size_t cov_fine_doubles(int p, double pairs);                  // (of any theta)
+size_t cov_fine_doubles(const CovParams &cp, double pairs);
 cudaError_t launch_fine_build(CovParams &cp, double *tab, double *fine, cudaStream_t s);
 // f(integral constant P) for p = 1 .. 4 variables.
 template <typename F>
@@ -362,7 +363,7 @@ size_t batch_desc_bytes();
 void batch_fill_desc(void *hdesc, int k, double *A, long long ld, int N, int n, const double *locs, const double *z,
                      const CovParams &cp);
 // Doubles of fine tables of a problem of n locations (0: it goes without).
-size_t batch_fine_doubles(int p, int n);
+size_t batch_fine_doubles(const CovParams &cp, int n);
 // Ticket table of the persistent launch (8 bytes per unit) for problems of orders N[0..count); returns the unit
 // count (out == NULL: only that).
 long long batch_units(const int *N, int count, void *out);
