@@ -173,7 +173,10 @@ def load_library(path: str = LIB_PATH) -> ctypes.CDLL:
 # ----------------------------------------------------------------------------
 
 def _doubles(values):
-    values = [float(v) for v in values]
+    try:
+        values = [float(v) for v in values]
+    except TypeError:   # rows of a 2-D array
+        values = np.asarray(values, dtype=np.float64).ravel().tolist()
     return (ctypes.c_double * max(1, len(values)))(*values)
 
 
