@@ -114,6 +114,13 @@ __device__ __forceinline__ void df_root(double d, double *l, double *inv) {
     *inv = __hiloint2double(__double2hiint(rec), below ? 1 : __double2loint(rec));
 }
 
+// The factor of a scaled tile, and its diagonal's reciprocals, as the tile's own (each warp its columns).
+__device__ __noinline__ void df_unscale(double (*S)[DLD], double *dinv, double sc, int lane, int w) {
+    const double si = df_inv_scale(sc);
+    for (int q = 0; q < 8; ++q) S[4 * q + w][lane] *= si;
+    if (w == 0) dinv[lane] *= sc;
+}
+
 // Cholesky factor of the 32 x 32 block S[col][row] (lower part) by one group, lane = row, columns w, w + 4, ...
 // in the registers of warp w.  Returns the first column without a positive pivot, or 32.  Panels of four
 // columns: the warps exchange the panel through shared memory (one barrier), then every warp factors it for
@@ -169,10 +176,7 @@ __device__ __forceinline__ int df_potrf32_plain(double (*S)[DLD], double (*buf)[
     }
     if (ext) {
         df_sync(grp);   // every warp has read the columns
-        const double si = df_inv_scale(sc);
-#pragma unroll
-        for (int q = 0; q < 8; ++q) S[4 * q + w][lane] *= si;
-        if (w == 0) dinv[lane] *= sc;
+        df_unscale(S, dinv, sc, lane, w);
     }
     return bad;
 }
@@ -228,8 +232,7 @@ __device__ __forceinline__ int df_potrf32(double (*S)[DLD], double (*buf)[4][DT]
     const unsigned ok = __ballot_sync(0xffffffffu, df_positive(d));
     double l, inv;
     df_root(d, &l, &inv);
-    if (w == 0) dinv[lane] = inv * sc;
-    const double si = df_inv_scale(sc);
+    if (w == 0) dinv[lane] = inv;
 #pragma unroll
     for (int q = 0; q < 8; ++q) {
         const int col = 4 * q + w;
@@ -238,7 +241,8 @@ __device__ __forceinline__ int df_potrf32(double (*S)[DLD], double (*buf)[4][DT]
     }
     df_sync(grp);   // every warp has read the diagonal
 #pragma unroll
-    for (int q = 0; q < 8; ++q) S[4 * q + w][lane] = ext ? v[q] * si : v[q];
+    for (int q = 0; q < 8; ++q) S[4 * q + w][lane] = v[q];
+    if (ext) df_unscale(S, dinv, sc, lane, w);
     return ok == 0xffffffffu ? DT : __ffs(~ok) - 1;
 }
 
