@@ -208,7 +208,8 @@ void drop_fine(geo_ctx *ctx, geo_factor *f) {
     double *lx = nullptr;
     // (the K_nu tables anew: as a call without fine tables makes them, so that its results are the same)
     if (cudaMalloc(&p, bytes) != cudaSuccess || cudaMemcpy(p, f->lx, bytes, cudaMemcpyDeviceToDevice) != cudaSuccess ||
-        launch_cheb_build(cp, (lx = (double *)p) + 2 * (size_t)f->n, 0) != cudaSuccess || cudaDeviceSynchronize() != cudaSuccess) {
+        launch_cheb_build(cp, (lx = (double *)p) + 2 * (size_t)f->n, 0) != cudaSuccess ||
+        cudaDeviceSynchronize() != cudaSuccess) {
         cudaGetLastError();
         cudaFree(p);
         return;
@@ -392,7 +393,8 @@ int theta_to_params(const geo_theta *th, CovParams *cp, std::string *err) {
             MaternConst &c = cp->m[i * p + j];
             const double nui = th->nu[i], nuj = th->nu[j];
             const double nij = 0.5 * (nui + nuj);
-            const long double rho = (long double)B[i][j] * sqrtl((long double)nui) * sqrtl((long double)nuj) / (long double)nij;
+            const long double rho = (long double)B[i][j] * sqrtl((long double)nui) * sqrtl((long double)nuj) /
+                                    (long double)nij;
             const long double c0 = rho * sqrtl((long double)th->sigma2[i]) * sqrtl((long double)th->sigma2[j]);
             c.nu = nij;
             c.c0 = (double)c0;
@@ -1320,7 +1322,8 @@ int geo_loglik_batch(geo_ctx *ctx, int count, const geo_batch_item *items, doubl
             const int p = items[k].theta.p, N = p * items[k].n;
             offs[k] = total;
             // matrix, then the theta's K_nu and fine tables
-            total += (size_t)round_up((long long)N + 1, 32) * N + GEO_TAB_DOUBLES + (fine ? batch_fine_doubles(cps[k], items[k].n) : 0);
+            total += (size_t)round_up((long long)N + 1, 32) * N + GEO_TAB_DOUBLES;
+            if (fine) total += batch_fine_doubles(cps[k], items[k].n);
         }
     };
     for (int k = 0; k < count; ++k) {
@@ -1802,7 +1805,8 @@ size_t loglik_device_bytes(int device, int n, int p, const geo_opts *opts) {
     const size_t N = (size_t)p * n;
     if (o.nb == 0) o.nb = resolve_nb(device, form_of(o), (int)N);
     const size_t nb = (size_t)std::max(o.nb, 64);
-    size_t b = sizeof(double) * (2 * (size_t)n + GEO_TAB_DOUBLES + cov_fine_doubles(p, 0.5 * n * (n + 1.0))) + sizeof(int) * 2 * n + sizeof(double) * N;
+    size_t b = sizeof(double) * (2 * (size_t)n + GEO_TAB_DOUBLES + cov_fine_doubles(p, 0.5 * n * (n + 1.0)));
+    b += sizeof(int) * 2 * n + sizeof(double) * N;
     if (o.prec == GEO_PREC_TLR) {
         const int kmax = std::min(o.tlr_kmax, (int)nb);
         const size_t T = (N + nb - 1) / nb;

@@ -223,7 +223,8 @@ __global__ void __launch_bounds__(DF_THREADS, 1) k_b_persistent(BatchDesc *d, co
             if (!diag)
                 sm.Bs[tx + 16 * (e % 2)][ty + 8 * (e / 2)] = -acc[e];
             else if (e < 5)
-                sm.Bs[dc[e % 5]][dr[e % 5]] = (dr[e % 5] < cb && dc[e % 5] < cb) ? -acc[e] : (dr[e % 5] == dc[e % 5] ? 1.0 : 0.0);
+                sm.Bs[dc[e % 5]][dr[e % 5]] =
+                    (dr[e % 5] < cb && dc[e % 5] < cb) ? -acc[e] : (dr[e % 5] == dc[e % 5] ? 1.0 : 0.0);
         }
         df_sync(grp);
         if (diag) {

@@ -810,7 +810,8 @@ __global__ void __launch_bounds__(JT, 1) k_jacobi_svd_cl(const SvdDesc *__restri
                     int c = 1 + (bb - 2 - p + st) % (bb - 1);
                     const bool act = p < bb / 2 && a < b && c < b && a != c;
                     if (!act) a = c = 0;
-                    pair(col(buf, w, min(a, c)), col(buf, w, max(a, c)), nrm(buf, w) + min(a, c), nrm(buf, w) + max(a, c), act);
+                    pair(col(buf, w, min(a, c)), col(buf, w, max(a, c)), nrm(buf, w) + min(a, c),
+                         nrm(buf, w) + max(a, c), act);
                     __syncthreads();
                 }
             }
@@ -823,7 +824,8 @@ __global__ void __launch_bounds__(JT, 1) k_jacobi_svd_cl(const SvdDesc *__restri
             // the circle method's move: first block 0 stays, the first blocks move up, the second ones down
             const int t0 = rank == 0 ? 0 : min(rank + 1, JC - 1), w0 = rank == JC - 1 ? 1 : 0;
             const int t1 = rank == 0 ? 1 : rank - 1, w1 = rank == 0 ? 0 : 1;
-            double *to0 = cluster.map_shared_rank(col(buf ^ 1, w0, 0), t0), *to1 = cluster.map_shared_rank(col(buf ^ 1, w1, 0), t1);
+            double *to0 = cluster.map_shared_rank(col(buf ^ 1, w0, 0), t0);
+            double *to1 = cluster.map_shared_rank(col(buf ^ 1, w1, 0), t1);
             for (int e = threadIdx.x; e < b * ROWS; e += JT) {
                 to0[e] = col(buf, 0, 0)[e];
                 to1[e] = col(buf, 1, 0)[e];

@@ -382,7 +382,8 @@ __global__ void __launch_bounds__(DF_THREADS, 1) k_chol_df(const DfArgs a) {
                 if (lr < cb && row < nr) a.W[(long long)(DT * e + row) * a.ldw + DT * c + lr] = -sm.Bs[lr][row];
             } else {
                 const int col = lc + 4 * u;
-                if (lr < nr && col < cb && (!diag || lr >= col)) R[(long long)(c0 + col) * rld + r0 + lr] = sm.Bs[col][lr];
+                if (lr < nr && col < cb && (!diag || lr >= col))
+                    R[(long long)(c0 + col) * rld + r0 + lr] = sm.Bs[col][lr];
             }
         }
         df_sync(grp);
@@ -450,7 +451,9 @@ cudaError_t launch_df(const DfArgs &a0, int sms, int cls, double flops, cudaStre
         return e != cudaSuccess ? e : launch_df(rest, sms, cls, 0.0, s);
     }
     const long long words = fixed + E;
-    const long long tickets = !a.factor ? (a.W ? T * (T + 1) / 2 : T * E) : a.W ? T * (T + E + 1) : T * (T + E) - T * (T - 1) / 2;
+    const long long tickets = !a.factor ? (a.W ? T * (T + 1) / 2 : T * E)
+                              : a.W     ? T * (T + E + 1)
+                                        : T * (T + E) - T * (T - 1) / 2;
     if (tickets == 0) return cudaSuccess;
     if (words > GEO_CHOL_SYNC_INTS || tickets > (1LL << 30)) return cudaErrorInvalidValue;
     a.tickets = (int)tickets;
@@ -471,15 +474,16 @@ cudaError_t launch_df(const DfArgs &a0, int sms, int cls, double flops, cudaStre
 
 // Factor the columns [j0, j0 + jb): the diagonal range, and the rows [x0, x1) below it (x0 >= j0 + jb;
 // x0 == x1 = none) solved against it.  factor_diag false: the diagonal range already holds L and only the
-// rows are solved (X <- X L^-T), or, without rows, only W is formed.  W (jb x jb, ldw) != NULL: also W = -L^-1, its strictly upper part must hold
-// zeros.  sms: at most that many CTAs, one per SM (0 = all).  sync: GEO_CHOL_SYNC_INTS device ints of scratch.
+// rows are solved (X <- X L^-T), or, without rows, only W is formed.  W (jb x jb, ldw) != NULL: also
+// W = -L^-1, its strictly upper part must hold zeros.  sms: at most that many CTAs, one per SM (0 = all).
+// sync: GEO_CHOL_SYNC_INTS device ints of scratch.
 cudaError_t chol64_panel(double *A, long long ld, int j0, int jb, int x0, int x1, DevStatus *st, int *sync,
                          cudaStream_t s, bool factor_diag, double *W, long long ldw, int sms, int order) {
     if (jb <= 0) return cudaSuccess;
     if (!factor_diag && W && x1 > x0) return cudaErrorInvalidValue;
     const int nx = std::max(0, x1 - x0);
-    DfArgs a{A, ld, j0, jb, A + x0, ld, nx, (jb + DT - 1) / DT, (nx + DT - 1) / DT, factor_diag ? 1 : 0, W, ldw, sync, 0, 0, 0, order == GEO_CHOL_BLOCK64,
-             order != GEO_CHOL_NATIVE, st, DF_WAIT_CYCLES};
+    DfArgs a{A, ld, j0, jb, A + x0, ld, nx, (jb + DT - 1) / DT, (nx + DT - 1) / DT, factor_diag ? 1 : 0, W, ldw, sync,
+             0, 0, 0, order == GEO_CHOL_BLOCK64, order != GEO_CHOL_NATIVE, st, DF_WAIT_CYCLES};
     const double j = jb, cubes = (factor_diag ? j * j * j / 3.0 : 0.0) + (W ? j * j * j / 3.0 : 0.0);
     return launch_df(a, sms, factor_diag ? GEO_K_POTRF : GEO_K_TRSM, cubes + nx * j * j, s);
 }
@@ -511,7 +515,8 @@ cudaError_t chol64_rhs_update(double *A, long long ld, int rC, int cC, int m, in
 cudaError_t chol64_factor(double *A, long long ld, int N, int nrows, DevStatus *st, int *sync, cudaStream_t s) {
     if (N <= 0) return cudaSuccess;
     const int nx = std::max(0, nrows - N);
-    DfArgs a{A, ld, 0, N, A + N, ld, nx, (N + DT - 1) / DT, (nx + DT - 1) / DT, 1, nullptr, 0, sync, 0, 0, 0, 0, 0, st, DF_WAIT_CYCLES};
+    DfArgs a{A, ld, 0, N, A + N, ld, nx, (N + DT - 1) / DT, (nx + DT - 1) / DT, 1, nullptr, 0, sync,
+             0, 0, 0, 0, 0, st, DF_WAIT_CYCLES};
     const double n = N;
     return launch_df(a, 0, GEO_K_GEMM, n * n * n / 3.0 + nx * n * n, s);
 }
@@ -520,6 +525,7 @@ cudaError_t chol64_factor(double *A, long long ld, int N, int nrows, DevStatus *
 cudaError_t chol64_solve_rows(double *X, long long ldx, int R, double *L, long long ldl, int N, DevStatus *st, int *sync,
                               cudaStream_t s) {
     if (R <= 0 || N <= 0) return cudaSuccess;
-    DfArgs a{L, ldl, 0, N, X, ldx, R, (N + DT - 1) / DT, (R + DT - 1) / DT, 0, nullptr, 0, sync, 0, 0, 0, 0, 0, st, DF_WAIT_CYCLES};
+    DfArgs a{L, ldl, 0, N, X, ldx, R, (N + DT - 1) / DT, (R + DT - 1) / DT, 0, nullptr, 0, sync,
+             0, 0, 0, 0, 0, st, DF_WAIT_CYCLES};
     return launch_df(a, 0, GEO_K_SOLVE, (double)R * N * N, s);
 }

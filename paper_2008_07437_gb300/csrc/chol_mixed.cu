@@ -478,9 +478,8 @@ size_t mixed_workspace_bytes(int N, int nb) { return panel_ws_bytes(N, nb); }
 // next panel's tile column; the diagonal tile of that panel is then factored
 // in FP64 on a second, high-priority stream while the rest of step j's
 // trailing update runs (its persistent tensor-core launch leaves a few SMs
-// free for it); the rows below it are solved after the join.  Every entry receives the same operations in the same order as
-// without the lookahead.
-
+// free for it); the rows below it are solved after the join.  Every entry
+// receives the same operations in the same order as without the lookahead.
 cudaError_t chol_mixed_factor(double *A, long long ld, int N, int nrows, int nb, int band, int lowp, void *ws,
                               size_t ws_bytes, DevStatus *st, int *sync, cudaStream_t s) {
     if (nb % 128 != 0 || nb <= 0) return cudaErrorInvalidValue;

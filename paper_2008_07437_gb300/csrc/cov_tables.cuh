@@ -75,7 +75,8 @@ __device__ __forceinline__ void fine_build_block(const CovParams &cp, double *ta
     matern_fine_bounds(idx, &mid, &half);
     if (k < n) {
         const double at = fma(half, cos22(2 * k + 1), mid);
-        val[w][k] = idx >= GEO_FINE_N && idx < GEO_FINE_N + GEO_FINE_FAR ? matern_far_node(at, c, nt) : matern_fine_node(at, c, nt);
+        const bool far = idx >= GEO_FINE_N && idx < GEO_FINE_N + GEO_FINE_FAR;
+        val[w][k] = far ? matern_far_node(at, c, nt) : matern_fine_node(at, c, nt);
     }
     __syncthreads();
     const double v0 = val[w][n / 2];   // t = 0

@@ -272,7 +272,8 @@ struct QrDesc {             // Householder QR of Y (m x r), in place, thin Q out
     double *Q;
     long long ldq;
     double *tau, *v0;       // r entries each
-    double *Rt;             // with house_qr_in_smem and not NULL: R' (r x r lower, ldr); with Q == NULL Y is then left as it is
+    double *Rt;             // with house_qr_in_smem and not NULL: R' (r x r lower, ldr); with Q == NULL Y is then
+                            // left as it is
     long long ldr;
 };
 struct SvdDesc {            // one-sided Jacobi SVD of M (r x r): M <- M V, sigma = its column norms

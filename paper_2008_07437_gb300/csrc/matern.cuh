@@ -480,7 +480,8 @@ GEO_DEV double matern_entry(double d2, const CovParams &cp, int i, int j) {
     if (cp.fine) {
         const double u = d2 * cp.inv_a2, *e = cp.fine + c.foff;
         if (matern_fine_pos(u, &idx, &t, &tf)) return matern_fine(e + (long long)idx * GEO_FINE_STRIDE, t, tf);
-        if (matern_outer_pos(u, cp.far, &idx, &t, &tf, &scale)) return scale * matern_fine(e + (long long)idx * GEO_FINE_STRIDE, t, tf);
+        if (matern_outer_pos(u, cp.far, &idx, &t, &tf, &scale))
+            return scale * matern_fine(e + (long long)idx * GEO_FINE_STRIDE, t, tf);
     }
     return matern_cov(sqrt(d2) * cp.inv_a, c, cp.tab);
 }

@@ -395,7 +395,8 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
             // every MMA issued so far has completed before TMEM can be freed
             mma_commit(&drain_bar);
             mbar_wait(&drain_bar, 0, tword, 26);
-            if (args.tc_flops && (!SPLIT || blockIdx.x % args.split == 0)) atomicAdd(args.tc_flops, nmma * (unsigned long long)(2 * OZ_BM * OZ_BN * 16));
+            if (args.tc_flops && (!SPLIT || blockIdx.x % args.split == 0))   // (a shared tile counts once)
+                atomicAdd(args.tc_flops, nmma * (unsigned long long)(2 * OZ_BM * OZ_BN * 16));
         }
         __syncwarp();
     } else {
@@ -624,7 +625,8 @@ __global__ void __launch_bounds__(256) k_oz_slice(const double *P, long long ld,
                 hi[i] = (unsigned int)(y >> 28);
                 lead[i] = (unsigned int)(y >> (7 * (S - 1)));
             }
-            unsigned int *o = reinterpret_cast<unsigned int *>(out + ((long long)(r0 + r) * Kp + (c0 + cq) / 16 * 16) * S + cq % 16);
+            const long long at = ((long long)(r0 + r) * Kp + (c0 + cq) / 16 * 16) * S + cq % 16;
+            unsigned int *o = reinterpret_cast<unsigned int *>(out + at);
 #pragma unroll
             for (int t = 0; t < 7; ++t)
                 if (t < S - 1) {
@@ -900,7 +902,8 @@ cudaError_t chol_oz_factor(double *A, long long ld, int N, int nrows, int nb, in
                 cudaSuccess)
                 return r;
             if (n1 >= N) {
-                r = chol64_panel(A, ld, t0, N - t0, N, nrows, st, sync, s, true, nullptr, 0, 0, order);   // last panel: diagonal tile + RHS rows
+                // last panel: diagonal tile + RHS rows
+                r = chol64_panel(A, ld, t0, N - t0, N, nrows, st, sync, s, true, nullptr, 0, 0, order);
                 if (r != cudaSuccess) return r;
                 j0 = t0;
                 continue;

@@ -75,8 +75,9 @@ struct Diag {
     double part[8][TH], rhs[TB], y[TH], e[TH];
 };
 
-// Loads the block and the reciprocals of its pivots (the diagonals of x) and, on request, inverts its triangles, column by column from the last: below the diagonal, minus the inverse
-// found so far times the column of L, over the pivot.  Four warps per triangle share a row's sum.
+// Loads the block and the reciprocals of its pivots (the diagonals of x) and, on request, inverts its triangles,
+// column by column from the last: below the diagonal, minus the inverse found so far times the column of L, over the
+// pivot.  Four warps per triangle share a row's sum.
 __device__ __forceinline__ void load_diag(const double *__restrict__ A, long long ld, int i0, int ib, Diag &d,
                                           bool invert) {
     for (int i = threadIdx.x; i < TB * TB; i += TT) {
