@@ -563,9 +563,7 @@ int geo_covgen(geo_ctx *ctx, const double *locs1_dev, int n1, const double *locs
     if (n1 == 0 || n2 == 0) return GEO_OK;
     // tables of theta: the K_nu ones, then (with enough pairs) the fine ones; closed forms alone cost so little that
     // it takes five times the pairs (one variable of order 1/2: 256 x 256 49 us without, 70 with, 404 x 404 66 and 71)
-    bool closed = true;
-    for (int q = 0; q < cp.p * cp.p; ++q) closed = closed && cp.m[q].kind != 0;
-    const size_t fine = cov_fine_doubles(cp, (closed ? 0.2 : 1.0) * n1 * n2);
+    const size_t fine = cov_fine_doubles(cp, (cov_closed(cp) ? 0.2 : 1.0) * n1 * n2);
     if (!ctx->ctab && (fine || cov_needs_tables(cp))) {
         // (in a capture too: nothing of it goes to the stream)
         cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;

@@ -89,7 +89,7 @@ __global__ void __launch_bounds__(TL *TR) k_covgen_sym_fine(const CovParams cp, 
 template <int P, bool FINE>
 __global__ void __launch_bounds__(TL *TR) k_covgen_rect(const CovParams cp, const double *__restrict__ l1, int n1,
                                                         const double *__restrict__ l2, int n2, double *out,
-                                                        long long ld) {
+                                                        long long ld, bool closed) {
     constexpr int RP = FINE ? RPT : 1;
     const int l = blockIdx.y * TL + (threadIdx.x % TL);
     if (l >= n1) return;
@@ -103,12 +103,22 @@ __global__ void __launch_bounds__(TL *TR) k_covgen_rect(const CovParams cp, cons
         if constexpr (FINE) {
             matern_pair<P>(d2, cp, v);
         } else {
-            double w[GEO_PMAX_DEV * GEO_PMAX_DEV];
-            cov_block(cp, sqrt(d2), w);
+            const double u = d2 * cp.inv_a2;
+            if (closed && u > 0x1p-900 && u < 0x1p900) {
+                // from u = x^2 as the tables' nodes are: x without the rounding of h / a, and the root's put back
+                const double h = sqrt(u), dh = fma(-h, h, u) / (2.0 * h), ex = exp(-h), emx = fma(-ex, dh, ex);
 #pragma unroll
-            for (int i = 0; i < P; ++i)
+                for (int i = 0; i < P; ++i)
 #pragma unroll
-                for (int j = 0; j < P; ++j) v[i * P + j] = w[i * GEO_PMAX_DEV + j];
+                    for (int j = 0; j < P; ++j) v[i * P + j] = matern_cov_e(h, emx, cp.m[i * P + j], nullptr);
+            } else {
+                double w[GEO_PMAX_DEV * GEO_PMAX_DEV];
+                cov_block(cp, sqrt(d2), w);
+#pragma unroll
+                for (int i = 0; i < P; ++i)
+#pragma unroll
+                    for (int j = 0; j < P; ++j) v[i * P + j] = w[i * GEO_PMAX_DEV + j];
+            }
         }
 #pragma unroll
         for (int j = 0; j < P; ++j) {
@@ -202,6 +212,12 @@ bool cov_needs_tables(const CovParams &cp) {
     return false;
 }
 
+bool cov_closed(const CovParams &cp) {
+    for (int q = 0; q < cp.p * cp.p; ++q)
+        if (cp.m[q].kind == 0) return false;
+    return true;
+}
+
 cudaError_t launch_cheb_build(CovParams &cp, double *tab, cudaStream_t s) {
     cp.tab = tab;
     if (!cov_needs_tables(cp)) return cudaSuccess;
@@ -212,7 +228,7 @@ cudaError_t launch_cheb_build(CovParams &cp, double *tab, cudaStream_t s) {
 }
 
 size_t cov_fine_doubles(int p, double pairs) {
-    // with fewer location pairs the tables (10,000 evaluations per C_ij) cost more than they save
+    // with fewer location pairs the tables (11,600 evaluations per C_ij) cost more than they save
     return pairs >= 32768.0 ? (size_t)p * (p + 1) / 2 * GEO_FINE_PER_PAIR : 0;
 }
 
@@ -252,11 +268,12 @@ cudaError_t launch_covgen_rect(const CovParams &cp, const double *l1, int n1, co
     const int per = cp.fine ? TR * RPT : TR;
     dim3 grid((n2 + per - 1) / per, (n1 + TL - 1) / TL);
     KScope ks(GEO_K_COVGEN, s, 0.0, 8.0 * cp.p * (double)n1 * cp.p * (double)n2);
+    const bool closed = cov_closed(cp);
     cov_by_p(cp.p, [&](auto P) {
         if (cp.fine)
-            k_covgen_rect<P.value, true><<<grid, TL * TR, 0, s>>>(cp, l1, n1, l2, n2, out, ld);
+            k_covgen_rect<P.value, true><<<grid, TL * TR, 0, s>>>(cp, l1, n1, l2, n2, out, ld, closed);
         else
-            k_covgen_rect<P.value, false><<<grid, TL * TR, 0, s>>>(cp, l1, n1, l2, n2, out, ld);
+            k_covgen_rect<P.value, false><<<grid, TL * TR, 0, s>>>(cp, l1, n1, l2, n2, out, ld, closed);
     });
     return cudaGetLastError();
 }

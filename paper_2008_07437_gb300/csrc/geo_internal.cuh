@@ -71,6 +71,7 @@ struct KScope {
 // afterwards reads them.  Nothing is launched when theta has no tabulated order.
 cudaError_t launch_cheb_build(CovParams &cp, double *tab, cudaStream_t s);
 bool cov_needs_tables(const CovParams &cp);
+bool cov_closed(const CovParams &cp);   // every order has a closed form (1/2, 3/2, 5/2)
 // Doubles of the fine tables (matern.cuh) of p variables, 0 where the number of location pairs does not pay
 // for them; and their construction on stream s together with the K_nu tables (tab, GEO_TAB_DOUBLES; NULL: only
 // the fine ones), with cp pointed at both.
