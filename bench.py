@@ -114,10 +114,10 @@ KERNEL_NAMES = {"gemm": "k_chol_df (native FP64 Cholesky: products, pivots and s
                       "trailing updates and panel solves)",
                 "sgemm": "k_sgemm_nt (FP32 SIMT diagonal/band and panel updates)",
                 "tcgemm": "k_tc_update (tcgen05 FP16x2 updates beyond the band)",
-                "covgen": "k_covgen_sym (FP64 Matern + Bessel K_nu)"}
+                "covgen": "k_covgen_sym_fine (C_ij from tables of (h / a)^2; k_covgen_sym for the reduced forms)"}
 TLR_KERNEL_NAMES = {"gemm": "k_bgemm (FP64 low-rank updates of the tile column, diagonal tiles)",
                     "tlr": "k_house_qr_col + k_jacobi_svd_cl (FP64 compression of the tiles)",
-                    "covgen": "k_covgen_block (FP64 Matern + Bessel K_nu)"}
+                    "covgen": "k_covgen_block (C_ij from tables of (h / a)^2)"}
 METRIC = "loglik evals/s"
 
 
